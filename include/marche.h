@@ -455,9 +455,9 @@ typedef struct {
   int32_t attention_kernel;      /* MARCHE_ATTENTION_*: AUTO picks by active rows and head_dim                 */
   int32_t attention_tc_min_rows; /* AUTO: tcgen05 attention above this many active rows (head_dim 64; 48)      */
   int32_t two_segment_attention; /* 1: the step uses marche_attention_two_segment instead of K5 + K3           */
-  int32_t gemm_kernel;           /* MARCHE_GEMM_*: AUTO = CTA-pair kernel above 128 rows                       */
+  int32_t gemm_kernel;           /* MARCHE_GEMM_*: AUTO = the kernel with the shorter estimated time           */
   int32_t tail_split;            /* 0 off, 1 cost model, 2 / 4 forced: column slices in a partial last round   */
-  int32_t tile_n;                /* 0 = 256-wide tiles whenever N allows, 128 = narrow tiles                   */
+  int32_t tile_n;                /* CTA-pair kernel: 0 = tile width by estimated time, 128 = narrow tiles      */
   int32_t pdl;                   /* 1: programmatic dependent launch along the kernel chain (process-wide)     */
 } marche_tuning;
 int marche_get_tuning(const marche_ctx* ctx, marche_tuning* out);

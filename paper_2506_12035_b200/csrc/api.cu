@@ -173,14 +173,16 @@ int score_slot(const marche_ctx* ctx, int l) {
   return -1;
 }
 
-// True when the QKV projection of M rows can write K and V into the cache itself (CTA-pair GEMM,
-// whole 256-column tiles per q / K / V range, 32-bit cache offsets): no scatter_kv launch then.
-bool qkv_scatter_fused(const marche_ctx* ctx, int M, int S) {
-  const marche_config& c = ctx->cfg;
-  return ctx->tune.fuse_qkv_scatter && ctx->bf16 && !ctx->tune.two_segment_attention && ctx->tune.tile_n != 128 &&
-         (ctx->tune.gemm_kernel == MARCHE_GEMM_PAIR || (ctx->tune.gemm_kernel == MARCHE_GEMM_AUTO && M > 128)) &&
-         c.width % 256 == 0 &&
-         (long)2 * c.batch * S * c.width < (1L << 31);
+// Which projection kernel an M x N x K projection of a 16-bit context runs on: the CTA-pair kernel or the split-K one.
+bool use_pair(const marche_ctx* ctx, int M, int N, int K) {
+  if (ctx->tune.gemm_kernel != MARCHE_GEMM_AUTO) return ctx->tune.gemm_kernel == MARCHE_GEMM_PAIR;
+  const double wide = gemm_tcgen05_2cta_cost(M, N, K, 256), narrow = gemm_tcgen05_2cta_cost(M, N, K, 128);
+  return gemm_splitk_cost(M, N, K, gemm_splitk_pick(M, N, K)) > (wide < narrow ? wide : narrow);
+}
+
+// True when the QKV projection writes K and V into the cache itself: no scatter_kv launch then.
+bool qkv_scatter_fused(const marche_ctx* ctx) {
+  return ctx->tune.fuse_qkv_scatter && ctx->bf16 && !ctx->tune.two_segment_attention;
 }
 
 int do_linear(marche_ctx* ctx, int cls, const void* a, int lda, int M, const void* w, const float* bias, int N, int K,
@@ -194,14 +196,15 @@ int do_linear(marche_ctx* ctx, int cls, const void* a, int lda, int M, const voi
   // 16-bit contexts run on the tensor cores or not at all
   if (N % 128 || K % 64) return MARCHE_ESHAPE;
   if (lda % 8 || (((uintptr_t)a | (uintptr_t)w | (uintptr_t)out) & 15)) return misaligned(ctx, "projection");
-  const bool pair = ctx->tune.gemm_kernel == MARCHE_GEMM_PAIR || (ctx->tune.gemm_kernel == MARCHE_GEMM_AUTO && M > 128);
+  const bool pair = use_pair(ctx, M, N, K);
   for (int r = 0; r < launches_of(ctx, cls); ++r) {
     if (M > 0) mark(ctx, cls, st);
     if (pair)
       MARCHE_TRY(launch_gemm_tcgen05_2cta(a, lda, M, w, bias, N, K, epi, out, ctx->a_bf16, ctx->status_dev, st,
                                           gemm_tuning(ctx), turn, kv), "gemm_tcgen05_2cta");
     else
-      MARCHE_TRY(launch_gemm_tcgen05(a, lda, M, w, bias, N, K, epi, out, ctx->a_bf16, ctx->status_dev, st), "gemm_tcgen05");
+      MARCHE_TRY(launch_gemm_splitk(a, lda, M, w, bias, N, K, epi, out, ctx->a_bf16, ctx->status_dev, st,
+                                    gemm_splitk_pick(M, N, K), kv), "gemm_splitk");
   }
   return MARCHE_OK;
 }
@@ -307,7 +310,7 @@ int run_blocks(marche_ctx* ctx, int l_begin, int l_end, const float* gather_src,
         MARCHE_TRY(launch_gather_layernorm(ctx->a_kind, x, nA, nullptr, B, nA, D, bw.ln1_g, bw.ln1_b, ctx->eps,
                                            nullptr, bf.u, st), "layernorm1");
     }
-    const bool fused_kv = qkv_scatter_fused(ctx, M, S);
+    const bool fused_kv = qkv_scatter_fused(ctx);
     const KvScatter kvs = {kv_idx, cache_l, nA, S, B, D};
     int rc = do_linear(ctx, MARCHE_KC_GEMM_QKV, bf.u, D, M, bw.w_qkv, bw.b_qkv, 3 * D, D, fused_kv ? 4 : MARCHE_EPI_BIAS,
                        bf.qkv, st, nullptr, fused_kv ? &kvs : nullptr);

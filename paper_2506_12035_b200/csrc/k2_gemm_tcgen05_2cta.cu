@@ -1,5 +1,5 @@
-// K2, 2-CTA flavour: the same projections as k2_gemm_tcgen05.cu with tcgen05.mma
-// cta_group::2.  Two CTAs on neighbouring SMs (a cluster of 2) share one 256 x BN output
+// K2 for many rows: out = epilogue(a * w^T + bias), the QKV, output and MLP projections of the active rows (Algorithm 1
+// lines 5 and 9), with tcgen05.mma cta_group::2.  Two CTAs on neighbouring SMs (a cluster of 2) share one 256 x BN output
 // tile: each CTA loads its own 128 rows of A and HALF of the W tile per K step, the pair's
 // tensor cores read both halves, and each CTA keeps its 128 x BN accumulator in its own
 // TMEM.  Per CTA a ring stage is 32 KB instead of 48 KB for the same MMA work, so the ring
@@ -39,8 +39,10 @@ template <int BN> struct PairCfg {
   static constexpr int STAGE_BYTES = A_BYTES + BH_BYTES;
   static constexpr int STAGES = (BN == 256) ? 5 : 6;
   static constexpr int RING_BYTES = STAGES * STAGE_BYTES;
-  static constexpr int STAGING_BYTES = 8 * 4096;                 // one 32-row x 128-byte box per epilogue warp
-  static constexpr int SMEM_BYTES = RING_BYTES + STAGING_BYTES + 1024 + 256;
+  static constexpr int STAGING_BYTES = 8 * 8192;                 // two 32-row x 128-byte boxes per epilogue warp
+  static constexpr int BIAS_BYTES = 2 * BN * 4;                  // one slot per accumulator
+  static constexpr int SMEM_BYTES = RING_BYTES + STAGING_BYTES + BIAS_BYTES + 256;
+  static_assert(SMEM_BYTES <= 227 * 1024, "shared memory of one CTA");
   static constexpr int TMEM_COLS = 2 * BN;
 };
 
@@ -54,22 +56,21 @@ gemm_tcgen05_2cta_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
                          const KvScatter kv, int tail_split, int a_bf16) {
   using Cfg = PairCfg<BN>;
   constexpr int STAGES = Cfg::STAGES;
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t raw = ptx::smem_u32(smem_raw);
-  const uint32_t base = (raw + 1023u) & ~1023u;
+  extern __shared__ __align__(1024) uint8_t smem_raw[];     // (swizzled tiles; there is no room to align by hand)
+  const uint32_t base = ptx::smem_u32(smem_raw);
   const uint32_t staging = base + Cfg::RING_BYTES;
-  const uint32_t bar_base = staging + Cfg::STAGING_BYTES;
+  const uint32_t bias_base = staging + Cfg::STAGING_BYTES;
+  const uint32_t bar_base = bias_base + Cfg::BIAS_BYTES;
   auto a_tile = [&](int s) { return base + (uint32_t)s * Cfg::STAGE_BYTES; };
   auto w_tile = [&](int s) { return base + (uint32_t)s * Cfg::STAGE_BYTES + A_BYTES; };
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
   auto tfull_bar = [&](int a) { return bar_base + 8u * (2 * STAGES + a); };
   auto tempty_bar = [&](int a) { return bar_base + 8u * (2 * STAGES + 2 + a); };
-  uint8_t* gen_base = smem_raw + (base - raw);
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gen_base + Cfg::RING_BYTES + Cfg::STAGING_BYTES + 8 * (2 * STAGES + 4));
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(gen_base + Cfg::RING_BYTES + Cfg::STAGING_BYTES + 8 * (2 * STAGES + 4) + 8);
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_raw + (bar_base - base) + 8 * (2 * STAGES + 4));
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_raw + (bar_base - base) + 8 * (2 * STAGES + 4) + 8);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = ptx::cluster_ctarank();           // 0 = leader
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   const int n_m2 = (M + 2 * BM - 1) / (2 * BM), n_n = N / BN, n_tiles = n_m2 * n_n, n_kb = K / BK;
@@ -152,28 +153,29 @@ gemm_tcgen05_2cta_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
   // Programmatic dependent launch: everything above overlapped the previous kernel's tail.  The
   // producer additionally fetches the first weight tiles (weights are never written by a kernel)
   // before it waits for the previous kernel; every other thread waits right here.
-  if (!(warp == 0 && lane == 0)) pdl_sync();
+  if (warp != 0) pdl_sync();
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer (both CTAs)
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       ptx::prefetch_tensormap(&tmap_a);
       ptx::prefetch_tensormap(&tmap_w);
       ptx::prefetch_tensormap(&tmap_out);
+      const uint32_t leader_full0 = ptx::mapa(full_bar(0), 0);
       int prefetched = 0;                                  // ring slots whose barrier is armed and W half loaded
       if (n_pieces > 0) {
         int tile, kb0, kb1, n_off, n_w;
         get_piece(0, tile, kb0, kb1, n_off, n_w);
         const int wrow0 = (tile % n_n) * BN + n_off + (int)rank * (n_w / 2);
         for (; prefetched < STAGES && kb0 + prefetched < kb1; ++prefetched) {
-          const uint32_t leader_full = ptx::mapa(full_bar(prefetched), 0);
           if (rank == 0) ptx::mbar_expect_tx(full_bar(prefetched), 2 * Cfg::STAGE_BYTES);
-          ptx::tma_load_2d_pair(w_tile(prefetched), &tmap_w, (kb0 + prefetched) * BK, wrow0, leader_full);
+          ptx::tma_load_2d_pair(w_tile(prefetched), &tmap_w, (kb0 + prefetched) * BK, wrow0, leader_full0 + 8u * prefetched);
         }
       }
       pdl_sync();
-      int it = 0;
       bool ok = true;
+      int s = 0, it = 0;
+      uint32_t phase = 1;                                  // an empty slot's first wait passes at once
       for (int i = 0; i < n_pieces && ok; ++i) {
         int tile, kb0, kb1, n_off, n_w;
         get_piece(i, tile, kb0, kb1, n_off, n_w);
@@ -181,25 +183,28 @@ gemm_tcgen05_2cta_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
         const int row0 = m2 * 2 * BM + (int)rank * BM;                // this CTA's 128 rows of A
         const int wrow0 = n_blk * BN + n_off + (int)rank * (n_w / 2);  // this CTA's half of the W rows of the slice
         for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const int s = it % STAGES;
-          const uint32_t leader_full = ptx::mapa(full_bar(s), 0);
-          if (it < prefetched) {                           // slot armed and W already in flight
-            ptx::tma_load_2d_pair(a_tile(s), &tmap_a, kb * BK, row0, leader_full);
-            continue;
+          if (it >= prefetched) {                          // else: slot armed and W already in flight
+            if (!ptx::mbar_wait(empty_bar(s), phase, abort_flag)) { ok = false; break; }
+            if (rank == 0) ptx::mbar_expect_tx(full_bar(s), 2 * Cfg::STAGE_BYTES);
           }
-          const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
-          if (!ptx::mbar_wait(empty_bar(s), ph ^ 1u, abort_flag)) { ok = false; break; }
-          if (rank == 0) ptx::mbar_expect_tx(full_bar(s), 2 * Cfg::STAGE_BYTES);
-          ptx::tma_load_2d_pair(a_tile(s), &tmap_a, kb * BK, row0, leader_full);
-          ptx::tma_load_2d_pair(w_tile(s), &tmap_w, kb * BK, wrow0, leader_full);
+          ptx::tma_load_2d_pair(a_tile(s), &tmap_a, kb * BK, row0, leader_full0 + 8u * s);
+          if (it >= prefetched) ptx::tma_load_2d_pair(w_tile(s), &tmap_w, kb * BK, wrow0, leader_full0 + 8u * s);
+          if (++s == STAGES) { s = 0; phase ^= 1u; }
         }
       }
       if (!ok) *(volatile int*)status = ST2_PRODUCER;
+    } else {
+      pdl_sync();
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer (leader only)
-    if (lane == 0 && rank == 0) {
-      int it = 0;
+    // Slot, phase and descriptors are stepped and the branch is an elected one: a K block costs 8 instructions or so
+    // per MMA.  Built per MMA inside a lane-0 branch they took 527 cycles a block, whatever the tile's width.
+    if (rank == 0 && ptx::elect_one()) {
+      const uint64_t a_desc0 = ptx::smem_desc_k_sw128(a_tile(0)), w_desc0 = ptx::smem_desc_k_sw128(w_tile(0));
+      uint64_t da = a_desc0, dw = w_desc0;
+      int s = 0;
+      uint32_t phase = 0;
       bool ok = true;
       for (int i = 0; i < n_pieces && ok; ++i) {
         int tile, kb0, kb1, n_off, n_w;
@@ -210,18 +215,16 @@ gemm_tcgen05_2cta_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
         if (!ptx::mbar_wait(tempty_bar(acc), acc_ph ^ 1u, abort_flag)) { ok = false; break; }
         ptx::tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const int s = it % STAGES;
-          const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
-          if (!ptx::mbar_wait(full_bar(s), ph, abort_flag)) { ok = false; break; }
+        for (int kb = kb0; kb < kb1; ++kb) {
+          if (!ptx::mbar_wait(full_bar(s), phase, abort_flag)) { ok = false; break; }
           ptx::tc_fence_after();
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            const uint64_t da = ptx::smem_desc_k_sw128(a_tile(s) + k * 32);
-            const uint64_t dw = ptx::smem_desc_k_sw128(w_tile(s) + k * 32);
-            ptx::umma_f16_pair(d_tmem, da, dw, idesc, (kb > kb0 || k) ? 1u : 0u);
-          }
+          for (int k = 0; k < BK / 16; ++k)
+            ptx::umma_f16_pair(d_tmem, da + 2 * k, dw + 2 * k, idesc, (kb > kb0 || k) ? 1u : 0u);
           ptx::umma_commit_pair(empty_bar(s), 3);           // frees the slot in both CTAs
+          da += Cfg::STAGE_BYTES >> 4;
+          dw += Cfg::STAGE_BYTES >> 4;
+          if (++s == STAGES) { s = 0; phase ^= 1u; da = a_desc0; dw = w_desc0; }
         }
         if (ok) ptx::umma_commit_pair(tfull_bar(acc), 3);   // accumulator complete in both CTAs
       }
@@ -231,6 +234,8 @@ gemm_tcgen05_2cta_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
     // ---------------------------------------------------------------- epilogue (warps 2..9, both CTAs)
     const int quarter = warp & 3;                           // TMEM lanes 32*quarter .. +31
     const int half = (warp - 2) >> 2;                       // which half of the BN columns
+    const uint32_t my_stage = staging + (uint32_t)(warp - 2) * 8192u;
+    int n_box = 0;
     bool ok = true;
     for (int i = 0; i < n_pieces && ok; ++i) {
       int tile, kb0, kb1, n_off, n_w;
@@ -238,11 +243,21 @@ gemm_tcgen05_2cta_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
       const int m2 = tile / n_n, n_blk = tile - m2 * n_n;
       const int acc = i & 1;
       const uint32_t acc_ph = (uint32_t)(i >> 1) & 1u;
+      constexpr int EC = EpiCols<EPI>::value;
+      const int col_tile = n_blk * BN + n_off;              // first output column of this piece
+      // the two warps of a TMEM lane quarter share the piece's n_w columns (a 64-column slice of a
+      // 64-column-box epilogue is handled by the first of them alone)
+      const int hw = n_w / 2 > EC ? n_w / 2 : EC;
+      const int c_begin = half * hw, c_end = (half + 1) * hw < n_w ? (half + 1) * hw : n_w;
+      const float* bias_tile = kb0 == 0 ? bias + col_tile : nullptr;     // the piece with K-block 0 adds the bias
+      const float4 my_bias = epilogue_bias_load(bias_tile ? bias_tile + c_begin : nullptr, c_end - c_begin, lane);
       if (!ptx::mbar_wait(tfull_bar(acc), acc_ph, abort_flag)) { ok = false; break; }
       ptx::tc_fence_after();
+      // (every warp has left the tile before last, so its bias slot is free)
+      const uint32_t bias_s = bias_base + (uint32_t)(acc * BN + c_begin) * 4u;
+      epilogue_bias_store(my_bias, c_end - c_begin, bias_s, lane);
       const int row0 = m2 * 2 * BM + (int)rank * BM + quarter * 32;
       const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN);
-      const uint32_t my_stage = staging + (uint32_t)(warp - 2) * 4096u;
       int* my_turn = turn ? turn + ((size_t)tile * 2 + rank) * 8 + (warp - 2) : nullptr;
       if (row0 < M) {
         if (my_turn && kb0 > 0) {
@@ -259,33 +274,22 @@ gemm_tcgen05_2cta_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
           __syncwarp();
           if (*abort_flag) { ok = false; break; }
         }
-        constexpr int EC = EpiCols<EPI>::value;
-        const int col_tile = n_blk * BN + n_off;                            // first output column of this piece
-        const float* bias_tile = kb0 == 0 ? bias + col_tile : nullptr;     // the piece with K-block 0 adds the bias
-        // the two warps of a TMEM lane quarter share the piece's n_w columns (a 64-column slice of a
-        // 64-column-box epilogue is handled by the first of them alone)
-        const int hw = n_w / 2 > EC ? n_w / 2 : EC;
-        const int c_begin = half * hw, c_end = (half + 1) * hw < n_w ? (half + 1) * hw : n_w;
         if (EPI == 4 && col_tile >= kv.D) {
           // a K or V tile of the fused QKV projection: straight into the cache rows of the active tokens
           const int which = col_tile / kv.D - 1;                            // 0 = K, 1 = V
           const int col0 = col_tile - (which + 1) * kv.D;
           const int grow = row0 + lane;
-          int dst_row = -1;
+          long dst_row = -1;
           if (grow < M) {
             const int b = grow / kv.n;
             const int t = kv.idx ? kv.idx[grow] : grow - b * kv.n;
-            dst_row = ((which * kv.B + b) * kv.S + t) * kv.D + col0;
+            dst_row = (((long)which * kv.B + b) * kv.S + t) * kv.D + col0;
           }
-#pragma unroll 1
-          for (int c0 = c_begin; c0 < c_end; c0 += 64)
-            epilogue_box_scatter(t_row + (uint32_t)c0, bias_tile + c0, (bf16*)kv.cache, dst_row < 0 ? -1 : dst_row + c0,
-                                 my_stage, lane);
+          epilogue_columns<0, true>(t_row, c_begin, c_end, bias_s, &tmap_out, col_tile, row0, my_stage, n_box, lane, false,
+                                    (bf16*)kv.cache, dst_row);
         } else {
-#pragma unroll 1
-          for (int c0 = c_begin; c0 < c_end; c0 += EC)
-            epilogue_box<(EPI == 4) ? 0 : EPI>(t_row + (uint32_t)c0, bias_tile ? bias_tile + c0 : nullptr, &tmap_out,
-                                               col_tile + c0, row0, my_stage, lane, a_bf16 != 0);
+          epilogue_columns<(EPI == 4) ? 0 : EPI, false>(t_row, c_begin, c_end, bias_s, &tmap_out, col_tile, row0, my_stage,
+                                                        n_box, lane, a_bf16 != 0);
         }
         if (my_turn && lane == 0) {
           if (kb0 == 0 && kb1 < n_kb) {
@@ -400,13 +404,27 @@ cudaError_t launch_pair(const CUtensorMap& ta, const CUtensorMap& tw, const CUte
 
 }  // namespace
 
-// Tile width: 256 whenever N allows it.  Measured on B200 at M = 4.3-5.8 k rows, the 128-wide
-// pair tile costs about 0.7x a 256-wide one (1.5x the operand bytes per flop), so it never wins
-// back what it gains in wave balance.  tile_n = 128 overrides (measurement only).
-int gemm_tcgen05_2cta_pick_bn(int M, int N, int tile_n) {
-  (void)M;
-  if (N % 256) return 128;
-  return tile_n == 128 ? 128 : 256;
+// Estimated time of a projection with this kernel in microseconds, for the choice of its tile width and between it and
+// the split-K kernel: a fixed cost (launch gap, first operands, the last tile's epilogue) and the K blocks of the tile
+// rounds at the measured 0.275 us (256 x 256) and 0.205 us (256 x 128) each; from two rounds on the narrow tiles' feed
+// from L2 slows to 0.24 us.  Measured, M x N x K: 700 x 3072 x 1024 9.3 (256) / 8.2 us (128), 2048 x 1024 x 4096 24.1 /
+// 17.7 us, 2624 x 1024 x 4096 26.6 / 23.2 us, 3500 x 1024 x 4096 26.4 / 28.3 us, 5248 x 3072 x 1024 27.7 / 31.8 us.
+double gemm_tcgen05_2cta_cost(int M, int N, int K, int bn) {
+  if (N % bn) return 1e30;
+  const int pairs = device_sm_count() / 2, n_tiles = ((M + 2 * BM - 1) / (2 * BM)) * (N / bn), left = n_tiles % pairs;
+  double rounds = n_tiles / pairs;
+  if (left > 0) {
+    if (K >= 2048 && n_tiles > pairs) rounds += (double)left / pairs;           // stream-K
+    else if (bn == 256 && n_tiles > pairs) rounds += left * 2 <= pairs ? 0.75 : 1.0;   // column slices
+    else rounds += 1.0;
+  }
+  const double kb = bn == 256 ? 0.275 : (rounds > 1.0 ? 0.24 : 0.205);
+  return (bn == 256 ? 5.4 : 4.6) + rounds * (K / BK) * kb;
+}
+
+int gemm_tcgen05_2cta_pick_bn(int M, int N, int K, int tile_n) {
+  if (tile_n == 128) return 128;
+  return gemm_tcgen05_2cta_cost(M, N, K, 256) <= gemm_tcgen05_2cta_cost(M, N, K, 128) ? 256 : 128;
 }
 
 size_t gemm_tcgen05_2cta_turn_bytes(int M, int N) {
@@ -420,14 +438,15 @@ cudaError_t launch_gemm_tcgen05_2cta(const void* a, int lda, int M, const void* 
   if (M == 0) return cudaSuccess;
   KvScatter kv = {nullptr, nullptr, 1, 1, 1, 1 << 30};
   if (epilogue == 4) {
-    // q, K and V column ranges must each be whole tiles, and cache offsets must fit 32 bits
-    if (!kv_scatter || !kv_scatter->cache || N != 3 * kv_scatter->D || kv_scatter->D % 256 ||
-        (long)2 * kv_scatter->B * kv_scatter->S * kv_scatter->D >= (1L << 31) || ((uintptr_t)kv_scatter->cache & 15))
+    // q, K and V column ranges must each be whole tiles
+    if (!kv_scatter || !kv_scatter->cache || N != 3 * kv_scatter->D || kv_scatter->D % 128 ||
+        ((uintptr_t)kv_scatter->cache & 15))
       return cudaErrorInvalidValue;
     kv = *kv_scatter;
   }
   if (N % 128 || K % BK || lda % 8 || ((uintptr_t)a & 15) || ((uintptr_t)w & 15)) return cudaErrorInvalidValue;
-  const int bn = gemm_tcgen05_2cta_pick_bn(M, N, tune.tile_n);
+  const int bn = gemm_tcgen05_2cta_pick_bn(M, N, K, tune.tile_n);
+  if (epilogue == 4 && kv.D % bn) return cudaErrorInvalidValue;
   CUtensorMap ta, tw, to;
   if (!make_map_2d(&ta, a, (uint64_t)M, (uint64_t)K, (uint64_t)lda, BM, !a_bf16)) return cudaErrorInvalidValue;
   if (!make_map_2d(&tw, w, (uint64_t)N, (uint64_t)K, (uint64_t)K, (uint32_t)(bn / 2), !a_bf16)) return cudaErrorInvalidValue;
@@ -437,7 +456,7 @@ cudaError_t launch_gemm_tcgen05_2cta(const void* a, int lda, int M, const void* 
   if (bn == BN_ && epilogue == EPI_)   \
     return launch_pair<BN_, EPI_>(ta, tw, to, M, N, K, bias, status, turn, kv, a_bf16 ? 1 : 0, tune, st);
   MARCHE_GEMM2_CASE(256, 0) MARCHE_GEMM2_CASE(256, 1) MARCHE_GEMM2_CASE(256, 2) MARCHE_GEMM2_CASE(256, 4)
-  MARCHE_GEMM2_CASE(128, 0) MARCHE_GEMM2_CASE(128, 1) MARCHE_GEMM2_CASE(128, 2)
+  MARCHE_GEMM2_CASE(128, 0) MARCHE_GEMM2_CASE(128, 1) MARCHE_GEMM2_CASE(128, 2) MARCHE_GEMM2_CASE(128, 4)
 #undef MARCHE_GEMM2_CASE
   return cudaErrorInvalidValue;
 }

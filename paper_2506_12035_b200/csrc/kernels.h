@@ -59,12 +59,6 @@ cudaError_t launch_topk(const float* partial, int H, float* scores, const uint8_
 cudaError_t launch_gemm_simt(const float* a, int lda, int M, const float* w, const float* bias,
                              int N, int K, int epilogue, float* out, cudaStream_t st);
 
-// K2 (16-bit operands, tcgen05/TMEM fed by TMA).  N % 128 == 0, K % 64 == 0, lda % 8 == 0, 16-byte aligned
-// operands.  a_bf16: both operands (and the GELU epilogue's output) are bf16, otherwise IEEE fp16.
-// `status` is a device-visible int that bounded waits set when they give up.
-cudaError_t launch_gemm_tcgen05(const void* a, int lda, int M, const void* w, const float* bias, int N, int K,
-                                int epilogue, void* out, bool a_bf16, int* status, cudaStream_t st);
-int gemm_tcgen05_pick_bn(int M, int N);
 // Where the K and V columns of a fused QKV projection go (Algorithm 1 line 11 done by the projection's
 // epilogue, epilogue code 4): row r of the GEMM is active token j = r % n of sample b = r / n, its cache row is
 // idx[r] (identity when idx is NULL).  cache is one block's [2][B][S][D] slice (bf16).  Needs N == 3 D,
@@ -75,20 +69,33 @@ struct KvScatter {
   int n, S, B, D;
 };
 
-// Same contract, tcgen05.mma cta_group::2: CTA pairs share 256 x BN tiles (cluster of 2, no multicast).
+// K2 (16-bit operands, tcgen05/TMEM fed by TMA), many rows: tcgen05.mma cta_group::2, CTA pairs share 256 x BN tiles
+// (cluster of 2, no multicast).  N % 128 == 0, K % 64 == 0, lda % 8 == 0, 16-byte aligned operands.  a_bf16: both
+// operands (and the GELU epilogue's output) are bf16, otherwise IEEE fp16.  `status` is a device-visible int that
+// bounded waits set when they give up.
 // `turn`: optional zero-filled device scratch of gemm_tcgen05_2cta_turn_bytes(M, N) bytes; with it the
 // residual epilogue may use stream-K (ordered reduce-adds; the flags are left zero again).
 struct GemmTuning {
   bool stream_k = true;   // residual epilogue: stream-K with ordered reduce-adds where it pays
   int tail_split = 1;     // partial last round of tiles cut into column slices: 0 off, 1 cost model, 2 / 4 forced
-  int tile_n = 0;         // 0: 256-wide tiles whenever N allows; 128 forces the narrow tile
+  int tile_n = 0;         // 0: tile width by estimated time; 128 forces the narrow tile
 };
 cudaError_t launch_gemm_tcgen05_2cta(const void* a, int lda, int M, const void* w, const float* bias, int N, int K,
                                      int epilogue, void* out, bool a_bf16, int* status, cudaStream_t st,
                                      const GemmTuning& tune, int* turn = nullptr,
                                      const KvScatter* kv_scatter = nullptr);
 size_t gemm_tcgen05_2cta_turn_bytes(int M, int N);
-int gemm_tcgen05_2cta_pick_bn(int M, int N, int tile_n);
+int gemm_tcgen05_2cta_pick_bn(int M, int N, int K, int tile_n);
+double gemm_tcgen05_2cta_cost(int M, int N, int K, int bn);   // microseconds, for the choice of a kernel
+
+// K2 for few rows: one CTA per (128 x bn output tile, K slice), the cs slices of a tile reduced through distributed
+// shared memory (a cluster of cs CTAs).  Same operand rules; epilogue 4 takes any D that is a multiple of bn.
+struct SplitKShape { int bn, cs; };
+SplitKShape gemm_splitk_pick(int M, int N, int K);
+double gemm_splitk_cost(int M, int N, int K, SplitKShape shape);   // microseconds, for the choice of a kernel
+cudaError_t launch_gemm_splitk(const void* a, int lda, int M, const void* w, const float* bias, int N, int K, int epilogue,
+                               void* out, bool a_bf16, int* status, cudaStream_t st, SplitKShape shape,
+                               const KvScatter* kv_scatter = nullptr);
 
 // K3 of the fp32 configuration (SIMT): attention of n queries per sample over all S cache rows.
 cudaError_t launch_attention_simt(const float* q, int ld_q, int B, int n, int S, int H, int dh,

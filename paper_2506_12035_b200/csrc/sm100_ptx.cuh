@@ -57,6 +57,44 @@ MARCHE_DEVINL bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_
   }
 }
 
+// The same wait for a barrier that other CTAs of the cluster arrive on after writing to this CTA's shared memory.
+MARCHE_DEVINL bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag,
+                                     long long limit = 2000000000LL) {
+  const long long t0 = clock64();
+  while (true) {
+    uint32_t done;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if (*abort_flag) return false;
+    if (clock64() - t0 > limit) {
+      *abort_flag = 1;
+      return false;
+    }
+  }
+}
+
+// True in exactly one lane of a converged warp.  A branch on it, unlike one on a lane index, tells the compiler that a
+// single thread follows, and it then issues MMAs and copies with uniform operands (375 -> 140 cycles for four MMAs).
+MARCHE_DEVINL bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "elect.sync _|p, 0xffffffff;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(p));
+  return p != 0;
+}
+
 // ---------------------------------------------------------------- TMA (tiled, 2-D / 3-D)
 MARCHE_DEVINL void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
   asm volatile(
@@ -96,6 +134,7 @@ MARCHE_DEVINL void tma_reduce_add_2d(const CUtensorMap* map, int c0, int c1, uin
 }
 MARCHE_DEVINL void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 MARCHE_DEVINL void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+MARCHE_DEVINL void bulk_wait_read_one() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 MARCHE_DEVINL void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 MARCHE_DEVINL void prefetch_tensormap(const CUtensorMap* map) {
@@ -146,6 +185,13 @@ MARCHE_DEVINL void tmem_ld_32x32(uint32_t taddr, uint32_t (&r)[32]) {
       : "memory");
 }
 MARCHE_DEVINL void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// The wait, tied to the registers it makes valid: no use of them can move in front of it.
+MARCHE_DEVINL void tmem_ld_wait(uint32_t (&r)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 32; ++i) asm volatile("" : "+r"(r[i]));
+}
 
 // ---------------------------------------------------------------- 2-CTA (cta_group::2) forms
 MARCHE_DEVINL uint32_t cluster_ctarank() {

@@ -370,6 +370,38 @@ def test_validate_indices():
         assert e.value.code == -5
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "bf16b"])
+@pytest.mark.parametrize("M,N,K", [(1, 128, 4096), (9, 640, 2560), (7, 256, 320), (127, 512, 448), (129, 512, 448),
+                                   (40, 3072, 1024), (128, 1024, 1024), (257, 384, 128), (640, 4096, 1024)])
+def test_linear_few_rows_split_k(dtype, M, N, K):
+    """Row counts at the edges of the A tile, every tile width and cluster size of the split-K kernel, K ranges that do
+    not divide evenly (5, 7, 40 blocks over 4, 4, 8 CTAs).  Products of unit size: |acc + bias| stays below 8, where
+    half a bf16 step is 0.016 (limit 0.02 with the fp32 sum), and an fp32 sum of K terms errs by sqrt(K) 2^-24."""
+    cfg, blocks, m = model_for(dtype, 256, 4, 1024, 68, 2)
+    rng = np.random.default_rng(M + N + K)
+    a = rng.standard_normal((M, K)).astype(np.float32)
+    w = (rng.standard_normal((N, K)) / math.sqrt(K)).astype(np.float32)
+    bias = rng.standard_normal(N).astype(np.float32)
+    acc = orc.linear(quant_a(a, dtype), quant_a(w, dtype), bias.astype(np.float64))
+    assert np.abs(acc).max() < 8.0
+    a_d, w_d, b_d = dev(a, adt(dtype)), dev(w, adt(dtype)), dev(bias)
+    out = torch.full((M + 3, N), 5.0, dtype=tdt(dtype), device="cuda")
+    m.linear(a_d, w_d, b_d, 0, out, M=M)
+    assert max_abs(host(out[:M]), acc) <= 2e-2 and (host(out[M:]) == 5.0).all()
+    res = rng.standard_normal((M, N)).astype(np.float32)
+    first = None
+    for _ in range(2):                                                   # bit-reproducible
+        out = dev(res)
+        m.linear(a_d, w_d, b_d, 1, out)
+        assert max_abs(host(out), acc + res) <= 2e-5
+        assert first is None or torch.equal(out, first)
+        first = out
+    out = torch.zeros(M, N, dtype=adt(dtype), device="cuda")
+    m.linear(a_d, w_d, b_d, 2, out)
+    assert max_abs(host(out), orc.gelu(acc)) <= 2e-2
+    assert m.device_status() == 0
+
+
 @pytest.mark.parametrize("M,N,K", [(4800, 1024, 256), (9000, 768, 128), (5248, 3072, 192), (19100, 256, 128)])
 def test_linear_many_tiles_all_epilogues(M, N, K):
     """Shapes with more output tiles than CTA pairs and a partial last round, where the pair GEMM

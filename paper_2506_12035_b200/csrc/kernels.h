@@ -101,7 +101,6 @@ cudaError_t launch_gemm_splitk(const void* a, int lda, int M, const void* w, con
 cudaError_t launch_attention_simt(const float* q, int ld_q, int B, int n, int S, int H, int dh,
                                   const float* cache_layer, const uint8_t* is_new, float* score_partial,
                                   float* o, cudaStream_t st);
-size_t attention_simt_smem(int S, int dh);
 
 // K3 (bf16 q / cache, TMA-staged K/V tiles, tensor-core QK^T and PV, fused score column sums).
 // head_dim 64 or 80; ld_q even; cache_layer 16-byte aligned.  o is written in the projections'

@@ -579,3 +579,47 @@ def test_attention_single_pass_tcgen05(operand, B, H, S, n):
                 want[:, c], _ = orc.softmax_attention(qq[b][:, c], cc[0, b][:, c], cc[1, b][:, c])
             assert rel_l2(got[b], want) <= 8e-3 and max_abs(got[b], want) <= 3e-2, \
                 "%s b=%d: max-abs %.3g rel-L2 %.3g" % (name, b, max_abs(got[b], want), rel_l2(got[b], want))
+
+
+@pytest.mark.parametrize("M,N,K", [(31, 64, 16), (33, 128, 144), (136, 1024, 256), (136, 256, 1024), (700, 192, 400),
+                                   (1776, 1024, 256), (2100, 640, 272)])
+def test_linear_f32_tiles_and_k_slices(M, N, K):
+    """The fp32 projection kernel: both tile sizes, one to four K slices, ragged rows, K chunks of fewer than 128 and a
+    wider row stride from an unaligned start.  Products of unit size: an fp32 sum of K terms errs by about sqrt(K) 2^-24 < 2e-6."""
+    cfg, blocks, m = model_for("f32", 256, 4, 1024, 68, 2)
+    rng = np.random.default_rng(M + N + K)
+    for lda, skip in ((K, 0), (K + 4, 1)):
+        a = rng.standard_normal((M, lda)).astype(np.float32)
+        w = (rng.standard_normal((N, K)) / math.sqrt(K)).astype(np.float32)
+        bias, res = rng.standard_normal(N).astype(np.float32), rng.standard_normal((M, N)).astype(np.float32)
+        acc = orc.linear(a[:, :K].astype(np.float64), w.astype(np.float64), bias.astype(np.float64))
+        a_d = torch.empty(M * lda + skip, device="cuda")[skip:].copy_(dev(a).view(-1))
+        w_d, b_d = dev(w), dev(bias)
+        for epi, start, want in ((0, np.full((M, N), 5.0, np.float32), acc), (1, res, acc + res), (2, res, orc.gelu(acc))):
+            out = torch.full((M + 3, N), 5.0, device="cuda")
+            out[:M] = dev(start)
+            m.linear(a_d, w_d, b_d, epi, out, M=M, lda=lda)
+            assert max_abs(host(out[:M]), want) <= 1e-5 and (host(out[M:]) == 5.0).all()
+
+
+@pytest.mark.parametrize("B,H,S,dh,n,nG", [(1, 2, 1, 64, 1, 1), (2, 4, 64, 64, 16, 3), (2, 4, 65, 32, 17, 17), (12, 4, 148, 64, 148, 5),
+                                           (1, 2, 2048, 128, 40, 11), (1, 8, 320, 16, 130, 0), (80, 8, 68, 16, 33, 9)])
+def test_attention_f32_query_clusters(B, H, S, dh, n, nG):
+    """The fp32 attention: one to eight CTAs per item, one to many 16-query tiles, ragged keys, both ring depths, scores
+    added over the cluster.  Weights sum to one, so an output errs by a few 2^-24 times the largest value (5)."""
+    cfg, blocks, m = model_for("f32", H * dh, H, 128, S, B)
+    rng = np.random.default_rng(B + S + n)
+    q = (rng.standard_normal((B * n, H * dh)) * 2.0).astype(np.float32)
+    cache = rng.standard_normal((2, B, S, H * dh)).astype(np.float32)
+    flags = np.zeros((B, n), dtype=np.uint8)
+    flags[:, rng.permutation(n)[:nG]] = 1
+    o, partial = torch.zeros(B * n, H * dh, device="cuda"), torch.full((B, H, S), -1.0, device="cuda")
+    m.attention(dev(q), H * dh, n, dev(cache), dev(flags), partial, o)
+    got_o, got_p = host(o).reshape(B, n, H * dh), host(partial)
+    for b in sorted({0, B // 2, B - 1}):
+        for h in range(H):
+            c = slice(h * dh, (h + 1) * dh)
+            z, p = orc.softmax_attention(q[b * n:(b + 1) * n, c].astype(np.float64), cache[0, b][:, c].astype(np.float64),
+                                         cache[1, b][:, c].astype(np.float64))
+            assert max_abs(got_o[b][:, c], z) <= 2e-5
+            assert max_abs(got_p[b, h], p[flags[b].astype(bool)].sum(axis=0)) <= 1e-5

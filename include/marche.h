@@ -447,7 +447,8 @@ int marche_attention_two_segment(marche_ctx* ctx, const void* qkv, int ld, int n
  * pin them to the same results.  None of them changes what is computed, only which kernel does it;
  * `pdl` is process-wide (it is a property of how kernels are launched). */
 enum { MARCHE_ATTENTION_AUTO = 0, MARCHE_ATTENTION_MMA = 1, MARCHE_ATTENTION_TCGEN05 = 2,
-       MARCHE_ATTENTION_TCGEN05_TWO_PASS = 3 /* the two-pass tcgen05 kernel also where no scores are taken */ };
+       MARCHE_ATTENTION_TCGEN05_TWO_PASS = 3 /* the two-pass tcgen05 kernel also where no scores are taken */,
+       MARCHE_ATTENTION_SPLIT = 4 /* keys split over a cluster, wherever it fits (at most 64 rows, no scores) */ };
 enum { MARCHE_GEMM_AUTO = 0, MARCHE_GEMM_SINGLE = 1, MARCHE_GEMM_PAIR = 2 };
 typedef struct {
   int32_t stream_k;              /* 1: fc2-sized residual projections use stream-K with ordered reduce-adds   */

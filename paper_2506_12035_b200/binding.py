@@ -17,7 +17,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libmarche.so")
 
 MARCHE_F32, MARCHE_BF16, MARCHE_BF16_F16OP = 0, 1, 2
-ATTENTION_AUTO, ATTENTION_MMA, ATTENTION_TCGEN05, ATTENTION_TCGEN05_TWO_PASS = 0, 1, 2, 3
+ATTENTION_AUTO, ATTENTION_MMA, ATTENTION_TCGEN05, ATTENTION_TCGEN05_TWO_PASS, ATTENTION_SPLIT = 0, 1, 2, 3, 4
 GEMM_AUTO, GEMM_SINGLE, GEMM_PAIR = 0, 1, 2
 EPI_BIAS, EPI_BIAS_RESIDUAL, EPI_BIAS_GELU = 0, 1, 2
 ERRORS = {-1: "EINVAL", -2: "ESHAPE", -3: "EWORKSPACE", -4: "ECACHE", -5: "EINDEX", -6: "ECUDA", -7: "ETIMEOUT"}

@@ -235,8 +235,17 @@ int do_attention(marche_ctx* ctx, const void* q, int ld_q, int n, const void* ca
   const bool tc5 = c.head_dim == 64 && ld_q % 8 == 0 && ((uintptr_t)q & 15) == 0 &&
                    (ak == MARCHE_ATTENTION_TCGEN05 || ak == MARCHE_ATTENTION_TCGEN05_TWO_PASS ||
                     (ak == MARCHE_ATTENTION_AUTO && n > tc_min));
+  // few items (or few key tiles): all tiles in flight, split over a cluster and over warps; measured beside the rule
+  const int items = c.batch * c.n_heads;
+  int split_cs, split_nk;
+  const bool split = !is_new && (ak == MARCHE_ATTENTION_SPLIT
+                                     ? attention_split_plan(n, S, c.head_dim, items, &split_cs, &split_nk)
+                                     : ak == MARCHE_ATTENTION_AUTO && attention_split_wins(n, S, c.head_dim, items));
+  if (split)
+    MARCHE_TRY(launch_attention_split(q, ld_q, c.batch, n, S, c.n_heads, c.head_dim, cache_layer, o, ctx->a_bf16,
+                                      ctx->status_dev, st), "attention_split");
   // plain flavour: single-pass streaming kernel; the relevance scores need final weights, i.e. two passes
-  if (tc5 && !is_new && ak != MARCHE_ATTENTION_TCGEN05_TWO_PASS)
+  else if (tc5 && !is_new && ak != MARCHE_ATTENTION_TCGEN05_TWO_PASS)
     MARCHE_TRY(launch_attention_tc_stream(q, ld_q, c.batch, n, S, c.n_heads, c.head_dim, cache_layer, o, ctx->a_bf16,
                                           ctx->status_dev, st), "attention_tc_stream");
   else if (tc5)
@@ -980,7 +989,7 @@ int marche_get_tuning(const marche_ctx* ctx, marche_tuning* out) {
 
 int marche_set_tuning(marche_ctx* ctx, const marche_tuning* t) {
   if (!ctx || !t) return MARCHE_EINVAL;
-  if (t->attention_kernel < MARCHE_ATTENTION_AUTO || t->attention_kernel > MARCHE_ATTENTION_TCGEN05_TWO_PASS) return MARCHE_EINVAL;
+  if (t->attention_kernel < MARCHE_ATTENTION_AUTO || t->attention_kernel > MARCHE_ATTENTION_SPLIT) return MARCHE_EINVAL;
   if (t->gemm_kernel < MARCHE_GEMM_AUTO || t->gemm_kernel > MARCHE_GEMM_PAIR) return MARCHE_EINVAL;
   if (t->tail_split != 0 && t->tail_split != 1 && t->tail_split != 2 && t->tail_split != 4) return MARCHE_EINVAL;
   if (t->tile_n != 0 && t->tile_n != 128) return MARCHE_EINVAL;

@@ -39,9 +39,6 @@ enum { STK_PRODUCER = 0x61, STK_MMA = 0x62, STK_EPILOGUE = 0x63 };
 
 MARCHE_DEVINL void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 MARCHE_DEVINL void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
-MARCHE_DEVINL void tma_prefetch_l2_2d(const CUtensorMap* map, int c0, int c1) {
-  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(c0), "r"(c1) : "memory");
-}
 MARCHE_DEVINL void st_cluster_v4(uint32_t addr, const uint32_t* v) {
   asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3])
                : "memory");
@@ -126,7 +123,7 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
       ptx::mbar_expect_tx(full_bar(loaded), a_bytes + W_BYTES);
       ptx::tma_load_2d(w_base + loaded * W_BYTES, &tmap_w, (kb0 + loaded) * BK, n_blk * BN, full_bar(loaded));
     }
-    for (int i = loaded; i < n_it; ++i) tma_prefetch_l2_2d(&tmap_w, (kb0 + i) * BK, n_blk * BN);
+    for (int i = loaded; i < n_it; ++i) ptx::tma_prefetch_l2_2d(&tmap_w, (kb0 + i) * BK, n_blk * BN);
   }
   __syncwarp();
   if (CS > 1) cluster_arrive();                            // our barriers exist

@@ -114,6 +114,13 @@ cudaError_t launch_attention_mma(const void* q, int ld_q, int B, int n, int S, i
 cudaError_t launch_attention_mma_persist(const void* q, int ld_q, int B, int n, int S, int H, int dh,
                                          const void* cache_layer, void* o, bool o_bf16, int* status, cudaStream_t st);
 
+// K3 for few items and n <= 64 rows without scores: all key tiles of an item in flight, split over a cluster of up to
+// eight CTAs and over warps.  ld_q even; q 4-byte, cache_layer and o 16-byte aligned.
+bool attention_split_plan(int n, int S, int dh, int items, int* cs, int* nk);
+bool attention_split_wins(int n, int S, int dh, int items);
+cudaError_t launch_attention_split(const void* q, int ld_q, int B, int n, int S, int H, int dh, const void* cache_layer,
+                                   void* o, bool o_bf16, int* status, cudaStream_t st);
+
 // K3 on tcgen05 (head_dim 64 only): S = Q K^T and O = P V as tcgen05.mma with TMEM accumulators.
 // ld_q % 8 == 0; q and cache_layer 16-byte aligned.
 cudaError_t launch_attention_tcgen05(const void* q, int ld_q, int B, int n, int S, int H, int dh,

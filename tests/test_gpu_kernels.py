@@ -623,3 +623,37 @@ def test_attention_f32_query_clusters(B, H, S, dh, n, nG):
                                          cache[1, b][:, c].astype(np.float64))
             assert max_abs(got_o[b][:, c], z) <= 2e-5
             assert max_abs(got_p[b, h], p[flags[b].astype(bool)].sum(axis=0)) <= 1e-5
+
+
+@pytest.mark.parametrize("dh,H", [(64, 4), (80, 8)])
+@pytest.mark.parametrize("B,S,n", [(1, 1, 1), (2, 64, 16), (1, 65, 17), (2, 320, 41), (2, 320, 64), (1, 1088, 48), (1, 2048, 33),
+                                   (3, 577, 5)])
+def test_attention_keys_split_over_a_cluster(dh, H, B, S, n):
+    """One to eight CTAs per item (one without a cluster), one to four key tiles per CTA and one to four query warps,
+    logits that grow along the keys (the ranks' maxima far apart) and one-hot rows; bit-reproducible."""
+    from paper_2506_12035_b200 import binding
+    D = H * dh
+    cfg, blocks, m = model_for("bf16", D, H, 128, S, B)
+    m.set_tuning(attention_kernel=binding.ATTENTION_SPLIT)
+    rng = np.random.default_rng(B + S + n + dh)
+    cache = rng.standard_normal((2, B, S, D)).astype(np.float32)
+    cache_ramp = cache.copy()
+    cache_ramp[0, :, :, 0::dh] = np.linspace(0.0, 40.0, S, dtype=np.float32)[None, :, None]
+    q = (rng.standard_normal((B * n, D)) * 3.0).astype(np.float32)
+    q_ramp = q.copy()
+    q_ramp[:, 0::dh] = 16.0
+    q_hot = np.stack([quant(cache, "bf16")[0, b, rng.integers(0, S, size=n)] for b in range(B)]).reshape(B * n, D).astype(np.float32) * 64.0
+    for qq, cc in ((q, cache), (q_ramp, cache_ramp), (q_hot, cache)):
+        outs = []
+        for _ in range(2):
+            o = torch.zeros(B * n, D, dtype=torch.float16, device="cuda")
+            m.attention(dev(qq, torch.bfloat16), D, n, dev(cc, torch.bfloat16), None, None, o)
+            outs.append(o)
+        assert torch.equal(outs[0], outs[1]) and m.device_status() == 0
+        qq, cc = quant(qq, "bf16"), quant(cc, "bf16")
+        want = np.zeros((B * n, D))
+        for b in range(B):
+            for h in range(H):
+                c = slice(h * dh, (h + 1) * dh)
+                want[b * n:(b + 1) * n, c], _ = orc.softmax_attention(qq[b * n:(b + 1) * n, c], cc[0, b][:, c], cc[1, b][:, c])
+        assert rel_l2(host(outs[0]), want) <= 8e-3 and max_abs(host(outs[0]), want) <= 3e-2

@@ -180,6 +180,13 @@ bool use_pair(const marche_ctx* ctx, int M, int N, int K) {
   return gemm_splitk_cost(M, N, K, gemm_splitk_pick(M, N, K)) > (wide < narrow ? wide : narrow);
 }
 
+// True when a projection of a step on M rows may run stream-K, whose turn flags in the workspace have to start at zero.
+// (Clearing them costs a few microseconds of a step on few rows: the kernels on either side of a memset do not overlap.)
+bool needs_turn(const marche_ctx* ctx, int M) {
+  const int D = ctx->cfg.width, F = ctx->cfg.mlp_dim;
+  return ctx->bf16 && ctx->tune.stream_k && ((F >= 2048 && use_pair(ctx, M, D, F)) || (D >= 2048 && use_pair(ctx, M, D, D)));
+}
+
 // True when the QKV projection writes K and V into the cache itself: no scatter_kv launch then.
 bool qkv_scatter_fused(const marche_ctx* ctx) {
   return ctx->tune.fuse_qkv_scatter && ctx->bf16 && !ctx->tune.two_segment_attention;
@@ -376,7 +383,7 @@ int run_stack(marche_ctx* ctx, const float* hidden, void* kv_cache, const int32_
   const StackBufs bf = carve(workspace, w);
 
   // the workspace is scratch between calls: make sure the stream-K turn flags start at zero
-  if (ctx->bf16 && ctx->tune.stream_k) MARCHE_TRY(cudaMemsetAsync(bf.turn, 0, w.turn_bytes, st), "memset");
+  if (needs_turn(ctx, B * nA)) MARCHE_TRY(cudaMemsetAsync(bf.turn, 0, w.turn_bytes, st), "memset");
   mark(ctx, MARCHE_KC_FLAGS, st);
   MARCHE_TRY(launch_step_flags(active_idx, nA, new_idx, n_new, excl_idx, n_excl, B, S, bf.is_new, bf.cand, st), "flags");
   const int rc = run_blocks(ctx, 0, L, hidden, S, active_idx, nA, bf.x, bf, kv_cache, bf.is_new, st);
@@ -406,7 +413,7 @@ int run_in_step(marche_ctx* ctx, const float* hidden, void* kv_cache, const int3
   if (ws_bytes < w.total) return MARCHE_EWORKSPACE;
   const StackBufs bf = carve(workspace, w);
   const int nA = n_new + n_prev + k;
-  if (ctx->bf16 && ctx->tune.stream_k) MARCHE_TRY(cudaMemsetAsync(bf.turn, 0, w.turn_bytes, st), "memset");
+  if (needs_turn(ctx, B * S) || needs_turn(ctx, B * nA)) MARCHE_TRY(cudaMemsetAsync(bf.turn, 0, w.turn_bytes, st), "memset");
 
   // phase 1: every token; generating rows flagged for the scores; candidates = all \ (new u prev)
   mark(ctx, MARCHE_KC_FLAGS, st);
@@ -449,7 +456,7 @@ int run_mar(marche_ctx* ctx, bool full_decoder, const float* tokens, const int32
   if (ws_bytes < w.total) return MARCHE_EWORKSPACE;
   const StackBufs bf = carve(workspace, w);
   const marche_mar_weights& mw = ctx->mar;
-  if (ctx->bf16 && ctx->tune.stream_k) MARCHE_TRY(cudaMemsetAsync(bf.turn, 0, w.turn_bytes, st), "memset");
+  if (needs_turn(ctx, B * S) || needs_turn(ctx, B * n_known) || needs_turn(ctx, B * nA)) MARCHE_TRY(cudaMemsetAsync(bf.turn, 0, w.turn_bytes, st), "memset");
 
   mark(ctx, MARCHE_KC_FLAGS, st);
   MARCHE_TRY(launch_step_flags(nullptr, S, new_idx, n_new, prev_idx, n_prev, B, S, bf.is_new, bf.cand, st), "flags");

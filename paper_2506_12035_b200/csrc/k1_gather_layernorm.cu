@@ -8,21 +8,33 @@
 #include "common.cuh"
 #include "kernels.h"
 #include "launch_pdl.h"
+#include "tma_host.h"
 
 namespace marche {
 
-constexpr int kLnWarps = 8;
+constexpr int kLnWarps = 8, kLnFewWarps = 4;
 
-template <typename TOut, int NV>
-__global__ void __launch_bounds__(kLnWarps * 32)
+// FEW: at most kLnFewWarps rows per SM.  Then a launch is one chain of latencies (1.0 us of it, plus 1.4 us of hand-overs),
+// so gamma and beta, which no kernel writes, are fetched ahead of the dependency wait (their first touch comes from HBM)
+// and a CTA has only as many warps as it takes to give every SM a row.  With many rows the 16 registers per 512 bytes of
+// row that this costs would halve the warps in flight, which is what hides the latency there.
+template <typename TOut, int NV, bool FEW>
+__global__ void __launch_bounds__((FEW ? kLnFewWarps : kLnWarps) * 32)
 gather_layernorm_kernel(const float* __restrict__ src, int src_rows, const int32_t* __restrict__ idx,
                         int n, int total_rows, const float* __restrict__ gamma,
                         const float* __restrict__ beta, float eps, float* __restrict__ x_out,
                         TOut* __restrict__ u_out, const int32_t* __restrict__ out_idx, int out_rows) {
   constexpr int D = NV * 128;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long r = (long)blockIdx.x * kLnWarps + warp;
+  const long r = (long)blockIdx.x * (blockDim.x >> 5) + warp;
   if (r >= total_rows) return;
+  const float4* g4 = reinterpret_cast<const float4*>(gamma);
+  const float4* b4 = reinterpret_cast<const float4*>(beta);
+  float4 gv[FEW ? NV : 1], bv[FEW ? NV : 1];
+  if (FEW) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) { gv[FEW ? i : 0] = __ldg(g4 + i * 32 + lane); bv[FEW ? i : 0] = __ldg(b4 + i * 32 + lane); }
+  }
   pdl_sync();
   const int b = (int)(r / n), j = (int)(r - (long)b * n);
   const int srow = idx ? idx[r] : j;
@@ -49,14 +61,12 @@ gather_layernorm_kernel(const float* __restrict__ src, int src_rows, const int32
 #pragma unroll
     for (int i = 0; i < NV; ++i) xo[i * 32 + lane] = v[i];
   }
-  const float4* g4 = reinterpret_cast<const float4*>(gamma);
-  const float4* b4 = reinterpret_cast<const float4*>(beta);
   // out_rows > 0: the normalised row goes to row out_idx[r] (identity when NULL) of a [B][out_rows][D] array
   const long orow = out_rows > 0 ? (long)b * out_rows + (out_idx ? out_idx[r] : j) : r;
   TOut* uo = u_out + orow * D;
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
-    const float4 g = __ldg(g4 + i * 32 + lane), be = __ldg(b4 + i * 32 + lane);
+    const float4 g = FEW ? gv[FEW ? i : 0] : __ldg(g4 + i * 32 + lane), be = FEW ? bv[FEW ? i : 0] : __ldg(b4 + i * 32 + lane);
     store4(uo + (i * 32 + lane) * 4,
            (v[i].x - mean) * rstd * g.x + be.x, (v[i].y - mean) * rstd * g.y + be.y,
            (v[i].z - mean) * rstd * g.z + be.z, (v[i].w - mean) * rstd * g.w + be.w);
@@ -69,12 +79,17 @@ static cudaError_t launch_ln_t(const float* src, int src_rows, const int32_t* id
                                cudaStream_t st, const int32_t* out_idx, int out_rows) {
   const long rows = (long)B * n;
   if (rows == 0) return cudaSuccess;
-  const unsigned grid = (unsigned)((rows + kLnWarps - 1) / kLnWarps);
+  const int sms = device_sm_count();
+  const bool few = rows <= (long)kLnFewWarps * sms;
+  const int warps = few ? (int)((rows + sms - 1) / sms) : kLnWarps;
+  const unsigned grid = (unsigned)((rows + warps - 1) / warps);
   cudaError_t err = cudaSuccess;
 #define MARCHE_LN_CASE(NV_)                                                                          \
   case NV_:                                                                                          \
-    err = launch_pdl(gather_layernorm_kernel<TOut, NV_>, dim3(grid), dim3(kLnWarps * 32), 0, st, src, src_rows, \
-                     idx, n, (int)rows, gamma, beta, eps, x_out, u_out, out_idx, out_rows);          \
+    err = few ? launch_pdl(gather_layernorm_kernel<TOut, NV_, true>, dim3(grid), dim3(warps * 32), 0, st, src, src_rows, \
+                           idx, n, (int)rows, gamma, beta, eps, x_out, u_out, out_idx, out_rows)     \
+              : launch_pdl(gather_layernorm_kernel<TOut, NV_, false>, dim3(grid), dim3(warps * 32), 0, st, src, src_rows, \
+                           idx, n, (int)rows, gamma, beta, eps, x_out, u_out, out_idx, out_rows);    \
     break;
   switch (D / 128) {
     MARCHE_LN_CASE(1) MARCHE_LN_CASE(2) MARCHE_LN_CASE(3) MARCHE_LN_CASE(4) MARCHE_LN_CASE(5)

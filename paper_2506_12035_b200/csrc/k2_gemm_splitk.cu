@@ -131,6 +131,12 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  constexpr int NQ = CS > 1 ? OWN / 4 : 1;                 // float4s that a thread finishes of its row
+  float4 bv[NQ];                                           // (the bias, too, is never written)
+  if (CS > 1 && warp >= 2) {
+#pragma unroll
+    for (int j = 0; j < NQ; ++j) bv[j] = __ldg(reinterpret_cast<const float4*>(bias + n_blk * BN + rank * OWN) + j);
+  }
   pdl_sync();                                              // everything above overlapped the previous kernel's tail
 
   bool ok = true;
@@ -213,37 +219,45 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
         if (lane == 0) ptx::bulk_wait_read_all();
       }
     } else {
-      // what the reduction will need is fetched under the main loop: bias, and (residual) the old values
-      constexpr int OB = EPI == 1 ? 4 : 2, NQ = OWN / 4;
+      // what the residual sum will need is fetched under the main loop: the old values
+      constexpr int OB = EPI == 1 ? 4 : 2;
       uint8_t* dst = !valid ? nullptr
                      : to_cache ? reinterpret_cast<uint8_t*>(kv.cache) + (kv_row * kv.D + kv_col) * OB
                                 : reinterpret_cast<uint8_t*>(out) + ((size_t)row * N + col0) * OB;
-      float4 res[NQ], bv[NQ];
+      float4 res[NQ];
 #pragma unroll
-      for (int j = 0; j < NQ; ++j) {
-        bv[j] = __ldg(reinterpret_cast<const float4*>(bias + col0) + j);
+      for (int j = 0; j < NQ; ++j)
         res[j] = EPI == 1 && valid ? reinterpret_cast<const float4*>(dst)[j] : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
       cluster_wait();                                      // every CTA of the cluster has started
       ok = ptx::mbar_wait(tfull_bar, 0, abort_flag);
       if (ok) {
         ptx::tc_fence_after();
         // ---- partial sums to the owners of the columns (consecutive lanes write consecutive 16 bytes)
         const uint32_t slot = recv + (uint32_t)(rank * NQ * BM + r) * 16u;
+        uint32_t v[BN / 32][32];
 #pragma unroll
-        for (int c0 = 0; c0 < BN; c0 += 32) {
-          uint32_t v[32];
-          ptx::tmem_ld_32x32(t_row + (uint32_t)c0, v);
-          ptx::tmem_ld_wait();
-          if (valid) {
+        for (int c = 0; c < BN / 32; ++c) ptx::tmem_ld_32x32(t_row + 32u * c, v[c]);
+#pragma unroll
+        for (int c = 0; c < BN / 32; ++c) ptx::tmem_ld_wait(v[c]);
+        ptx::tc_fence_before();
+        if (valid) {
+#pragma unroll
+          for (int c = 0; c < BN / 32; ++c)
 #pragma unroll
             for (int q = 0; q < 8; ++q)
-              st_cluster_v4(ptx::mapa(slot, (uint32_t)((c0 + 4 * q) / OWN)) + (uint32_t)((c0 + 4 * q) % OWN) * (BM * 4u),
-                            v + 4 * q);
-          }
+              st_cluster_v4(ptx::mapa(slot, (uint32_t)((32 * c + 4 * q) / OWN)) + (uint32_t)((32 * c + 4 * q) % OWN) * (BM * 4u),
+                            v[c] + 4 * q);
         }
         __syncwarp();
         if (lane < CS) ptx::mbar_arrive_cluster(ptx::mapa(recv_bar, (uint32_t)lane));
+      }
+      // tensor memory is given back while the other CTAs' partial sums arrive, not after them
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      if (warp == 2) {
+        ptx::tc_fence_after();
+        ptx::tmem_dealloc(tmem_base, BN);
+      }
+      if (ok) {
         // ---- the sum over the cluster, in rank order
         ok = ptx::mbar_wait_cluster(recv_bar, 0, abort_flag);
         if (ok && valid) {
@@ -266,7 +280,7 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
   if (CS > 1 && warp < 2) cluster_wait();
   ptx::tc_fence_before();
   __syncthreads();
-  if (warp == 2) {
+  if (CS == 1 && warp == 2) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem_base, BN);
   }

@@ -12,9 +12,9 @@
 //                      predecessor's tail; only the A tiles wait for it.
 //   warp 1 (one lane)  issues tcgen05.mma (M 128, N BN, K 16), accumulator in BN columns of tensor memory
 //   warps 2-5          partial sums to the owners, reduction, epilogue; one thread per output row
-// A CTA takes at most 112 KB of shared memory and BN columns of tensor memory, so the next kernel's CTAs become
-// resident beside it and run their set-up early (programmatic dependent launch).  A tiles are only as high as the
-// rows that exist (rounded up to 8): the MMA's remaining rows read whatever the ring holds and are never stored.
+// A CTA takes at most 112 KB of shared memory (but for clusters on 128-column tiles) and BN columns of tensor memory, so
+// the next kernel's CTAs become resident beside it and run their set-up early (programmatic dependent launch).  A tiles are
+// only as high as their share of the rows: the MMA's remaining rows read whatever the ring holds and are never stored.
 // All waits are bounded; a CTA that gave up stays until its cluster has left, so nobody writes to a CTA that is gone.
 #include <cuda.h>
 
@@ -35,6 +35,7 @@ constexpr int BK = 64;
 constexpr int kThreads = 192;
 constexpr int kMaxStages = 8;
 constexpr int kSmemBudget = 112 * 1024;   // two CTAs per SM
+constexpr int kSmemBudgetWide = 224 * 1024;   // one: a 128-column tile's partial sums take 64 KB
 enum { STK_PRODUCER = 0x61, STK_MMA = 0x62, STK_EPILOGUE = 0x63 };
 
 MARCHE_DEVINL void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
@@ -71,7 +72,7 @@ MARCHE_DEVINL void finish4(float4 v, void* dst, float4 res, bool a_bf16) {
 
 // Grid: x = CS * (n_m * n_n) CTAs, clusters of CS consecutive ones share an output tile and split its K blocks.
 template <int BN, int CS, int EPI>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, BN == 128 && CS > 1 ? 1 : 2)
 gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w,
                    const __grid_constant__ CUtensorMap tmap_out, int M, int N, int K, int a_rows, int n_stages,
                    int ring_bytes, const float* __restrict__ bias, void* __restrict__ out,
@@ -151,7 +152,7 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
           ptx::mbar_expect_tx(full_bar(s), a_bytes + W_BYTES);
           ptx::tma_load_2d(w_base + s * W_BYTES, &tmap_w, x, n_blk * BN, full_bar(s));
         }
-        ptx::tma_load_2d(base + s * a_bytes, &tmap_a, x, m_blk * BM, full_bar(s));
+        ptx::tma_load_2d(base + s * a_bytes, &tmap_a, x, m_blk * a_rows, full_bar(s));
         if (++s == n_stages) { s = 0; phase ^= 1u; }
       }
       if (!ok) {
@@ -189,8 +190,8 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
   } else {
     // ---------------------------------------------------------------- epilogue (warps 2..5)
     const int quarter = warp & 3;
-    const int r = quarter * 32 + lane, row = m_blk * BM + r;
-    const bool valid = row < M;
+    const int r = quarter * 32 + lane, row = m_blk * a_rows + r;
+    const bool valid = r < a_rows && row < M;
     const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16);
     const int col0 = n_blk * BN + rank * OWN;              // first output column this CTA finishes
     const bool to_cache = EPI == 4 && col0 >= kv.D;        // a K or V column: into the cache row of the token
@@ -208,13 +209,14 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
       ptx::tc_fence_after();
       // every MMA has completed, so the ring is free: it becomes the warps' staging boxes
       const uint32_t stage = base + (uint32_t)(warp - 2) * 8192u;
-      if (ok && m_blk * BM + quarter * 32 < M) {
+      const int row0 = m_blk * a_rows + quarter * 32;
+      if (ok && quarter * 32 < a_rows && row0 < M) {
         int n_box = 0;
         if (to_cache)
-          epilogue_columns<0, true>(t_row, 0, BN, recv, &tmap_out, col0, m_blk * BM + quarter * 32, stage, n_box, lane,
+          epilogue_columns<0, true>(t_row, 0, BN, recv, &tmap_out, col0, row0, stage, n_box, lane,
                                     false, (bf16*)kv.cache, kv_row < 0 ? -1L : kv_row * kv.D + kv_col);
         else
-          epilogue_columns<EPI == 4 ? 0 : EPI, false>(t_row, 0, BN, recv, &tmap_out, col0, m_blk * BM + quarter * 32,
+          epilogue_columns<EPI == 4 ? 0 : EPI, false>(t_row, 0, BN, recv, &tmap_out, col0, row0,
                                                       stage, n_box, lane, a_bf16 != 0);
         if (lane == 0) ptx::bulk_wait_read_all();
       }
@@ -297,7 +299,8 @@ cudaError_t launch_one(const CUtensorMap& ta, const CUtensorMap& tw, const CUten
   const int fixed = 1024 + 256 + (CS > 1 ? BM * BN * 4 : BN * 4);
   const int stage = a_rows * BK * 2 + BN * BK * 2;
   const int n_it = (K / BK + CS - 1) / CS;
-  int stages = (kSmemBudget - fixed) / stage;
+  constexpr int budget = BN == 128 && CS > 1 ? kSmemBudgetWide : kSmemBudget;
+  int stages = (budget - fixed) / stage;
   if (stages > kMaxStages) stages = kMaxStages;
   if (stages > n_it) stages = n_it;
   // The MMA reads 128 rows of A from the last slot on, whatever they hold, and without a cluster the ring ends as the
@@ -308,7 +311,7 @@ cudaError_t launch_one(const CUtensorMap& ta, const CUtensorMap& tw, const CUten
   if (CS == 1 && ring < 32768) ring = 32768;
   const size_t smem = fixed + ring;
   static size_t smem_set[kMaxDevices] = {};
-  cudaError_t e = ensure_dynamic_smem(gemm_splitk_kernel<BN, CS, EPI>, (size_t)kSmemBudget, smem_set);
+  cudaError_t e = ensure_dynamic_smem(gemm_splitk_kernel<BN, CS, EPI>, (size_t)budget, smem_set);
   if (e != cudaSuccess) return e;
   return launch_pdl_cluster(gemm_splitk_kernel<BN, CS, EPI>, dim3(n_tiles * CS), dim3(kThreads), smem, CS, st, ta, tw, to, M, N,
                             K, a_rows, stages, (int)ring, bias, out, kv, a_bf16, status);
@@ -316,26 +319,36 @@ cudaError_t launch_one(const CUtensorMap& ta, const CUtensorMap& tw, const CUten
 
 }  // namespace
 
-// Estimated time of one shape in microseconds: a fixed cost, the K loop (a 64-wide block costs about 0.14 us of
-// hand-overs or its bytes at the 114 KB/us that a 128 x BN tile is fed with, whichever is more), what two CTAs on one
-// SM take from each other, and the exchange of partial sums (27 KB/us of distributed shared memory).
+// Rows of A per tile: the row blocks share the rows evenly, so that the last one is not a tile of padding that costs as
+// much to feed as the others.  A whole number of 8-row swizzle atoms, or of 32-row store boxes where TMA stores.
+static int rows_per_tile(int M, int cs) {
+  const int n_m = (M + BM - 1) / BM, step = cs > 1 || n_m == 1 ? 8 : 32;
+  return ((M + n_m - 1) / n_m + step - 1) / step * step;
+}
+
+// Estimated time of one shape in microseconds: a fixed cost, the K loop (hand-overs of a 64-wide block, or its bytes at
+// the 114 KB/us that an SM is fed with from L2, whichever is more), and with a cluster its start, the exchange of partial
+// sums through distributed shared memory and the second CTA of an SM (without one, two CTAs of an SM hide each other).
+// The constants are fitted to 156 measured shapes (M 8 to 5248, the projections of widths 768, 1024 and 1280, every tile
+// and cluster size): the choice costs 0.5 % over the fastest shape on average; before the fit, without the 128-column
+// clusters, 3.6 %.  M x N x K, us: 8 x 4096 x 1024 5.0 -> 4.0, 82 x 2304 x 768 4.3 -> 4.0, 390 x 4096 x 1024 9.5 -> 7.7,
+// 390 x 1024 x 4096 12.4 -> 10.1, 520 x 1024 x 4096 15.4 -> 12.6, 390 x 1280 x 5120 18.7 -> 15.0.
 double gemm_splitk_cost(int M, int N, int K, SplitKShape shape) {
   const int bn = shape.bn, cs = shape.cs;
-  const int n_kb = K / BK, rows = M < BM ? (M + 7) & ~7 : BM;
+  const int n_kb = K / BK, rows = rows_per_tile(M, cs);
   if (N % bn || n_kb < cs) return 1e30;
-  const double ctas = (double)((M + BM - 1) / BM) * (N / bn) * cs, sms = device_sm_count();
-  const double load = ctas / sms;
-  const double share = load <= 1.0 ? 1.0 : (cs == 1 && load <= 2.0 ? 0.55 + 0.45 * load : std::ceil(load));
-  double kb = (rows + bn) * 128 / 114e3;
-  if (kb < 0.14) kb = 0.14;
-  double t = 2.1 + 0.004 * ctas + share * ((n_kb + cs - 1) / cs) * kb;
-  if (cs > 1) t += 0.45 + share * rows * bn * 4 * (cs - 1) / cs / 27.5e3;
-  else t += 0.3 * bn / 64;
-  return load > 1.0 && cs > 1 ? t + 1.2 : t;
+  const double ctas = (double)((M + BM - 1) / BM) * (N / bn) * cs, load = ctas / device_sm_count();
+  const double share = load <= 1.0 ? 1.0 : (cs == 1 && load <= 2.0 ? 0.956 + 0.044 * load : std::ceil(load));
+  const double feed = (rows + bn) * 128 / 114e3, hand_over = rows > 32 ? 0.11 : 0.184;
+  double t = 1.81 + 0.006 * ctas + share * ((n_kb + cs - 1) / cs) * (feed > hand_over ? feed : hand_over);
+  if (cs == 1) return t + 0.41 * bn / 64;
+  t += 0.68 + 0.157 * cs + share * rows * bn * 4 * (cs - 1) / cs / 28.6e3;
+  if (load > 1.0) t += 1.34;
+  return bn == 128 ? t + 0.15 : t;
 }
 
 SplitKShape gemm_splitk_pick(int M, int N, int K) {
-  static const SplitKShape shapes[] = {{64, 1}, {64, 2}, {64, 4}, {64, 8}, {32, 2}, {32, 4}, {128, 1}};
+  static const SplitKShape shapes[] = {{64, 1}, {64, 2}, {64, 4}, {64, 8}, {32, 2}, {32, 4}, {128, 1}, {128, 2}, {128, 4}, {128, 8}};
   SplitKShape best = {128, 1};
   double t = 1e30;
   for (const SplitKShape& s : shapes) {
@@ -359,7 +372,7 @@ cudaError_t launch_gemm_splitk(const void* a, int lda, int M, const void* w, con
       return cudaErrorInvalidValue;
     kv = *kv_scatter;
   }
-  const int a_rows = M >= BM ? BM : (M + 7) & ~7;
+  const int a_rows = rows_per_tile(M, cs);
   CUtensorMap ta, tw, to;
   if (!tma_make_store_map(&to, out, (uint64_t)M, (uint64_t)N, epilogue == 1 ? 4 : 2)) return cudaErrorInvalidValue;
   {
@@ -381,7 +394,7 @@ cudaError_t launch_gemm_splitk(const void* a, int lda, int M, const void* w, con
   }
   MARCHE_SPLITK_CASE(32, 2) MARCHE_SPLITK_CASE(32, 4)
   MARCHE_SPLITK_CASE(64, 1) MARCHE_SPLITK_CASE(64, 2) MARCHE_SPLITK_CASE(64, 4) MARCHE_SPLITK_CASE(64, 8)
-  MARCHE_SPLITK_CASE(128, 1)
+  MARCHE_SPLITK_CASE(128, 1) MARCHE_SPLITK_CASE(128, 2) MARCHE_SPLITK_CASE(128, 4) MARCHE_SPLITK_CASE(128, 8)
 #undef MARCHE_SPLITK_CASE
   return cudaErrorInvalidValue;
 }

@@ -406,20 +406,18 @@ cudaError_t launch_pair(const CUtensorMap& ta, const CUtensorMap& tw, const CUte
 
 // Estimated time of a projection with this kernel in microseconds, for the choice of its tile width and between it and
 // the split-K kernel: a fixed cost (launch gap, first operands, the last tile's epilogue) and the K blocks of the tile
-// rounds at the measured 0.275 us (256 x 256) and 0.205 us (256 x 128) each; from two rounds on the narrow tiles' feed
-// from L2 slows to 0.24 us.  Measured, M x N x K: 700 x 3072 x 1024 9.3 (256) / 8.2 us (128), 2048 x 1024 x 4096 24.1 /
-// 17.7 us, 2624 x 1024 x 4096 26.6 / 23.2 us, 3500 x 1024 x 4096 26.4 / 28.3 us, 5248 x 3072 x 1024 27.7 / 31.8 us.
+// rounds.  The constants are fitted together with gemm_splitk_cost (see there).
 double gemm_tcgen05_2cta_cost(int M, int N, int K, int bn) {
   if (N % bn) return 1e30;
   const int pairs = device_sm_count() / 2, n_tiles = ((M + 2 * BM - 1) / (2 * BM)) * (N / bn), left = n_tiles % pairs;
   double rounds = n_tiles / pairs;
   if (left > 0) {
-    if (K >= 2048 && n_tiles > pairs) rounds += (double)left / pairs;           // stream-K
+    if (K >= 2048 && n_tiles > pairs) rounds += 0.38 + (double)left / pairs;           // stream-K
     else if (bn == 256 && n_tiles > pairs) rounds += left * 2 <= pairs ? 0.75 : 1.0;   // column slices
     else rounds += 1.0;
   }
-  const double kb = bn == 256 ? 0.275 : (rounds > 1.0 ? 0.24 : 0.205);
-  return (bn == 256 ? 5.4 : 4.6) + rounds * (K / BK) * kb;
+  const double kb = bn == 256 ? 0.243 : (rounds > 1.0 ? 0.188 : 0.18);
+  return (bn == 256 ? 5.1 : 4.73) + rounds * (K / BK) * kb;
 }
 
 int gemm_tcgen05_2cta_pick_bn(int M, int N, int K, int tile_n) {

@@ -372,7 +372,8 @@ def test_validate_indices():
 
 @pytest.mark.parametrize("dtype", ["bf16", "bf16b"])
 @pytest.mark.parametrize("M,N,K", [(1, 128, 4096), (9, 640, 2560), (7, 256, 320), (127, 512, 448), (129, 512, 448),
-                                   (40, 3072, 1024), (128, 1024, 1024), (257, 384, 128), (640, 4096, 1024)])
+                                   (40, 3072, 1024), (128, 1024, 1024), (257, 384, 128), (640, 4096, 1024),
+                                   (8, 4096, 1024), (161, 384, 192), (390, 1024, 4096), (521, 1280, 5120)])
 def test_linear_few_rows_split_k(dtype, M, N, K):
     """Row counts at the edges of the A tile, every tile width and cluster size of the split-K kernel, K ranges that do
     not divide evenly (5, 7, 40 blocks over 4, 4, 8 CTAs).  Products of unit size: |acc + bias| stays below 8, where

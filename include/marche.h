@@ -267,7 +267,7 @@ int marche_mar_step(marche_ctx* ctx, int full_decoder, const float* tokens,
  * highest relevance scores"): scores device float [B][S] (finite); candidates
  * are all tokens outside new_idx and exclude_idx; writes refresh_idx device
  * int32 [B][k] ascending; order (score descending, index ascending); -0 == +0.
- * `mask_scratch` is device scratch of B*S bytes.  MARCHE_EINVAL if
+ * `mask_scratch` is device scratch of B*S bytes (not written: the selection keeps its marks on chip).  MARCHE_EINVAL if
  * k > S - n_new - n_excl or k < 0; k == 0 enqueues nothing. */
 int marche_select_refresh(marche_ctx* ctx, const float* scores,
                           const int32_t* new_idx, int n_new,
@@ -293,17 +293,9 @@ int marche_select_refresh_policy(marche_ctx* ctx, const float* scores,
  * whose memory was sized up front, a latency-critical serving loop that must never touch the
  * allocator, a plug-in that is handed only its input and output tensors).  The paper has no
  * counterpart; this is a packaging variant of the same kernels.
- *   - The candidate mask lives in a fixed array inside the library, MARCHE_STATIC_SCRATCH_BYTES
- *     (256 KiB) per GPU, which every GPU that loads the library holds until the process exits.
- *     batch*seq_len must not exceed that size; otherwise MARCHE_EWORKSPACE is returned, nothing
- *     is enqueued and marche_last_error() names both numbers.
- *   - No device memory is allocated or freed by this call, now or later.  Its first call on a
- *     device looks up the array's device address (a synchronous, one-time driver query), so make
- *     that first call before starting any stream capture on that device.
- *   - All calls on a device, from every context, share the one array and it keeps the bytes of
- *     the last call.  Each call rewrites every byte it reads, so stale contents are harmless, but
- *     two calls whose kernels overlap on the GPU (different streams, no dependency) race on it:
- *     keep them on one stream or order them with events.
+ *   - batch*seq_len must not exceed MARCHE_STATIC_SCRATCH_BYTES (256 Ki); otherwise MARCHE_EWORKSPACE is
+ *     returned, nothing is enqueued and marche_last_error() names both numbers.
+ *   - No device memory is allocated or freed by this call, now or later, and none is shared between calls.
  * Arguments, result and errors otherwise exactly as marche_select_refresh without mask_scratch. */
 #define MARCHE_STATIC_SCRATCH_BYTES (256 * 1024)
 int marche_select_refresh_static(marche_ctx* ctx, const float* scores,
@@ -447,8 +439,7 @@ int marche_attention_two_segment(marche_ctx* ctx, const void* qkv, int ld, int n
  * pin them to the same results.  None of them changes what is computed, only which kernel does it;
  * `pdl` is process-wide (it is a property of how kernels are launched). */
 enum { MARCHE_ATTENTION_AUTO = 0, MARCHE_ATTENTION_MMA = 1, MARCHE_ATTENTION_TCGEN05 = 2,
-       MARCHE_ATTENTION_TCGEN05_TWO_PASS = 3 /* the two-pass tcgen05 kernel also where no scores are taken */,
-       MARCHE_ATTENTION_SPLIT = 4 /* keys split over a cluster, wherever it fits (at most 64 rows, no scores) */ };
+       MARCHE_ATTENTION_TCGEN05_TWO_PASS = 3 /* the two-pass tcgen05 kernel also where no scores are taken */ };
 enum { MARCHE_GEMM_AUTO = 0, MARCHE_GEMM_SINGLE = 1, MARCHE_GEMM_PAIR = 2 };
 typedef struct {
   int32_t stream_k;              /* 1: fc2-sized residual projections use stream-K with ordered reduce-adds   */

@@ -17,7 +17,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libmarche.so")
 
 MARCHE_F32, MARCHE_BF16, MARCHE_BF16_F16OP = 0, 1, 2
-ATTENTION_AUTO, ATTENTION_MMA, ATTENTION_TCGEN05, ATTENTION_TCGEN05_TWO_PASS, ATTENTION_SPLIT = 0, 1, 2, 3, 4
+ATTENTION_AUTO, ATTENTION_MMA, ATTENTION_TCGEN05, ATTENTION_TCGEN05_TWO_PASS = 0, 1, 2, 3
 GEMM_AUTO, GEMM_SINGLE, GEMM_PAIR = 0, 1, 2
 EPI_BIAS, EPI_BIAS_RESIDUAL, EPI_BIAS_GELU = 0, 1, 2
 ERRORS = {-1: "EINVAL", -2: "ESHAPE", -3: "EWORKSPACE", -4: "ECACHE", -5: "EINDEX", -6: "ECUDA", -7: "ETIMEOUT"}
@@ -128,8 +128,9 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 
 def _stream(stream: Optional[torch.cuda.Stream]) -> Optional[int]:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream or None
+    if stream is None:                    # (building a torch.cuda.Stream object costs more than the ctypes call)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) or None
+    return stream.cuda_stream or None
 
 
 def _operand_dtype(dtype: str, operand: str) -> torch.dtype:
@@ -303,8 +304,7 @@ class Marche:
             _ptr(mask_scratch), _stream(stream)))
 
     def select_refresh_static(self, scores, new_idx, exclude_idx, k, refresh_idx, stream=None):
-        """select_refresh without a caller-supplied scratch buffer: the candidate mask lives in a
-        fixed 256 KiB array inside the library (B*S must fit).  Nothing is allocated."""
+        """select_refresh without a caller-supplied scratch buffer (B*S at most 256 Ki).  Nothing is allocated."""
         rc = self.lib.marche_select_refresh_static(
             self.h, _ptr(scores), _ptr(new_idx), 0 if new_idx is None else new_idx.shape[1],
             _ptr(exclude_idx), 0 if exclude_idx is None else exclude_idx.shape[1], k, _ptr(refresh_idx),

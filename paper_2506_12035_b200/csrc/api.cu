@@ -56,7 +56,7 @@ namespace {
 inline size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 struct WsLayout {
-  size_t scores, partial, cand, is_new, turn, turn_bytes, x, x2, x3, u, qkv, o, g, total;
+  size_t scores, partial, is_new, turn, turn_bytes, x, x2, x3, u, qkv, o, g, total;
 };
 
 WsLayout ws_layout(const marche_ctx* c, int nA) {
@@ -66,7 +66,6 @@ WsLayout ws_layout(const marche_ctx* c, int nA) {
   size_t off = 0;
   w.scores = off;  off += align256(B * S * sizeof(float));
   w.partial = off; off += align256((1 + c->extra_score_layers.size()) * B * H * S * sizeof(float));
-  w.cand = off;    off += align256(B * S);
   w.is_new = off;  off += align256(M);
   w.turn_bytes = gemm_tcgen05_2cta_turn_bytes((int)M, (int)D);   // stream-K turn flags of the residual GEMMs
   w.turn = off;    off += align256(w.turn_bytes);
@@ -243,11 +242,7 @@ int do_attention(marche_ctx* ctx, const void* q, int ld_q, int n, const void* ca
                    (ak == MARCHE_ATTENTION_TCGEN05 || ak == MARCHE_ATTENTION_TCGEN05_TWO_PASS ||
                     (ak == MARCHE_ATTENTION_AUTO && n > tc_min));
   // few items (or few key tiles): all tiles in flight, split over a cluster and over warps; measured beside the rule
-  const int items = c.batch * c.n_heads;
-  int split_cs, split_nk;
-  const bool split = !is_new && (ak == MARCHE_ATTENTION_SPLIT
-                                     ? attention_split_plan(n, S, c.head_dim, items, &split_cs, &split_nk)
-                                     : ak == MARCHE_ATTENTION_AUTO && attention_split_wins(n, S, c.head_dim, items));
+  const bool split = !is_new && ak == MARCHE_ATTENTION_AUTO && attention_split_wins(n, S, c.head_dim, c.batch * c.n_heads);
   if (split)
     MARCHE_TRY(launch_attention_split(q, ld_q, c.batch, n, S, c.n_heads, c.head_dim, cache_layer, o, ctx->a_bf16,
                                       ctx->status_dev, st), "attention_split");
@@ -271,7 +266,7 @@ int do_attention(marche_ctx* ctx, const void* q, int ld_q, int n, const void* ca
 }
 
 struct StackBufs {
-  float* scores; float* partial; uint8_t* cand; uint8_t* is_new;
+  float* scores; float* partial; uint8_t* is_new;
   float* x; float* x2; float* x3; char* u; char* qkv; char* o; char* g;
   int* turn;
 };
@@ -281,7 +276,6 @@ StackBufs carve(void* workspace, const WsLayout& w) {
   StackBufs b;
   b.scores = (float*)(ws + w.scores);
   b.partial = (float*)(ws + w.partial);
-  b.cand = (uint8_t*)(ws + w.cand);
   b.is_new = (uint8_t*)(ws + w.is_new);
   b.turn = (int*)(ws + w.turn);
   b.x = (float*)(ws + w.x);
@@ -385,13 +379,14 @@ int run_stack(marche_ctx* ctx, const float* hidden, void* kv_cache, const int32_
   // the workspace is scratch between calls: make sure the stream-K turn flags start at zero
   if (needs_turn(ctx, B * nA)) MARCHE_TRY(cudaMemsetAsync(bf.turn, 0, w.turn_bytes, st), "memset");
   mark(ctx, MARCHE_KC_FLAGS, st);
-  MARCHE_TRY(launch_step_flags(active_idx, nA, new_idx, n_new, excl_idx, n_excl, B, S, bf.is_new, bf.cand, st), "flags");
+  MARCHE_TRY(launch_step_flags(active_idx, nA, new_idx, n_new, B, S, bf.is_new, st), "flags");
   const int rc = run_blocks(ctx, 0, L, hidden, S, active_idx, nA, bf.x, bf, kv_cache, bf.is_new, st);
   if (rc) return rc;
   mark(ctx, MARCHE_KC_SCATTER_ROWS, st);
   MARCHE_TRY(launch_scatter_rows(bf.x, active_idx, B, nA, S, D, hidden_out, st), "scatter_rows");
   mark(ctx, MARCHE_KC_TOPK, st);
-  MARCHE_TRY(launch_topk(bf.partial, H, bf.scores, bf.cand, B, S, k, refresh_idx, st), "topk");
+  MARCHE_TRY(launch_topk(bf.partial, H, bf.scores, new_idx, n_new, excl_idx, n_excl, B, S, k, refresh_idx, st),
+             "topk");
   return MARCHE_OK;
 }
 
@@ -417,11 +412,12 @@ int run_in_step(marche_ctx* ctx, const float* hidden, void* kv_cache, const int3
 
   // phase 1: every token; generating rows flagged for the scores; candidates = all \ (new u prev)
   mark(ctx, MARCHE_KC_FLAGS, st);
-  MARCHE_TRY(launch_step_flags(nullptr, S, new_idx, n_new, prev_idx, n_prev, B, S, bf.is_new, bf.cand, st), "flags");
+  MARCHE_TRY(launch_step_flags(nullptr, S, new_idx, n_new, B, S, bf.is_new, st), "flags");
   int rc = run_blocks(ctx, 0, sl + 1, hidden, S, nullptr, S, bf.x, bf, kv_cache, bf.is_new, st);
   if (rc) return rc;
   mark(ctx, MARCHE_KC_TOPK, st);
-  MARCHE_TRY(launch_topk(bf.partial, H, bf.scores, bf.cand, B, S, k, refresh_idx, st), "topk");
+  MARCHE_TRY(launch_topk(bf.partial, H, bf.scores, new_idx, n_new, prev_idx, n_prev, B, S, k, refresh_idx, st),
+             "topk");
   mark(ctx, MARCHE_KC_OTHER, st);
   MARCHE_TRY(launch_build_active(new_idx, n_new, prev_idx, n_prev, forced_refresh ? forced_refresh : refresh_idx, k, B,
                                  active_idx, st), "build_active");
@@ -459,7 +455,7 @@ int run_mar(marche_ctx* ctx, bool full_decoder, const float* tokens, const int32
   if (needs_turn(ctx, B * S) || needs_turn(ctx, B * n_known) || needs_turn(ctx, B * nA)) MARCHE_TRY(cudaMemsetAsync(bf.turn, 0, w.turn_bytes, st), "memset");
 
   mark(ctx, MARCHE_KC_FLAGS, st);
-  MARCHE_TRY(launch_step_flags(nullptr, S, new_idx, n_new, prev_idx, n_prev, B, S, bf.is_new, bf.cand, st), "flags");
+  MARCHE_TRY(launch_step_flags(nullptr, S, new_idx, n_new, B, S, bf.is_new, st), "flags");
   // ---- Eq. 1: encoder on the compacted known tokens; its K/V live only inside this step
   int rc = run_blocks(ctx, 0, E, tokens, S, known_idx, n_known, bf.x, bf, kv_cache, nullptr, st, n_known);
   if (rc) return rc;
@@ -482,7 +478,8 @@ int run_mar(marche_ctx* ctx, bool full_decoder, const float* tokens, const int32
     rc = run_blocks(ctx, E, L, bf.x3, S, nullptr, S, bf.x, bf, kv_cache, bf.is_new, st);
     if (rc) return rc;
     mark(ctx, MARCHE_KC_TOPK, st);
-    MARCHE_TRY(launch_topk(bf.partial, H, bf.scores, bf.cand, B, S, k, refresh_idx, st), "topk");
+    MARCHE_TRY(launch_topk(bf.partial, H, bf.scores, new_idx, n_new, prev_idx, n_prev, B, S, k, refresh_idx, st),
+             "topk");
     mark(ctx, MARCHE_KC_GATHER_LN, st);
     MARCHE_TRY(launch_gather_layernorm(OUT_F32, bf.x, S, nullptr, B, S, D, mw.dec_norm_g, mw.dec_norm_b, ctx->eps,
                                        nullptr, z_out, st), "decoder_norm");
@@ -491,7 +488,8 @@ int run_mar(marche_ctx* ctx, bool full_decoder, const float* tokens, const int32
   rc = run_blocks(ctx, E, sl + 1, bf.x3, S, nullptr, S, bf.x, bf, kv_cache, bf.is_new, st);
   if (rc) return rc;
   mark(ctx, MARCHE_KC_TOPK, st);
-  MARCHE_TRY(launch_topk(bf.partial, H, bf.scores, bf.cand, B, S, k, refresh_idx, st), "topk");
+  MARCHE_TRY(launch_topk(bf.partial, H, bf.scores, new_idx, n_new, prev_idx, n_prev, B, S, k, refresh_idx, st),
+             "topk");
   mark(ctx, MARCHE_KC_OTHER, st);
   MARCHE_TRY(launch_build_active(new_idx, n_new, prev_idx, n_prev, forced_refresh ? forced_refresh : refresh_idx, k, B,
                                  active_idx, st), "build_active");
@@ -675,12 +673,9 @@ int marche_select_refresh_policy(marche_ctx* ctx, const float* scores, const int
   if (k == 0) return MARCHE_OK;
   if (!refresh_idx) return MARCHE_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
-  mark(ctx, MARCHE_KC_FLAGS, st);
-  MARCHE_TRY(launch_step_flags(nullptr, 0, new_idx, n_new, exclude_idx, n_excl, B, S, nullptr, (uint8_t*)mask_scratch,
-                               st), "flags");
   mark(ctx, MARCHE_KC_TOPK, st);
-  MARCHE_TRY(launch_topk(nullptr, 0, const_cast<float*>(scores), (const uint8_t*)mask_scratch, B, S, k, refresh_idx,
-                         st, policy, seed), "topk");
+  MARCHE_TRY(launch_topk(nullptr, 0, const_cast<float*>(scores), new_idx, n_new, exclude_idx, n_excl, B, S, k, refresh_idx, st,
+                         policy, seed), "topk");
   return MARCHE_OK;
 }
 
@@ -707,7 +702,7 @@ int marche_get_layer_scores(marche_ctx* ctx, void* workspace, int layer, float* 
   const float* partial = (const float*)((const char*)workspace + w.partial) + (size_t)slot * c.batch * c.n_heads * c.seq_len;
   mark(ctx, MARCHE_KC_TOPK, (cudaStream_t)stream);
   // k = 0: the kernel only adds the per-head partials in head order and writes the sums
-  MARCHE_TRY(launch_topk(partial, c.n_heads, scores_out, nullptr, c.batch, c.seq_len, 0, nullptr, (cudaStream_t)stream),
+  MARCHE_TRY(launch_topk(partial, c.n_heads, scores_out, nullptr, 0, nullptr, 0, c.batch, c.seq_len, 0, nullptr, (cudaStream_t)stream),
              "score_sum");
   return MARCHE_OK;
 }
@@ -934,30 +929,6 @@ const char* marche_kernel_class_name(int cls) {
 }
 
 // ---------------------------------------------------------------- allocation-free selection
-// Candidate-mask scratch of marche_select_refresh_static.  It lives in the library image, so every
-// GPU that loads the library holds these bytes until the process exits.  In host code the name
-// below is only a stand-in for the device object; its device address is obtained once per device
-// with cudaGetSymbolAddress and handed to the kernels.
-static __device__ __align__(256) uint8_t g_static_mask_scratch[MARCHE_STATIC_SCRATCH_BYTES];
-
-namespace {
-uint8_t* g_static_mask_ptr[kMaxDevices] = {};
-
-// Device address of the scratch array on device `dev`, which must be the current device (looked up on
-// first use: cudaGetSymbolAddress answers for the current device).
-cudaError_t static_mask_address(int dev, uint8_t** out) {
-  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-  if (!g_static_mask_ptr[dev]) {
-    void* p = nullptr;
-    const cudaError_t e = cudaGetSymbolAddress(&p, g_static_mask_scratch);
-    if (e != cudaSuccess) return e;
-    g_static_mask_ptr[dev] = static_cast<uint8_t*>(p);
-  }
-  *out = g_static_mask_ptr[dev];
-  return cudaSuccess;
-}
-}  // namespace
-
 int marche_select_refresh_static(marche_ctx* ctx, const float* scores, const int32_t* new_idx, int n_new,
                                  const int32_t* exclude_idx, int n_excl, int k, int32_t* refresh_idx,
                                  marche_stream stream) {
@@ -975,15 +946,10 @@ int marche_select_refresh_static(marche_ctx* ctx, const float* scores, const int
     ctx->last_error = msg;
     return MARCHE_EWORKSPACE;
   }
-  uint8_t* mask = nullptr;
-  MARCHE_TRY(static_mask_address(ctx->device, &mask), "cudaGetSymbolAddress");
   cudaStream_t st = (cudaStream_t)stream;
-  // The mask kernel writes all B*S bytes it uses, so nothing left over from an earlier call
-  // (of this or any other context) can leak into this one.
-  mark(ctx, MARCHE_KC_FLAGS, st);
-  MARCHE_TRY(launch_step_flags(nullptr, 0, new_idx, n_new, exclude_idx, n_excl, B, S, nullptr, mask, st), "flags");
   mark(ctx, MARCHE_KC_TOPK, st);
-  MARCHE_TRY(launch_topk(nullptr, 0, const_cast<float*>(scores), mask, B, S, k, refresh_idx, st), "topk");
+  MARCHE_TRY(launch_topk(nullptr, 0, const_cast<float*>(scores), new_idx, n_new, exclude_idx, n_excl, B, S, k, refresh_idx, st),
+             "topk");
   return MARCHE_OK;
 }
 
@@ -996,7 +962,7 @@ int marche_get_tuning(const marche_ctx* ctx, marche_tuning* out) {
 
 int marche_set_tuning(marche_ctx* ctx, const marche_tuning* t) {
   if (!ctx || !t) return MARCHE_EINVAL;
-  if (t->attention_kernel < MARCHE_ATTENTION_AUTO || t->attention_kernel > MARCHE_ATTENTION_SPLIT) return MARCHE_EINVAL;
+  if (t->attention_kernel < MARCHE_ATTENTION_AUTO || t->attention_kernel > MARCHE_ATTENTION_TCGEN05_TWO_PASS) return MARCHE_EINVAL;
   if (t->gemm_kernel < MARCHE_GEMM_AUTO || t->gemm_kernel > MARCHE_GEMM_PAIR) return MARCHE_EINVAL;
   if (t->tail_split != 0 && t->tail_split != 1 && t->tail_split != 2 && t->tail_split != 4) return MARCHE_EINVAL;
   if (t->tile_n != 0 && t->tile_n != 128) return MARCHE_EINVAL;

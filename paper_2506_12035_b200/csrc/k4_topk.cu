@@ -4,7 +4,13 @@
 // kernel are summed in fixed head order (bit-reproducible run to run, unlike atomics),
 // then the K-th best candidate under (score descending, index ascending) is found by a
 // radix select and the K best are emitted in ascending index order through a block
-// scan.  S <= 2048, so all keys of a sample live in shared memory.
+// scan.  S <= 2048: a thread keeps its share of the candidates, at most eight, in registers.
+//
+// Bound by latency (64 samples of 1088 tokens are 0.3 MB): what counts is how many barriers stand in a row.  The
+// tokens that must not be chosen are marked in shared memory by the same launch; the digits start at the first bit
+// in which the candidates differ, which leaves one to three of a thousand scores in the crossing bin of the first pass;
+// every warp scans the 512 bins for itself.  Six to eight barriers and one launch, where four fixed passes of four
+// barriers took two launches.
 #include "common.cuh"
 #include "kernels.h"
 #include "launch_pdl.h"
@@ -34,124 +40,146 @@ MARCHE_DEVINL uint32_t mix32(uint32_t seed, uint32_t b, uint32_t t) {
 // policy 0: highest score first (Section 4.2); 1: lowest score first and 2: random order (the
 // selection ablations of Section 5.3).  Ties always go to the lower token index.
 //
-// Every candidate gets a 44-bit composite (32-bit order key, then 2047 - index, plus one so that
-// 0 can mean "not a candidate"); composites are distinct, a larger one ranks earlier.  The k-th
-// largest composite is found by a most-significant-digit-first radix select, four passes of 11
-// bits over a 2048-bin histogram in shared memory, and every candidate at or above it is emitted.
-// O(S) work per sample instead of the S^2 of ranking by counting; the result is the same set.
-constexpr int kRadixBits = 11, kRadixBins = 1 << kRadixBits, kRadixPasses = 4;
+// Every candidate gets a 43-bit composite (32-bit order key, then 2047 - index); composites are distinct, a larger one
+// ranks earlier.  Each pass deals those in the current range over 512 bins by their next nine bits and keeps the bin in
+// which the k-th largest lies; it is over when that bin is wanted whole or holds one value.
+constexpr int kIdxBits = 11, kBinBits = 9, kBins = 1 << kBinBits, kMaxPasses = (32 + kIdxBits + kBinBits - 1) / kBinBits;
+constexpr int kPerThread = 2048 / kTopkThreads, kTopkWarps = kTopkThreads / 32;
 
 __global__ void __launch_bounds__(kTopkThreads)
-topk_kernel(const float* __restrict__ partial, int H, float* __restrict__ scores,
-            const uint8_t* __restrict__ cand, int S, int k, int policy, uint32_t seed,
+topk_kernel(const float* __restrict__ partial, int H, float* __restrict__ scores, const int32_t* __restrict__ new_idx,
+            int n_new, const int32_t* __restrict__ excl_idx, int n_excl, int S, int k, int policy, uint32_t seed,
             int32_t* __restrict__ refresh_idx) {
-  extern __shared__ unsigned long long comp[];          // [S] composites; 0 = not a candidate
-  __shared__ unsigned int hist[kRadixBins];
-  __shared__ int warp_tot[kTopkThreads / 32];
-  __shared__ unsigned int sel_digit, sel_above;
+  __shared__ uint4 hist[kMaxPasses][kBins / 4];          // one histogram per pass: none has to be cleared again
+  __shared__ uint32_t taken[2048 / 4];                   // a byte per token: generating or excluded
+  __shared__ uint32_t warp_min[kTopkWarps], warp_max[kTopkWarps];
+  __shared__ int warp_tot[kTopkWarps];
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int i = tid; i < kMaxPasses * kBins / 4; i += kTopkThreads) (&hist[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (int i = tid; i < 2048 / 4; i += kTopkThreads) taken[i] = 0u;
+  __syncthreads();
   pdl_sync();
 
-  for (int t = tid; t < S; t += kTopkThreads) {
-    float s;
-    if (partial) {
-      s = 0.f;
-      for (int h = 0; h < H; ++h) s += partial[((long)b * H + h) * S + t];
-      scores[(long)b * S + t] = s;
-    } else {
-      s = scores[(long)b * S + t];
+  uint8_t* mark = reinterpret_cast<uint8_t*>(taken);
+  if (k > 0) {
+    for (int i = tid; i < n_new; i += kTopkThreads) mark[new_idx[(long)b * n_new + i]] = 1;
+    for (int i = tid; i < n_excl; i += kTopkThreads) mark[excl_idx[(long)b * n_excl + i]] = 1;
+  }
+  // a thread owns consecutive tokens, so that the selected ones come out in ascending order
+  const int per = (S + kTopkThreads - 1) / kTopkThreads, t0 = tid * per;
+  uint32_t key[kPerThread];
+#pragma unroll
+  for (int i = 0; i < kPerThread; ++i) {
+    const int t = t0 + i;
+    key[i] = 0u;
+    if (i < per && t < S) {
+      float s;
+      if (partial) {
+        s = 0.f;
+        for (int h = 0; h < H; ++h) s += partial[((long)b * H + h) * S + t];
+        scores[(long)b * S + t] = s;
+      } else {
+        s = scores[(long)b * S + t];
+      }
+      key[i] = policy == 0 ? score_key(s) : (policy == 1 ? ~score_key(s) : ~mix32(seed, (uint32_t)b, (uint32_t)t));
     }
-    const uint32_t key = policy == 0 ? score_key(s) : (policy == 1 ? ~score_key(s) : ~mix32(seed, (uint32_t)b, (uint32_t)t));
-    comp[t] = (k > 0 && cand[(long)b * S + t])
-                  ? ((((unsigned long long)key << kRadixBits) | (unsigned long long)(kRadixBins - 1 - t)) + 1ull)
-                  : 0ull;
   }
   if (k <= 0) return;
-
-  // ---- radix select of the k-th largest composite
-  unsigned long long prefix = 0ull, decided = 0ull;     // bits fixed so far and their mask
-  int remaining = k;
-#pragma unroll 1
-  for (int pass = 0; pass < kRadixPasses; ++pass) {
-    const int shift = kRadixBits * (kRadixPasses - 1 - pass);
-    for (int i = tid; i < kRadixBins; i += kTopkThreads) hist[i] = 0u;
-    __syncthreads();                                     // also orders the writes of comp before the reads
-    for (int t = tid; t < S; t += kTopkThreads) {
-      const unsigned long long c = comp[t];
-      if (c != 0ull && (c & decided) == prefix) atomicAdd(&hist[(unsigned)(c >> shift) & (kRadixBins - 1)], 1u);
-    }
-    __syncthreads();
-    // With fewer than `remaining` candidates left no bin crosses: digit 0 then keeps every candidate.
-    // (Reset here: all threads have passed this pass's first barrier, so none still reads the last pass's values.)
-    if (tid == 0) { sel_digit = 0u; sel_above = 0u; }
-    // thread i owns PER consecutive bins; suffix sums from the top bin downwards
-    constexpr int PER = kRadixBins / kTopkThreads;
-    unsigned int h[PER], mine = 0u;
+  __syncthreads();                                       // the marks
+  unsigned cand = 0;                                     // bit i: token t0 + i is a candidate
+  uint32_t lo32 = 0xffffffffu, hi32 = 0u;
 #pragma unroll
-    for (int j = 0; j < PER; ++j) { h[j] = hist[tid * PER + j]; mine += h[j]; }
-    unsigned int inc = mine;                             // inclusive scan over threads in DESCENDING thread order
+  for (int i = 0; i < kPerThread; ++i)
+    if (i < per && t0 + i < S && !mark[t0 + i]) {
+      cand |= 1u << i;
+      lo32 = min(lo32, key[i]);
+      hi32 = max(hi32, key[i]);
+    }
+  lo32 = __reduce_min_sync(0xffffffffu, lo32);
+  hi32 = __reduce_max_sync(0xffffffffu, hi32);
+  if (lane == 0) { warp_min[warp] = lo32; warp_max[warp] = hi32; }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kTopkWarps; ++w) { lo32 = min(lo32, warp_min[w]); hi32 = max(hi32, warp_max[w]); }
+
+  // ---- radix select of the k-th largest composite; with fewer than k candidates all of them stay
+  auto composite = [&](int i) { return ((unsigned long long)key[i] << kIdxBits) | (unsigned)((1 << kIdxBits) - 1 - (t0 + i)); };
+  unsigned long long lo = (unsigned long long)lo32 << kIdxBits;
+  unsigned long long range = hi32 >= lo32 ? (((unsigned long long)(hi32 - lo32) << kIdxBits) | ((1 << kIdxBits) - 1)) : 0ull;
+  unsigned int remaining = (unsigned)k;
+  unsigned in_range = cand;
+#pragma unroll 1
+  for (int pass = 0; pass < kMaxPasses; ++pass) {
+    const int bits = 64 - __clzll((long long)range), shift = bits > kBinBits ? bits - kBinBits : 0;
+    unsigned int* h = reinterpret_cast<unsigned int*>(hist[pass]);
+#pragma unroll
+    for (int i = 0; i < kPerThread; ++i)
+      if (in_range & (1u << i)) atomicAdd(&h[(unsigned)((composite(i) - lo) >> shift)], 1u);
+    __syncthreads();
+    unsigned int c[kBins / 32], mine = 0u;               // a lane's consecutive bins
+#pragma unroll
+    for (int j = 0; j < kBins / 128; ++j) {
+      const uint4 v = hist[pass][lane * (kBins / 128) + j];
+      c[4 * j] = v.x; c[4 * j + 1] = v.y; c[4 * j + 2] = v.z; c[4 * j + 3] = v.w;
+      mine += (v.x + v.y) + (v.z + v.w);
+    }
+    unsigned int above = mine;                           // suffix sums from the top bin downwards
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const unsigned int v = __shfl_down_sync(0xffffffffu, inc, o);
-      if (lane + o < 32) inc += v;
+      const unsigned int v = __shfl_down_sync(0xffffffffu, above, o);
+      if (lane + o < 32) above += v;
     }
-    if (lane == 0) warp_tot[warp] = (int)inc;
-    __syncthreads();
-    unsigned int above = inc - mine;                     // candidates in bins above this thread's bins
-    for (int w = warp + 1; w < kTopkThreads / 32; ++w) above += (unsigned)warp_tot[w];
-    // the crossing bin: the highest bin d with (count in bins >= d) >= remaining
-    if (above < (unsigned)remaining && above + mine >= (unsigned)remaining) {
-      unsigned int acc = above;
+    const bool here = above >= remaining && above - mine < remaining;
+    const unsigned who = __ballot_sync(0xffffffffu, here);
+    if (who == 0u) break;                                // fewer candidates than remaining
+    above -= mine;
+    int digit = 0;
+    unsigned int before = 0u, held = 0u;
 #pragma unroll
-      for (int j = PER - 1; j >= 0; --j) {
-        if (acc < (unsigned)remaining && acc + h[j] >= (unsigned)remaining) {
-          sel_digit = (unsigned)(tid * PER + j);
-          sel_above = acc;
-        }
-        acc += h[j];
-      }
+    for (int j = kBins / 32 - 1; j >= 0; --j) {
+      if (above < remaining && above + c[j] >= remaining) { digit = lane * (kBins / 32) + j; before = above; held = c[j]; }
+      above += c[j];
     }
-    __syncthreads();
-    prefix |= (unsigned long long)sel_digit << shift;
-    decided |= (unsigned long long)(kRadixBins - 1) << shift;
-    remaining -= (int)sel_above;
+    const int src = __ffs((int)who) - 1;
+    digit = __shfl_sync(0xffffffffu, digit, src);
+    before = __shfl_sync(0xffffffffu, before, src);
+    held = __shfl_sync(0xffffffffu, held, src);
+    lo += (unsigned long long)digit << shift;
+    range = (1ull << shift) - 1ull;
+    remaining -= before;
+    if (held == remaining || shift == 0) break;
+#pragma unroll
+    for (int i = 0; i < kPerThread; ++i)
+      if ((in_range & (1u << i)) && (composite(i) < lo || composite(i) - lo > range)) in_range &= ~(1u << i);
   }
-  const unsigned long long threshold = prefix;           // the k-th largest composite itself
 
-  // Each thread owns a contiguous chunk of token indices so the scan below emits ascending indices.
-  const int per = (S + kTopkThreads - 1) / kTopkThreads;
-  const int t0 = tid * per;
-  unsigned sel_mask = 0;   // per <= 8 for S <= 2048
-  int cnt = 0;
-  for (int i = 0; i < per; ++i) {
-    const int t = t0 + i;
-    if (t < S) {
-      const unsigned long long me = comp[t];
-      if (me != 0ull && me >= threshold) { sel_mask |= 1u << i; ++cnt; }
-    }
-  }
-  // exclusive block scan of cnt
-  int inc2 = cnt;
+  // ---- every candidate at or above the bound, in ascending order of index
+  unsigned sel = 0;
+#pragma unroll
+  for (int i = 0; i < kPerThread; ++i)
+    if ((cand & (1u << i)) && composite(i) >= lo) sel |= 1u << i;
+  const int cnt = __popc(sel);
+  int inc = cnt;                                         // inclusive scan over the block
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, inc2, o);
-    if (lane >= o) inc2 += v;
+    const int v = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += v;
   }
-  __syncthreads();                                       // warp_tot is reused
-  if (lane == 31) warp_tot[warp] = inc2;
+  if (lane == 31) warp_tot[warp] = inc;
   __syncthreads();
-  int base = 0;
-  for (int w = 0; w < warp; ++w) base += warp_tot[w];
-  int pos = base + inc2 - cnt;
-  for (int i = 0; i < per; ++i)
-    if (sel_mask & (1u << i)) refresh_idx[(long)b * k + pos++] = t0 + i;
+  int pos = inc - cnt;
+  for (int w = 0; w < warp; ++w) pos += warp_tot[w];
+#pragma unroll
+  for (int i = 0; i < kPerThread; ++i)
+    if (sel & (1u << i)) refresh_idx[(long)b * k + pos++] = t0 + i;
 }
 
-cudaError_t launch_topk(const float* partial, int H, float* scores, const uint8_t* cand, int B, int S, int k,
-                        int32_t* refresh_idx, cudaStream_t st, int policy, uint32_t seed) {
+cudaError_t launch_topk(const float* partial, int H, float* scores, const int32_t* new_idx, int n_new,
+                        const int32_t* excl_idx, int n_excl, int B, int S, int k, int32_t* refresh_idx, cudaStream_t st,
+                        int policy, uint32_t seed) {
   if (S > 2048) return cudaErrorInvalidValue;
-  return launch_pdl(topk_kernel, dim3(B), dim3(kTopkThreads), (size_t)S * sizeof(unsigned long long), st, partial, H,
-                    scores, cand, S, k, policy, seed, refresh_idx);
+  return launch_pdl(topk_kernel, dim3(B), dim3(kTopkThreads), 0, st, partial, H, scores, new_idx, n_new, excl_idx, n_excl, S,
+                    k, policy, seed, refresh_idx);
 }
 
 }  // namespace marche

@@ -91,25 +91,19 @@ fill_mask_rows_kernel(const float4* __restrict__ mask_token, const float4* __res
   }
 }
 
-// One CTA per sample.  mark bit0 = generating token, bit1 = excluded token.
+// One CTA per sample.
 __global__ void __launch_bounds__(256)
 step_flags_kernel(const int32_t* __restrict__ active_idx, int n_active, const int32_t* __restrict__ new_idx,
-                  int n_new, const int32_t* __restrict__ excl_idx, int n_excl, int S,
-                  uint8_t* __restrict__ is_new, uint8_t* __restrict__ cand) {
+                  int n_new, int S, uint8_t* __restrict__ is_new) {
   extern __shared__ uint8_t mark[];
   const int b = blockIdx.x;
-  pdl_sync();
   for (int t = threadIdx.x; t < S; t += blockDim.x) mark[t] = 0;
   __syncthreads();
+  pdl_sync();
   for (int i = threadIdx.x; i < n_new; i += blockDim.x) mark[new_idx[(long)b * n_new + i]] = 1;
   __syncthreads();
-  for (int i = threadIdx.x; i < n_excl; i += blockDim.x) mark[excl_idx[(long)b * n_excl + i]] |= 2;
-  __syncthreads();
-  if (is_new)
-    for (int j = threadIdx.x; j < n_active; j += blockDim.x)
-      is_new[(long)b * n_active + j] = active_idx ? (mark[active_idx[(long)b * n_active + j]] & 1) : (mark[j] & 1);
-  if (cand)
-    for (int t = threadIdx.x; t < S; t += blockDim.x) cand[(long)b * S + t] = mark[t] ? 0 : 1;
+  for (int j = threadIdx.x; j < n_active; j += blockDim.x)
+    is_new[(long)b * n_active + j] = mark[active_idx ? active_idx[(long)b * n_active + j] : j];
 }
 
 __global__ void build_active_kernel(const int32_t* __restrict__ a, int na, const int32_t* __restrict__ b, int nb,
@@ -205,11 +199,9 @@ cudaError_t launch_fill_mask_rows(const float* mask_token, const float* pos, int
                     (const float4*)mask_token, (const float4*)pos, S, D / 4, total, (float4*)out);
 }
 
-cudaError_t launch_step_flags(const int32_t* active_idx, int n_active, const int32_t* new_idx, int n_new,
-                              const int32_t* excl_idx, int n_excl, int B, int S, uint8_t* is_new,
-                              uint8_t* cand, cudaStream_t st) {
-  return launch_pdl(step_flags_kernel, dim3(B), dim3(256), (size_t)S, st, active_idx, n_active, new_idx, n_new, excl_idx,
-                    n_excl, S, is_new, cand);
+cudaError_t launch_step_flags(const int32_t* active_idx, int n_active, const int32_t* new_idx, int n_new, int B, int S,
+                              uint8_t* is_new, cudaStream_t st) {
+  return launch_pdl(step_flags_kernel, dim3(B), dim3(256), (size_t)S, st, active_idx, n_active, new_idx, n_new, S, is_new);
 }
 
 cudaError_t launch_build_active(const int32_t* a, int na, const int32_t* b, int nb, const int32_t* c, int nc,

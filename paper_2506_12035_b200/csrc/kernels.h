@@ -37,10 +37,9 @@ cudaError_t launch_gather_table_rows(const float* table, const int32_t* idx, lon
 cudaError_t launch_fill_mask_rows(const float* mask_token, const float* pos, int B, int S, int D, float* out,
                                   cudaStream_t st);
 
-// a0 prologue: is_new[b][j] (may be NULL with n_active = 0) and the candidate mask cand[b][t].
-cudaError_t launch_step_flags(const int32_t* active_idx, int n_active, const int32_t* new_idx, int n_new,
-                              const int32_t* excl_idx, int n_excl, int B, int S, uint8_t* is_new,
-                              uint8_t* cand, cudaStream_t st);
+// a0 prologue: is_new[b][j] = active row j of sample b is a generating token (active_idx NULL = identity).
+cudaError_t launch_step_flags(const int32_t* active_idx, int n_active, const int32_t* new_idx, int n_new, int B, int S,
+                              uint8_t* is_new, cudaStream_t st);
 
 cudaError_t launch_build_active(const int32_t* a, int na, const int32_t* b, int nb, const int32_t* c, int nc,
                                 int B, int32_t* out, cudaStream_t st);
@@ -49,11 +48,12 @@ cudaError_t launch_build_active(const int32_t* a, int na, const int32_t* b, int 
 cudaError_t launch_validate(const int32_t* active_idx, int n_active, const int32_t* new_idx, int n_new,
                             const int32_t* excl_idx, int n_excl, int B, int S, int* status, cudaStream_t st);
 
-// K4: optional fixed-order head reduction of score partials [B][H][S] into scores [B][S],
-// then top-k among cand (k may be 0: reduction only).
+// K4: optional fixed-order head reduction of score partials [B][H][S] into scores [B][S], then top-k among the tokens
+// in neither new_idx [B][n_new] nor excl_idx [B][n_excl] (k may be 0: reduction only).
 // policy 0 = highest scores, 1 = lowest scores, 2 = random (counter-based hash of seed, sample, token).
-cudaError_t launch_topk(const float* partial, int H, float* scores, const uint8_t* cand, int B, int S, int k,
-                        int32_t* refresh_idx, cudaStream_t st, int policy = 0, uint32_t seed = 0);
+cudaError_t launch_topk(const float* partial, int H, float* scores, const int32_t* new_idx, int n_new,
+                        const int32_t* excl_idx, int n_excl, int B, int S, int k, int32_t* refresh_idx, cudaStream_t st,
+                        int policy = 0, uint32_t seed = 0);
 
 // K2 of the fp32 configuration (SIMT, fp32 operands and outputs).
 cudaError_t launch_gemm_simt(const float* a, int lda, int M, const float* w, const float* bias,

@@ -188,7 +188,7 @@ bool needs_turn(const marche_ctx* ctx, int M) {
 
 // True when the QKV projection writes K and V into the cache itself: no scatter_kv launch then.
 bool qkv_scatter_fused(const marche_ctx* ctx) {
-  return ctx->tune.fuse_qkv_scatter && ctx->bf16 && !ctx->tune.two_segment_attention;
+  return ctx->tune.fuse_qkv_scatter && !(ctx->bf16 && ctx->tune.two_segment_attention);
 }
 
 int do_linear(marche_ctx* ctx, int cls, const void* a, int lda, int M, const void* w, const float* bias, int N, int K,
@@ -196,7 +196,7 @@ int do_linear(marche_ctx* ctx, int cls, const void* a, int lda, int M, const voi
   if (skipped(ctx, cls)) return MARCHE_OK;
   if (!ctx->bf16) {
     if (M > 0) mark(ctx, cls, st);
-    MARCHE_TRY(launch_gemm_simt((const float*)a, lda, M, (const float*)w, bias, N, K, epi, (float*)out, st), "gemm");
+    MARCHE_TRY(launch_gemm_simt((const float*)a, lda, M, (const float*)w, bias, N, K, epi, (float*)out, st, kv), "gemm");
     return MARCHE_OK;
   }
   // 16-bit contexts run on the tensor cores or not at all

@@ -11,6 +11,8 @@
 // order through distributed shared memory: bit-reproducible either way.  K chunks of 128 arrive by cp.async, two in
 // flight, the weights' first ones before the dependency wait (no kernel writes weights).  With this and the fp32 attention
 // in clusters a tiny eight-step run (2 x 68 tokens, width 256, 4 blocks) went from 7.38 ms to 1.24 ms.
+#include <cmath>
+
 #include "common.cuh"
 #include "kernels.h"
 #include "launch_pdl.h"
@@ -39,7 +41,7 @@ MARCHE_DEVINL void copy4(uint32_t dst, const float* src, bool valid, bool vec) {
 template <int T, int CS, int EPI>
 __global__ void __launch_bounds__(kGemmThreads)
 gemm_simt_kernel(const float* __restrict__ a, int lda, int M, const float* __restrict__ w, const float* __restrict__ bias,
-                 int N, int K, float* __restrict__ out, int vec) {
+                 int N, int K, float* __restrict__ out, const KvScatter kv, int vec) {
   constexpr int TM = T / 8, LD = KC + kRowPad, STAGE = 2 * T * LD;
   constexpr int NV = T * T / 4 / kGemmThreads;           // float4s of the tile per thread
   constexpr int OWN = T * T / 4 / CS;                    // float4s of the tile that one CTA of the cluster finishes
@@ -168,13 +170,18 @@ gemm_simt_kernel(const float* __restrict__ a, int lda, int M, const float* __res
     v.x += bv[i].x; v.y += bv[i].y; v.z += bv[i].z; v.w += bv[i].w;
     if (EPI == 1) { v.x += res[i].x; v.y += res[i].y; v.z += res[i].z; v.w += res[i].w; }
     if (EPI == 2) { v.x = gelu_erf(v.x); v.y = gelu_erf(v.y); v.z = gelu_erf(v.z); v.w = gelu_erf(v.w); }
-    *reinterpret_cast<float4*>(out + (long)row * N + col) = v;
+    float* dst = out + (long)row * N + col;
+    if (EPI == 4 && col >= kv.D) {                       // a K or V column: into the cache row of the token
+      const int which = col / kv.D - 1, b = row / kv.n, token = kv.idx ? kv.idx[row] : row - b * kv.n;
+      dst = reinterpret_cast<float*>(kv.cache) + (((long)which * kv.B + b) * kv.S + token) * kv.D + col - (which + 1) * kv.D;
+    }
+    *reinterpret_cast<float4*>(dst) = v;
   }
 }
 
 template <int T, int CS, int EPI>
 cudaError_t launch_one(const float* a, int lda, int M, const float* w, const float* bias, int N, int K, float* out,
-                       cudaStream_t st) {
+                       const KvScatter& kv, cudaStream_t st) {
   const size_t smem = ((size_t)kStagesSimt * 2 * T * (KC + kRowPad) + (CS > 1 ? T * T : 0)) * sizeof(float);
   static_assert(kStagesSimt * 2 * (KC + kRowPad) >= kGroups * T, "the groups' partial sums lie over the ring");
   static size_t smem_set[kMaxDevices] = {};
@@ -182,41 +189,47 @@ cudaError_t launch_one(const float* a, int lda, int M, const float* w, const flo
   if (e != cudaSuccess) return e;
   const int vec = lda % 4 == 0 && ((((uintptr_t)a | (uintptr_t)w)) & 15) == 0;
   return launch_pdl_cluster(gemm_simt_kernel<T, CS, EPI>, dim3(CS * (N / T) * ((M + T - 1) / T)), dim3(kGemmThreads), smem, CS,
-                            st, a, lda, M, w, bias, N, K, out, vec);
+                            st, a, lda, M, w, bias, N, K, out, kv, vec);
 }
 
-// Estimated microseconds: a fixed cost, the cluster exchange, then the FMA work of the busiest SM at 128 a clock over the
-// share of it that the micro-tiles reach: 8 x 8 load 16 words per 64 FMAs, 4 x 4 8 words per 16.
+// Estimated microseconds, fitted to the measured times of every tile and cluster size (M 10 to 1700, N 256 to 1024, K 256 and
+// 1024): a K column of a 32 x 32 tile takes 14.6 ns alone on an SM and 12.1 with others, one of a 64 x 64 tile 35 and 42
+// (LDS.128 issue bounds both: 8 loads per 64 and 16 per 256 FMAs); a cluster costs its start and exchange, more so where
+// CTAs queue.  M x N x K, us, one CTA per tile -> chosen: 20 x 256 x 1024 15.6 -> 3.6, 40 x 768 x 256 4.4 -> 3.9.
 double simt_cost(int M, int N, int K, int t, int cs) {
   if (N % t || K % (16 * cs)) return 1e30;
-  const double ctas = (double)((M + t - 1) / t) * (N / t) * cs;
-  double rounds = ctas / device_sm_count();
-  if (rounds < 1.0) rounds = 1.0;
-  const double fma_us = (double)t * t * K / cs / 128.0 / 1900.0;
-  return 2.5 + (cs > 1 ? 0.8 : 0.0) + rounds * fma_us * (t == 64 ? 1.4 : 2.2);
+  const double load = (double)((M + t - 1) / t) * (N / t) * cs / device_sm_count(), k = (double)K / cs;
+  const double cost = load <= 1.0 ? 0.8 + k * (t == 32 ? 14.6e-3 : 35e-3) : 0.6 + std::ceil(load) * k * (t == 32 ? 12.1e-3 : 42e-3);
+  return cs == 1 ? cost : cost + 0.4 + 0.15 * cs + (load > 1.0 ? 2.0 : 0.0);
 }
 
 }  // namespace
 
 cudaError_t launch_gemm_simt(const float* a, int lda, int M, const float* w, const float* bias,
-                             int N, int K, int epilogue, float* out, cudaStream_t st) {
+                             int N, int K, int epilogue, float* out, cudaStream_t st, const KvScatter* kv_scatter) {
   if (M == 0) return cudaSuccess;
   if (N % 64 || K % 16) return cudaErrorInvalidValue;
+  KvScatter kv = {nullptr, nullptr, 1, 1, 1, 1 << 30};
+  if (epilogue == 4) {
+    if (!kv_scatter || !kv_scatter->cache || N != 3 * kv_scatter->D || ((uintptr_t)kv_scatter->cache & 15)) return cudaErrorInvalidValue;
+    kv = *kv_scatter;
+  }
   int t = 64, cs = 1;
   double best = 1e30;
   for (int ti = 32; ti <= 64; ti *= 2)
-    for (int c = 1; c <= 4; c *= 2) {
+    for (int c = 1; c <= (ti == 32 ? 8 : 1); c *= 2) {
       const double cost = simt_cost(M, N, K, ti, c);
       if (cost < best) { best = cost; t = ti; cs = c; }
     }
 #define MARCHE_SIMT_CASE(T_, CS_)                                                                          \
   if (t == T_ && cs == CS_) {                                                                              \
-    if (epilogue == 0) return launch_one<T_, CS_, 0>(a, lda, M, w, bias, N, K, out, st);                   \
-    if (epilogue == 1) return launch_one<T_, CS_, 1>(a, lda, M, w, bias, N, K, out, st);                   \
-    if (epilogue == 2) return launch_one<T_, CS_, 2>(a, lda, M, w, bias, N, K, out, st);                   \
+    if (epilogue == 0) return launch_one<T_, CS_, 0>(a, lda, M, w, bias, N, K, out, kv, st);               \
+    if (epilogue == 1) return launch_one<T_, CS_, 1>(a, lda, M, w, bias, N, K, out, kv, st);               \
+    if (epilogue == 2) return launch_one<T_, CS_, 2>(a, lda, M, w, bias, N, K, out, kv, st);               \
+    if (epilogue == 4) return launch_one<T_, CS_, 4>(a, lda, M, w, bias, N, K, out, kv, st);               \
   }
   MARCHE_SIMT_CASE(32, 1) MARCHE_SIMT_CASE(32, 2) MARCHE_SIMT_CASE(32, 4)
-  MARCHE_SIMT_CASE(64, 1) MARCHE_SIMT_CASE(64, 2) MARCHE_SIMT_CASE(64, 4)
+  MARCHE_SIMT_CASE(32, 8) MARCHE_SIMT_CASE(64, 1)
 #undef MARCHE_SIMT_CASE
   return cudaErrorInvalidValue;
 }

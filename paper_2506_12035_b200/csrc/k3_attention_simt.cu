@@ -20,19 +20,19 @@ namespace marche {
 
 namespace {
 
-constexpr int kAttWarps = 8, kRows = 16, kKeys = 64;
+constexpr int kAttWarps = 8, kAttThreads = kAttWarps * 32, kKeys = 64;
 
 struct SimtLayout {                                      // in floats
   int ld, p_ld, tile, q, p, colsum, kv, total;
 };
-__host__ __device__ inline SimtLayout simt_layout(int S, int dh, int stages) {
+__host__ __device__ inline SimtLayout simt_layout(int S, int dh, int stages, int rows) {
   SimtLayout l;
   l.ld = dh + 4;                                         // rows 16 bytes apart modulo 128: conflict-free 128-bit reads
   l.p_ld = (S + kKeys - 1) / kKeys * kKeys + 4;
   l.tile = kKeys * l.ld;
   l.q = 0;
-  l.p = l.q + kRows * l.ld;
-  l.colsum = l.p + kRows * l.p_ld;
+  l.p = l.q + rows * l.ld;
+  l.colsum = l.p + rows * l.p_ld;
   l.kv = l.colsum + (S + 3) / 4 * 4;
   l.total = l.kv + stages * l.tile;
   return l;
@@ -42,15 +42,16 @@ MARCHE_DEVINL float dot4(float4 x, float4 y, float acc) {
   return fmaf(x.w, y.w, fmaf(x.z, y.z, fmaf(x.y, y.y, fmaf(x.x, y.x, acc))));
 }
 
-// NST K/V tiles in flight.  vec: q and the cache allow 16-byte copies.
-template <int NST>
-__global__ void __launch_bounds__(kAttWarps * 32)
+// NST K/V tiles in flight, RW queries per warp.  vec: the cache allows 16-byte copies.
+template <int NST, int RW>
+__global__ void __launch_bounds__(kAttThreads)
 attention_simt_kernel(const float* __restrict__ q, int ld_q, int n, int S, int H, int dh, int cs,
                       const float* __restrict__ cache_layer, long kv_stride, const uint8_t* __restrict__ is_new,
                       float* __restrict__ score_partial, float* __restrict__ o, int vec) {
+  constexpr int kRows = RW * kAttWarps;
   extern __shared__ float4 smem_f4[];
   float* smem = reinterpret_cast<float*>(smem_f4);
-  const SimtLayout l = simt_layout(S, dh, NST);
+  const SimtLayout l = simt_layout(S, dh, NST, kRows);
   float *qs = smem + l.q, *p = smem + l.p, *colsum = smem + l.colsum, *kv = smem + l.kv;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rank = cs > 1 ? (int)ptx::cluster_ctarank() : 0, item = (int)blockIdx.x / cs;
@@ -60,96 +61,124 @@ attention_simt_kernel(const float* __restrict__ q, int ld_q, int n, int S, int H
   const int n_kv = (S + kKeys - 1) / kKeys, dv = dh / 4;
   const float scale = rsqrtf((float)dh);
   const uint32_t kv_base = ptx::smem_u32(kv);
+  __shared__ bool flag[kRows];                           // scoring queries among the CTA's
   if (is_new)
-    for (int t = tid; t < S; t += kAttWarps * 32) colsum[t] = 0.f;
+    for (int t = tid; t < S; t += kAttThreads) colsum[t] = 0.f;
   pdl_sync();
 
   for (int r0 = row_begin; r0 < row_end; r0 += kRows) {
     const int rows = row_end - r0 < kRows ? row_end - r0 : kRows;
-    auto load = [&](int i) {                             // K tiles 0 .. n_kv - 1, then the V tiles
+    // tile i of K tiles 0 .. n_kv - 1, then the V tiles; whole groups of four keys, zeros beyond S
+    auto load = [&](int i) {
       if (i < 2 * n_kv) {
         const int t0 = (i < n_kv ? i : i - n_kv) * kKeys;
         const float* src = Kb + (i < n_kv ? 0 : kv_stride);
         const uint32_t dst = kv_base + 4u * (uint32_t)((i % NST) * l.tile);
-        for (int e = tid; e < kKeys * dv; e += kAttWarps * 32) {
-          const int t = e / dv, v = e - t * dv, bytes = t0 + t < S ? (vec ? 16 : 4) : 0;
-          const float* s = src + (long)(t0 + t < S ? t0 + t : 0) * D + 4 * v;
-          const uint32_t d = dst + 4u * (uint32_t)(t * l.ld + 4 * v);
-          if (vec) {
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(s), "r"(bytes) : "memory");
-          } else {
+        for (int t = tid >> 4; t < kKeys && t0 + (t & ~3) < S; t += kAttThreads / 16)
+          for (int v = tid & 15; v < dv; v += 16) {
+            const bool ok = t0 + t < S;
+            const float* s = src + (ok ? (long)(t0 + t) * D : 0L) + 4 * v;
+            const uint32_t d = dst + 4u * (uint32_t)(t * l.ld + 4 * v);
+            if (vec) {
+              asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(s), "r"(ok ? 16 : 0) : "memory");
+            } else {
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-              asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d + 4 * j), "l"(s + j), "r"(bytes) : "memory");
+              for (int j = 0; j < 4; ++j)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d + 4 * j), "l"(s + j), "r"(ok ? 4 : 0) : "memory");
+            }
           }
-        }
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
     for (int i = 0; i < NST - 1; ++i) load(i);
-    for (int e = tid; e < kRows * dh; e += kAttWarps * 32) {
-      const int r = e / dh, c = e - r * dh;
-      qs[r * l.ld + c] = r < rows ? q[((long)b * n + r0 + r) * ld_q + h * dh + c] * scale : 0.f;
+    // a warp's queries are rows warp, warp + 8; it loads them itself, so no barrier stands between
+    bool live[RW];
+    const float* qr[RW];
+    float* pr[RW];
+#pragma unroll
+    for (int r = 0; r < RW; ++r) {
+      const int row = warp + r * kAttWarps;
+      live[r] = row < rows;
+      if (is_new && lane == 0) flag[row] = live[r] && is_new[(long)b * n + r0 + row];
+      qr[r] = qs + row * l.ld;
+      pr[r] = p + row * l.p_ld;
+      for (int c = lane; c < dh; c += 32)
+        qs[row * l.ld + c] = live[r] ? q[((long)b * n + r0 + row) * ld_q + h * dh + c] * scale : 0.f;
     }
-    const int ra = warp, rb = warp + kAttWarps;          // this warp's two queries
-    float o_acc[2][2][2] = {};                           // [query][64-column half of the head][column of the lane's pair]
+    float o_acc[RW][2][2] = {};                          // [query][64-column half of the head][column of the lane's pair]
 
     for (int i = 0; i < 2 * n_kv; ++i) {
       asm volatile("cp.async.wait_group %0;" ::"n"(NST - 2) : "memory");
       __syncthreads();                                   // tile i has landed; every warp is done with tile i - 1
       load(i + NST - 1);
       const float* tile = kv + (i % NST) * l.tile;
+      const int t0 = (i < n_kv ? i : i - n_kv) * kKeys, keys = S - t0 < kKeys ? S - t0 : kKeys;
       if (i < n_kv) {
-        float s[2][2] = {};                              // logits: queries ra, rb x keys lane, lane + 32
-        const float *qa = qs + ra * l.ld, *qb = qs + rb * l.ld, *k0 = tile + lane * l.ld, *k1 = k0 + 32 * l.ld;
+        if (live[0]) {
+          float s[2][RW] = {};                           // logits: this warp's queries x keys lane, lane + 32
+          const float* kr = tile + lane * l.ld;
+          if (keys > 32) {
 #pragma unroll 4
-        for (int c = 0; c < dh; c += 4) {
-          const float4 x0 = *reinterpret_cast<const float4*>(k0 + c), x1 = *reinterpret_cast<const float4*>(k1 + c);
-          const float4 ya = *reinterpret_cast<const float4*>(qa + c), yb = *reinterpret_cast<const float4*>(qb + c);
-          s[0][0] = dot4(x0, ya, s[0][0]);
-          s[0][1] = dot4(x1, ya, s[0][1]);
-          s[1][0] = dot4(x0, yb, s[1][0]);
-          s[1][1] = dot4(x1, yb, s[1][1]);
-        }
-        const int t = i * kKeys + lane;
-        p[ra * l.p_ld + t] = t < S ? s[0][0] : -INFINITY;
-        p[ra * l.p_ld + t + 32] = t + 32 < S ? s[0][1] : -INFINITY;
-        p[rb * l.p_ld + t] = t < S ? s[1][0] : -INFINITY;
-        p[rb * l.p_ld + t + 32] = t + 32 < S ? s[1][1] : -INFINITY;
-        if (i == n_kv - 1) {
-          // ---- exact softmax of the two queries (each lane reads back what it wrote itself)
+            for (int c = 0; c < dh; c += 4) {
+              const float4 x0 = *reinterpret_cast<const float4*>(kr + c), x1 = *reinterpret_cast<const float4*>(kr + 32 * l.ld + c);
 #pragma unroll
-          for (int r = 0; r < 2; ++r) {
-            float* pr = p + (r ? rb : ra) * l.p_ld;
+              for (int r = 0; r < RW; ++r) {
+                const float4 y = *reinterpret_cast<const float4*>(qr[r] + c);
+                s[0][r] = dot4(x0, y, s[0][r]);
+                s[1][r] = dot4(x1, y, s[1][r]);
+              }
+            }
+          } else {
+#pragma unroll 4
+            for (int c = 0; c < dh; c += 4) {
+              const float4 x0 = *reinterpret_cast<const float4*>(kr + c);
+#pragma unroll
+              for (int r = 0; r < RW; ++r) s[0][r] = dot4(x0, *reinterpret_cast<const float4*>(qr[r] + c), s[0][r]);
+            }
+          }
+#pragma unroll
+          for (int r = 0; r < RW; ++r) {
+            pr[r][t0 + lane] = lane < keys ? s[0][r] : -INFINITY;
+            pr[r][t0 + lane + 32] = lane + 32 < keys ? s[1][r] : -INFINITY;
+          }
+        }
+        if (i == n_kv - 1) {
+          // ---- exact softmax (each lane reads back what it wrote itself)
+#pragma unroll
+          for (int r = 0; r < RW; ++r) {
+            if (!live[r]) continue;
             float mx = -INFINITY, sum = 0.f;
-            for (int u = lane; u < n_kv * kKeys; u += 32) mx = fmaxf(mx, pr[u]);
+            for (int u = lane; u < n_kv * kKeys; u += 32) mx = fmaxf(mx, pr[r][u]);
             mx = warp_max(mx);
             for (int u = lane; u < n_kv * kKeys; u += 32) {
-              const float e = expf(pr[u] - mx);
-              pr[u] = e;
+              const float e = expf(pr[r][u] - mx);
+              pr[r][u] = e;
               sum += e;
             }
             const float inv = 1.0f / warp_sum(sum);
-            for (int u = lane; u < n_kv * kKeys; u += 32) pr[u] *= inv;
+            for (int u = lane; u < n_kv * kKeys; u += 32) pr[r][u] *= inv;
           }
           __syncwarp();
           if (is_new) {
-            __syncthreads();                             // all 16 queries' probabilities
-            for (int t2 = tid; t2 < S; t2 += kAttWarps * 32) {
-              float cs_t = colsum[t2];
-              for (int r = 0; r < rows; ++r)
-                if (is_new[(long)b * n + r0 + r]) cs_t += p[r * l.p_ld + t2];
-              colsum[t2] = cs_t;
+            __syncthreads();                             // the CTA's probabilities, added in query order
+            for (int t = tid; t < S; t += kAttThreads) {
+              float sum = colsum[t];
+#pragma unroll
+              for (int r = 0; r < kRows; ++r)
+                if (flag[r]) sum += p[r * l.p_ld + t];
+              colsum[t] = sum;
             }
           }
         }
-      } else {
-        const int t0 = (i - n_kv) * kKeys;
-        const float *pa = p + ra * l.p_ld + t0, *pb = p + rb * l.p_ld + t0;
+      } else if (live[0]) {
 #pragma unroll 4
-        for (int t = 0; t < kKeys; t += 4) {             // (keys beyond S: zero probabilities times zeros)
-          const float4 wa = *reinterpret_cast<const float4*>(pa + t), wb = *reinterpret_cast<const float4*>(pb + t);
-          const float va[4] = {wa.x, wa.y, wa.z, wa.w}, vb[4] = {wb.x, wb.y, wb.z, wb.w};
+        for (int t = 0; t < keys; t += 4) {              // (the last group may reach beyond S: zero weights times zeros)
+          float w[RW][4];
+#pragma unroll
+          for (int r = 0; r < RW; ++r) {
+            const float4 x = *reinterpret_cast<const float4*>(pr[r] + t0 + t);
+            w[r][0] = x.x; w[r][1] = x.y; w[r][2] = x.z; w[r][3] = x.w;
+          }
 #pragma unroll
           for (int half = 0; half < 2; ++half) {
             const int c = 64 * half + 2 * lane;
@@ -157,10 +186,11 @@ attention_simt_kernel(const float* __restrict__ q, int ld_q, int n, int S, int H
 #pragma unroll
               for (int u = 0; u < 4; ++u) {
                 const float2 x = *reinterpret_cast<const float2*>(tile + (t + u) * l.ld + c);
-                o_acc[0][half][0] = fmaf(va[u], x.x, o_acc[0][half][0]);
-                o_acc[0][half][1] = fmaf(va[u], x.y, o_acc[0][half][1]);
-                o_acc[1][half][0] = fmaf(vb[u], x.x, o_acc[1][half][0]);
-                o_acc[1][half][1] = fmaf(vb[u], x.y, o_acc[1][half][1]);
+#pragma unroll
+                for (int r = 0; r < RW; ++r) {
+                  o_acc[r][half][0] = fmaf(w[r][u], x.x, o_acc[r][half][0]);
+                  o_acc[r][half][1] = fmaf(w[r][u], x.y, o_acc[r][half][1]);
+                }
               }
             }
           }
@@ -168,25 +198,25 @@ attention_simt_kernel(const float* __restrict__ q, int ld_q, int n, int S, int H
       }
     }
 #pragma unroll
-    for (int r = 0; r < 2; ++r)
+    for (int r = 0; r < RW; ++r)
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
-        const int row = r ? rb : ra, c = 64 * half + 2 * lane;
-        if (row < rows && c < dh) {
-          float* dst = o + ((long)b * n + r0 + row) * D + h * dh + c;
+        const int c = 64 * half + 2 * lane;
+        if (live[r] && c < dh) {
+          float* dst = o + ((long)b * n + r0 + warp + r * kAttWarps) * D + h * dh + c;
           dst[0] = o_acc[r][half][0];
           dst[1] = o_acc[r][half][1];
         }
       }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncthreads();                                     // the next 16 queries reuse the buffers
+    __syncthreads();                                     // the next queries reuse the buffers
   }
 
   if (is_new) {
     // ---- column sums of the cluster, rank r finishing every cs-th group of keys
     __syncthreads();
     if (cs > 1) ptx::cluster_sync_all();
-    for (int t = rank * kAttWarps * 32 + tid; t < S; t += cs * kAttWarps * 32) {
+    for (int t = rank * kAttThreads + tid; t < S; t += cs * kAttThreads) {
       float sum = 0.f;
       for (int src = 0; src < cs; ++src) {
         float v;
@@ -199,15 +229,15 @@ attention_simt_kernel(const float* __restrict__ q, int ld_q, int n, int S, int H
   }
 }
 
-template <int NST>
+template <int NST, int RW>
 cudaError_t launch_stages(const float* q, int ld_q, int B, int n, int S, int H, int dh, int cs, const float* cache_layer,
                           const uint8_t* is_new, float* score_partial, float* o, cudaStream_t st) {
-  const size_t smem = (size_t)simt_layout(S, dh, NST).total * sizeof(float);
+  const size_t smem = (size_t)simt_layout(S, dh, NST, RW * kAttWarps).total * sizeof(float);
   static size_t smem_set[kMaxDevices] = {};
-  cudaError_t e = ensure_dynamic_smem(attention_simt_kernel<NST>, smem, smem_set);
+  cudaError_t e = ensure_dynamic_smem(attention_simt_kernel<NST, RW>, smem, smem_set);
   if (e != cudaSuccess) return e;
   const int vec = (((uintptr_t)cache_layer) & 15) == 0;
-  return launch_pdl_cluster(attention_simt_kernel<NST>, dim3(B * H * cs), dim3(kAttWarps * 32), smem, cs, st, q, ld_q, n, S, H,
+  return launch_pdl_cluster(attention_simt_kernel<NST, RW>, dim3(B * H * cs), dim3(kAttThreads), smem, cs, st, q, ld_q, n, S, H,
                             dh, cs, cache_layer, (long)B * S * H * dh, is_new, score_partial, o, vec);
 }
 
@@ -217,13 +247,18 @@ cudaError_t launch_attention_simt(const float* q, int ld_q, int B, int n, int S,
                                   const float* cache_layer, const uint8_t* is_new, float* score_partial,
                                   float* o, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  // CTAs per item: one per 16 queries, as long as the launch stays within a few CTAs per SM
+  // CTAs per item: one per 8 queries (one query per warp) while the launch stays within a few CTAs per SM; with more
+  // queries than that a warp takes two, which share every key and value it reads
   int cs = 1;
-  while (cs < 8 && cs * kRows < n && B * H * cs * 2 <= 4 * device_sm_count()) cs *= 2;
+  while (cs < 8 && cs * kAttWarps < n && B * H * cs * 2 <= 4 * device_sm_count()) cs *= 2;
+  const bool one = cs * kAttWarps >= n;
   // four tiles in flight where two CTAs per SM still fit, else two
-  return simt_layout(S, dh, 4).total * sizeof(float) <= 112 * 1024
-             ? launch_stages<4>(q, ld_q, B, n, S, H, dh, cs, cache_layer, is_new, score_partial, o, st)
-             : launch_stages<2>(q, ld_q, B, n, S, H, dh, cs, cache_layer, is_new, score_partial, o, st);
+  const bool deep = simt_layout(S, dh, 4, one ? kAttWarps : 2 * kAttWarps).total * sizeof(float) <= 112 * 1024;
+  if (one)
+    return deep ? launch_stages<4, 1>(q, ld_q, B, n, S, H, dh, cs, cache_layer, is_new, score_partial, o, st)
+                : launch_stages<2, 1>(q, ld_q, B, n, S, H, dh, cs, cache_layer, is_new, score_partial, o, st);
+  return deep ? launch_stages<4, 2>(q, ld_q, B, n, S, H, dh, cs, cache_layer, is_new, score_partial, o, st)
+              : launch_stages<2, 2>(q, ld_q, B, n, S, H, dh, cs, cache_layer, is_new, score_partial, o, st);
 }
 
 }  // namespace marche

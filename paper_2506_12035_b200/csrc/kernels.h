@@ -55,19 +55,21 @@ cudaError_t launch_topk(const float* partial, int H, float* scores, const int32_
                         const int32_t* excl_idx, int n_excl, int B, int S, int k, int32_t* refresh_idx, cudaStream_t st,
                         int policy = 0, uint32_t seed = 0);
 
-// K2 of the fp32 configuration (SIMT, fp32 operands and outputs).
-cudaError_t launch_gemm_simt(const float* a, int lda, int M, const float* w, const float* bias,
-                             int N, int K, int epilogue, float* out, cudaStream_t st);
-
 // Where the K and V columns of a fused QKV projection go (Algorithm 1 line 11 done by the projection's
 // epilogue, epilogue code 4): row r of the GEMM is active token j = r % n of sample b = r / n, its cache row is
-// idx[r] (identity when idx is NULL).  cache is one block's [2][B][S][D] slice (bf16).  Needs N == 3 D,
+// idx[r] (identity when idx is NULL).  cache is one block's [2][B][S][D] slice (bf16, or fp32
+// in an fp32 context).  Needs N == 3 D,
 // D a multiple of 256 and 2 B S D < 2^31.
 struct KvScatter {
   const int32_t* idx;
   void* cache;
   int n, S, B, D;
 };
+
+// K2 of the fp32 configuration (SIMT, fp32 operands and outputs).
+cudaError_t launch_gemm_simt(const float* a, int lda, int M, const float* w, const float* bias,
+                             int N, int K, int epilogue, float* out, cudaStream_t st,
+                             const KvScatter* kv_scatter = nullptr);
 
 // K2 (16-bit operands, tcgen05/TMEM fed by TMA), many rows: tcgen05.mma cta_group::2, CTA pairs share 256 x BN tiles
 // (cluster of 2, no multicast).  N % 128 == 0, K % 64 == 0, lda % 8 == 0, 16-byte aligned operands.  a_bf16: both

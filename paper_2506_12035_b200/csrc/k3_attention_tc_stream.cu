@@ -213,12 +213,13 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
     asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
    if (warp < W_MMA) {
     // ---------------------------------------------------------------- TMA producer of stream j
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       const int j = warp - W_PROD;
       ptx::prefetch_tensormap(&tmap_kv);
       ptx::prefetch_tensormap(&tmap_q);
       const uint64_t stream_once = ptx::l2_policy_evict_first();
-      int tl = 0;                                          // K/V tiles issued so far
+      int tl = 0, s = 0;                                   // K/V tiles issued so far; ring slot of the next
+      uint32_t phase = 1;                                  // an empty slot's first wait passes at once
       bool ok = true;
       for (int u = 0; u < n_units[j] && ok; ++u) {
         const Unit un = unit_of(j, u, n_qt, H);
@@ -226,12 +227,12 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
         ptx::mbar_expect_tx(bar(j, B_Q_FULL), Q_BYTES);
         ptx::tma_load_3d(base + OFF_Q + j * Q_BYTES, &tmap_q, un.h * DH, un.qt * QT, un.b, bar(j, B_Q_FULL));
         for (int kt = 0; kt < n_kv; ++kt, ++tl) {
-          const int s = tl % NST;
-          if (!ptx::mbar_wait(bar(j, B_KV_EMPTY + s), ((uint32_t)(tl / NST) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+          if (!ptx::mbar_wait(bar(j, B_KV_EMPTY + s), phase, abort_flag)) { ok = false; break; }
           const uint32_t dst = base + OFF_KV + (j * NST + s) * STAGE_BYTES;
           ptx::mbar_expect_tx(bar(j, B_KV_FULL + s), STAGE_BYTES);
           ptx::tma_load_3d_hint(dst, &tmap_kv, un.h * DH, kt * KT, un.b, bar(j, B_KV_FULL + s), stream_once);
           ptx::tma_load_3d_hint(dst + K_BYTES, &tmap_kv, un.h * DH, kt * KT, B + un.b, bar(j, B_KV_FULL + s), stream_once);
+          if (++s == NST) { s = 0; phase ^= 1u; }
         }
       }
       if (!ok) {
@@ -247,44 +248,66 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
     // ---------------------------------------------------------------- MMA issuer of stream j
     // Within a stream the events arrive in a fixed order (S buffer handed back, then the weights of the same
     // tile), so a plain sequence of waits is optimal: S(0); for each tile t: [S buffer free] S(t+1), [weights] P V(t).
-    if (lane == 0) {
+    // Slots, phases and descriptors are stepped and the branch is an elected one: with divisions by the tile count and
+    // descriptors built per MMA in a lane-0 branch the issuer's own instructions were a third of a tile's chain.
+    if (ptx::elect_one()) {
       const int j = warp - W_MMA;
       constexpr uint32_t idesc_s = idesc_bf16(QT, KT, false);
       constexpr uint32_t idesc_o = idesc_bf16(QT, DH, true);
       const int total = n_units[j] * n_kv;
-      const uint32_t q_addr = base + OFF_Q + j * Q_BYTES;
+      const uint32_t kv0 = base + OFF_KV + j * NST * STAGE_BYTES;
+      const uint32_t d_s = tmem_base + COL_S + (uint32_t)(j * KT), d_p = tmem_base + COL_P + (uint32_t)(j * (KT / 2)),
+                     d_o = tmem_base + COL_O + (uint32_t)(j * DH);
+      const uint64_t dq = ptx::smem_desc_k_sw128(base + OFF_Q + j * Q_BYTES), dk0 = ptx::smem_desc_k_sw128(kv0),
+                     dv0 = smem_desc_mn_sw128(kv0 + K_BYTES);
       bool ok = true;
-      auto issue_s = [&](int t) -> bool {                  // t: tile counter of the stream
-        const int i = t % n_kv, u = t / n_kv;
-        if (t > 0 && !ptx::mbar_wait(bar(j, B_S_EMPTY), (uint32_t)(t - 1) & 1u, abort_flag)) return false;
-        if (i == 0 && !ptx::mbar_wait(bar(j, B_Q_FULL), (uint32_t)u & 1u, abort_flag)) return false;
-        if (!ptx::mbar_wait(bar(j, B_KV_FULL + t % NST), (uint32_t)(t / NST) & 1u, abort_flag)) return false;
-        const uint32_t k_addr = base + OFF_KV + (j * NST + t % NST) * STAGE_BYTES;
+      uint64_t dk = dk0;                                   // state of the S = Q K^T sequence
+      int s_slot = 0, s_i = 0;
+      uint32_t s_kv_phase = 0, s_free_phase = 1, q_phase = 0;   // (a wait for the phase before the first passes at once)
+      auto issue_s = [&]() -> bool {
+        if (!ptx::mbar_wait(bar(j, B_S_EMPTY), s_free_phase, abort_flag)) return false;
+        s_free_phase ^= 1u;
+        if (s_i == 0) {
+          if (!ptx::mbar_wait(bar(j, B_Q_FULL), q_phase, abort_flag)) return false;
+          q_phase ^= 1u;
+        }
+        if (!ptx::mbar_wait(bar(j, B_KV_FULL + s_slot), s_kv_phase, abort_flag)) return false;
         ptx::tc_fence_after();
 #pragma unroll
-        for (int k = 0; k < DH / 16; ++k)
-          ptx::umma_f16(tmem_base + COL_S + (uint32_t)(j * KT), ptx::smem_desc_k_sw128(q_addr + k * 32),
-                        ptx::smem_desc_k_sw128(k_addr + k * 32), idesc_s, k ? 1u : 0u);
+        for (int k = 0; k < DH / 16; ++k) ptx::umma_f16(d_s, dq + 2 * k, dk + 2 * k, idesc_s, k ? 1u : 0u);
         ptx::umma_commit(bar(j, B_S_FULL));
-        if (i == n_kv - 1) ptx::umma_commit(bar(j, B_Q_EMPTY));   // the unit's last Q K^T: Q_j may be overwritten
+        if (++s_i == n_kv) {                               // the unit's last Q K^T: Q_j may be overwritten
+          s_i = 0;
+          ptx::umma_commit(bar(j, B_Q_EMPTY));
+        }
+        dk += STAGE_BYTES >> 4;
+        if (++s_slot == NST) { s_slot = 0; s_kv_phase ^= 1u; dk = dk0; }
         return true;
       };
-      if (total > 0) ok = issue_s(0);
+      uint64_t dv = dv0;                                   // state of the O += P V sequence
+      int o_slot = 0, o_i = 0;
+      uint32_t p_phase = 0, o_free_phase = 1;
+      if (total > 0) ok = issue_s();
       for (int t = 0; t < total && ok; ++t) {
-        const int i = t % n_kv, u = t / n_kv;
-        if (t + 1 < total && !issue_s(t + 1)) { ok = false; break; }
+        if (t + 1 < total && !issue_s()) { ok = false; break; }
         // O_j += P_j V: needs the weights, and for a unit's first tile the previous output read out
-        if (!ptx::mbar_wait(bar(j, B_P_FULL), (uint32_t)t & 1u, abort_flag)) { ok = false; break; }
-        if (i == 0 && u > 0 && !ptx::mbar_wait(bar(j, B_O_FREE), (uint32_t)(u - 1) & 1u, abort_flag)) { ok = false; break; }
-        const uint32_t v_addr = base + OFF_KV + (j * NST + t % NST) * STAGE_BYTES + K_BYTES;
+        if (!ptx::mbar_wait(bar(j, B_P_FULL), p_phase, abort_flag)) { ok = false; break; }
+        p_phase ^= 1u;
+        if (o_i == 0) {
+          if (!ptx::mbar_wait(bar(j, B_O_FREE), o_free_phase, abort_flag)) { ok = false; break; }
+          o_free_phase ^= 1u;
+        }
         ptx::tc_fence_after();
 #pragma unroll
-        for (int k = 0; k < KT / 16; ++k)
-          umma_f16_ts(tmem_base + COL_O + (uint32_t)(j * DH), tmem_base + COL_P + (uint32_t)(j * (KT / 2) + k * 8),
-                      smem_desc_mn_sw128(v_addr + k * 2048), idesc_o, (i == 0 && k == 0) ? 0u : 1u);
-        ptx::umma_commit(bar(j, B_KV_EMPTY + t % NST));    // K was read by the S of this tile, V just now
+        for (int k = 0; k < KT / 16; ++k) umma_f16_ts(d_o, d_p + 8u * k, dv + 128 * k, idesc_o, (o_i | k) ? 1u : 0u);
+        ptx::umma_commit(bar(j, B_KV_EMPTY + o_slot));     // K was read by the S of this tile, V just now
         ptx::umma_commit(bar(j, B_P_EMPTY));
-        if (i == n_kv - 1) ptx::umma_commit(bar(j, B_O_FULL));
+        if (++o_i == n_kv) {
+          o_i = 0;
+          ptx::umma_commit(bar(j, B_O_FULL));
+        }
+        dv += STAGE_BYTES >> 4;
+        if (++o_slot == NST) { o_slot = 0; dv = dv0; }
       }
       if (!ok) *(volatile int*)status = ST_ATT_STREAM;
     }
@@ -336,13 +359,30 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
           // lazy reference maximum: move it only when this tile exceeds it by more than 2^8
           move = (tmax - m_ref) * c_log2 > 8.0f;           // also true for a unit's first tile (m_ref = -inf)
         }
+        const float f = move ? ex2_approx((m_ref - tmax) * c_log2) : 1.0f;   // (0 for a unit's first tile)
+        if (move) m_ref = tmax;
+        const float neg = -m_ref * c_log2;
+        // weights: p = 2^((s - m_ref) / sqrt(d) * log2 e), packed bf16 pairs, in place (pair c -> v[c]).  The first half is
+        // computed while the previous P_j V still runs
+        float ls[4] = {0.f, 0.f, 0.f, 0.f};
+        auto weights = [&](int c) {
+          float x0, x1;
+          ffma2_bcast(__uint_as_float(v[2 * c]), __uint_as_float(v[2 * c + 1]), c_log2, neg, x0, x1);
+          const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
+          fadd2(ls[2 * (c & 1)], ls[2 * (c & 1) + 1], p0, p1);
+          v[c] = pack_bf16x2(p0, p1);
+        };
+        if (warp_valid && lim >= KT) {
+#pragma unroll
+          for (int c = 0; c < KT / 4; ++c) weights(c);
+        }
         // the previous P_j V has read the weights we are about to overwrite, and has finished adding to O_j
         if (t > 0 && !ptx::mbar_wait(bar(j, B_P_EMPTY), (uint32_t)(t - 1) & 1u, abort_flag)) { ok = false; break; }
         ptx::tc_fence_after();
         if (warp_valid) {
+          if (lim >= KT) tmem_st_32x16(t_p, v);            // on its way while the second half is computed
           if (i > 0 && __any_sync(0xffffffffu, move)) {
             // rescale this row's accumulator in tensor memory to the new reference
-            const float f = move ? ex2_approx((m_ref - tmax) * c_log2) : 1.0f;
 #pragma unroll 1
             for (int qc = 0; qc < 4; ++qc) {
               uint32_t ov[16];
@@ -352,24 +392,11 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
               for (int c = 0; c < 16; ++c) ov[c] = __float_as_uint(__uint_as_float(ov[c]) * f);
               tmem_st_32x16(t_o + (uint32_t)(qc * 16), ov);
             }
-            l *= f;
           }
-          if (move) m_ref = tmax;
-          const float neg = -m_ref * c_log2;
-          // weights: p = 2^((s - m_ref) / sqrt(d) * log2 e), packed bf16 pairs, in place (pair c -> v[c])
-          float ls[4] = {0.f, 0.f, 0.f, 0.f};
-          bool half_stored = false;
           if (lim >= KT) {                                 // (two copies of the loop: no per-element selects on the
 #pragma unroll                                             //  common, full tile)
-            for (int c = 0; c < KT / 2; ++c) {
-              float x0, x1;
-              ffma2_bcast(__uint_as_float(v[2 * c]), __uint_as_float(v[2 * c + 1]), c_log2, neg, x0, x1);
-              const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
-              fadd2(ls[2 * (c & 1)], ls[2 * (c & 1) + 1], p0, p1);
-              v[c] = pack_bf16x2(p0, p1);
-              if (c == KT / 4 - 1) tmem_st_32x16(t_p, v);  // first half on its way while the second is computed
-            }
-            half_stored = true;
+            for (int c = KT / 4; c < KT / 2; ++c) weights(c);
+            tmem_st_32x16(t_p + 16u, v + 16);
           } else {
 #pragma unroll
             for (int c = 0; c < KT / 2; ++c) {
@@ -380,10 +407,9 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
               ls[c & 3] += p0 + p1;
               v[c] = pack_bf16x2(p0, p1);
             }
+            tmem_st_32x32(t_p, v);
           }
-          l += (ls[0] + ls[1]) + (ls[2] + ls[3]);
-          if (half_stored) tmem_st_32x16(t_p + 16u, v + 16);
-          else tmem_st_32x32(t_p, v);
+          l = (i > 0 ? l * f : 0.f) + ((ls[0] + ls[1]) + (ls[2] + ls[3]));
           tmem_st_wait();
         }
         ptx::tc_fence_before();

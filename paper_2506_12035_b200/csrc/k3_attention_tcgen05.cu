@@ -120,7 +120,7 @@ attention_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __gr
   bool ok = true;
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       ptx::prefetch_tensormap(&tmap_kv);
       ptx::prefetch_tensormap(&tmap_q);
       int it = 0;                                          // K/V loads issued so far
@@ -143,25 +143,25 @@ attention_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __gr
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       constexpr uint32_t idesc_s = idesc_bf16(QT, KT, false);
       constexpr uint32_t idesc_o = idesc_bf16(QT, DH, true);
-      const uint32_t q_addr = base + OFF_Q;
+      const uint64_t dq = ptx::smem_desc_k_sw128(base + OFF_Q), dk0 = ptx::smem_desc_k_sw128(base + OFF_KV),
+                     dp0 = ptx::smem_desc_k_sw128(base + OFF_P), dv0 = smem_desc_mn_sw128(base + OFF_KV + TILE_BYTES);
       int it = 0;        // K/V tiles consumed (ring index)
       int sc = 0;        // S accumulators produced
       int pc = 0;        // P tiles consumed
       auto s_mma = [&](int s, int a) {
 #pragma unroll
         for (int k = 0; k < DH / 16; ++k)
-          ptx::umma_f16(tmem_base + (uint32_t)(a * KT), ptx::smem_desc_k_sw128(q_addr + k * 32),
-                        ptx::smem_desc_k_sw128(base + OFF_KV + s * STAGE_BYTES + k * 32), idesc_s, k ? 1u : 0u);
+          ptx::umma_f16(tmem_base + (uint32_t)(a * KT), dq + 2 * k, dk0 + (uint32_t)(s * (STAGE_BYTES >> 4)) + 2 * k, idesc_s,
+                        k ? 1u : 0u);
       };
       auto pv_mma = [&](int s, int a, bool first) {
 #pragma unroll
         for (int k = 0; k < KT / 16; ++k)
-          ptx::umma_f16(tmem_base + 128u, ptx::smem_desc_k_sw128(base + OFF_P + a * P_BYTES + k * 32),
-                        smem_desc_mn_sw128(base + OFF_KV + s * STAGE_BYTES + TILE_BYTES + k * 2048), idesc_o,
-                        (first && k == 0) ? 0u : 1u);
+          ptx::umma_f16(tmem_base + 128u, dp0 + (uint32_t)(a * (P_BYTES >> 4)) + 2 * k,
+                        dv0 + (uint32_t)(s * (STAGE_BYTES >> 4)) + 128 * k, idesc_o, (first && k == 0) ? 0u : 1u);
       };
       for (int qt = 0; qt < n_qt && ok; ++qt) {
         if (!ptx::mbar_wait(bar(B_Q_FULL), (uint32_t)qt & 1u, abort_flag)) { ok = false; break; }

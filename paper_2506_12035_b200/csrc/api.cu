@@ -216,10 +216,10 @@ int do_linear(marche_ctx* ctx, int cls, const void* a, int lda, int M, const voi
 }
 
 int do_attention(marche_ctx* ctx, const void* q, int ld_q, int n, const void* cache_layer, const uint8_t* is_new,
-                 float* partial, void* o, cudaStream_t st, int S_kv = 0) {
+                 float* partial, void* o, cudaStream_t st, int n_new, int S_kv = 0) {
   const marche_config& c = ctx->cfg;
   const int S = S_kv > 0 ? S_kv : c.seq_len;            // tokens per sample in cache_layer [2][B][S][D]
-  if (skipped(ctx, MARCHE_KC_ATTENTION)) return MARCHE_OK;
+  if (!ctx->bf16 && skipped(ctx, MARCHE_KC_ATTENTION)) return MARCHE_OK;
   if (!ctx->bf16) {
     if (n > 0) mark(ctx, MARCHE_KC_ATTENTION, st);
     MARCHE_TRY(launch_attention_simt((const float*)q, ld_q, c.batch, n, S, c.n_heads, c.head_dim, (const float*)cache_layer,
@@ -227,6 +227,15 @@ int do_attention(marche_ctx* ctx, const void* q, int ld_q, int n, const void* ca
     return MARCHE_OK;
   }
   if (ld_q % 2 || ((uintptr_t)q & 3) || ((uintptr_t)cache_layer & 15) || ((uintptr_t)o & 15)) return misaligned(ctx, "attention");
+  if (is_new && ctx->tune.attention_kernel == MARCHE_ATTENTION_AUTO &&
+      attention_scores_wins(n, n_new, S, c.head_dim, c.batch * c.n_heads)) {
+    // the scores of the generating rows alone, then the plain attention of all rows
+    mark(ctx, MARCHE_KC_OTHER, st);
+    MARCHE_TRY(launch_attention_scores(q, ld_q, c.batch, n, S, c.n_heads, c.head_dim, cache_layer, is_new, partial,
+                                       ctx->status_dev, st), "attention_scores");
+    is_new = nullptr;
+  }
+  if (skipped(ctx, MARCHE_KC_ATTENTION)) return MARCHE_OK;
   for (int rep_i = 0; rep_i < launches_of(ctx, MARCHE_KC_ATTENTION); ++rep_i) {
   if (n > 0) mark(ctx, MARCHE_KC_ATTENTION, st);
   // Three tensor-core kernels.  At small active sets the step is bound by streaming the cache and the
@@ -291,12 +300,12 @@ StackBufs carve(void* workspace, const WsLayout& w) {
 // Blocks [l_begin, l_end) for M = B*nA rows whose token positions are idx (nullptr = identity,
 // nA == S).  When gather_src is non-null the first block's LayerNorm gathers its rows from
 // gather_src[b][idx][:] (float [B][src_rows][D]) and writes the compact residual rows to x;
-// otherwise x already holds them.  is_new (flags of the scoring queries) is used at the scoring block.
+// otherwise x already holds them.  is_new (flags of the scoring queries, n_new per sample) is used at the scoring block.
 // S_kv > 0: these blocks keep only S_kv tokens per sample, laid out [2][B][S_kv][D] at the start of each
 // block's cache slice (the encoder over the known tokens, whose K/V do not outlive the step).
 int run_blocks(marche_ctx* ctx, int l_begin, int l_end, const float* gather_src, int src_rows, const int32_t* idx,
-               int nA, float* x, const StackBufs& bf, void* kv_cache, const uint8_t* is_new, cudaStream_t st,
-               int S_kv = 0) {
+               int nA, float* x, const StackBufs& bf, void* kv_cache, const uint8_t* is_new, int n_new,
+               cudaStream_t st, int S_kv = 0) {
   const marche_config& c = ctx->cfg;
   const int B = c.batch, S = S_kv > 0 ? S_kv : c.seq_len, D = c.width, F = c.mlp_dim;
   const int M = B * nA;
@@ -327,7 +336,7 @@ int run_blocks(marche_ctx* ctx, int l_begin, int l_end, const float* gather_src,
     if (rc) return rc;
     if (fused_kv) {
       // the projection's epilogue has written K and V into the cache (Algorithm 1 line 11)
-      rc = do_attention(ctx, bf.qkv, 3 * D, nA, cache_l, flags_l, partial_l, bf.o, st, S);
+      rc = do_attention(ctx, bf.qkv, 3 * D, nA, cache_l, flags_l, partial_l, bf.o, st, n_new, S);
       if (rc) return rc;
     } else if (ctx->tune.two_segment_attention && ctx->bf16) {
       // two-segment attention: fresh K/V read in place, cache write-back by the same kernel
@@ -339,7 +348,7 @@ int run_blocks(marche_ctx* ctx, int l_begin, int l_end, const float* gather_src,
       mark(ctx, MARCHE_KC_SCATTER_KV, st);
       MARCHE_TRY(launch_scatter_kv(ctx->bf16, bf.qkv + (size_t)D * eb, bf.qkv + (size_t)2 * D * eb, 3 * D, kv_idx, B, nA,
                                    S, D, cache_l, st), "scatter_kv");
-      rc = do_attention(ctx, bf.qkv, 3 * D, nA, cache_l, flags_l, partial_l, bf.o, st,
+      rc = do_attention(ctx, bf.qkv, 3 * D, nA, cache_l, flags_l, partial_l, bf.o, st, n_new,
                         S);
       if (rc) return rc;
     }
@@ -380,7 +389,7 @@ int run_stack(marche_ctx* ctx, const float* hidden, void* kv_cache, const int32_
   if (needs_turn(ctx, B * nA)) MARCHE_TRY(cudaMemsetAsync(bf.turn, 0, w.turn_bytes, st), "memset");
   mark(ctx, MARCHE_KC_FLAGS, st);
   MARCHE_TRY(launch_step_flags(active_idx, nA, new_idx, n_new, B, S, bf.is_new, st), "flags");
-  const int rc = run_blocks(ctx, 0, L, hidden, S, active_idx, nA, bf.x, bf, kv_cache, bf.is_new, st);
+  const int rc = run_blocks(ctx, 0, L, hidden, S, active_idx, nA, bf.x, bf, kv_cache, bf.is_new, n_new, st);
   if (rc) return rc;
   mark(ctx, MARCHE_KC_SCATTER_ROWS, st);
   MARCHE_TRY(launch_scatter_rows(bf.x, active_idx, B, nA, S, D, hidden_out, st), "scatter_rows");
@@ -413,7 +422,7 @@ int run_in_step(marche_ctx* ctx, const float* hidden, void* kv_cache, const int3
   // phase 1: every token; generating rows flagged for the scores; candidates = all \ (new u prev)
   mark(ctx, MARCHE_KC_FLAGS, st);
   MARCHE_TRY(launch_step_flags(nullptr, S, new_idx, n_new, B, S, bf.is_new, st), "flags");
-  int rc = run_blocks(ctx, 0, sl + 1, hidden, S, nullptr, S, bf.x, bf, kv_cache, bf.is_new, st);
+  int rc = run_blocks(ctx, 0, sl + 1, hidden, S, nullptr, S, bf.x, bf, kv_cache, bf.is_new, n_new, st);
   if (rc) return rc;
   mark(ctx, MARCHE_KC_TOPK, st);
   MARCHE_TRY(launch_topk(bf.partial, H, bf.scores, new_idx, n_new, prev_idx, n_prev, B, S, k, refresh_idx, st),
@@ -422,7 +431,7 @@ int run_in_step(marche_ctx* ctx, const float* hidden, void* kv_cache, const int3
   MARCHE_TRY(launch_build_active(new_idx, n_new, prev_idx, n_prev, forced_refresh ? forced_refresh : refresh_idx, k, B,
                                  active_idx, st), "build_active");
   // phase 2: rows of A, gathered from the full residual rows of phase 1
-  rc = run_blocks(ctx, sl + 1, L, bf.x, S, active_idx, nA, bf.x2, bf, kv_cache, nullptr, st);
+  rc = run_blocks(ctx, sl + 1, L, bf.x, S, active_idx, nA, bf.x2, bf, kv_cache, nullptr, 0, st);
   if (rc) return rc;
   mark(ctx, MARCHE_KC_SCATTER_ROWS, st);
   MARCHE_TRY(launch_scatter_rows(bf.x2, active_idx, B, nA, S, D, hidden_out, st), "scatter_rows");
@@ -457,7 +466,7 @@ int run_mar(marche_ctx* ctx, bool full_decoder, const float* tokens, const int32
   mark(ctx, MARCHE_KC_FLAGS, st);
   MARCHE_TRY(launch_step_flags(nullptr, S, new_idx, n_new, B, S, bf.is_new, st), "flags");
   // ---- Eq. 1: encoder on the compacted known tokens; its K/V live only inside this step
-  int rc = run_blocks(ctx, 0, E, tokens, S, known_idx, n_known, bf.x, bf, kv_cache, nullptr, st, n_known);
+  int rc = run_blocks(ctx, 0, E, tokens, S, known_idx, n_known, bf.x, bf, kv_cache, nullptr, 0, st, n_known);
   if (rc) return rc;
   // ---- Eq. 2: x3[b][s] = mask + pos[s];  x3[b][known] = W_de * LN(h_enc) + b_de + pos[known]
   mark(ctx, MARCHE_KC_GATHER_LN, st);
@@ -475,7 +484,7 @@ int run_mar(marche_ctx* ctx, bool full_decoder, const float* tokens, const int32
 
   // ---- decoder
   if (full_decoder) {
-    rc = run_blocks(ctx, E, L, bf.x3, S, nullptr, S, bf.x, bf, kv_cache, bf.is_new, st);
+    rc = run_blocks(ctx, E, L, bf.x3, S, nullptr, S, bf.x, bf, kv_cache, bf.is_new, n_new, st);
     if (rc) return rc;
     mark(ctx, MARCHE_KC_TOPK, st);
     MARCHE_TRY(launch_topk(bf.partial, H, bf.scores, new_idx, n_new, prev_idx, n_prev, B, S, k, refresh_idx, st),
@@ -485,7 +494,7 @@ int run_mar(marche_ctx* ctx, bool full_decoder, const float* tokens, const int32
                                        nullptr, z_out, st), "decoder_norm");
     return MARCHE_OK;
   }
-  rc = run_blocks(ctx, E, sl + 1, bf.x3, S, nullptr, S, bf.x, bf, kv_cache, bf.is_new, st);
+  rc = run_blocks(ctx, E, sl + 1, bf.x3, S, nullptr, S, bf.x, bf, kv_cache, bf.is_new, n_new, st);
   if (rc) return rc;
   mark(ctx, MARCHE_KC_TOPK, st);
   MARCHE_TRY(launch_topk(bf.partial, H, bf.scores, new_idx, n_new, prev_idx, n_prev, B, S, k, refresh_idx, st),
@@ -493,7 +502,7 @@ int run_mar(marche_ctx* ctx, bool full_decoder, const float* tokens, const int32
   mark(ctx, MARCHE_KC_OTHER, st);
   MARCHE_TRY(launch_build_active(new_idx, n_new, prev_idx, n_prev, forced_refresh ? forced_refresh : refresh_idx, k, B,
                                  active_idx, st), "build_active");
-  rc = run_blocks(ctx, sl + 1, L, bf.x, S, active_idx, nA, bf.x2, bf, kv_cache, nullptr, st);
+  rc = run_blocks(ctx, sl + 1, L, bf.x, S, active_idx, nA, bf.x2, bf, kv_cache, nullptr, 0, st);
   if (rc) return rc;
   mark(ctx, MARCHE_KC_GATHER_LN, st);
   MARCHE_TRY(launch_gather_layernorm(OUT_F32, bf.x2, nA, nullptr, B, nA, D, mw.dec_norm_g, mw.dec_norm_b, ctx->eps,
@@ -813,7 +822,7 @@ int marche_attention(marche_ctx* ctx, const void* q, int ld_q, int n, const void
     return MARCHE_EINVAL;
   if (is_new && !score_partial) return MARCHE_EINVAL;
   MARCHE_ENTER(ctx);
-  return do_attention(ctx, q, ld_q, n, cache_layer, is_new, score_partial, o, (cudaStream_t)stream);
+  return do_attention(ctx, q, ld_q, n, cache_layer, is_new, score_partial, o, (cudaStream_t)stream, n);
 }
 
 int marche_gather_rows(marche_ctx* ctx, const float* src, const int32_t* idx, int n, float* rows_out,

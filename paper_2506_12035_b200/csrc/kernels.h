@@ -123,6 +123,12 @@ bool attention_split_wins(int n, int S, int dh, int items);
 cudaError_t launch_attention_split(const void* q, int ld_q, int B, int n, int S, int H, int dh, const void* cache_layer,
                                    void* o, bool o_bf16, int* status, cudaStream_t st);
 
+// K3, relevance scores of the rows flagged in is_new [B][n] alone (no attention output), for the scoring block beside a
+// plain attention.  Same alignment rules as launch_attention_mma.
+bool attention_scores_wins(int n, int n_new, int S, int dh, int items);
+cudaError_t launch_attention_scores(const void* q, int ld_q, int B, int n, int S, int H, int dh, const void* cache_layer,
+                                    const uint8_t* is_new, float* score_partial, int* status, cudaStream_t st);
+
 // K3 on tcgen05 (head_dim 64 only): S = Q K^T and O = P V as tcgen05.mma with TMEM accumulators.
 // ld_q % 8 == 0; q and cache_layer 16-byte aligned.
 cudaError_t launch_attention_tcgen05(const void* q, int ld_q, int B, int n, int S, int H, int dh,

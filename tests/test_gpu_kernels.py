@@ -657,3 +657,31 @@ def test_attention_keys_split_over_a_cluster(dh, H, B, S, n):
                 c = slice(h * dh, (h + 1) * dh)
                 want[b * n:(b + 1) * n, c], _ = orc.softmax_attention(qq[b * n:(b + 1) * n, c], cc[0, b][:, c], cc[1, b][:, c])
         assert rel_l2(host(outs[0]), want) <= 8e-3 and max_abs(host(outs[0]), want) <= 3e-2
+
+
+@pytest.mark.parametrize("dh,H", [(64, 4), (80, 8)])
+@pytest.mark.parametrize("B,S,n,nG", [(1, 1, 1, 1), (2, 64, 16, 16), (2, 65, 17, 17), (3, 320, 32, 5), (2, 1088, 32, 31), (1, 1200, 20, 0)])
+def test_attention_scores_of_the_generating_rows(dh, H, B, S, n, nG):
+    """The kernel that scores the flagged rows alone: none, one group of 16 (four warps share the tiles) and two, one to
+    nineteen key tiles; weights in fp32 from bf16 logits, so a score errs by the logits' rounding as in the attention."""
+    D = H * dh
+    cfg, blocks, m = model_for("bf16", D, H, 128, S, B)
+    rng = np.random.default_rng(B + S + n + dh)
+    q, cache = (rng.standard_normal((B * n, D)) * 3.0).astype(np.float32), rng.standard_normal((2, B, S, D)).astype(np.float32)
+    flags = np.zeros((B, n), dtype=np.uint8)
+    for b in range(B):
+        flags[b, rng.permutation(n)[:nG]] = 1
+    got = []
+    for _ in range(2):
+        o, partial = torch.zeros(B * n, D, dtype=torch.float16, device="cuda"), torch.full((B, H, S), -1.0, device="cuda")
+        m.attention(dev(q, torch.bfloat16), D, n, dev(cache, torch.bfloat16), dev(flags), partial, o)
+        got.append(partial)
+    assert torch.equal(got[0], got[1]) and m.device_status() == 0
+    qq, cc = quant(q, "bf16"), quant(cache, "bf16")
+    want = np.zeros((B, H, S))
+    for b in range(B):
+        for h in range(H):
+            c = slice(h * dh, (h + 1) * dh)
+            _, p = orc.softmax_attention(qq[b * n:(b + 1) * n, c], cc[0, b][:, c], cc[1, b][:, c])
+            want[b, h] = p[flags[b].astype(bool)].sum(axis=0)
+    assert max_abs(host(got[0]), want) <= 2e-4 * max(1, nG) and np.allclose(host(got[0]).sum(-1), nG, rtol=1e-4, atol=1e-6)

@@ -3,25 +3,29 @@
 // Appendix A), with the running-maximum / running-sum merge of Eq. 6-10 applied tile by tile.
 //
 // Persistent CTAs (one per SM).  The work of a CTA is a list of units, one unit = one 128-row query
-// tile of one (sample, head) item against all S keys; THREE independent streams inside the CTA take
+// tile of one (sample, head) item against all S keys; FOUR independent streams inside the CTA take
 // the units in turn.  A unit is a latency chain (Q K^T -> read logits -> exponentials -> write weights
-// -> P V ...), and the exponentials - 16 per clock and SM - are the scarce resource once the active set
-// is large; three chains in flight per SM partition keep those units and the tensor core busy while
-// each chain waits on its own hand-overs.  Each stream owns a query buffer, a 3-deep TMA ring of 64-key
-// K/V tiles that runs ahead across units (the HBM queue never drains between items) and accumulators in
-// tensor memory: S_j 64 columns (fp32 logits), P_j 32 columns (weights as packed bf16), O_j 64 columns.
-// Roles (20 warps; the eight control warps hand most of their registers to the twelve softmax warps):
-//   warps 0-11    softmax: warps 4j .. 4j+3 serve stream j, one thread per query row.  A thread pulls its
-//                 S row into registers (tcgen05.ld), hands the S buffer straight back so that the next
-//                 tile's Q K^T runs during the exponentials, and writes the weights to tensor memory
+// -> P V -> next Q K^T ...), and the exponentials - 16 per clock and SM - are the scarce resource once the active set
+// is large; four chains in flight per SM partition keep those units busy while each chain waits on its hand-overs.
+// Each stream owns a query buffer, TMA rings of 64-key tiles (three of K, two of V: a K tile is used up a step earlier)
+// that run ahead across units and 128 columns of tensor memory: S_j 64 columns (fp32 logits), whose first 32 the
+// weights P_j (packed bf16) overwrite, and O_j 64 columns.  So P V of a tile and Q K^T of the next are issued together,
+// in the order in which the tensor core executes them, and one barrier per tile tells the softmax that both are done:
+// its weights may be overwritten, its accumulator rescaled, its logits read.
+// Roles (24 warps of 80 registers a thread):
+//   warps 0-15    softmax: warps 4j .. 4j+3 serve stream j, one thread per query row.  A thread pulls its
+//                 S row into registers (tcgen05.ld; the first half again for its exponentials, since 80 registers do
+//                 not hold a row and its weights) and writes the weights to tensor memory
 //                 (tcgen05.st), from where the tensor core reads them as the A operand of P V
-//   warps 12-14   TMA producer of stream 0 / 1 / 2: Q tile per unit, K/V ring
-//   warps 15-17   issue tcgen05.mma for stream 0 / 1 / 2: S_j = Q_j K^T (M128 x N64 x K64) as soon as the S
-//                 buffer is free, O_j += P_j V (M128 x N64 x K64, V as an MN-major operand from shared
-//                 memory) as soon as the weights are there; warp 17 also allocates / frees tensor memory
+//   warps 16-19   TMA producer of stream 0 .. 3: Q tile per unit, K and V rings
+//   warps 20-23   issue tcgen05.mma for stream 0 .. 3: O_j += P_j V (M128 x N64 x K64, V as an MN-major operand from
+//                 shared memory) as soon as the weights are there, then S_j = Q_j K^T (M128 x N64 x K64) of the next
+//                 tile; warp 23 also allocates / frees tensor memory
+// A warp can only reach the tensor-memory lanes of its quarter, and a quarter is one SM partition.  A query tile of
+// fewer than 97 rows is therefore placed on other lanes by other streams, so that the partitions share the work.
 // Online softmax with a lazy reference maximum: the exponent reference of a row only moves when a
 // tile's maximum exceeds it by more than 2^8 in the exponent, and only then is the row's O accumulator
-// rescaled in tensor memory (by the row's own thread, after the previous P V has completed); weights
+// rescaled in tensor memory (by the row's own thread); weights
 // therefore never exceed 256 and the final division by the row sum makes the result exact up to
 // rounding.  All waits are bounded and report through the status word.
 #include <cuda.h>
@@ -38,29 +42,28 @@ namespace {
 constexpr int DH = 64;
 constexpr int QT = 128;                    // query rows per unit (= TMEM lanes)
 constexpr int KT = 64;                     // keys per tile
-constexpr int NS = 3;                      // streams per CTA
-constexpr int NST = 3;                     // K/V ring stages per stream
-constexpr int K_BYTES = KT * DH * 2;       // 8 KB
-constexpr int STAGE_BYTES = 2 * K_BYTES;   // K tile then V tile
+constexpr int NS = 4;                      // streams per CTA
+constexpr int NK = 3, NV = 2;              // K and V tiles in flight per stream
+constexpr int T_BYTES = KT * DH * 2;       // a K or V tile: 8 KB
 constexpr int Q_BYTES = QT * DH * 2;       // 16 KB
-constexpr int kThreads = 640;               // 12 softmax warps, then 8 control warps: 3 producers, 3 MMA issuers, 2 idle
+constexpr int kThreads = 768;               // 16 softmax warps, 4 producers, 4 MMA issuers
 constexpr int W_PROD = NS * 4, W_MMA = NS * 5;   // (whole groups of four warps, as the register reallocation requires)
 constexpr int TMEM_COLS = 512;
-constexpr uint32_t COL_S = 0;                       // S_j: KT columns each
-constexpr uint32_t COL_P = NS * KT;                 // P_j: KT / 2 columns each (KT bf16)
-constexpr uint32_t COL_O = COL_P + NS * (KT / 2);   // O_j: 64 columns each
-static_assert(COL_O + NS * DH <= TMEM_COLS, "tensor memory budget");
+constexpr uint32_t COL_STREAM = 128, COL_O = 64;   // stream j: S_j (and P_j over it) at 128 j, O_j at 128 j + 64
+static_assert(NS * COL_STREAM <= TMEM_COLS, "tensor memory budget");
 enum { ST_ATT_STREAM = 0x51 };
 
 // shared memory (from a 1024-byte aligned base)
 constexpr int OFF_Q = 0;                                   // [stream]
-constexpr int OFF_KV = OFF_Q + NS * Q_BYTES;               // [stream][stage]
-constexpr int OFF_BAR = OFF_KV + NS * NST * STAGE_BYTES;
+constexpr int OFF_K = OFF_Q + NS * Q_BYTES;                // [stream][slot]
+constexpr int OFF_V = OFF_K + NS * NK * T_BYTES;           // [stream][slot]
+constexpr int OFF_BAR = OFF_V + NS * NV * T_BYTES;
 // barriers of one stream (8 bytes each); stream j's block starts at j * NB
-enum { B_KV_FULL = 0, B_KV_EMPTY = NST, B_Q_FULL = 2 * NST, B_Q_EMPTY, B_S_FULL, B_S_EMPTY, B_P_FULL, B_P_EMPTY, B_O_FULL,
-       B_O_FREE, NB };
+enum { B_K_FULL = 0, B_K_EMPTY = B_K_FULL + NK, B_V_FULL = B_K_EMPTY + NK, B_V_EMPTY = B_V_FULL + NV, B_Q_FULL = B_V_EMPTY + NV,
+       B_Q_EMPTY, B_S_FULL, B_P_FULL, B_O_FULL, NB };
 constexpr int OFF_MISC = OFF_BAR + 8 * NS * NB;            // tmem slot (4), abort flags (8)
 constexpr int SMEM_BYTES = OFF_MISC + 32 + 1024;
+static_assert(SMEM_BYTES <= 227 * 1024, "shared memory of one CTA");
 
 MARCHE_DEVINL constexpr uint32_t idesc_bf16(int M, int N, bool b_mn_major) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (b_mn_major ? (1u << 16) : 0u) | ((uint32_t)(N >> 3) << 17) |
@@ -86,13 +89,6 @@ MARCHE_DEVINL void umma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc
       : "memory");
 }
 // 32 lanes x N consecutive 32-bit columns: thread i of the warp accesses lane (base + i).
-MARCHE_DEVINL void tmem_ld_32x64(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, %48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%64];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]), "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]), "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
-      : "r"(taddr)
-      : "memory");
-}
 MARCHE_DEVINL void tmem_ld_32x16(uint32_t taddr, uint32_t* r) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
@@ -104,17 +100,6 @@ MARCHE_DEVINL void tmem_st_32x16(uint32_t taddr, const uint32_t* r) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
       ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-      : "memory");
-}
-MARCHE_DEVINL void tmem_st_32x32(uint32_t taddr, const uint32_t* r) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]),
-        "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]),
-        "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
       : "memory");
 }
 MARCHE_DEVINL void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
@@ -151,16 +136,30 @@ MARCHE_DEVINL float ex2_approx(float x) {
   return y;
 }
 
-// The CTA's units in order: unit k = query tile (k % n_qt) of the CTA's (k / n_qt)-th item; stream j
-// takes k = j, j + NS, ...
-struct Unit { int b, h, qt; };
-MARCHE_DEVINL Unit unit_of(int j, int u, int n_qt, int H) {
-  const int k = NS * u + j;
-  const int item = (int)blockIdx.x + (k / n_qt) * (int)gridDim.x;
+// Unit k of a CTA: query tile (k % n_qt) of its (k / n_qt)-th item; stream j takes k = j, j + NS, ...  Items are dealt to the
+// CTAs in turn, so that CTAs that run at the same time read neighbouring heads of the same cache rows (consecutive
+// ranges per CTA: 59 -> 65 us at S 1088, 41 rows).  Where all units of the launch can run at once the units are dealt
+// instead: with more items than SMs but less than four units per SM some CTAs would get a second round of units (192 items
+// of three tiles, S 320: 25.7 -> 17.5 us).
+struct Unit { int b, h, start, row0; };    // the tile's first query row; the row on lane 0 (up to 96 before it)
+MARCHE_DEVINL Unit unit_of(int j, int u, bool deal_units, int n_qt, int n, int H) {
+  int k = NS * u + j, item, qt;
+  if (deal_units) {
+    k = (int)blockIdx.x + k * (int)gridDim.x;
+    item = k / n_qt;
+    qt = k - item * n_qt;
+  } else {
+    item = k / n_qt;
+    qt = k - item * n_qt;
+    item = (int)blockIdx.x + item * (int)gridDim.x;
+  }
   Unit r;
   r.b = item / H;
   r.h = item - r.b * H;
-  r.qt = k % n_qt;
+  r.start = qt * QT;
+  // a tile that needs one, two or three of the four lane quarters starts at another quarter in another stream
+  const int quarters = n - r.start >= QT ? 4 : (n - r.start + 31) / 32;
+  r.row0 = r.start - 32 * (quarters == 1 ? j : (quarters == 4 ? 0 : (j & 1) * (4 - quarters)));
   return r;
 }
 
@@ -178,21 +177,14 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int D = H * DH;
   const int n_kv = (S + KT - 1) / KT, n_qt = (n + QT - 1) / QT;
-  const int n_items = B * H;
-  const int items_cta = (n_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-  const int units_cta = items_cta * n_qt;
-  int n_units[NS];
-#pragma unroll
-  for (int j = 0; j < NS; ++j) n_units[j] = (units_cta + NS - 1 - j) / NS;
-  const float c_log2 = rsqrtf((float)DH) * 1.4426950408889634f;
+  const bool deal_units = B * H * n_qt <= NS * (int)gridDim.x;
+  const int dealt = deal_units ? B * H * n_qt : B * H;     // units or items over the CTAs
+  const int units_cta = (dealt - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x * (deal_units ? 1 : n_qt);
+  constexpr float c_log2 = 0.125f * 1.4426950408889634f;   // log2(e) / sqrt(head_dim)
 
   if (threadIdx.x == 0) {
     for (int j = 0; j < NS; ++j) {
-      for (int s = 0; s < NST; ++s) { ptx::mbar_init(bar(j, B_KV_FULL + s), 1); ptx::mbar_init(bar(j, B_KV_EMPTY + s), 1); }
-      ptx::mbar_init(bar(j, B_Q_FULL), 1);   ptx::mbar_init(bar(j, B_Q_EMPTY), 1);
-      ptx::mbar_init(bar(j, B_S_FULL), 1);   ptx::mbar_init(bar(j, B_S_EMPTY), 4);
-      ptx::mbar_init(bar(j, B_P_FULL), 4);   ptx::mbar_init(bar(j, B_P_EMPTY), 1);
-      ptx::mbar_init(bar(j, B_O_FULL), 1);   ptx::mbar_init(bar(j, B_O_FREE), 4);
+      for (int i = 0; i < NB; ++i) ptx::mbar_init(bar(j, i), i == B_P_FULL ? 4 : 1);
     }
     abort_flag[0] = 0;
     abort_flag[1] = 0;
@@ -208,181 +200,186 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   pdl_sync();
-  // Register reallocation (per group of four warps): 256 control threads x 40 + 384 softmax threads x 128 <= 640 x 96.
   if (warp >= W_PROD) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
    if (warp < W_MMA) {
     // ---------------------------------------------------------------- TMA producer of stream j
     if (ptx::elect_one()) {
-      const int j = warp - W_PROD;
+      const int j = warp - W_PROD, n_units = (units_cta + NS - 1 - j) / NS;
       ptx::prefetch_tensormap(&tmap_kv);
       ptx::prefetch_tensormap(&tmap_q);
       const uint64_t stream_once = ptx::l2_policy_evict_first();
-      int tl = 0, s = 0;                                   // K/V tiles issued so far; ring slot of the next
-      uint32_t phase = 1;                                  // an empty slot's first wait passes at once
+      const uint32_t k0 = base + OFF_K + j * NK * T_BYTES, v0 = base + OFF_V + j * NV * T_BYTES;
+      int n_k = 0, n_v = 0, ks = 0, vs = 0;                // K and V tiles issued so far; slots of the next
+      uint32_t k_phase = 1, v_phase = 1;                   // an empty slot's first wait passes at once
       bool ok = true;
-      for (int u = 0; u < n_units[j] && ok; ++u) {
-        const Unit un = unit_of(j, u, n_qt, H);
+      for (int u = 0; u < n_units && ok; ++u) {
+        const Unit un = unit_of(j, u, deal_units, n_qt, n, H);
         if (!ptx::mbar_wait(bar(j, B_Q_EMPTY), ((uint32_t)u & 1u) ^ 1u, abort_flag)) { ok = false; break; }
         ptx::mbar_expect_tx(bar(j, B_Q_FULL), Q_BYTES);
-        ptx::tma_load_3d(base + OFF_Q + j * Q_BYTES, &tmap_q, un.h * DH, un.qt * QT, un.b, bar(j, B_Q_FULL));
-        for (int kt = 0; kt < n_kv; ++kt, ++tl) {
-          if (!ptx::mbar_wait(bar(j, B_KV_EMPTY + s), phase, abort_flag)) { ok = false; break; }
-          const uint32_t dst = base + OFF_KV + (j * NST + s) * STAGE_BYTES;
-          ptx::mbar_expect_tx(bar(j, B_KV_FULL + s), STAGE_BYTES);
-          ptx::tma_load_3d_hint(dst, &tmap_kv, un.h * DH, kt * KT, un.b, bar(j, B_KV_FULL + s), stream_once);
-          ptx::tma_load_3d_hint(dst + K_BYTES, &tmap_kv, un.h * DH, kt * KT, B + un.b, bar(j, B_KV_FULL + s), stream_once);
-          if (++s == NST) { s = 0; phase ^= 1u; }
+        ptx::tma_load_3d(base + OFF_Q + j * Q_BYTES, &tmap_q, un.h * DH, un.row0, un.b, bar(j, B_Q_FULL));
+        for (int kt = 0; kt < n_kv; ++kt) {
+          if (!ptx::mbar_wait(bar(j, B_K_EMPTY + ks), k_phase, abort_flag)) { ok = false; break; }
+          ptx::mbar_expect_tx(bar(j, B_K_FULL + ks), T_BYTES);
+          ptx::tma_load_3d_hint(k0 + ks * T_BYTES, &tmap_kv, un.h * DH, kt * KT, un.b, bar(j, B_K_FULL + ks), stream_once);
+          ++n_k;
+          if (++ks == NK) { ks = 0; k_phase ^= 1u; }
+          if (!ptx::mbar_wait(bar(j, B_V_EMPTY + vs), v_phase, abort_flag)) { ok = false; break; }
+          ptx::mbar_expect_tx(bar(j, B_V_FULL + vs), T_BYTES);
+          ptx::tma_load_3d_hint(v0 + vs * T_BYTES, &tmap_kv, un.h * DH, kt * KT, B + un.b, bar(j, B_V_FULL + vs), stream_once);
+          ++n_v;
+          if (++vs == NV) { vs = 0; v_phase ^= 1u; }
         }
       }
       if (!ok) {
         *(volatile int*)status = ST_ATT_STREAM;
         // let copies already issued land before the CTA's shared memory is released
-        for (int back = 1; back <= NST && back <= tl; ++back) {
-          const int i2 = tl - back;
-          ptx::mbar_wait(bar(j, B_KV_FULL + i2 % NST), (uint32_t)(i2 / NST) & 1u, abort_flag + 1, 20000000LL);
-        }
+        for (int back = 1; back <= NK && back <= n_k; ++back)
+          ptx::mbar_wait(bar(j, B_K_FULL + (n_k - back) % NK), (uint32_t)((n_k - back) / NK) & 1u, abort_flag + 1, 20000000LL);
+        for (int back = 1; back <= NV && back <= n_v; ++back)
+          ptx::mbar_wait(bar(j, B_V_FULL + (n_v - back) % NV), (uint32_t)((n_v - back) / NV) & 1u, abort_flag + 1, 20000000LL);
       }
     }
    } else if (warp < W_MMA + NS) {
     // ---------------------------------------------------------------- MMA issuer of stream j
-    // Within a stream the events arrive in a fixed order (S buffer handed back, then the weights of the same
-    // tile), so a plain sequence of waits is optimal: S(0); for each tile t: [S buffer free] S(t+1), [weights] P V(t).
     // Slots, phases and descriptors are stepped and the branch is an elected one: with divisions by the tile count and
-    // descriptors built per MMA in a lane-0 branch the issuer's own instructions were a third of a tile's chain.
+    // descriptors built per MMA in a lane-0 branch the issuer's own instructions were a fifth of a tile's chain.
     if (ptx::elect_one()) {
-      const int j = warp - W_MMA;
+      const int j = warp - W_MMA, n_units = (units_cta + NS - 1 - j) / NS;
       constexpr uint32_t idesc_s = idesc_bf16(QT, KT, false);
       constexpr uint32_t idesc_o = idesc_bf16(QT, DH, true);
-      const int total = n_units[j] * n_kv;
-      const uint32_t kv0 = base + OFF_KV + j * NST * STAGE_BYTES;
-      const uint32_t d_s = tmem_base + COL_S + (uint32_t)(j * KT), d_p = tmem_base + COL_P + (uint32_t)(j * (KT / 2)),
-                     d_o = tmem_base + COL_O + (uint32_t)(j * DH);
-      const uint64_t dq = ptx::smem_desc_k_sw128(base + OFF_Q + j * Q_BYTES), dk0 = ptx::smem_desc_k_sw128(kv0),
-                     dv0 = smem_desc_mn_sw128(kv0 + K_BYTES);
+      const int total = n_units * n_kv;
+      const uint32_t d_s = tmem_base + (uint32_t)j * COL_STREAM, d_o = d_s + COL_O;
+      const uint64_t dq = ptx::smem_desc_k_sw128(base + OFF_Q + j * Q_BYTES),
+                     dk0 = ptx::smem_desc_k_sw128(base + OFF_K + j * NK * T_BYTES),
+                     dv0 = smem_desc_mn_sw128(base + OFF_V + j * NV * T_BYTES);
       bool ok = true;
-      uint64_t dk = dk0;                                   // state of the S = Q K^T sequence
-      int s_slot = 0, s_i = 0;
-      uint32_t s_kv_phase = 0, s_free_phase = 1, q_phase = 0;   // (a wait for the phase before the first passes at once)
-      auto issue_s = [&]() -> bool {
-        if (!ptx::mbar_wait(bar(j, B_S_EMPTY), s_free_phase, abort_flag)) return false;
-        s_free_phase ^= 1u;
+      int s_slot = 0, s_i = 0, o_slot = 0, o_i = 0;        // ring slot and tile of the unit, of the next S and of the next O
+      uint32_t k_phase = 0, v_phase = 0, q_phase = 0;
+      // operands of the next S = Q K^T are there
+      auto wait_s = [&]() -> bool {
         if (s_i == 0) {
           if (!ptx::mbar_wait(bar(j, B_Q_FULL), q_phase, abort_flag)) return false;
           q_phase ^= 1u;
         }
-        if (!ptx::mbar_wait(bar(j, B_KV_FULL + s_slot), s_kv_phase, abort_flag)) return false;
-        ptx::tc_fence_after();
+        return ptx::mbar_wait(bar(j, B_K_FULL + s_slot), k_phase, abort_flag);
+      };
+      auto issue_s = [&]() {
+        const uint64_t dk = dk0 + (uint32_t)(s_slot * (T_BYTES >> 4));
 #pragma unroll
         for (int k = 0; k < DH / 16; ++k) ptx::umma_f16(d_s, dq + 2 * k, dk + 2 * k, idesc_s, k ? 1u : 0u);
-        ptx::umma_commit(bar(j, B_S_FULL));
+        ptx::umma_commit(bar(j, B_S_FULL));                // covers the P V before it, too
+        ptx::umma_commit(bar(j, B_K_EMPTY + s_slot));
         if (++s_i == n_kv) {                               // the unit's last Q K^T: Q_j may be overwritten
           s_i = 0;
           ptx::umma_commit(bar(j, B_Q_EMPTY));
         }
-        dk += STAGE_BYTES >> 4;
-        if (++s_slot == NST) { s_slot = 0; s_kv_phase ^= 1u; dk = dk0; }
-        return true;
+        if (++s_slot == NK) { s_slot = 0; k_phase ^= 1u; }
       };
-      uint64_t dv = dv0;                                   // state of the O += P V sequence
-      int o_slot = 0, o_i = 0;
-      uint32_t p_phase = 0, o_free_phase = 1;
-      if (total > 0) ok = issue_s();
-      for (int t = 0; t < total && ok; ++t) {
-        if (t + 1 < total && !issue_s()) { ok = false; break; }
-        // O_j += P_j V: needs the weights, and for a unit's first tile the previous output read out
-        if (!ptx::mbar_wait(bar(j, B_P_FULL), p_phase, abort_flag)) { ok = false; break; }
-        p_phase ^= 1u;
-        if (o_i == 0) {
-          if (!ptx::mbar_wait(bar(j, B_O_FREE), o_free_phase, abort_flag)) { ok = false; break; }
-          o_free_phase ^= 1u;
-        }
+      if (total > 0) {
+        ok = wait_s();
         ptx::tc_fence_after();
+        if (ok) issue_s();
+      }
+      for (int t = 0; t < total && ok; ++t) {
+        // a wait costs 110 cycles even if nothing is waited for, so those for the tiles come before the one for the weights
+        if ((t + 1 < total && !wait_s()) || !ptx::mbar_wait(bar(j, B_V_FULL + o_slot), v_phase, abort_flag) ||
+            // (for a unit's first tile the previous output has been read out: every softmax warp did so before it wrote)
+            !ptx::mbar_wait(bar(j, B_P_FULL), (uint32_t)t & 1u, abort_flag)) { ok = false; break; }
+        ptx::tc_fence_after();
+        const uint64_t dv = dv0 + (uint32_t)(o_slot * (T_BYTES >> 4));
 #pragma unroll
-        for (int k = 0; k < KT / 16; ++k) umma_f16_ts(d_o, d_p + 8u * k, dv + 128 * k, idesc_o, (o_i | k) ? 1u : 0u);
-        ptx::umma_commit(bar(j, B_KV_EMPTY + o_slot));     // K was read by the S of this tile, V just now
-        ptx::umma_commit(bar(j, B_P_EMPTY));
+        for (int k = 0; k < KT / 16; ++k) umma_f16_ts(d_o, d_s + 8u * k, dv + 128 * k, idesc_o, (o_i | k) ? 1u : 0u);
         if (++o_i == n_kv) {
           o_i = 0;
           ptx::umma_commit(bar(j, B_O_FULL));
         }
-        dv += STAGE_BYTES >> 4;
-        if (++o_slot == NST) { o_slot = 0; dv = dv0; }
+        // behind it, in the order of execution, the next logits over these weights
+        if (t + 1 < total) issue_s();
+        ptx::umma_commit(bar(j, B_V_EMPTY + o_slot));
+        if (++o_slot == NV) { o_slot = 0; v_phase ^= 1u; }
       }
       if (!ok) *(volatile int*)status = ST_ATT_STREAM;
     }
    }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 128;");
     // ---------------------------------------------------------------- softmax streams (one thread per row)
     const int j = warp >> 2;                               // stream (warps 4j .. 4j+3)
+    const int n_units = (units_cta + NS - 1 - j) / NS;
     const int quarter = warp & 3;
     const int r = quarter * 32 + lane;                     // row inside the query tile = TMEM lane
     const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16);
-    const uint32_t t_s = t_lane + COL_S + (uint32_t)(j * KT);
-    const uint32_t t_p = t_lane + COL_P + (uint32_t)(j * (KT / 2));
-    const uint32_t t_o = t_lane + COL_O + (uint32_t)(j * DH);
+    const uint32_t t_s = t_lane + (uint32_t)j * COL_STREAM, t_o = t_s + COL_O;   // (the weights go to t_s, too)
     bool ok = true;
     int t = 0;                                             // tiles of this stream so far
-    for (int u = 0; u < n_units[j] && ok; ++u) {
-      const Unit un = unit_of(j, u, n_qt, H);
-      const int row = un.qt * QT + r;
-      const bool warp_valid = (un.qt * QT + quarter * 32) < n;
+    for (int u = 0; u < n_units && ok; ++u) {
+      const Unit un = unit_of(j, u, deal_units, n_qt, n, H);
+      const int row = un.row0 + r, row_w = un.row0 + quarter * 32;   // this thread's query row, the warp's first one
+      const bool warp_valid = row_w >= un.start && row_w < n;
       float m_ref = -INFINITY, l = 0.f;                    // exponent reference (raw logit units), running sum
-      uint32_t v[KT];
       for (int i = 0; i < n_kv; ++i, ++t) {
+        // S_j of this tile is there, and the previous P V is done: it has read the weights and added to O_j
         if (!ptx::mbar_wait(bar(j, B_S_FULL), (uint32_t)t & 1u, abort_flag)) { ok = false; break; }
         ptx::tc_fence_after();
         const int lim = S - i * KT;                        // keys of this tile that exist
         if (warp_valid) {
-          tmem_ld_32x64(t_s, v);
-          ptx::tmem_ld_wait();
-        }
-        // the row is in registers: the next tile's logits may overwrite S_j while we work on this one
-        ptx::tc_fence_before();
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(bar(j, B_S_EMPTY));
-        bool move = false;
-        float tmax = -INFINITY;
-        if (warp_valid) {
+          uint32_t va[KT / 2], vb[KT / 2];                 // logits of the first and second 32 keys
+          ptx::tmem_ld_32x32(t_s, va);
+          ptx::tmem_ld_32x32(t_s + KT / 2, vb);
+          ptx::tmem_ld_wait(va);
+          ptx::tmem_ld_wait(vb);
           float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
           if (lim >= KT) {
 #pragma unroll
-            for (int c = 0; c < KT; c += 2)
-              mx[(c >> 1) & 3] = max3(mx[(c >> 1) & 3], __uint_as_float(v[c]), __uint_as_float(v[c + 1]));
+            for (int c = 0; c < KT / 2; c += 2) {
+              mx[c & 2] = max3(mx[c & 2], __uint_as_float(va[c]), __uint_as_float(va[c + 1]));
+              mx[(c & 2) + 1] = max3(mx[(c & 2) + 1], __uint_as_float(vb[c]), __uint_as_float(vb[c + 1]));
+            }
           } else {
 #pragma unroll
-            for (int c = 0; c < KT; ++c)
-              if (c < lim) mx[c & 3] = fmaxf(mx[c & 3], __uint_as_float(v[c]));
+            for (int c = 0; c < KT / 2; ++c) {
+              if (c < lim) mx[c & 1] = fmaxf(mx[c & 1], __uint_as_float(va[c]));
+              if (c + KT / 2 < lim) mx[2 + (c & 1)] = fmaxf(mx[2 + (c & 1)], __uint_as_float(vb[c]));
+            }
           }
-          tmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+          ptx::tmem_ld_32x32(t_s, va);                     // again, for the exponentials
+          const float tmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
           // lazy reference maximum: move it only when this tile exceeds it by more than 2^8
-          move = (tmax - m_ref) * c_log2 > 8.0f;           // also true for a unit's first tile (m_ref = -inf)
-        }
-        const float f = move ? ex2_approx((m_ref - tmax) * c_log2) : 1.0f;   // (0 for a unit's first tile)
-        if (move) m_ref = tmax;
-        const float neg = -m_ref * c_log2;
-        // weights: p = 2^((s - m_ref) / sqrt(d) * log2 e), packed bf16 pairs, in place (pair c -> v[c]).  The first half is
-        // computed while the previous P_j V still runs
-        float ls[4] = {0.f, 0.f, 0.f, 0.f};
-        auto weights = [&](int c) {
-          float x0, x1;
-          ffma2_bcast(__uint_as_float(v[2 * c]), __uint_as_float(v[2 * c + 1]), c_log2, neg, x0, x1);
-          const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
-          fadd2(ls[2 * (c & 1)], ls[2 * (c & 1) + 1], p0, p1);
-          v[c] = pack_bf16x2(p0, p1);
-        };
-        if (warp_valid && lim >= KT) {
+          const bool move = (tmax - m_ref) * c_log2 > 8.0f;   // also true for a unit's first tile (m_ref = -inf)
+          const bool rescale = i > 0 && __any_sync(0xffffffffu, move);
+          const float f = move ? ex2_approx((m_ref - tmax) * c_log2) : 1.0f;
+          if (move) m_ref = tmax;
+          const float neg = -m_ref * c_log2;
+          // weights: p = 2^((s - m_ref) / sqrt(d) * log2 e), packed bf16 pairs, in place (pair c -> v[c])
+          float ls[4] = {0.f, 0.f, 0.f, 0.f};
+          auto weights = [&](uint32_t (&v)[KT / 2], int left) {   // left: keys of this half that exist
+            if (left >= KT / 2) {                          // (two copies: no per-element selects for the full half)
 #pragma unroll
-          for (int c = 0; c < KT / 4; ++c) weights(c);
-        }
-        // the previous P_j V has read the weights we are about to overwrite, and has finished adding to O_j
-        if (t > 0 && !ptx::mbar_wait(bar(j, B_P_EMPTY), (uint32_t)(t - 1) & 1u, abort_flag)) { ok = false; break; }
-        ptx::tc_fence_after();
-        if (warp_valid) {
-          if (lim >= KT) tmem_st_32x16(t_p, v);            // on its way while the second half is computed
-          if (i > 0 && __any_sync(0xffffffffu, move)) {
-            // rescale this row's accumulator in tensor memory to the new reference
+              for (int c = 0; c < KT / 4; ++c) {
+                float x0, x1;
+                ffma2_bcast(__uint_as_float(v[2 * c]), __uint_as_float(v[2 * c + 1]), c_log2, neg, x0, x1);
+                const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
+                fadd2(ls[2 * (c & 1)], ls[2 * (c & 1) + 1], p0, p1);
+                v[c] = pack_bf16x2(p0, p1);
+              }
+            } else {
+#pragma unroll
+              for (int c = 0; c < KT / 4; ++c) {
+                float p0 = ex2_approx(fmaf(__uint_as_float(v[2 * c]), c_log2, neg));
+                float p1 = ex2_approx(fmaf(__uint_as_float(v[2 * c + 1]), c_log2, neg));
+                if (2 * c >= left) p0 = 0.f;
+                if (2 * c + 1 >= left) p1 = 0.f;
+                ls[c & 3] += p0 + p1;
+                v[c] = pack_bf16x2(p0, p1);
+              }
+            }
+          };
+          weights(vb, lim - KT / 2);
+          ptx::tmem_ld_wait(va);
+          tmem_st_32x16(t_s + KT / 4, vb);                 // over logits that have been read
+          weights(va, lim);
+          tmem_st_32x16(t_s, va);
+          if (rescale) {
+            // this row's accumulator in tensor memory moves to the new reference
 #pragma unroll 1
             for (int qc = 0; qc < 4; ++qc) {
               uint32_t ov[16];
@@ -392,24 +389,9 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
               for (int c = 0; c < 16; ++c) ov[c] = __float_as_uint(__uint_as_float(ov[c]) * f);
               tmem_st_32x16(t_o + (uint32_t)(qc * 16), ov);
             }
+            l *= f;
           }
-          if (lim >= KT) {                                 // (two copies of the loop: no per-element selects on the
-#pragma unroll                                             //  common, full tile)
-            for (int c = KT / 4; c < KT / 2; ++c) weights(c);
-            tmem_st_32x16(t_p + 16u, v + 16);
-          } else {
-#pragma unroll
-            for (int c = 0; c < KT / 2; ++c) {
-              float p0 = ex2_approx(fmaf(__uint_as_float(v[2 * c]), c_log2, neg));
-              float p1 = ex2_approx(fmaf(__uint_as_float(v[2 * c + 1]), c_log2, neg));
-              if (2 * c >= lim) p0 = 0.f;
-              if (2 * c + 1 >= lim) p1 = 0.f;
-              ls[c & 3] += p0 + p1;
-              v[c] = pack_bf16x2(p0, p1);
-            }
-            tmem_st_32x32(t_p, v);
-          }
-          l = (i > 0 ? l * f : 0.f) + ((ls[0] + ls[1]) + (ls[2] + ls[3]));
+          l += (ls[0] + ls[1]) + (ls[2] + ls[3]);
           tmem_st_wait();
         }
         ptx::tc_fence_before();
@@ -420,30 +402,34 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
       // ---- end of the unit: O / l -> output rows
       if (!ptx::mbar_wait(bar(j, B_O_FULL), (uint32_t)u & 1u, abort_flag)) { ok = false; break; }
       ptx::tc_fence_after();
-      const float inv = 1.0f / l;
-      uint4* dst = reinterpret_cast<uint4*>(o + ((size_t)un.b * n + row) * D + un.h * DH);
-#pragma unroll 1
-      for (int qc = 0; qc < 4; ++qc) {                       // 16 output columns at a time
-        uint32_t ov[16];
-        if (warp_valid) {
-          tmem_ld_32x16(t_o + (uint32_t)(qc * 16), ov);
-          ptx::tmem_ld_wait();
-        }
-        if (qc == 3) {
-          ptx::tc_fence_before();
-          __syncwarp();
-          if (lane == 0) ptx::mbar_arrive(bar(j, B_O_FREE));
-        }
-        if (warp_valid && row < n) {
+      if (warp_valid) {
+        const float inv = 1.0f / l;
+        uint16_t* dst = o + ((size_t)un.b * n + row) * D + un.h * DH;
+        uint32_t oa[DH / 2], ob[DH / 2];
+        ptx::tmem_ld_32x32(t_o, oa);
+        ptx::tmem_ld_32x32(t_o + DH / 2, ob);
+        ptx::tmem_ld_wait(oa);
+        ptx::tmem_ld_wait(ob);
+        // 16 columns per store, a whole 32-byte sector where the output is so aligned
+        auto store = [&](const uint32_t (&x)[DH / 2], uint16_t* to) {
 #pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            uint4 w;
-            w.x = pack_a16x2(__uint_as_float(ov[8 * q + 0]) * inv, __uint_as_float(ov[8 * q + 1]) * inv, o_bf16 != 0);
-            w.y = pack_a16x2(__uint_as_float(ov[8 * q + 2]) * inv, __uint_as_float(ov[8 * q + 3]) * inv, o_bf16 != 0);
-            w.z = pack_a16x2(__uint_as_float(ov[8 * q + 4]) * inv, __uint_as_float(ov[8 * q + 5]) * inv, o_bf16 != 0);
-            w.w = pack_a16x2(__uint_as_float(ov[8 * q + 6]) * inv, __uint_as_float(ov[8 * q + 7]) * inv, o_bf16 != 0);
-            dst[2 * qc + q] = w;
+          for (int q = 0; q < DH / 32; ++q) {
+            uint32_t w[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+              w[e] = pack_a16x2(__uint_as_float(x[16 * q + 2 * e]) * inv, __uint_as_float(x[16 * q + 2 * e + 1]) * inv, o_bf16 != 0);
+            if ((reinterpret_cast<uintptr_t>(o) & 31) == 0) {
+              asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(to + 16 * q), "r"(w[0]), "r"(w[1]),
+                           "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+            } else {
+              reinterpret_cast<uint4*>(to + 16 * q)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+              reinterpret_cast<uint4*>(to + 16 * q)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+            }
           }
+        };
+        if (row < n) {
+          store(oa, dst);
+          store(ob, dst + DH / 2);
         }
       }
     }
@@ -483,7 +469,8 @@ cudaError_t launch_attention_tc_stream(const void* q, int ld_q, int B, int n, in
   cudaError_t e = ensure_dynamic_smem(attention_tc_stream_kernel, (size_t)SMEM_BYTES, smem_set);
   if (e != cudaSuccess) return e;
   const int sms = device_sm_count();
-  const int grid = B * H < sms ? B * H : sms;
+  const long units = (long)B * H * ((n + QT - 1) / QT);
+  const int grid = units < sms ? (int)units : sms;
   return launch_pdl(attention_tc_stream_kernel, dim3(grid), dim3(kThreads), (size_t)SMEM_BYTES, st, tkv, tq, n, S, H, B,
                     (uint16_t*)o, o_bf16 ? 1 : 0, status);
 }

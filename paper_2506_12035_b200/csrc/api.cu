@@ -241,11 +241,11 @@ int do_attention(marche_ctx* ctx, const void* q, int ld_q, int n, const void* ca
   // Three tensor-core kernels.  At small active sets the step is bound by streaming the cache and the
   // mma.sync kernel (several small CTAs per SM, one pass) is fastest: 40 us vs 50 us at n = 41..48 (S 320).
   // From 49 rows, where the mma.sync kernel needs a fourth consumer warp and drops to two CTAs per SM, the
-  // single-pass tcgen05 kernel wins (S 320: 50 vs 56 us at n = 49..64, 54 vs 110 us at n = 77, 141 vs 303 us at
-  // n = 320; S 1088: 77 vs 82 us at n = 49..64, 81 vs 252 us at n = 116, 129 vs 256 us at n = 159).  The
-  // relevance scores need final weights, hence the two-pass tcgen05 kernel there (74 vs 143 us at n = 77).
+  // single-pass tcgen05 kernel wins (S 320: 43 vs 58 us at n = 60, 48 vs 110 us at n = 77, 128 vs 303 us at n = 320); over
+  // long sequences (S >= 512) from 33 rows (S 1088: 57 vs 62 us at n = 41, 57 vs 84 us at n = 60, 67 vs 252 us at n = 116).
+  // The relevance scores need final weights, hence the two-pass tcgen05 kernel there (74 vs 143 us at n = 77).
   // marche_tuning.attention_kernel forces one of them; head_dim 80 has only the mma.sync kernel.
-  const int tc_min = is_new ? 64 : ctx->tune.attention_tc_min_rows;
+  const int tc_min = is_new ? 64 : (S >= 512 ? ctx->tune.attention_tc_min_rows * 2 / 3 : ctx->tune.attention_tc_min_rows);
   const int ak = ctx->tune.attention_kernel;
   const bool tc5 = c.head_dim == 64 && ld_q % 8 == 0 && ((uintptr_t)q & 15) == 0 &&
                    (ak == MARCHE_ATTENTION_TCGEN05 || ak == MARCHE_ATTENTION_TCGEN05_TWO_PASS ||

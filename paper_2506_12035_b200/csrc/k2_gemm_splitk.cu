@@ -50,24 +50,46 @@ MARCHE_DEVINL float4 ld_shared_v4(uint32_t addr) {
   return v;
 }
 
-// Four finished columns of one output row: epilogue and store.
+MARCHE_DEVINL void st_global_v8(void* dst, const uint32_t* v) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
+               "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+}
+
+// 32 bytes of one finished output row (8 fp32 or 16 16-bit columns, the sums in f): epilogue and store.  A lane holds a
+// row, so that a warp's store touches 32 rows whatever its width: whole sectors where the output is so aligned.
 template <int EPI>
-MARCHE_DEVINL void finish4(float4 v, void* dst, float4 res, bool a_bf16) {
-  if (EPI == 1) {
-    *reinterpret_cast<float4*>(dst) = make_float4(res.x + v.x, res.y + v.y, res.z + v.z, res.w + v.w);
-  } else {
-    uint2 u;
-    if (EPI == 2) {
-      gelu_erf_pair(v.x, v.y);
-      gelu_erf_pair(v.z, v.w);
-      u.x = pack_a16x2(v.x, v.y, a_bf16);
-      u.y = pack_a16x2(v.z, v.w, a_bf16);
+MARCHE_DEVINL void finish32(float4 (&f)[EPI == 1 ? 2 : 4], uint8_t* dst, bool sector, bool a_bf16) {
+  uint32_t v[8];
+#pragma unroll
+  for (int j = 0; j < (EPI == 1 ? 2 : 4); ++j) {
+    if (EPI == 1) {
+      v[4 * j % 8] = __float_as_uint(f[j].x); v[(4 * j + 1) % 8] = __float_as_uint(f[j].y);
+      v[(4 * j + 2) % 8] = __float_as_uint(f[j].z); v[(4 * j + 3) % 8] = __float_as_uint(f[j].w);
+    } else if (EPI == 2) {
+      gelu_erf_pair(f[j].x, f[j].y);
+      gelu_erf_pair(f[j].z, f[j].w);
+      v[2 * j] = pack_a16x2(f[j].x, f[j].y, a_bf16);
+      v[2 * j + 1] = pack_a16x2(f[j].z, f[j].w, a_bf16);
     } else {
-      u.x = pack_bf16x2(v.x, v.y);
-      u.y = pack_bf16x2(v.z, v.w);
+      v[2 * j] = pack_bf16x2(f[j].x, f[j].y);
+      v[2 * j + 1] = pack_bf16x2(f[j].z, f[j].w);
     }
-    *reinterpret_cast<uint2*>(dst) = u;
   }
+  if (sector) {
+    st_global_v8(dst, v);
+  } else {
+    reinterpret_cast<uint4*>(dst)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+    reinterpret_cast<uint4*>(dst)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+  }
+}
+
+// The same for eight 16-bit columns.
+template <int EPI>
+MARCHE_DEVINL void finish16(float4 a, float4 b, uint8_t* dst, bool a_bf16) {
+  if (EPI == 2) { gelu_erf_pair(a.x, a.y); gelu_erf_pair(a.z, a.w); gelu_erf_pair(b.x, b.y); gelu_erf_pair(b.z, b.w); }
+  const bool bf = EPI != 2 || a_bf16;
+  *reinterpret_cast<uint4*>(dst) = make_uint4(pack_a16x2(a.x, a.y, bf), pack_a16x2(a.z, a.w, bf), pack_a16x2(b.x, b.y, bf),
+                                              pack_a16x2(b.z, b.w, bf));
 }
 
 // Grid: x = CS * (n_m * n_n) CTAs, clusters of CS consecutive ones share an output tile and split its K blocks.
@@ -263,8 +285,9 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
         // ---- the sum over the cluster, in rank order
         ok = ptx::mbar_wait_cluster(recv_bar, 0, abort_flag);
         if (ok && valid) {
-#pragma unroll
-          for (int j = 0; j < NQ; ++j) {
+          constexpr int NG = EPI == 1 ? 2 : 4;              // float4s per 32 bytes of output
+          const bool sector = (reinterpret_cast<uintptr_t>(dst) & 31) == 0;
+          auto total = [&](int j) -> float4 {
             float4 f = ld_shared_v4(recv + (uint32_t)(j * BM + r) * 16u);
 #pragma unroll
             for (int src = 1; src < CS; ++src) {
@@ -272,7 +295,22 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
               f.x += p.x; f.y += p.y; f.z += p.z; f.w += p.w;
             }
             f.x += bv[j].x; f.y += bv[j].y; f.z += bv[j].z; f.w += bv[j].w;
-            finish4<EPI>(f, dst + 4 * j * OB, res[j], a_bf16 != 0);
+            if (EPI == 1) { f.x += res[j].x; f.y += res[j].y; f.z += res[j].z; f.w += res[j].w; }
+            return f;
+          };
+          if (NQ % NG == 0) {
+#pragma unroll
+            for (int j = 0; j < NQ / NG; ++j) {
+              float4 f[NG];
+#pragma unroll
+              for (int e = 0; e < NG; ++e) f[e] = total((NG * j + e) % NQ);
+              finish32<EPI>(f, dst + 32 * j, sector, a_bf16 != 0);
+            }
+          } else {                                         // eight 16-bit columns: half of that
+            float4 f[NG] = {};
+#pragma unroll
+            for (int e = 0; e < NQ && e < NG; ++e) f[e] = total(e);
+            finish16<EPI>(f[0], f[1], dst, a_bf16 != 0);
           }
         }
       }

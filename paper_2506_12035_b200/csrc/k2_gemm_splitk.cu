@@ -19,6 +19,7 @@
 #include <cuda.h>
 
 #include <cmath>
+#include <type_traits>
 
 #include "gemm_epilogue.cuh"
 #include "kernels.h"
@@ -92,11 +93,14 @@ MARCHE_DEVINL void finish16(float4 a, float4 b, uint8_t* dst, bool a_bf16) {
                                               pack_a16x2(b.z, b.w, bf));
 }
 
+// TMA stores the output only where no cluster finishes it: the other launches do not carry its map.
+template <int CS> using OutMap = typename std::conditional<CS == 1, CUtensorMap, char>::type;
+
 // Grid: x = CS * (n_m * n_n) CTAs, clusters of CS consecutive ones share an output tile and split its K blocks.
 template <int BN, int CS, int EPI>
 __global__ void __launch_bounds__(kThreads, BN == 128 && CS > 1 ? 1 : 2)
 gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w,
-                   const __grid_constant__ CUtensorMap tmap_out, int M, int N, int K, int a_rows, int n_stages,
+                   const __grid_constant__ OutMap<CS> tmap_out, int M, int N, int K, int a_rows, int n_stages,
                    int ring_bytes, const float* __restrict__ bias, void* __restrict__ out,
                    const KvScatter kv, int a_bf16, int* __restrict__ status) {
   constexpr int W_BYTES = BN * BK * 2;
@@ -225,7 +229,7 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
       const int t = kv.idx ? kv.idx[row] : row - b * kv.n;
       kv_row = ((long)which * kv.B + b) * kv.S + t;
     }
-    if (CS == 1) {
+    if constexpr (CS == 1) {
       epilogue_bias_store(epilogue_bias_load(bias + col0, BN, lane), BN, recv, lane);
       ok = ptx::mbar_wait(tfull_bar, 0, abort_flag);
       ptx::tc_fence_after();
@@ -331,7 +335,7 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
 }
 
 template <int BN, int CS, int EPI>
-cudaError_t launch_one(const CUtensorMap& ta, const CUtensorMap& tw, const CUtensorMap& to, int M, int N, int K, int a_rows, const float* bias,
+cudaError_t launch_one(const CUtensorMap& ta, const CUtensorMap& tw, int M, int N, int K, int a_rows, const float* bias,
                        void* out, const KvScatter& kv, int a_bf16, int* status, cudaStream_t st) {
   const int n_tiles = ((M + BM - 1) / BM) * (N / BN);
   const int fixed = 1024 + 256 + (CS > 1 ? BM * BN * 4 : BN * 4);
@@ -348,6 +352,9 @@ cudaError_t launch_one(const CUtensorMap& ta, const CUtensorMap& tw, const CUten
   if (CS > 1 ? reach > ring + BM * BN * 4 : reach > ring) ring = reach;
   if (CS == 1 && ring < 32768) ring = 32768;
   const size_t smem = fixed + ring;
+  OutMap<CS> to = {};
+  if constexpr (CS == 1)
+    if (!tma_make_store_map(&to, out, (uint64_t)M, (uint64_t)N, EPI == 1 ? 4 : 2)) return cudaErrorInvalidValue;
   static size_t smem_set[kMaxDevices] = {};
   cudaError_t e = ensure_dynamic_smem(gemm_splitk_kernel<BN, CS, EPI>, (size_t)budget, smem_set);
   if (e != cudaSuccess) return e;
@@ -411,8 +418,7 @@ cudaError_t launch_gemm_splitk(const void* a, int lda, int M, const void* w, con
     kv = *kv_scatter;
   }
   const int a_rows = rows_per_tile(M, cs);
-  CUtensorMap ta, tw, to;
-  if (!tma_make_store_map(&to, out, (uint64_t)M, (uint64_t)N, epilogue == 1 ? 4 : 2)) return cudaErrorInvalidValue;
+  CUtensorMap ta, tw;
   {
     const uint64_t dims[2] = {(uint64_t)K, (uint64_t)M}, strides[1] = {(uint64_t)lda * 2};
     const uint32_t box[2] = {BK, (uint32_t)a_rows};
@@ -425,10 +431,10 @@ cudaError_t launch_gemm_splitk(const void* a, int lda, int M, const void* w, con
   }
 #define MARCHE_SPLITK_CASE(BN_, CS_)                                                                                   \
   if (bn == BN_ && cs == CS_) {                                                                                        \
-    if (epilogue == 0) return launch_one<BN_, CS_, 0>(ta, tw, to, M, N, K, a_rows, bias, out, kv, a_bf16, status, st);      \
-    if (epilogue == 1) return launch_one<BN_, CS_, 1>(ta, tw, to, M, N, K, a_rows, bias, out, kv, a_bf16, status, st);      \
-    if (epilogue == 2) return launch_one<BN_, CS_, 2>(ta, tw, to, M, N, K, a_rows, bias, out, kv, a_bf16, status, st);      \
-    if (epilogue == 4) return launch_one<BN_, CS_, 4>(ta, tw, to, M, N, K, a_rows, bias, out, kv, a_bf16, status, st);      \
+    if (epilogue == 0) return launch_one<BN_, CS_, 0>(ta, tw, M, N, K, a_rows, bias, out, kv, a_bf16, status, st);      \
+    if (epilogue == 1) return launch_one<BN_, CS_, 1>(ta, tw, M, N, K, a_rows, bias, out, kv, a_bf16, status, st);      \
+    if (epilogue == 2) return launch_one<BN_, CS_, 2>(ta, tw, M, N, K, a_rows, bias, out, kv, a_bf16, status, st);      \
+    if (epilogue == 4) return launch_one<BN_, CS_, 4>(ta, tw, M, N, K, a_rows, bias, out, kv, a_bf16, status, st);      \
   }
   MARCHE_SPLITK_CASE(32, 2) MARCHE_SPLITK_CASE(32, 4)
   MARCHE_SPLITK_CASE(64, 1) MARCHE_SPLITK_CASE(64, 2) MARCHE_SPLITK_CASE(64, 4) MARCHE_SPLITK_CASE(64, 8)

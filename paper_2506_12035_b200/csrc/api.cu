@@ -238,33 +238,32 @@ int do_attention(marche_ctx* ctx, const void* q, int ld_q, int n, const void* ca
   if (skipped(ctx, MARCHE_KC_ATTENTION)) return MARCHE_OK;
   for (int rep_i = 0; rep_i < launches_of(ctx, MARCHE_KC_ATTENTION); ++rep_i) {
   if (n > 0) mark(ctx, MARCHE_KC_ATTENTION, st);
-  // Three tensor-core kernels.  At small active sets the step is bound by streaming the cache and the
-  // mma.sync kernel (several small CTAs per SM, one pass) is fastest: 40 us vs 50 us at n = 41..48 (S 320).
-  // From 49 rows, where the mma.sync kernel needs a fourth consumer warp and drops to two CTAs per SM, the
-  // single-pass tcgen05 kernel wins (S 320: 43 vs 58 us at n = 60, 48 vs 110 us at n = 77, 128 vs 303 us at n = 320); over
-  // long sequences (S >= 512) from 33 rows (S 1088: 57 vs 62 us at n = 41, 57 vs 84 us at n = 60, 67 vs 252 us at n = 116).
-  // The relevance scores need final weights, hence the two-pass tcgen05 kernel there (74 vs 143 us at n = 77).
-  // marche_tuning.attention_kernel forces one of them; head_dim 80 has only the mma.sync kernel.
-  const int tc_min = is_new ? 64 : (S >= 512 ? ctx->tune.attention_tc_min_rows * 2 / 3 : ctx->tune.attention_tc_min_rows);
-  const int ak = ctx->tune.attention_kernel;
-  const bool tc5 = c.head_dim == 64 && ld_q % 8 == 0 && ((uintptr_t)q & 15) == 0 &&
-                   (ak == MARCHE_ATTENTION_TCGEN05 || ak == MARCHE_ATTENTION_TCGEN05_TWO_PASS ||
-                    (ak == MARCHE_ATTENTION_AUTO && n > tc_min));
-  // few items (or few key tiles): all tiles in flight, split over a cluster and over warps; measured beside the rule
-  const bool split = !is_new && ak == MARCHE_ATTENTION_AUTO && attention_split_wins(n, S, c.head_dim, c.batch * c.n_heads);
+  // The plain attention has four tensor-core kernels; which one runs is a matter of query rows, keys, head_dim and items, by
+  // rules that stand beside the kernels with both sides measured:
+  //   few items (or few key tiles)      all tiles in flight, split over a cluster and over warps (attention_split_wins)
+  //   more than 48 rows, or nearly so   four tcgen05 streams per SM (attention_tc_stream_wins)
+  //   32 rows or fewer                  the persistent mma.sync launch (31 vs 34 us at n = 8, 32 vs 36 us at n = 24..32, S 320)
+  //   else                              mma.sync with one CTA per item
+  // Where relevance scores are taken in the same kernel their final weights take two passes: on tcgen05 above 64 rows (head_dim
+  // 64; 74 vs 143 us at n = 77), else the two-pass mma.sync flavour.  marche_tuning.attention_kernel forces one of them.
+  const int ak = ctx->tune.attention_kernel, items = c.batch * c.n_heads;
+  const bool aligned = ld_q % 8 == 0 && ((uintptr_t)q & 15) == 0, automatic = ak == MARCHE_ATTENTION_AUTO;
+  const bool split = !is_new && automatic && attention_split_wins(n, S, c.head_dim, items);
+  const bool stream = !is_new && aligned && (ak == MARCHE_ATTENTION_TCGEN05 ||
+                      (automatic && attention_tc_stream_wins(n, S, c.head_dim, items, ctx->tune.attention_tc_min_rows)));
+  const bool two_pass = aligned && c.head_dim == 64 &&
+                        (ak == MARCHE_ATTENTION_TCGEN05_TWO_PASS ||
+                         (is_new && (ak == MARCHE_ATTENTION_TCGEN05 || (automatic && n > 64))));
   if (split)
     MARCHE_TRY(launch_attention_split(q, ld_q, c.batch, n, S, c.n_heads, c.head_dim, cache_layer, o, ctx->a_bf16,
                                       ctx->status_dev, st), "attention_split");
-  // plain flavour: single-pass streaming kernel; the relevance scores need final weights, i.e. two passes
-  else if (tc5 && !is_new && ak != MARCHE_ATTENTION_TCGEN05_TWO_PASS)
+  else if (stream)
     MARCHE_TRY(launch_attention_tc_stream(q, ld_q, c.batch, n, S, c.n_heads, c.head_dim, cache_layer, o, ctx->a_bf16,
                                           ctx->status_dev, st), "attention_tc_stream");
-  else if (tc5)
+  else if (two_pass)
     MARCHE_TRY(launch_attention_tcgen05(q, ld_q, c.batch, n, S, c.n_heads, c.head_dim, cache_layer, is_new,
                                         partial, o, ctx->a_bf16, ctx->status_dev, st), "attention_tcgen05");
-  else if (!is_new && n <= 32 && ld_q % 8 == 0 && ((uintptr_t)q & 15) == 0)
-    // very small active sets, no scores: the persistent launch of the same arithmetic (31 vs 34 us at n = 8,
-    // 32 vs 36 us at n = 24..32, S 320); above 32 rows one CTA per item is as fast or faster
+  else if (!is_new && n <= 32 && aligned)
     MARCHE_TRY(launch_attention_mma_persist(q, ld_q, c.batch, n, S, c.n_heads, c.head_dim, cache_layer, o, ctx->a_bf16,
                                             ctx->status_dev, st), "attention_mma_persist");
   else

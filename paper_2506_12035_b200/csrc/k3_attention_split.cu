@@ -301,20 +301,19 @@ bool attention_split_plan(int n, int S, int dh, int items, int* cs, int* nk) {
   return true;
 }
 
-// Where it beats the kernels with one CTA per item and a ring (us, 41 rows unless stated): always below one CTA per SM
-// (S 320: 6.9 -> 4.5 at 32 items; S 1088: 17.8 -> 6.8); up to two per SM for five key tiles (288 items: 9.8 -> 8.2); for three
-// tiles, which leave room for four CTAs, without limit from 33 rows at head_dim 64 (2048 items: 29.2 -> 26.6), else up to
-// four per SM (512 items, 20 rows: 7.8 -> 7.0).  With a fourth group of queries the ring kernels lose more: up to four per
-// SM at head_dim 64 (512 items, S 320: 20.2 -> 16.9; 768 items 23.8 and 24.2), without limit at head_dim 80, which has no
-// tcgen05 kernel (2048 items, S 320: 98 -> 68).
+// Where it beats the other kernels (us, 45 rows unless stated): always below one CTA per SM (S 320: 6.9 -> 4.5 at 32 items;
+// S 1088: 17.8 -> 6.8); up to two per SM for five key tiles (288 items: 9.6 -> 8.2; 384 items, 60 rows: 13.5 against 12.5 of
+// the tcgen05 kernel); for three tiles, which leave room for four CTAs, up to four per SM (512 items, 20 rows: 7.8 -> 7.0; 576
+// items, 60 rows: 11.2 either way) and with three groups of queries at head_dim 64 without limit (2048 items: 29.7 -> 26.6).
+// At head_dim 80 with 33 rows or more up to one and a half per SM (S 320: 192 items 9.6 against 9.9, 288 items 11.5 and 10.4).
 bool attention_split_wins(int n, int S, int dh, int items) {
   int cs, nk;
   if (!attention_split_plan(n, S, dh, items, &cs, &nk)) return false;
   const int n_kv = (S + KT - 1) / KT, nq = (n + 15) / 16, sms = device_sm_count();
   if (items * cs <= sms) return true;
   if (cs > 1 || n_kv > 5) return false;
-  if (nq == 4) return dh == 80 || items <= 4 * sms;
-  if (n_kv <= 3) return dh == 64 ? (nq == 3 || items <= 4 * sms) : items <= 2 * sms;
+  if (dh == 80 && nq >= 3) return 2 * items <= 3 * sms;
+  if (dh == 64 && n_kv <= 3) return nq == 3 || items <= 4 * sms;
   return items <= 2 * sms;
 }
 

@@ -1,18 +1,18 @@
-// K3 on the 5th-generation tensor cores, single pass (head_dim 64, no relevance scores): attention of
+// K3 on the 5th-generation tensor cores, single pass (head_dim 64 or 80, no relevance scores): attention of
 // the active queries over all S cached rows of one block (Algorithm 1 lines 6-8 == Eq. 5 by
 // Appendix A), with the running-maximum / running-sum merge of Eq. 6-10 applied tile by tile.
 //
 // Persistent CTAs (one per SM).  The work of a CTA is a list of units, one unit = one 128-row query
-// tile of one (sample, head) item against all S keys; FOUR independent streams inside the CTA take
-// the units in turn.  A unit is a latency chain (Q K^T -> read logits -> exponentials -> write weights
+// tile of one (sample, head) item against all S keys; FOUR independent streams (three at head_dim 80, whose buffers are
+// larger) inside the CTA take the units in turn.  A unit is a latency chain (Q K^T -> read logits -> exponentials -> write weights
 // -> P V -> next Q K^T ...), and the exponentials - 16 per clock and SM - are the scarce resource once the active set
 // is large; four chains in flight per SM partition keep those units busy while each chain waits on its hand-overs.
 // Each stream owns a query buffer, TMA rings of 64-key tiles (three of K, two of V: a K tile is used up a step earlier)
-// that run ahead across units and 128 columns of tensor memory: S_j 64 columns (fp32 logits), whose first 32 the
-// weights P_j (packed bf16) overwrite, and O_j 64 columns.  So P V of a tile and Q K^T of the next are issued together,
+// that run ahead across units and 128 (144) columns of tensor memory: S_j 64 columns (fp32 logits), whose first 32 the
+// weights P_j (packed bf16) overwrite, and O_j.  So P V of a tile and Q K^T of the next are issued together,
 // in the order in which the tensor core executes them, and one barrier per tile tells the softmax that both are done:
 // its weights may be overwritten, its accumulator rescaled, its logits read.
-// Roles (24 warps of 80 registers a thread):
+// Roles, for four streams (24 warps of 80 registers a thread):
 //   warps 0-15    softmax: warps 4j .. 4j+3 serve stream j, one thread per query row.  A thread pulls its
 //                 S row into registers (tcgen05.ld; the first half again for its exponentials, since 80 registers do
 //                 not hold a row and its weights) and writes the weights to tensor memory
@@ -23,6 +23,9 @@
 //                 tile; warp 23 also allocates / frees tensor memory
 // A warp can only reach the tensor-memory lanes of its quarter, and a quarter is one SM partition.  A query tile of
 // fewer than 97 rows is therefore placed on other lanes by other streams, so that the partitions share the work.
+// head_dim 80: a tile arrives as two boxes, columns 0-63 in rows of 128 bytes under the 128-byte swizzle and columns 64-79
+// behind them in rows of 32 bytes under the 32-byte swizzle; Q K^T takes a fifth K = 16 step from the second one, P V a second
+// MMA of 16 columns per step.
 // Online softmax with a lazy reference maximum: the exponent reference of a row only moves when a
 // tile's maximum exceeds it by more than 2^8 in the exponent, and only then is the row's O accumulator
 // rescaled in tensor memory (by the row's own thread); weights
@@ -39,31 +42,33 @@ namespace marche {
 
 namespace {
 
-constexpr int DH = 64;
 constexpr int QT = 128;                    // query rows per unit (= TMEM lanes)
 constexpr int KT = 64;                     // keys per tile
-constexpr int NS = 4;                      // streams per CTA
 constexpr int NK = 3, NV = 2;              // K and V tiles in flight per stream
-constexpr int T_BYTES = KT * DH * 2;       // a K or V tile: 8 KB
-constexpr int Q_BYTES = QT * DH * 2;       // 16 KB
-constexpr int kThreads = 768;               // 16 softmax warps, 4 producers, 4 MMA issuers
-constexpr int W_PROD = NS * 4, W_MMA = NS * 5;   // (whole groups of four warps, as the register reallocation requires)
 constexpr int TMEM_COLS = 512;
-constexpr uint32_t COL_STREAM = 128, COL_O = 64;   // stream j: S_j (and P_j over it) at 128 j, O_j at 128 j + 64
-static_assert(NS * COL_STREAM <= TMEM_COLS, "tensor memory budget");
+constexpr uint32_t COL_O = KT;             // O_j's first column in its stream's share: behind S_j (and P_j over it)
 enum { ST_ATT_STREAM = 0x51 };
-
-// shared memory (from a 1024-byte aligned base)
-constexpr int OFF_Q = 0;                                   // [stream]
-constexpr int OFF_K = OFF_Q + NS * Q_BYTES;                // [stream][slot]
-constexpr int OFF_V = OFF_K + NS * NK * T_BYTES;           // [stream][slot]
-constexpr int OFF_BAR = OFF_V + NS * NV * T_BYTES;
 // barriers of one stream (8 bytes each); stream j's block starts at j * NB
 enum { B_K_FULL = 0, B_K_EMPTY = B_K_FULL + NK, B_V_FULL = B_K_EMPTY + NK, B_V_EMPTY = B_V_FULL + NV, B_Q_FULL = B_V_EMPTY + NV,
        B_Q_EMPTY, B_S_FULL, B_P_FULL, B_O_FULL, NB };
-constexpr int OFF_MISC = OFF_BAR + 8 * NS * NB;            // tmem slot (4), abort flags (8)
-constexpr int SMEM_BYTES = OFF_MISC + 32 + 1024;
-static_assert(SMEM_BYTES <= 227 * 1024, "shared memory of one CTA");
+
+template <int DH> struct Cfg {
+  static constexpr int NS = DH == 64 ? 4 : 3;                // streams per CTA
+  static constexpr int THREADS = NS * 6 * 32;                // per stream four softmax warps, a producer, an MMA issuer
+  static constexpr int W_PROD = NS * 4, W_MMA = NS * 5;
+  static constexpr int T_MAIN = KT * 128, T_BYTES = KT * DH * 2;   // a K or V tile; its columns 0-63
+  static constexpr int Q_MAIN = QT * 128, Q_BYTES = QT * DH * 2;
+  static constexpr uint32_t COL_STREAM = DH == 64 ? 128 : 160;
+  // shared memory (from a 1024-byte aligned base)
+  static constexpr int OFF_Q = 0;                            // [stream]
+  static constexpr int OFF_K = OFF_Q + NS * Q_BYTES;         // [stream][slot]
+  static constexpr int OFF_V = OFF_K + NS * NK * T_BYTES;    // [stream][slot]
+  static constexpr int OFF_BAR = OFF_V + NS * NV * T_BYTES;
+  static constexpr int OFF_MISC = OFF_BAR + 8 * NS * NB;     // tmem slot (4), abort flags (8)
+  static constexpr int SMEM_BYTES = OFF_MISC + 32 + 1024;
+  static_assert(NS * COL_STREAM <= TMEM_COLS && COL_O + DH <= COL_STREAM, "tensor memory budget");
+  static_assert(SMEM_BYTES <= 227 * 1024 && T_BYTES % 1024 == 0 && Q_BYTES % 1024 == 0, "shared memory of one CTA");
+};
 
 MARCHE_DEVINL constexpr uint32_t idesc_bf16(int M, int N, bool b_mn_major) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (b_mn_major ? (1u << 16) : 0u) | ((uint32_t)(N >> 3) << 17) |
@@ -74,6 +79,13 @@ MARCHE_DEVINL constexpr uint32_t idesc_bf16(int M, int N, bool b_mn_major) {
 MARCHE_DEVINL uint64_t smem_desc_mn_sw128(uint32_t addr) {
   const uint32_t lo = ((addr & 0x3FFFFu) >> 4) | ((1024u >> 4) << 16);
   const uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+  return ((uint64_t)hi << 32) | lo;
+}
+// The same for tiles of 32-byte rows (16 elements) under the 32-byte swizzle: 8 rows form a 256-byte atom.  K-major: one
+// K = 16 step of an operand; MN-major: 16 columns.
+MARCHE_DEVINL uint64_t smem_desc_sw32(uint32_t addr) {
+  const uint32_t lo = ((addr & 0x3FFFFu) >> 4) | ((256u >> 4) << 16);
+  const uint32_t hi = (256u >> 4) | (1u << 14) | (6u << 29);
   return ((uint64_t)hi << 32) | lo;
 }
 // D[tmem] (+)= A[tmem] * B[smem desc]: the A operand (128 lanes x K 16-bit values, two per column) is
@@ -142,6 +154,7 @@ MARCHE_DEVINL float ex2_approx(float x) {
 // instead: with more items than SMs but less than four units per SM some CTAs would get a second round of units (192 items
 // of three tiles, S 320: 25.7 -> 17.5 us).
 struct Unit { int b, h, start, row0; };    // the tile's first query row; the row on lane 0 (up to 96 before it)
+template <int NS>
 MARCHE_DEVINL Unit unit_of(int j, int u, bool deal_units, int n_qt, int n, int H) {
   int k = NS * u + j, item, qt;
   if (deal_units) {
@@ -163,16 +176,20 @@ MARCHE_DEVINL Unit unit_of(int j, int u, bool deal_units, int n_qt, int n, int H
   return r;
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
+// tmap_kv, tmap_q: columns 0-63 of a head; the tails: columns 64-79 (unused at head_dim 64).
+template <int DH>
+__global__ void __launch_bounds__(Cfg<DH>::THREADS, 1)
 attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid_constant__ CUtensorMap tmap_q,
-                           int n, int S, int H, int B, uint16_t* __restrict__ o, int o_bf16, int* __restrict__ status) {
+                           const __grid_constant__ CUtensorMap tmap_kv_tail, const __grid_constant__ CUtensorMap tmap_q_tail, int n, int S, int H, int B, uint16_t* __restrict__ o, int o_bf16, int* __restrict__ status) {
+  using C = Cfg<DH>;
+  constexpr int NS = C::NS;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = ptx::smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* gen = smem_raw + (base - raw);
-  auto bar = [&](int j, int i) { return base + OFF_BAR + 8u * (uint32_t)(j * NB + i); };
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gen + OFF_MISC);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(gen + OFF_MISC + 8);
+  auto bar = [&](int j, int i) { return base + C::OFF_BAR + 8u * (uint32_t)(j * NB + i); };
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gen + C::OFF_MISC);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(gen + C::OFF_MISC + 8);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int D = H * DH;
@@ -180,7 +197,7 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
   const bool deal_units = B * H * n_qt <= NS * (int)gridDim.x;
   const int dealt = deal_units ? B * H * n_qt : B * H;     // units or items over the CTAs
   const int units_cta = (dealt - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x * (deal_units ? 1 : n_qt);
-  constexpr float c_log2 = 0.125f * 1.4426950408889634f;   // log2(e) / sqrt(head_dim)
+  constexpr float c_log2 = (DH == 64 ? 0.125f : 0.111803399f) * 1.4426950408889634f;   // log2(e) / sqrt(head_dim)
 
   if (threadIdx.x == 0) {
     for (int j = 0; j < NS; ++j) {
@@ -191,7 +208,7 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
     ptx::fence_barrier_init();
     ptx::fence_proxy_async();
   }
-  if (warp == W_MMA + NS - 1) {
+  if (warp == C::W_MMA + NS - 1) {
     ptx::tmem_alloc(ptx::smem_u32((const void*)tmem_slot), TMEM_COLS);
     ptx::tmem_relinquish();
   }
@@ -200,32 +217,41 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   pdl_sync();
-  if (warp >= W_PROD) {
-   if (warp < W_MMA) {
+  if (warp >= C::W_PROD) {
+   if (warp < C::W_MMA) {
     // ---------------------------------------------------------------- TMA producer of stream j
     if (ptx::elect_one()) {
-      const int j = warp - W_PROD, n_units = (units_cta + NS - 1 - j) / NS;
+      const int j = warp - C::W_PROD, n_units = (units_cta + NS - 1 - j) / NS;
       ptx::prefetch_tensormap(&tmap_kv);
       ptx::prefetch_tensormap(&tmap_q);
       const uint64_t stream_once = ptx::l2_policy_evict_first();
-      const uint32_t k0 = base + OFF_K + j * NK * T_BYTES, v0 = base + OFF_V + j * NV * T_BYTES;
+      const uint32_t k0 = base + C::OFF_K + j * NK * C::T_BYTES, v0 = base + C::OFF_V + j * NV * C::T_BYTES;
       int n_k = 0, n_v = 0, ks = 0, vs = 0;                // K and V tiles issued so far; slots of the next
       uint32_t k_phase = 1, v_phase = 1;                   // an empty slot's first wait passes at once
       bool ok = true;
       for (int u = 0; u < n_units && ok; ++u) {
-        const Unit un = unit_of(j, u, deal_units, n_qt, n, H);
+        const Unit un = unit_of<NS>(j, u, deal_units, n_qt, n, H);
         if (!ptx::mbar_wait(bar(j, B_Q_EMPTY), ((uint32_t)u & 1u) ^ 1u, abort_flag)) { ok = false; break; }
-        ptx::mbar_expect_tx(bar(j, B_Q_FULL), Q_BYTES);
-        ptx::tma_load_3d(base + OFF_Q + j * Q_BYTES, &tmap_q, un.h * DH, un.row0, un.b, bar(j, B_Q_FULL));
+        ptx::mbar_expect_tx(bar(j, B_Q_FULL), C::Q_BYTES);
+        ptx::tma_load_3d(base + C::OFF_Q + j * C::Q_BYTES, &tmap_q, un.h * DH, un.row0, un.b, bar(j, B_Q_FULL));
+        if (DH > 64)
+          ptx::tma_load_3d(base + C::OFF_Q + j * C::Q_BYTES + C::Q_MAIN, &tmap_q_tail, un.h * DH + 64, un.row0, un.b,
+                           bar(j, B_Q_FULL));
         for (int kt = 0; kt < n_kv; ++kt) {
           if (!ptx::mbar_wait(bar(j, B_K_EMPTY + ks), k_phase, abort_flag)) { ok = false; break; }
-          ptx::mbar_expect_tx(bar(j, B_K_FULL + ks), T_BYTES);
-          ptx::tma_load_3d_hint(k0 + ks * T_BYTES, &tmap_kv, un.h * DH, kt * KT, un.b, bar(j, B_K_FULL + ks), stream_once);
+          ptx::mbar_expect_tx(bar(j, B_K_FULL + ks), C::T_BYTES);
+          ptx::tma_load_3d_hint(k0 + ks * C::T_BYTES, &tmap_kv, un.h * DH, kt * KT, un.b, bar(j, B_K_FULL + ks), stream_once);
+          if (DH > 64)
+            ptx::tma_load_3d_hint(k0 + ks * C::T_BYTES + C::T_MAIN, &tmap_kv_tail, un.h * DH + 64, kt * KT, un.b,
+                                  bar(j, B_K_FULL + ks), stream_once);
           ++n_k;
           if (++ks == NK) { ks = 0; k_phase ^= 1u; }
           if (!ptx::mbar_wait(bar(j, B_V_EMPTY + vs), v_phase, abort_flag)) { ok = false; break; }
-          ptx::mbar_expect_tx(bar(j, B_V_FULL + vs), T_BYTES);
-          ptx::tma_load_3d_hint(v0 + vs * T_BYTES, &tmap_kv, un.h * DH, kt * KT, B + un.b, bar(j, B_V_FULL + vs), stream_once);
+          ptx::mbar_expect_tx(bar(j, B_V_FULL + vs), C::T_BYTES);
+          ptx::tma_load_3d_hint(v0 + vs * C::T_BYTES, &tmap_kv, un.h * DH, kt * KT, B + un.b, bar(j, B_V_FULL + vs), stream_once);
+          if (DH > 64)
+            ptx::tma_load_3d_hint(v0 + vs * C::T_BYTES + C::T_MAIN, &tmap_kv_tail, un.h * DH + 64, kt * KT, B + un.b,
+                                  bar(j, B_V_FULL + vs), stream_once);
           ++n_v;
           if (++vs == NV) { vs = 0; v_phase ^= 1u; }
         }
@@ -239,19 +265,22 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
           ptx::mbar_wait(bar(j, B_V_FULL + (n_v - back) % NV), (uint32_t)((n_v - back) / NV) & 1u, abort_flag + 1, 20000000LL);
       }
     }
-   } else if (warp < W_MMA + NS) {
+   } else if (warp < C::W_MMA + NS) {
     // ---------------------------------------------------------------- MMA issuer of stream j
     // Slots, phases and descriptors are stepped and the branch is an elected one: with divisions by the tile count and
     // descriptors built per MMA in a lane-0 branch the issuer's own instructions were a fifth of a tile's chain.
     if (ptx::elect_one()) {
-      const int j = warp - W_MMA, n_units = (units_cta + NS - 1 - j) / NS;
+      const int j = warp - C::W_MMA, n_units = (units_cta + NS - 1 - j) / NS;
       constexpr uint32_t idesc_s = idesc_bf16(QT, KT, false);
-      constexpr uint32_t idesc_o = idesc_bf16(QT, DH, true);
+      constexpr uint32_t idesc_o = idesc_bf16(QT, 64, true), idesc_tail = idesc_bf16(QT, 16, true);
       const int total = n_units * n_kv;
-      const uint32_t d_s = tmem_base + (uint32_t)j * COL_STREAM, d_o = d_s + COL_O;
-      const uint64_t dq = ptx::smem_desc_k_sw128(base + OFF_Q + j * Q_BYTES),
-                     dk0 = ptx::smem_desc_k_sw128(base + OFF_K + j * NK * T_BYTES),
-                     dv0 = smem_desc_mn_sw128(base + OFF_V + j * NV * T_BYTES);
+      const uint32_t d_s = tmem_base + (uint32_t)j * C::COL_STREAM, d_o = d_s + COL_O;
+      const uint64_t dq = ptx::smem_desc_k_sw128(base + C::OFF_Q + j * C::Q_BYTES),
+                     dk0 = ptx::smem_desc_k_sw128(base + C::OFF_K + j * NK * C::T_BYTES),
+                     dv0 = smem_desc_mn_sw128(base + C::OFF_V + j * NV * C::T_BYTES),
+                     dq_tail = smem_desc_sw32(base + C::OFF_Q + j * C::Q_BYTES + C::Q_MAIN),
+                     dk_tail0 = smem_desc_sw32(base + C::OFF_K + j * NK * C::T_BYTES + C::T_MAIN),
+                     dv_tail0 = smem_desc_sw32(base + C::OFF_V + j * NV * C::T_BYTES + C::T_MAIN);
       bool ok = true;
       int s_slot = 0, s_i = 0, o_slot = 0, o_i = 0;        // ring slot and tile of the unit, of the next S and of the next O
       uint32_t k_phase = 0, v_phase = 0, q_phase = 0;
@@ -264,9 +293,10 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
         return ptx::mbar_wait(bar(j, B_K_FULL + s_slot), k_phase, abort_flag);
       };
       auto issue_s = [&]() {
-        const uint64_t dk = dk0 + (uint32_t)(s_slot * (T_BYTES >> 4));
+        const uint64_t dk = dk0 + (uint32_t)(s_slot * (C::T_BYTES >> 4));
 #pragma unroll
-        for (int k = 0; k < DH / 16; ++k) ptx::umma_f16(d_s, dq + 2 * k, dk + 2 * k, idesc_s, k ? 1u : 0u);
+        for (int k = 0; k < 4; ++k) ptx::umma_f16(d_s, dq + 2 * k, dk + 2 * k, idesc_s, k ? 1u : 0u);
+        if (DH > 64) ptx::umma_f16(d_s, dq_tail, dk_tail0 + (uint32_t)(s_slot * (C::T_BYTES >> 4)), idesc_s, 1u);
         ptx::umma_commit(bar(j, B_S_FULL));                // covers the P V before it, too
         ptx::umma_commit(bar(j, B_K_EMPTY + s_slot));
         if (++s_i == n_kv) {                               // the unit's last Q K^T: Q_j may be overwritten
@@ -286,9 +316,14 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
             // (for a unit's first tile the previous output has been read out: every softmax warp did so before it wrote)
             !ptx::mbar_wait(bar(j, B_P_FULL), (uint32_t)t & 1u, abort_flag)) { ok = false; break; }
         ptx::tc_fence_after();
-        const uint64_t dv = dv0 + (uint32_t)(o_slot * (T_BYTES >> 4));
+        const uint64_t dv = dv0 + (uint32_t)(o_slot * (C::T_BYTES >> 4));
 #pragma unroll
-        for (int k = 0; k < KT / 16; ++k) umma_f16_ts(d_o, d_s + 8u * k, dv + 128 * k, idesc_o, (o_i | k) ? 1u : 0u);
+        for (int k = 0; k < KT / 16; ++k) {
+          umma_f16_ts(d_o, d_s + 8u * k, dv + 128 * k, idesc_o, (o_i | k) ? 1u : 0u);
+          if (DH > 64)
+            umma_f16_ts(d_o + 64u, d_s + 8u * k, dv_tail0 + (uint32_t)(o_slot * (C::T_BYTES >> 4)) + 32 * k, idesc_tail,
+                        (o_i | k) ? 1u : 0u);
+        }
         if (++o_i == n_kv) {
           o_i = 0;
           ptx::umma_commit(bar(j, B_O_FULL));
@@ -308,11 +343,11 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
     const int quarter = warp & 3;
     const int r = quarter * 32 + lane;                     // row inside the query tile = TMEM lane
     const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16);
-    const uint32_t t_s = t_lane + (uint32_t)j * COL_STREAM, t_o = t_s + COL_O;   // (the weights go to t_s, too)
+    const uint32_t t_s = t_lane + (uint32_t)j * C::COL_STREAM, t_o = t_s + COL_O;   // (the weights go to t_s, too)
     bool ok = true;
     int t = 0;                                             // tiles of this stream so far
     for (int u = 0; u < n_units && ok; ++u) {
-      const Unit un = unit_of(j, u, deal_units, n_qt, n, H);
+      const Unit un = unit_of<NS>(j, u, deal_units, n_qt, n, H);
       const int row = un.row0 + r, row_w = un.row0 + quarter * 32;   // this thread's query row, the warp's first one
       const bool warp_valid = row_w >= un.start && row_w < n;
       float m_ref = -INFINITY, l = 0.f;                    // exponent reference (raw logit units), running sum
@@ -381,7 +416,7 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
           if (rescale) {
             // this row's accumulator in tensor memory moves to the new reference
 #pragma unroll 1
-            for (int qc = 0; qc < 4; ++qc) {
+            for (int qc = 0; qc < DH / 16; ++qc) {
               uint32_t ov[16];
               tmem_ld_32x16(t_o + (uint32_t)(qc * 16), ov);
               ptx::tmem_ld_wait();
@@ -405,31 +440,35 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
       if (warp_valid) {
         const float inv = 1.0f / l;
         uint16_t* dst = o + ((size_t)un.b * n + row) * D + un.h * DH;
-        uint32_t oa[DH / 2], ob[DH / 2];
+        uint32_t oa[32], ob[32], oc[16];
         ptx::tmem_ld_32x32(t_o, oa);
-        ptx::tmem_ld_32x32(t_o + DH / 2, ob);
+        ptx::tmem_ld_32x32(t_o + 32u, ob);
         ptx::tmem_ld_wait(oa);
         ptx::tmem_ld_wait(ob);
         // 16 columns per store, a whole 32-byte sector where the output is so aligned
-        auto store = [&](const uint32_t (&x)[DH / 2], uint16_t* to) {
+        auto store = [&](const uint32_t* x, uint16_t* to) {
+          uint32_t w[8];
 #pragma unroll
-          for (int q = 0; q < DH / 32; ++q) {
-            uint32_t w[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e)
-              w[e] = pack_a16x2(__uint_as_float(x[16 * q + 2 * e]) * inv, __uint_as_float(x[16 * q + 2 * e + 1]) * inv, o_bf16 != 0);
-            if ((reinterpret_cast<uintptr_t>(o) & 31) == 0) {
-              asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(to + 16 * q), "r"(w[0]), "r"(w[1]),
-                           "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
-            } else {
-              reinterpret_cast<uint4*>(to + 16 * q)[0] = make_uint4(w[0], w[1], w[2], w[3]);
-              reinterpret_cast<uint4*>(to + 16 * q)[1] = make_uint4(w[4], w[5], w[6], w[7]);
-            }
+          for (int e = 0; e < 8; ++e)
+            w[e] = pack_a16x2(__uint_as_float(x[2 * e]) * inv, __uint_as_float(x[2 * e + 1]) * inv, o_bf16 != 0);
+          if ((reinterpret_cast<uintptr_t>(o) & 31) == 0) {
+            asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(to), "r"(w[0]), "r"(w[1]),
+                         "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+          } else {
+            reinterpret_cast<uint4*>(to)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+            reinterpret_cast<uint4*>(to)[1] = make_uint4(w[4], w[5], w[6], w[7]);
           }
         };
         if (row < n) {
           store(oa, dst);
-          store(ob, dst + DH / 2);
+          store(oa + 16, dst + 16);
+          store(ob, dst + 32);
+          store(ob + 16, dst + 48);
+        }
+        if (DH > 64) {
+          tmem_ld_32x16(t_o + 64u, oc);
+          ptx::tmem_ld_wait();
+          if (row < n) store(oc, dst + 64);
         }
       }
     }
@@ -438,41 +477,62 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
 
   ptx::tc_fence_before();
   __syncthreads();
-  if (warp == W_MMA + NS - 1) {
+  if (warp == C::W_MMA + NS - 1) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem_base, TMEM_COLS);
   }
 }
 
-}  // namespace
-
-cudaError_t launch_attention_tc_stream(const void* q, int ld_q, int B, int n, int S, int H, int dh,
-                                       const void* cache_layer, void* o, bool o_bf16, int* status, cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  if (dh != DH || ld_q % 8 || ((uintptr_t)q & 15) || ((uintptr_t)cache_layer & 15) || ((uintptr_t)o & 15) || S > 2048)
+template <int DH>
+cudaError_t launch_stream(const void* q, int ld_q, int B, int n, int S, int H, const void* cache_layer, void* o, bool o_bf16,
+                          int* status, cudaStream_t st) {
+  using C = Cfg<DH>;
+  const int D = H * DH;
+  // columns 0-63 of a head as 128-byte rows, columns 64-79 as 32-byte rows, both swizzled
+  CUtensorMap tkv, tq, tkv_tail, tq_tail;
+  auto make = [&](CUtensorMap* map, const void* p, int ld, int rows, int samples, uint32_t box_rows, bool tail) {
+    const uint64_t dims[3] = {(uint64_t)ld, (uint64_t)rows, (uint64_t)samples};
+    const uint64_t strides[2] = {(uint64_t)ld * 2, (uint64_t)rows * ld * 2};
+    const uint32_t box[3] = {tail ? 16u : 64u, box_rows, 1};
+    return tma_make_map_bf16(map, p, 3, dims, strides, box, !tail, false, tail);
+  };
+  if (!make(&tkv, cache_layer, D, S, 2 * B, KT, false) || !make(&tq, q, ld_q, n, B, QT, false)) return cudaErrorInvalidValue;
+  tkv_tail = tkv;
+  tq_tail = tq;
+  if (DH > 64 && (!make(&tkv_tail, cache_layer, D, S, 2 * B, KT, true) || !make(&tq_tail, q, ld_q, n, B, QT, true)))
     return cudaErrorInvalidValue;
-  const int D = H * dh;
-  CUtensorMap tkv, tq;
-  {
-    const uint64_t dims[3] = {(uint64_t)D, (uint64_t)S, (uint64_t)2 * B};
-    const uint64_t strides[2] = {(uint64_t)D * 2, (uint64_t)S * D * 2};
-    const uint32_t box[3] = {(uint32_t)DH, KT, 1};
-    if (!tma_make_map_bf16(&tkv, cache_layer, 3, dims, strides, box, true)) return cudaErrorInvalidValue;
-  }
-  {
-    const uint64_t dims[3] = {(uint64_t)ld_q, (uint64_t)n, (uint64_t)B};
-    const uint64_t strides[2] = {(uint64_t)ld_q * 2, (uint64_t)n * ld_q * 2};
-    const uint32_t box[3] = {(uint32_t)DH, QT, 1};
-    if (!tma_make_map_bf16(&tq, q, 3, dims, strides, box, true)) return cudaErrorInvalidValue;
-  }
   static size_t smem_set[kMaxDevices] = {};
-  cudaError_t e = ensure_dynamic_smem(attention_tc_stream_kernel, (size_t)SMEM_BYTES, smem_set);
+  cudaError_t e = ensure_dynamic_smem(attention_tc_stream_kernel<DH>, (size_t)C::SMEM_BYTES, smem_set);
   if (e != cudaSuccess) return e;
   const int sms = device_sm_count();
   const long units = (long)B * H * ((n + QT - 1) / QT);
   const int grid = units < sms ? (int)units : sms;
-  return launch_pdl(attention_tc_stream_kernel, dim3(grid), dim3(kThreads), (size_t)SMEM_BYTES, st, tkv, tq, n, S, H, B,
-                    (uint16_t*)o, o_bf16 ? 1 : 0, status);
+  return launch_pdl(attention_tc_stream_kernel<DH>, dim3(grid), dim3(C::THREADS), (size_t)C::SMEM_BYTES, st, tkv, tq, tkv_tail,
+                    tq_tail, n, S, H, B, (uint16_t*)o, o_bf16 ? 1 : 0, status);
+}
+
+}  // namespace
+
+// Against the mma.sync kernels (us), which take 48 rows or fewer (min_rows, marche_tuning) with up to five CTAs per SM and
+// drop to two from 49 rows: S 320, head_dim 64: 60 rows 42 and 58, 77 rows 47 and 110, 320 rows 125 and 303; head_dim 80: 60
+// rows 46 and 98, 320 rows 134 and 350.  33 to 48 rows: over long sequences at head_dim 64 (S 1088, 41 rows: 57 and 62; S 320:
+// 41 and 42, nothing in a whole step); at head_dim 80 over five key tiles or more (S 320: 45 and 49), unless the last
+// round of units leaves the streams (three per SM) idle: 576 items on 444 streams 19 and 16, 1024 items 29 either way.
+bool attention_tc_stream_wins(int n, int S, int dh, int items, int min_rows) {
+  if (n > min_rows) return true;
+  if (3 * n <= 2 * min_rows) return false;
+  if (dh == 64) return S >= 512;
+  const int streams = Cfg<80>::NS * device_sm_count(), rounds = (items + streams - 1) / streams;
+  return S > 4 * KT && (rounds == 1 || 4 * items >= 3 * rounds * streams);
+}
+
+cudaError_t launch_attention_tc_stream(const void* q, int ld_q, int B, int n, int S, int H, int dh,
+                                       const void* cache_layer, void* o, bool o_bf16, int* status, cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  if ((dh != 64 && dh != 80) || ld_q % 8 || ((uintptr_t)q & 15) || ((uintptr_t)cache_layer & 15) || ((uintptr_t)o & 15) || S > 2048)
+    return cudaErrorInvalidValue;
+  return dh == 64 ? launch_stream<64>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st)
+                  : launch_stream<80>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
 }
 
 }  // namespace marche

@@ -136,7 +136,8 @@ cudaError_t launch_attention_tcgen05(const void* q, int ld_q, int B, int n, int 
                                      bool o_bf16, int* status, cudaStream_t st);
 
 // K3 on tcgen05, single pass with online softmax, persistent over (sample, head) items, P kept in tensor
-// memory (head_dim 64, no relevance scores).  Same alignment rules as launch_attention_tcgen05, o 16-byte aligned.
+// memory (head_dim 64 or 80, no relevance scores).  Same alignment rules as launch_attention_tcgen05, o 16-byte aligned.
+bool attention_tc_stream_wins(int n, int S, int dh, int items, int min_rows);
 cudaError_t launch_attention_tc_stream(const void* q, int ld_q, int B, int n, int S, int H, int dh,
                                        const void* cache_layer, void* o, bool o_bf16, int* status, cudaStream_t st);
 

@@ -685,3 +685,31 @@ def test_attention_scores_of_the_generating_rows(dh, H, B, S, n, nG):
             _, p = orc.softmax_attention(qq[b * n:(b + 1) * n, c], cc[0, b][:, c], cc[1, b][:, c])
             want[b, h] = p[flags[b].astype(bool)].sum(axis=0)
     assert max_abs(host(got[0]), want) <= 2e-4 * max(1, nG) and np.allclose(host(got[0]).sum(-1), nG, rtol=1e-4, atol=1e-6)
+
+
+@pytest.mark.parametrize("dh,H", [(64, 4), (80, 8)])
+@pytest.mark.parametrize("B,S,n", [(1, 1, 1), (2, 65, 33), (3, 320, 70), (2, 128, 128), (60, 130, 129), (2, 1088, 150), (25, 577, 300)])
+def test_attention_single_pass_streams(dh, H, B, S, n):
+    """The single-pass tcgen05 kernel at both head sizes: query tiles on one to four lane quarters (alone and behind full
+    ones), units dealt one by one (few) and by items (more than run at once), ragged keys, row maxima that keep growing."""
+    from paper_2506_12035_b200 import binding
+    D = H * dh
+    cfg, blocks, m = model_for("bf16", D, H, 128, S, B)
+    m.set_tuning(attention_kernel=binding.ATTENTION_TCGEN05)
+    rng = np.random.default_rng(B + S + n + dh)
+    cache = rng.standard_normal((2, B, S, D)).astype(np.float32)
+    q = (rng.standard_normal((B * n, D)) * 3.0).astype(np.float32)
+    ramp, q_ramp = cache.copy(), q.copy()
+    ramp[0, :, :, dh - 1::dh] = np.linspace(0.0, 40.0, S, dtype=np.float32)[None, :, None]
+    q_ramp[:, dh - 1::dh] = 16.0
+    for qq, cc in ((q, cache), (q_ramp, ramp)):
+        o = torch.zeros(B * n, D, dtype=torch.float16, device="cuda")
+        m.attention(dev(qq, torch.bfloat16), D, n, dev(cc, torch.bfloat16), None, None, o)
+        assert m.device_status() == 0
+        got, qq, cc = host(o).reshape(B, n, D), quant(qq, "bf16").reshape(B, n, D), quant(cc, "bf16")
+        for b in sorted({0, B // 2, B - 1}):
+            want = np.zeros((n, D))
+            for h in range(H):
+                c = slice(h * dh, (h + 1) * dh)
+                want[:, c], _ = orc.softmax_attention(qq[b][:, c], cc[0, b][:, c], cc[1, b][:, c])
+            assert rel_l2(got[b], want) <= 8e-3 and max_abs(got[b], want) <= 3e-2

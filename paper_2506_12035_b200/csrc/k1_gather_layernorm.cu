@@ -86,10 +86,16 @@ static cudaError_t launch_ln_t(const float* src, int src_rows, const int32_t* id
   cudaError_t err = cudaSuccess;
 #define MARCHE_LN_CASE(NV_)                                                                          \
   case NV_:                                                                                          \
-    err = few ? launch_pdl(gather_layernorm_kernel<TOut, NV_, true>, dim3(grid), dim3(warps * 32), 0, st, src, src_rows, \
-                           idx, n, (int)rows, gamma, beta, eps, x_out, u_out, out_idx, out_rows)     \
-              : launch_pdl(gather_layernorm_kernel<TOut, NV_, false>, dim3(grid), dim3(warps * 32), 0, st, src, src_rows, \
-                           idx, n, (int)rows, gamma, beta, eps, x_out, u_out, out_idx, out_rows);    \
+    if (few) {                                                                                       \
+      static bool carved[kMaxDevices] = {};                                                          \
+      err = prefer_shared_memory(gather_layernorm_kernel<TOut, NV_, true>, carved);                  \
+      if (err == cudaSuccess)                                                                        \
+        err = launch_pdl(gather_layernorm_kernel<TOut, NV_, true>, dim3(grid), dim3(warps * 32), 0, st, src, src_rows, \
+                         idx, n, (int)rows, gamma, beta, eps, x_out, u_out, out_idx, out_rows);      \
+    } else {                                                                                         \
+      err = launch_pdl(gather_layernorm_kernel<TOut, NV_, false>, dim3(grid), dim3(warps * 32), 0, st, src, src_rows, \
+                       idx, n, (int)rows, gamma, beta, eps, x_out, u_out, out_idx, out_rows);        \
+    }                                                                                                \
     break;
   switch (D / 128) {
     MARCHE_LN_CASE(1) MARCHE_LN_CASE(2) MARCHE_LN_CASE(3) MARCHE_LN_CASE(4) MARCHE_LN_CASE(5)

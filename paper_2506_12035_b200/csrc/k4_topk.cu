@@ -178,6 +178,9 @@ cudaError_t launch_topk(const float* partial, int H, float* scores, const int32_
                         const int32_t* excl_idx, int n_excl, int B, int S, int k, int32_t* refresh_idx, cudaStream_t st,
                         int policy, uint32_t seed) {
   if (S > 2048) return cudaErrorInvalidValue;
+  static bool carved[kMaxDevices] = {};
+  const cudaError_t e = prefer_shared_memory(topk_kernel, carved);
+  if (e != cudaSuccess) return e;
   return launch_pdl(topk_kernel, dim3(B), dim3(kTopkThreads), 0, st, partial, H, scores, new_idx, n_new, excl_idx, n_excl, S,
                     k, policy, seed, refresh_idx);
 }

@@ -170,6 +170,9 @@ cudaError_t launch_scatter_rows(const float* rows, const int32_t* idx, int B, in
   if (D % 4) return cudaErrorInvalidValue;
   const long total = (long)B * n;
   if (total == 0) return cudaSuccess;
+  static bool carved[kMaxDevices] = {};
+  const cudaError_t e = prefer_shared_memory(scatter_rows_kernel, carved);
+  if (e != cudaSuccess) return e;
   return launch_pdl(scatter_rows_kernel, dim3((unsigned)((total + 7) / 8)), dim3(256), 0, st, (const float4*)rows, idx,
                     n, S, D / 4, total, (float4*)dst);
 }
@@ -179,6 +182,9 @@ cudaError_t launch_gather_rows(const float* src, const int32_t* idx, int B, int 
   if (D % 4) return cudaErrorInvalidValue;
   const long total = (long)B * n;
   if (total == 0) return cudaSuccess;
+  static bool carved[kMaxDevices] = {};
+  const cudaError_t e = prefer_shared_memory(gather_rows_kernel, carved);
+  if (e != cudaSuccess) return e;
   return launch_pdl(gather_rows_kernel, dim3((unsigned)((total + 7) / 8)), dim3(256), 0, st, (const float4*)src, idx, n,
                     S, D / 4, total, (float4*)out);
 }
@@ -187,6 +193,9 @@ cudaError_t launch_gather_table_rows(const float* table, const int32_t* idx, lon
                                      cudaStream_t st) {
   if (D % 4) return cudaErrorInvalidValue;
   if (total_rows == 0) return cudaSuccess;
+  static bool carved[kMaxDevices] = {};
+  const cudaError_t e = prefer_shared_memory(gather_table_rows_kernel, carved);
+  if (e != cudaSuccess) return e;
   return launch_pdl(gather_table_rows_kernel, dim3((unsigned)((total_rows + 7) / 8)), dim3(256), 0, st,
                     (const float4*)table, idx, D / 4, total_rows, (float4*)out);
 }
@@ -195,12 +204,18 @@ cudaError_t launch_fill_mask_rows(const float* mask_token, const float* pos, int
                                   cudaStream_t st) {
   if (D % 4) return cudaErrorInvalidValue;
   const long total = (long)B * S;
+  static bool carved[kMaxDevices] = {};
+  const cudaError_t e = prefer_shared_memory(fill_mask_rows_kernel, carved);
+  if (e != cudaSuccess) return e;
   return launch_pdl(fill_mask_rows_kernel, dim3((unsigned)((total + 7) / 8)), dim3(256), 0, st,
                     (const float4*)mask_token, (const float4*)pos, S, D / 4, total, (float4*)out);
 }
 
 cudaError_t launch_step_flags(const int32_t* active_idx, int n_active, const int32_t* new_idx, int n_new, int B, int S,
                               uint8_t* is_new, cudaStream_t st) {
+  static bool carved[kMaxDevices] = {};
+  const cudaError_t e = prefer_shared_memory(step_flags_kernel, carved);
+  if (e != cudaSuccess) return e;
   return launch_pdl(step_flags_kernel, dim3(B), dim3(256), (size_t)S, st, active_idx, n_active, new_idx, n_new, S, is_new);
 }
 
@@ -208,6 +223,9 @@ cudaError_t launch_build_active(const int32_t* a, int na, const int32_t* b, int 
                                 int B, int32_t* out, cudaStream_t st) {
   const long total = (long)B * (na + nb + nc);
   if (total == 0) return cudaSuccess;
+  static bool carved[kMaxDevices] = {};
+  const cudaError_t e = prefer_shared_memory(build_active_kernel, carved);
+  if (e != cudaSuccess) return e;
   return launch_pdl(build_active_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, a, na, b, nb, c, nc,
                     B, out);
 }

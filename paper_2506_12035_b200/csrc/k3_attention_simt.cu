@@ -3,13 +3,14 @@
 // the active rows' fresh K, V are in the cache), with the relevance reduction of
 // Section 4.2 fused in.  fp32 arithmetic and storage; serves the fp32 configuration only.
 //
-// Bound by latency at that configuration's sizes (a handful of samples, 4 heads, about a hundred rows): the queries of
-// a (sample, head) item are therefore dealt to a cluster of up to eight CTAs, 16 queries at a time, and the K and V
-// tiles (64 keys, coalesced cp.async) are all on their way at once where shared memory holds them.  A warp owns two
-// queries: their logits, softmax and output never leave it.  The probabilities of a tile's 16 queries stay in shared
-// memory, so the softmax is the exact two-pass form and the column sums use final probabilities; they are added in
-// query order within a CTA and in rank order over the cluster: scores are bit-reproducible.  (One CTA per item, reading
-// a key row per lane and a value row at a time from global memory, was most of the 7.4 ms that an eight-step run took.)
+// Bound by latency at that configuration's sizes (a handful of samples, 4 heads, about a hundred rows), then by shared
+// memory, from which every warp reads every key and value: the queries of a (sample, head) item are dealt to up to eight
+// CTAs (a cluster where they add scores together), and a warp takes two, for which it reads a key once.  K and V tiles (64
+// keys, coalesced cp.async) are on their way up to four at once.  A warp's logits, softmax and output never leave it.  The
+// probabilities of a CTA's queries stay in shared memory, so the softmax is the exact two-pass form and the column sums
+// use final probabilities; they are added in query order within a CTA and in rank order over the cluster: scores are
+// bit-reproducible.  (One CTA per item, reading a key row per lane and a value row at a time from global memory, was most
+// of the 7.4 ms that an eight-step run took.)
 #include "common.cuh"
 #include "kernels.h"
 #include "launch_pdl.h"
@@ -21,18 +22,19 @@ namespace marche {
 namespace {
 
 constexpr int kAttWarps = 8, kAttThreads = kAttWarps * 32, kKeys = 64;
+constexpr int RW = 2, kRows = RW * kAttWarps;            // queries per warp and per CTA at a time
 
 struct SimtLayout {                                      // in floats
   int ld, p_ld, tile, q, p, colsum, kv, total;
 };
-__host__ __device__ inline SimtLayout simt_layout(int S, int dh, int stages, int rows) {
+__host__ __device__ inline SimtLayout simt_layout(int S, int dh, int stages) {
   SimtLayout l;
   l.ld = dh + 4;                                         // rows 16 bytes apart modulo 128: conflict-free 128-bit reads
   l.p_ld = (S + kKeys - 1) / kKeys * kKeys + 4;
   l.tile = kKeys * l.ld;
   l.q = 0;
-  l.p = l.q + rows * l.ld;
-  l.colsum = l.p + rows * l.p_ld;
+  l.p = l.q + kRows * l.ld;
+  l.colsum = l.p + kRows * l.p_ld;
   l.kv = l.colsum + (S + 3) / 4 * 4;
   l.total = l.kv + stages * l.tile;
   return l;
@@ -42,23 +44,22 @@ MARCHE_DEVINL float dot4(float4 x, float4 y, float acc) {
   return fmaf(x.w, y.w, fmaf(x.z, y.z, fmaf(x.y, y.y, fmaf(x.x, y.x, acc))));
 }
 
-// NST K/V tiles in flight, RW queries per warp.  vec: the cache allows 16-byte copies.
-template <int NST, int RW>
+// NST K/V tiles in flight; HALVES 64-column halves of a head.  vec: the cache allows 16-byte copies.
+template <int NST, int HALVES>
 __global__ void __launch_bounds__(kAttThreads)
 attention_simt_kernel(const float* __restrict__ q, int ld_q, int n, int S, int H, int dh, int cs,
                       const float* __restrict__ cache_layer, long kv_stride, const uint8_t* __restrict__ is_new,
                       float* __restrict__ score_partial, float* __restrict__ o, int vec) {
-  constexpr int kRows = RW * kAttWarps;
   extern __shared__ float4 smem_f4[];
   float* smem = reinterpret_cast<float*>(smem_f4);
-  const SimtLayout l = simt_layout(S, dh, NST, kRows);
+  const SimtLayout l = simt_layout(S, dh, NST);
   float *qs = smem + l.q, *p = smem + l.p, *colsum = smem + l.colsum, *kv = smem + l.kv;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int rank = cs > 1 ? (int)ptx::cluster_ctarank() : 0, item = (int)blockIdx.x / cs;
+  const int item = (int)blockIdx.x / cs, rank = (int)blockIdx.x - item * cs;   // (clusters are consecutive CTAs)
   const int b = item / H, h = item - b * H, D = H * dh;
   const int row_begin = (int)((long)n * rank / cs), row_end = (int)((long)n * (rank + 1) / cs);
   const float* Kb = cache_layer + (long)b * S * D + h * dh;
-  const int n_kv = (S + kKeys - 1) / kKeys, dv = dh / 4;
+  const int n_kv = (S + kKeys - 1) / kKeys;
   const float scale = rsqrtf((float)dh);
   const uint32_t kv_base = ptx::smem_u32(kv);
   __shared__ bool flag[kRows];                           // scoring queries among the CTA's
@@ -74,38 +75,52 @@ attention_simt_kernel(const float* __restrict__ q, int ld_q, int n, int S, int H
         const int t0 = (i < n_kv ? i : i - n_kv) * kKeys;
         const float* src = Kb + (i < n_kv ? 0 : kv_stride);
         const uint32_t dst = kv_base + 4u * (uint32_t)((i % NST) * l.tile);
-        for (int t = tid >> 4; t < kKeys && t0 + (t & ~3) < S; t += kAttThreads / 16)
-          for (int v = tid & 15; v < dv; v += 16) {
-            const bool ok = t0 + t < S;
-            const float* s = src + (ok ? (long)(t0 + t) * D : 0L) + 4 * v;
-            const uint32_t d = dst + 4u * (uint32_t)(t * l.ld + 4 * v);
+        const int keys4 = S - t0 < kKeys ? (S - t0 + 3) & ~3 : kKeys;
+        const float* s = src + (t0 + (tid >> 4)) * D + 4 * (tid & 15);
+        uint32_t d = dst + 4u * (uint32_t)((tid >> 4) * l.ld + 4 * (tid & 15));
+        for (int t = tid >> 4; t < keys4; t += kAttThreads / 16, s += kAttThreads / 16 * D, d += 4u * (kAttThreads / 16) * l.ld) {
+          const bool ok = t0 + t < S;
+#pragma unroll
+          for (int half = 0; half < HALVES; ++half) {
+            if (64 * half + 4 * (tid & 15) >= dh) break;
+            const float* from = ok ? s + 64 * half : src;
             if (vec) {
-              asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(s), "r"(ok ? 16 : 0) : "memory");
+              asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d + 256u * half), "l"(from), "r"(ok ? 16 : 0) : "memory");
             } else {
 #pragma unroll
-              for (int j = 0; j < 4; ++j)
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d + 4 * j), "l"(s + j), "r"(ok ? 4 : 0) : "memory");
+              for (int e = 0; e < 4; ++e)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d + 256u * half + 4 * e), "l"(from + (ok ? e : 0)),
+                             "r"(ok ? 4 : 0) : "memory");
             }
           }
+        }
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    for (int i = 0; i < NST - 1; ++i) load(i);
-    // a warp's queries are rows warp, warp + 8; it loads them itself, so no barrier stands between
+    // a warp's queries are rows RW * warp, ...; it loads them itself, so no barrier stands between
     bool live[RW];
     const float* qr[RW];
     float* pr[RW];
+    float qv[RW][2 * HALVES];
 #pragma unroll
     for (int r = 0; r < RW; ++r) {
-      const int row = warp + r * kAttWarps;
+      const int row = RW * warp + r;
       live[r] = row < rows;
       if (is_new && lane == 0) flag[row] = live[r] && is_new[(long)b * n + r0 + row];
       qr[r] = qs + row * l.ld;
       pr[r] = p + row * l.p_ld;
-      for (int c = lane; c < dh; c += 32)
-        qs[row * l.ld + c] = live[r] ? q[((long)b * n + r0 + row) * ld_q + h * dh + c] * scale : 0.f;
+#pragma unroll
+      for (int e = 0; e < 2 * HALVES; ++e)
+        qv[r][e] = live[r] && lane + 32 * e < dh ? q[((long)b * n + r0 + row) * ld_q + h * dh + lane + 32 * e] : 0.f;
     }
-    float o_acc[RW][2][2] = {};                          // [query][64-column half of the head][column of the lane's pair]
+    for (int i = 0; i < NST - 1; ++i) load(i);
+#pragma unroll
+    for (int r = 0; r < RW; ++r)
+#pragma unroll
+      for (int e = 0; e < 2 * HALVES; ++e)
+        if (lane + 32 * e < dh) qs[(RW * warp + r) * l.ld + lane + 32 * e] = qv[r][e] * scale;
+    __syncwarp();
+    float o_acc[RW][HALVES][2] = {};                     // [query][64-column half of the head][column of the lane's pair]
 
     for (int i = 0; i < 2 * n_kv; ++i) {
       asm volatile("cp.async.wait_group %0;" ::"n"(NST - 2) : "memory");
@@ -148,14 +163,17 @@ attention_simt_kernel(const float* __restrict__ q, int ld_q, int n, int S, int H
           for (int r = 0; r < RW; ++r) {
             if (!live[r]) continue;
             float mx = -INFINITY, sum = 0.f;
+#pragma unroll 4
             for (int u = lane; u < n_kv * kKeys; u += 32) mx = fmaxf(mx, pr[r][u]);
             mx = warp_max(mx);
+#pragma unroll 2
             for (int u = lane; u < n_kv * kKeys; u += 32) {
               const float e = expf(pr[r][u] - mx);
               pr[r][u] = e;
               sum += e;
             }
             const float inv = 1.0f / warp_sum(sum);
+#pragma unroll 4
             for (int u = lane; u < n_kv * kKeys; u += 32) pr[r][u] *= inv;
           }
           __syncwarp();
@@ -180,7 +198,7 @@ attention_simt_kernel(const float* __restrict__ q, int ld_q, int n, int S, int H
             w[r][0] = x.x; w[r][1] = x.y; w[r][2] = x.z; w[r][3] = x.w;
           }
 #pragma unroll
-          for (int half = 0; half < 2; ++half) {
+          for (int half = 0; half < HALVES; ++half) {
             const int c = 64 * half + 2 * lane;
             if (c < dh) {
 #pragma unroll
@@ -200,10 +218,10 @@ attention_simt_kernel(const float* __restrict__ q, int ld_q, int n, int S, int H
 #pragma unroll
     for (int r = 0; r < RW; ++r)
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
+      for (int half = 0; half < HALVES; ++half) {
         const int c = 64 * half + 2 * lane;
         if (live[r] && c < dh) {
-          float* dst = o + ((long)b * n + r0 + warp + r * kAttWarps) * D + h * dh + c;
+          float* dst = o + ((long)b * n + r0 + RW * warp + r) * D + h * dh + c;
           dst[0] = o_acc[r][half][0];
           dst[1] = o_acc[r][half][1];
         }
@@ -229,15 +247,15 @@ attention_simt_kernel(const float* __restrict__ q, int ld_q, int n, int S, int H
   }
 }
 
-template <int NST, int RW>
+template <int NST, int HALVES>
 cudaError_t launch_stages(const float* q, int ld_q, int B, int n, int S, int H, int dh, int cs, const float* cache_layer,
                           const uint8_t* is_new, float* score_partial, float* o, cudaStream_t st) {
-  const size_t smem = (size_t)simt_layout(S, dh, NST, RW * kAttWarps).total * sizeof(float);
+  const size_t smem = (size_t)simt_layout(S, dh, NST).total * sizeof(float);
   static size_t smem_set[kMaxDevices] = {};
-  cudaError_t e = ensure_dynamic_smem(attention_simt_kernel<NST, RW>, smem, smem_set);
+  cudaError_t e = ensure_dynamic_smem(attention_simt_kernel<NST, HALVES>, smem, smem_set);
   if (e != cudaSuccess) return e;
   const int vec = (((uintptr_t)cache_layer) & 15) == 0;
-  return launch_pdl_cluster(attention_simt_kernel<NST, RW>, dim3(B * H * cs), dim3(kAttThreads), smem, cs, st, q, ld_q, n, S, H,
+  return launch_pdl_cluster(attention_simt_kernel<NST, HALVES>, dim3(B * H * cs), dim3(kAttThreads), smem, is_new ? cs : 1, st, q, ld_q, n, S, H,
                             dh, cs, cache_layer, (long)B * S * H * dh, is_new, score_partial, o, vec);
 }
 
@@ -247,14 +265,12 @@ cudaError_t launch_attention_simt(const float* q, int ld_q, int B, int n, int S,
                                   const float* cache_layer, const uint8_t* is_new, float* score_partial,
                                   float* o, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  // CTAs per item: one per 8 queries (one query per warp) while the launch stays within a few CTAs per SM; with more
-  // queries than that a warp takes two, which share every key and value it reads
+  // CTAs per item: one per eight queries (four warps) while the launch stays within a few CTAs per SM
   int cs = 1;
   while (cs < 8 && cs * kAttWarps < n && B * H * cs * 2 <= 4 * device_sm_count()) cs *= 2;
-  const bool one = cs * kAttWarps >= n;
   // four tiles in flight where two CTAs per SM still fit, else two
-  const bool deep = simt_layout(S, dh, 4, one ? kAttWarps : 2 * kAttWarps).total * sizeof(float) <= 112 * 1024;
-  if (one)
+  const bool deep = simt_layout(S, dh, 4).total * sizeof(float) <= 112 * 1024;
+  if (dh <= 64)
     return deep ? launch_stages<4, 1>(q, ld_q, B, n, S, H, dh, cs, cache_layer, is_new, score_partial, o, st)
                 : launch_stages<2, 1>(q, ld_q, B, n, S, H, dh, cs, cache_layer, is_new, score_partial, o, st);
   return deep ? launch_stages<4, 2>(q, ld_q, B, n, S, H, dh, cs, cache_layer, is_new, score_partial, o, st)

@@ -51,7 +51,8 @@ enum { ST2_PRODUCER = 0x31, ST2_MMA = 0x32, ST2_EPILOGUE = 0x33 };
 template <int BN, int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 gemm_tcgen05_2cta_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w,
-                         const __grid_constant__ CUtensorMap tmap_out, int M, int N, int K,
+                         const __grid_constant__ CUtensorMap tmap_ws, const __grid_constant__ CUtensorMap tmap_out,
+                         int M, int N, int K,
                          const float* __restrict__ bias, int* __restrict__ status, int* __restrict__ turn,
                          const KvScatter kv, int tail_split, int a_bf16) {
   using Cfg = PairCfg<BN>;
@@ -88,7 +89,7 @@ gemm_tcgen05_2cta_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
   //  * tail_split > 1 (whole-tile mode only): the tiles left over after the last full round
   //    (n_tiles mod n_pairs of them) are cut along N into tail_split column slices each, and the slices
   //    are dealt round-robin, so the last round costs about 1/tail_split of a tile instead of a whole one.
-  //    A slice loads the same W box (only its first rows are used) and issues MMAs with N = BN / tail_split.
+  //    A slice loads its own rows of W only (tmap_ws) and issues MMAs with N = BN / tail_split.
   int n_pieces, sk_u0 = 0, sk_u1 = 0, sk_t_last = 0, full_rounds = 0;
   if (turn) {
     const long U = (long)n_tiles * n_kb;
@@ -168,8 +169,8 @@ gemm_tcgen05_2cta_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
         get_piece(0, tile, kb0, kb1, n_off, n_w);
         const int wrow0 = (tile % n_n) * BN + n_off + (int)rank * (n_w / 2);
         for (; prefetched < STAGES && kb0 + prefetched < kb1; ++prefetched) {
-          if (rank == 0) ptx::mbar_expect_tx(full_bar(prefetched), 2 * Cfg::STAGE_BYTES);
-          ptx::tma_load_2d_pair(w_tile(prefetched), &tmap_w, (kb0 + prefetched) * BK, wrow0, leader_full0 + 8u * prefetched);
+          if (rank == 0) ptx::mbar_expect_tx(full_bar(prefetched), 2 * (A_BYTES + n_w * BK));
+          ptx::tma_load_2d_pair(w_tile(prefetched), n_w < BN ? &tmap_ws : &tmap_w, (kb0 + prefetched) * BK, wrow0, leader_full0 + 8u * prefetched);
         }
       }
       pdl_sync();
@@ -182,13 +183,15 @@ gemm_tcgen05_2cta_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
         const int m2 = tile / n_n, n_blk = tile - m2 * n_n;
         const int row0 = m2 * 2 * BM + (int)rank * BM;                // this CTA's 128 rows of A
         const int wrow0 = n_blk * BN + n_off + (int)rank * (n_w / 2);  // this CTA's half of the W rows of the slice
+        const CUtensorMap* w_map = n_w < BN ? &tmap_ws : &tmap_w;
+        const uint32_t bytes = 2 * (A_BYTES + n_w * BK);               // of both CTAs: n_w / 2 rows of 2 BK bytes each
         for (int kb = kb0; kb < kb1; ++kb, ++it) {
           if (it >= prefetched) {                          // else: slot armed and W already in flight
             if (!ptx::mbar_wait(empty_bar(s), phase, abort_flag)) { ok = false; break; }
-            if (rank == 0) ptx::mbar_expect_tx(full_bar(s), 2 * Cfg::STAGE_BYTES);
+            if (rank == 0) ptx::mbar_expect_tx(full_bar(s), bytes);
           }
           ptx::tma_load_2d_pair(a_tile(s), &tmap_a, kb * BK, row0, leader_full0 + 8u * s);
-          if (it >= prefetched) ptx::tma_load_2d_pair(w_tile(s), &tmap_w, kb * BK, wrow0, leader_full0 + 8u * s);
+          if (it >= prefetched) ptx::tma_load_2d_pair(w_tile(s), w_map, kb * BK, wrow0, leader_full0 + 8u * s);
           if (++s == STAGES) { s = 0; phase ^= 1u; }
         }
       }
@@ -363,8 +366,8 @@ cudaError_t max_resident_pairs(int* out) {
 }
 
 template <int BN, int EPI>
-cudaError_t launch_pair(const CUtensorMap& ta, const CUtensorMap& tw, const CUtensorMap& to, int M, int N, int K,
-                        const float* bias, int* status, int* turn, const KvScatter& kv, int a_bf16, const GemmTuning& tune,
+cudaError_t launch_pair(const CUtensorMap& ta, const CUtensorMap& tw, const CUtensorMap& to, const void* w, int M, int N,
+                        int K, const float* bias, int* status, int* turn, const KvScatter& kv, int a_bf16, const GemmTuning& tune,
                         cudaStream_t st) {
   static size_t smem_set[kMaxDevices] = {};
   cudaError_t e = ensure_dynamic_smem(gemm_tcgen05_2cta_kernel<BN, EPI>, (size_t)PairCfg<BN>::SMEM_BYTES, smem_set);
@@ -393,13 +396,18 @@ cudaError_t launch_pair(const CUtensorMap& ta, const CUtensorMap& tw, const CUte
     double best = 1.0;
     for (int sp = 2; sp <= 4; sp *= 2) {
       // measured at K = 1024: a half-width slice costs about 0.75 of a tile, a quarter-width one about 0.65
-      // (every slice loads the whole A tile again and pays its own ramp and epilogue)
+      // (every slice loads the whole A tile again and pays its own ramp and epilogue).  With the W rows of the slice
+      // only instead of a tile's 128 a CTA, N x K at M = 5248, back to back, us: 3072 x 1024 31.1 -> 30.4, 1024 x 1024
+      // 15.4 -> 15.0, 1024 x 4096 45.9 -> 44.7, 1280 x 5120 66.4 -> 65.2.
       const double cost = (double)((left * sp + pairs - 1) / pairs) * (1.0 / sp + (sp == 2 ? 0.25 : 0.40));
       if (cost < best - 0.05) { best = cost; tail_split = sp; }
     }
   }
+  CUtensorMap tws = tw;
+  if (tail_split > 1 && !make_map_2d(&tws, w, (uint64_t)N, (uint64_t)K, (uint64_t)K, (uint32_t)(BN / 2 / tail_split), !a_bf16))
+    return cudaErrorInvalidValue;
   return launch_pdl(gemm_tcgen05_2cta_kernel<BN, EPI>, dim3(2 * pairs), dim3(kThreads), (size_t)PairCfg<BN>::SMEM_BYTES,
-                    st, ta, tw, to, M, N, K, bias, status, use_turn, kv, tail_split, a_bf16);
+                    st, ta, tw, tws, to, M, N, K, bias, status, use_turn, kv, tail_split, a_bf16);
 }
 
 }  // namespace
@@ -452,7 +460,7 @@ cudaError_t launch_gemm_tcgen05_2cta(const void* a, int lda, int M, const void* 
     return cudaErrorInvalidValue;
 #define MARCHE_GEMM2_CASE(BN_, EPI_) \
   if (bn == BN_ && epilogue == EPI_)   \
-    return launch_pair<BN_, EPI_>(ta, tw, to, M, N, K, bias, status, turn, kv, a_bf16 ? 1 : 0, tune, st);
+    return launch_pair<BN_, EPI_>(ta, tw, to, w, M, N, K, bias, status, turn, kv, a_bf16 ? 1 : 0, tune, st);
   MARCHE_GEMM2_CASE(256, 0) MARCHE_GEMM2_CASE(256, 1) MARCHE_GEMM2_CASE(256, 2) MARCHE_GEMM2_CASE(256, 4)
   MARCHE_GEMM2_CASE(128, 0) MARCHE_GEMM2_CASE(128, 1) MARCHE_GEMM2_CASE(128, 2) MARCHE_GEMM2_CASE(128, 4)
 #undef MARCHE_GEMM2_CASE

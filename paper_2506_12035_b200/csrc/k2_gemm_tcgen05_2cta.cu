@@ -54,7 +54,7 @@ gemm_tcgen05_2cta_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
                          const __grid_constant__ CUtensorMap tmap_ws, const __grid_constant__ CUtensorMap tmap_out,
                          int M, int N, int K,
                          const float* __restrict__ bias, int* __restrict__ status, int* __restrict__ turn,
-                         const KvScatter kv, int tail_split, int a_bf16) {
+                         const KvScatter kv, int tail_split, int sk_num, int sk_den, int a_bf16) {
   using Cfg = PairCfg<BN>;
   constexpr int STAGES = Cfg::STAGES;
   extern __shared__ __align__(1024) uint8_t smem_raw[];     // (swizzled tiles; there is no room to align by hand)
@@ -79,9 +79,10 @@ gemm_tcgen05_2cta_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
   // Work list of this CTA pair, as pieces (tile, K-block range).
   //  * turn == nullptr: whole tiles, pair p takes tiles p, p + n_pairs, ...
   //  * turn != nullptr (residual epilogue only): stream-K.  The tiles' K-blocks, laid end to end, are cut
-  //    into n_pairs equal ranges, so no pair idles in a partial last wave.  A range is at least one
-  //    tile long, hence a tile is shared by at most two pairs: the one that owns its first K-blocks
-  //    (it adds the bias) and the one that owns the rest.  Each pair walks its range from the LAST tile
+  //    into n_pairs ranges of sk_num / sk_den tiles, so hardly any pair idles in a partial last wave, and no piece is
+  //    shorter than 1 / sk_den of a tile: a piece of a few K-blocks could not hide the epilogue of the one before it.
+  //    A range is at least one tile long, hence a tile is shared by at most two pairs: the one that owns its first
+  //    K-blocks (it adds the bias) and the one that owns the rest.  Each pair walks its range from the LAST tile
   //    to the first, so the piece that starts at K-block 0 is computed early and the completing piece
   //    late; the two TMA reduce-adds into the fp32 output are ordered by a per-(tile, rank, warp) turn
   //    flag in global memory (0 -> 1 by the first piece, back to 0 by the second), which keeps the
@@ -93,9 +94,9 @@ gemm_tcgen05_2cta_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
   int n_pieces, sk_u0 = 0, sk_u1 = 0, sk_t_last = 0, full_rounds = 0;
   if (turn) {
     const long U = (long)n_tiles * n_kb;
-    const long W = (U + n_pairs - 1) / n_pairs;
-    sk_u0 = (int)((long)pair * W < U ? (long)pair * W : U);
-    sk_u1 = (int)((long)sk_u0 + W < U ? (long)sk_u0 + W : U);
+    const long u0 = (long)pair * sk_num * n_kb / sk_den, u1 = (long)(pair + 1) * sk_num * n_kb / sk_den;
+    sk_u0 = (int)(u0 < U ? u0 : U);
+    sk_u1 = (int)(u1 < U ? u1 : U);
     sk_t_last = sk_u1 > sk_u0 ? (sk_u1 - 1) / n_kb : 0;
     n_pieces = sk_u1 > sk_u0 ? sk_t_last - sk_u0 / n_kb + 1 : 0;
   } else if (tail_split > 1) {
@@ -385,6 +386,16 @@ cudaError_t launch_pair(const CUtensorMap& ta, const CUtensorMap& tw, const CUte
   // work, the out-projection) cannot hide: measured 18 us with and without stream-K there.
   int* use_turn = (EPI == 1 && turn && tune.stream_k && K >= 2048 && n_tiles > max_pairs && n_tiles % max_pairs != 0 &&
                    n_tiles < 4 * max_pairs) ? turn : nullptr;
+  int sk_num = 1, sk_den = 1;
+  if (use_turn) {
+    // The shortest range of sk_num / sk_den tiles that covers the tiles, in pieces of at least 8 K blocks.  Against exactly
+    // equal ranges, in the step, sustained: N 1024, K 4096, 84 tiles (8/7 for 1.135) 43.6 -> 42.1 us; N 1280, K 5120, 105
+    // tiles (10/7 for 1.419) 66.2 -> 65.6; N 1024, K 4096, 116 tiles (11/7 for 1.568) 81.7 -> 81.2.
+    for (int den = 1; den <= K / BK / 8; ++den) {
+      const int num = (n_tiles * den + pairs - 1) / pairs;
+      if (den == 1 || num * sk_den < sk_num * den) { sk_num = num; sk_den = den; }
+    }
+  }
   // Whole-tile mode: cut the tiles of the last, partial round into 2 or 4 column slices when that
   // shortens the round (cost model in tile units, below).
   const int split_on = tune.tail_split;              // 0 off, 1 cost model, 2 / 4 forced (measurement only)
@@ -407,7 +418,7 @@ cudaError_t launch_pair(const CUtensorMap& ta, const CUtensorMap& tw, const CUte
   if (tail_split > 1 && !make_map_2d(&tws, w, (uint64_t)N, (uint64_t)K, (uint64_t)K, (uint32_t)(BN / 2 / tail_split), !a_bf16))
     return cudaErrorInvalidValue;
   return launch_pdl(gemm_tcgen05_2cta_kernel<BN, EPI>, dim3(2 * pairs), dim3(kThreads), (size_t)PairCfg<BN>::SMEM_BYTES,
-                    st, ta, tw, tws, to, M, N, K, bias, status, use_turn, kv, tail_split, a_bf16);
+                    st, ta, tw, tws, to, M, N, K, bias, status, use_turn, kv, tail_split, sk_num, sk_den, a_bf16);
 }
 
 }  // namespace

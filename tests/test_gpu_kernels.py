@@ -351,6 +351,28 @@ def test_select_refresh_policies_bit_exact(policy, name):
         assert np.array_equal(out.cpu().numpy(), orc.select_refresh(sc, new, excl, k, policy=name, seed=1234))
 
 
+@pytest.mark.parametrize("F,S,B", [(2048, 300, 64), (4096, 320, 64), (3072, 330, 100)])
+def test_fc2_shared_tiles_equal_whole_tiles(F, S, B):
+    """75, 80 and 129 tiles of 256 x 256 dealt to the CTA pairs in whole tiles or in ranges of 5/4, 9/8 and 7/4 tiles (74
+    pairs), where a pair completes what its neighbour began.  Everything before fc2 is the same launch; the sums of K
+    terms of order 1/16 differ by sqrt(K) 2^-24 at most, the additions to |hidden| < 8 by half a step, 2.4e-7, each."""
+    cfg, blocks, m = model_for("bf16", 256, 4, F, S, B)
+    hidden = torch.randn(B, S, 256, device="cuda", generator=torch.Generator(device="cuda").manual_seed(S))
+    cache, ws = m.alloc_cache(), m.alloc_workspace(S)
+    new = idx_dev(np.tile(np.arange(4, dtype=np.int32), (B, 1)))
+    refresh = torch.zeros(B * S, dtype=torch.int32, device="cuda")
+    m.set_tuning(gemm_kernel=2)
+    outs = []
+    for stream_k in (0, 1, 1):
+        m.set_tuning(stream_k=stream_k)
+        outs.append(torch.full((B, S, 256), 5.0, device="cuda"))
+        m.full_step(hidden, cache, new, None, 0.1, outs[-1], refresh, ws)
+    m.check_status()
+    assert outs[0].abs().max() < 8.0 and (outs[0] - hidden).abs().max() > 0.01
+    assert (outs[1] - outs[0]).abs().max() <= 1e-5
+    assert torch.equal(outs[1], outs[2])                                 # bit-reproducible
+
+
 def test_validate_indices():
     from paper_2506_12035_b200.binding import MarcheError
     S, B = 68, 2

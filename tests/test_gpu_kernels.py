@@ -558,6 +558,31 @@ def test_attention_small_sets_persistent(operand, dh, B, H, S, n):
             "b=%d: max-abs %.3g rel-L2 %.3g" % (b, max_abs(got[b], want), rel_l2(got[b], want))
 
 
+@pytest.mark.parametrize("dh", [64, 80])
+@pytest.mark.parametrize("S,n", [(33, 30), (64, 32), (100, 30), (164, 17), (192, 30), (192, 16)])
+def test_attention_persistent_rows_of_every_item(dh, S, n):
+    """2048 items, several per CTA, whose one to three key tiles fit the ring, so that an item's query rows are on their way
+    while the one before is computed: every row of every item, and the same bits in every launch.  Weights are bf16 (2^-9
+    each, of both signs over S keys, values below 6) and the output fp16: 3e-2 as in the other attention tests."""
+    from paper_2506_12035_b200 import binding
+    B, H = 128, 16
+    D = H * dh
+    cfg, blocks, m = model_for("bf16", D, H, 128, S, B)
+    m.set_tuning(attention_kernel=binding.ATTENTION_MMA)
+    gen = torch.Generator(device="cuda").manual_seed(S + n + dh)
+    q = (torch.randn(B * n, D, generator=gen, device="cuda") * 2.0).to(torch.bfloat16)
+    cache = torch.randn(2, B, S, D, generator=gen, device="cuda").to(torch.bfloat16)
+    heads = lambda t: t.view(B, -1, H, dh).transpose(1, 2).double()
+    want = torch.softmax(heads(q) @ heads(cache[0]).transpose(2, 3) / math.sqrt(dh), -1) @ heads(cache[1])
+    first = None
+    for _ in range(20):
+        o = torch.zeros(B * n, D, dtype=torch.float16, device="cuda")
+        m.attention(q, D, n, cache, None, None, o)
+        assert first is None or torch.equal(o, first)
+        first = o
+    assert (heads(first) - want).abs().max() <= 3e-2 and m.device_status() == 0
+
+
 @pytest.mark.parametrize("operand", ["bf16", "bf16b"])
 @pytest.mark.parametrize("B,H,S,n", [(2, 4, 68, 5), (2, 4, 128, 128), (3, 4, 320, 41), (40, 4, 320, 41), (2, 4, 320, 129),
                                      (2, 4, 320, 320), (100, 4, 320, 77), (2, 16, 1088, 122), (2, 16, 1088, 159),

@@ -183,7 +183,7 @@ bool use_pair(const marche_ctx* ctx, int M, int N, int K) {
 // (Clearing them costs a few microseconds of a step on few rows: the kernels on either side of a memset do not overlap.)
 bool needs_turn(const marche_ctx* ctx, int M) {
   const int D = ctx->cfg.width, F = ctx->cfg.mlp_dim;
-  return ctx->bf16 && ctx->tune.stream_k && ((F >= 2048 && use_pair(ctx, M, D, F)) || (D >= 2048 && use_pair(ctx, M, D, D)));
+  return M > 0 && ctx->bf16 && ctx->tune.stream_k && ((F >= 2048 && use_pair(ctx, M, D, F)) || (D >= 2048 && use_pair(ctx, M, D, D)));
 }
 
 // True when the QKV projection writes K and V into the cache itself: no scatter_kv launch then.
@@ -202,6 +202,7 @@ int do_linear(marche_ctx* ctx, int cls, const void* a, int lda, int M, const voi
   // 16-bit contexts run on the tensor cores or not at all
   if (N % 128 || K % 64) return MARCHE_ESHAPE;
   if (lda % 8 || (((uintptr_t)a | (uintptr_t)w | (uintptr_t)out) & 15)) return misaligned(ctx, "projection");
+  if (M == 0) return MARCHE_OK;                         // no rows: no estimate of a kernel's time either
   const bool pair = use_pair(ctx, M, N, K);
   for (int r = 0; r < launches_of(ctx, cls); ++r) {
     if (M > 0) mark(ctx, cls, st);

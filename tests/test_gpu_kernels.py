@@ -156,6 +156,19 @@ def test_linear_strided_input_and_row_guard(dtype):
     assert (host(out[M:]) == 5.0).all()
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "bf16b"])
+@pytest.mark.parametrize("gemm_kernel", [0, 1, 2])
+def test_linear_of_no_rows(dtype, gemm_kernel):
+    """M = 0 is a valid call that enqueues nothing, whichever kernel would run."""
+    cfg, blocks, m = model_for(dtype, 256, 4, 1024, 68, 2)
+    m.set_tuning(gemm_kernel=gemm_kernel)
+    a, w, bias = torch.zeros(8, 256, dtype=adt(dtype), device="cuda"), torch.zeros(512, 256, dtype=adt(dtype), device="cuda"), torch.zeros(512, device="cuda")
+    for epi, t in ((0, tdt(dtype)), (1, torch.float32), (2, adt(dtype))):
+        out = torch.full((8, 512), 5.0, dtype=t, device="cuda")
+        m.linear(a, w, bias, epi, out, M=0)
+        assert (out == 5.0).all()
+
+
 # ------------------------------------------------------------------ K5 scatter
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("n", [1, 7, 41])

@@ -773,7 +773,7 @@ int marche_gather_layernorm(marche_ctx* ctx, const float* src, int src_rows, con
   if (!idx && n > src_rows) return MARCHE_EINVAL;
   mark(ctx, MARCHE_KC_GATHER_LN, (cudaStream_t)stream);
   MARCHE_TRY(launch_gather_layernorm(ctx->a_kind, src, src_rows, idx, ctx->cfg.batch, n, ctx->cfg.width, gamma, beta,
-                                     ctx->eps, x_out, u_out, (cudaStream_t)stream), "gather_layernorm");
+                                     ctx->eps, x_out, u_out, (cudaStream_t)stream, nullptr, 0, false), "gather_layernorm");
   return MARCHE_OK;
 }
 

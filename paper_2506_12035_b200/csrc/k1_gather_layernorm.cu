@@ -15,15 +15,16 @@ namespace marche {
 constexpr int kLnWarps = 8, kLnFewWarps = 4;
 
 // FEW: at most kLnFewWarps rows per SM.  Then a launch is one chain of latencies (1.0 us of it, plus 1.4 us of hand-overs),
-// so gamma and beta, which no kernel writes, are fetched ahead of the dependency wait (their first touch comes from HBM)
-// and a CTA has only as many warps as it takes to give every SM a row.  With many rows the 16 registers per 512 bytes of
-// row that this costs would halve the warps in flight, which is what hides the latency there.
+// so a CTA has only as many warps as it takes to give every SM a row, and gamma and beta are fetched ahead of the
+// dependency wait (their first touch comes from HBM) where params_ready says that they were complete before the preceding
+// launch: a stack's weights are, those of a single call may have been written by it.  With many rows the 16 registers per
+// 512 bytes of row that this costs would halve the warps in flight, which is what hides the latency there.
 template <typename TOut, int NV, bool FEW>
 __global__ void __launch_bounds__((FEW ? kLnFewWarps : kLnWarps) * 32)
 gather_layernorm_kernel(const float* __restrict__ src, int src_rows, const int32_t* __restrict__ idx,
                         int n, int total_rows, const float* __restrict__ gamma,
                         const float* __restrict__ beta, float eps, float* __restrict__ x_out,
-                        TOut* __restrict__ u_out, const int32_t* __restrict__ out_idx, int out_rows) {
+                        TOut* __restrict__ u_out, const int32_t* __restrict__ out_idx, int out_rows, int params_ready) {
   constexpr int D = NV * 128;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long r = (long)blockIdx.x * (blockDim.x >> 5) + warp;
@@ -32,6 +33,7 @@ gather_layernorm_kernel(const float* __restrict__ src, int src_rows, const int32
   const float4* b4 = reinterpret_cast<const float4*>(beta);
   float4 gv[FEW ? NV : 1], bv[FEW ? NV : 1];
   if (FEW) {
+    if (!params_ready) pdl_sync();
 #pragma unroll
     for (int i = 0; i < NV; ++i) { gv[FEW ? i : 0] = __ldg(g4 + i * 32 + lane); bv[FEW ? i : 0] = __ldg(b4 + i * 32 + lane); }
   }
@@ -76,7 +78,7 @@ gather_layernorm_kernel(const float* __restrict__ src, int src_rows, const int32
 template <typename TOut>
 static cudaError_t launch_ln_t(const float* src, int src_rows, const int32_t* idx, int B, int n, int D,
                                const float* gamma, const float* beta, float eps, float* x_out, TOut* u_out,
-                               cudaStream_t st, const int32_t* out_idx, int out_rows) {
+                               cudaStream_t st, const int32_t* out_idx, int out_rows, bool params_ready) {
   const long rows = (long)B * n;
   if (rows == 0) return cudaSuccess;
   const int sms = device_sm_count();
@@ -91,10 +93,10 @@ static cudaError_t launch_ln_t(const float* src, int src_rows, const int32_t* id
       err = prefer_shared_memory(gather_layernorm_kernel<TOut, NV_, true>, carved);                  \
       if (err == cudaSuccess)                                                                        \
         err = launch_pdl(gather_layernorm_kernel<TOut, NV_, true>, dim3(grid), dim3(warps * 32), 0, st, src, src_rows, \
-                         idx, n, (int)rows, gamma, beta, eps, x_out, u_out, out_idx, out_rows);      \
+                         idx, n, (int)rows, gamma, beta, eps, x_out, u_out, out_idx, out_rows, (int)params_ready);      \
     } else {                                                                                         \
       err = launch_pdl(gather_layernorm_kernel<TOut, NV_, false>, dim3(grid), dim3(warps * 32), 0, st, src, src_rows, \
-                       idx, n, (int)rows, gamma, beta, eps, x_out, u_out, out_idx, out_rows);        \
+                       idx, n, (int)rows, gamma, beta, eps, x_out, u_out, out_idx, out_rows, (int)params_ready);        \
     }                                                                                                \
     break;
   switch (D / 128) {
@@ -111,13 +113,16 @@ static cudaError_t launch_ln_t(const float* src, int src_rows, const int32_t* id
 cudaError_t launch_gather_layernorm(int out_kind, const float* src, int src_rows, const int32_t* idx,
                                     int B, int n, int D, const float* gamma, const float* beta, float eps,
                                     float* x_out, void* u_out, cudaStream_t st, const int32_t* out_idx,
-                                    int out_rows) {
+                                    int out_rows, bool params_ready) {
   if (D % 128 != 0) return cudaErrorInvalidValue;
   if (out_kind == OUT_F16)
-    return launch_ln_t<f16>(src, src_rows, idx, B, n, D, gamma, beta, eps, x_out, (f16*)u_out, st, out_idx, out_rows);
+    return launch_ln_t<f16>(src, src_rows, idx, B, n, D, gamma, beta, eps, x_out, (f16*)u_out, st, out_idx, out_rows,
+                            params_ready);
   if (out_kind == OUT_BF16)
-    return launch_ln_t<bf16>(src, src_rows, idx, B, n, D, gamma, beta, eps, x_out, (bf16*)u_out, st, out_idx, out_rows);
-  return launch_ln_t<float>(src, src_rows, idx, B, n, D, gamma, beta, eps, x_out, (float*)u_out, st, out_idx, out_rows);
+    return launch_ln_t<bf16>(src, src_rows, idx, B, n, D, gamma, beta, eps, x_out, (bf16*)u_out, st, out_idx, out_rows,
+                            params_ready);
+  return launch_ln_t<float>(src, src_rows, idx, B, n, D, gamma, beta, eps, x_out, (float*)u_out, st, out_idx, out_rows,
+                            params_ready);
 }
 
 }  // namespace marche

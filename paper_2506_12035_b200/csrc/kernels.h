@@ -12,10 +12,11 @@ namespace marche {
 enum { OUT_F32 = 0, OUT_F16 = 1, OUT_BF16 = 2 };
 
 // K1: gather + LayerNorm (output type out_kind).  rows = B*n; src row of (b, j) is src[b][idx ? idx[b][j] : j].
+// params_ready: gamma and beta were complete before the preceding launch of the stream.
 cudaError_t launch_gather_layernorm(int out_kind, const float* src, int src_rows, const int32_t* idx,
                                     int B, int n, int D, const float* gamma, const float* beta, float eps,
                                     float* x_out, void* u_out, cudaStream_t st, const int32_t* out_idx = nullptr,
-                                    int out_rows = 0);
+                                    int out_rows = 0, bool params_ready = true);
 
 // K5: K/V write-back into one block's cache slice [2][B][S][D]; idx NULL = identity.
 cudaError_t launch_scatter_kv(bool bf16_t, const void* k, const void* v, int ld_kv, const int32_t* idx,

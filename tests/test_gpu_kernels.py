@@ -76,6 +76,26 @@ def test_gather_layernorm(dtype, D, H, n):
     assert_close(host(u_out), want, dtype, "LN identity", scale=1.0 if dtype in LOW else 10.0)
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("D", [256, 2048])
+def test_gather_layernorm_of_parameters_just_gathered(dtype, D):
+    """gamma and beta come from the call right before (rows picked from a table): few rows, whose launch is set up while
+    that call still runs, must not read them before it has written them."""
+    S, B, n = 320, 2, 41
+    cfg, blocks, m = model_for(dtype, D, D // 64, 128, S, B)
+    gen = torch.Generator(device="cuda").manual_seed(D)
+    table, x = torch.randn(B, S, D, generator=gen, device="cuda"), torch.randn(B, S, D, generator=gen, device="cuda")
+    xn = torch.nn.functional.layer_norm(x[:, :n].double(), (D,), eps=cfg.ln_eps).reshape(B * n, D)
+    picked = torch.zeros(B, S, D, device="cuda")
+    u = torch.zeros(B * n, D, dtype=adt(dtype), device="cuda")
+    for t in range(8):
+        order = torch.randperm(S, generator=gen, device="cuda").to(torch.int32).expand(B, S).contiguous()
+        m.gather_rows(table, order, picked)
+        m.gather_layernorm(x, None, n, picked[1, S - 2], picked[1, S - 1], None, u)
+        want = xn * table[1, order[0, S - 2]].double() + table[1, order[0, S - 1]].double()
+        assert (u.double() - want).abs().max() <= (2e-2 if dtype in LOW else 1e-4)     # |want| < 32: half an fp16 step 8e-3
+
+
 # ------------------------------------------------------------------ K2 projections
 @pytest.mark.parametrize("dtype", ["f32", "bf16", "bf16b"])
 @pytest.mark.parametrize("M", [1, 24, 62, 129, 300])

@@ -470,10 +470,10 @@ int marche_device_status(const marche_ctx* ctx);
  * invalid; marche_device_status() names the kernel) or MARCHE_OK.  Synchronous.  The other
  * synchronous calls, marche_validate_indices and marche_profile_end, report the same condition. */
 int marche_check_status(marche_ctx* ctx, marche_stream stream);
-/* Test hook for that path: enqueues a one-warp kernel whose single waiting thread uses the library's
- * bounded wait on a barrier that nothing arrives on.  After `limit_cycles` SM clock cycles (1 ..
- * 2e9; a million is about half a millisecond) the wait gives up, the status word is set and the
- * kernel returns; nothing traps and the context stays usable.  Asynchronous. */
+/* Test hook for that path: enqueues a kernel of two one-warp CTAs (a cluster) in which one thread uses the
+ * library's bounded wait on a barrier that nothing arrives on.  After `limit_cycles` SM clock cycles (1 ..
+ * 2e9; a million is about half a millisecond) the wait gives up, the cluster is told, the other CTA sets the
+ * status word and the kernel returns; nothing traps and the context stays usable.  Asynchronous. */
 int marche_debug_bounded_wait(marche_ctx* ctx, long long limit_cycles, marche_stream stream);
 /* Number of kernels this context has launched so far. */
 unsigned long long marche_launch_count(const marche_ctx* ctx);

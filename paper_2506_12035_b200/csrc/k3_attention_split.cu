@@ -11,7 +11,8 @@
 // dependency wait: the L2 is where a concurrent write-back of fresh rows lands too, so nothing stale can be kept.
 // Arithmetic as in the ring kernel (mma.sync m16n8k16, fp32 softmax statistics).  16 heads, head_dim 64, us before -> after:
 // 32 items: S 320, 41 rows 6.9 -> 4.5, 5 rows 5.5 -> 3.1; S 1088, 41 rows 17.8 -> 6.8; 160 items, S 320, 41 rows 8.7 -> 7.0.
-// Every wait is bounded; all threads of a cluster reach both cluster barriers, whatever happened.
+// Every wait is bounded; all threads of a cluster reach both cluster barriers, whatever happened, and no CTA of a cluster
+// stores a row after one of them gave up.
 #include <cuda.h>
 
 #include "attention_common.cuh"
@@ -194,10 +195,14 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid
       }
     }
   }
-  if (!ok && lane == 0) {
-    *(volatile int*)status = ST_ATTENTION_SPLIT;
-    // let copies already issued land before the CTA's shared memory is released
-    for (int i = 0; i < n_tiles; ++i) ptx::mbar_wait(full0 + 8u * i, 0, abort_flag + 1, 20000000LL);
+  ok = __all_sync(0xffffffffu, ok);
+  if (!ok) {
+    if (lane == 0) {
+      *(volatile int*)status = ST_ATTENTION_SPLIT;
+      // let copies already issued land before the CTA's shared memory is released
+      for (int i = 0; i < n_tiles; ++i) ptx::mbar_wait(full0 + 8u * i, 0, abort_flag + 1, 20000000LL);
+    }
+    __syncwarp();
   }
 
   if (n_parts == 1) {
@@ -216,6 +221,7 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid
     // ---- partial results to the owners of the rows
     if (cs > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // every CTA of the cluster has started
     else __syncthreads();                                // the tiles are used up
+    if (cs > 1 && !ok) ptx::cluster_raise(ptx::smem_u32(abort_flags), cs, lane);         // nobody merges what is missing
     if (warp_active && ok) {
 #pragma unroll
       for (int r = 0; r < 2; ++r) {

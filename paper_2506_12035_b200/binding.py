@@ -127,9 +127,15 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return t.data_ptr()
 
 
+# (building a torch.cuda.Stream object costs more than the ctypes call; the short cut is private to torch and may go)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream: Optional[torch.cuda.Stream]) -> Optional[int]:
-    if stream is None:                    # (building a torch.cuda.Stream object costs more than the ctypes call)
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) or None
+    if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device()) or None
+        stream = torch.cuda.current_stream()
     return stream.cuda_stream or None
 
 

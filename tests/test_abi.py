@@ -94,3 +94,20 @@ int main(void) {
                     "-Wl,-rpath," + os.path.dirname(so)], check=True)
     out = subprocess.run([str(exe)], capture_output=True, text=True)
     assert out.returncode == 0 and "abi ok" in out.stdout, (out.returncode, out.stdout, out.stderr)
+
+
+@pytest.mark.parametrize("raw", [None, lambda device: 0x5000 + device])
+def test_current_stream_with_and_without_the_private_short_cut(monkeypatch, raw):
+    """Calls go to torch's current stream, also where torch has no raw-stream getter."""
+    import torch
+    from paper_2506_12035_b200 import binding
+
+    class Stream:
+        def __init__(self, handle):
+            self.cuda_stream = handle
+
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream(0x5003))
+    monkeypatch.setattr(binding, "_raw_stream", raw)
+    assert binding._stream(None) == 0x5003
+    assert binding._stream(Stream(0x7000)) == 0x7000 and binding._stream(Stream(0)) is None

@@ -355,7 +355,7 @@ int marche_gather_rows(marche_ctx* ctx, const float* src, const int32_t* idx, in
  *   h_new_idx       host int32 [B][n_new] (G);  h_excl_idx host int32 [B][n_excl] or NULL
  *   refresh_in      device int32 [B][n_refresh_in]: the previous call's refresh_out
  *   refresh_out     device int32, room for B*floor(ratio*S+1/2) entries (the next call's
- *                   refresh_in; use two buffers alternately)
+ *                   refresh_in; use two buffers alternately); NULL where that is no entry
  *   h_out_rows      host float [B][n_new][D] or NULL: hidden_out rows of new_idx
  *   h_refresh_out   host int32 [B][K] or NULL;  n_refresh host int, receives K
  *   staging         device scratch of marche_staging_bytes(ctx, max_new), 256-byte aligned,

@@ -849,8 +849,9 @@ int marche_step_host(marche_ctx* ctx, int full, float* hidden, void* kv_cache, c
                      float refresh_ratio, float* hidden_out, int32_t* refresh_out, float* h_out_rows,
                      int32_t* h_refresh_out, int* n_refresh, int max_new, void* staging, size_t staging_bytes,
                      void* workspace, size_t workspace_bytes, marche_stream stream) {
-  if (!ctx || !hidden || !staging || !refresh_out || n_prev < 0 || n_new < 0 || n_excl < 0 || n_refresh_in < 0)
-    return MARCHE_EINVAL;
+  if (!ctx || !hidden || !staging || n_prev < 0 || n_new < 0 || n_excl < 0 || n_refresh_in < 0) return MARCHE_EINVAL;
+  // (no list of refreshed tokens where none are to be refreshed)
+  if (!refresh_out && refresh_count(refresh_ratio, ctx->cfg.seq_len, ctx->cfg.seq_len - n_new - n_excl) > 0) return MARCHE_EINVAL;
   if (n_prev > max_new || n_new > max_new || n_excl > max_new) return MARCHE_EINVAL;
   if ((n_prev && (!h_prev_rows || !h_prev_idx)) || (n_new && !h_new_idx) || (n_excl && !h_excl_idx) ||
       (n_refresh_in && !refresh_in))

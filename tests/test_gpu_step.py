@@ -287,6 +287,45 @@ def test_host_driven_step_matches_device_loop():
     assert all(v[0] >= 0 for v in prof.values())
 
 
+def test_host_driven_step_without_refresh():
+    """With ratio 0 there is no list of refreshed tokens: marche_step_host takes NULL (or an empty tensor) for it and gives the
+    rows of the device-resident calls; with a ratio that selects tokens NULL stays an error."""
+    cfg = synth.CONFIGS["tiny"].replace(dtype="bf16")
+    blocks = synth.make_weights(cfg)
+    m = make_model(cfg, blocks)
+    B, S, D = cfg.B, cfg.S, cfg.D
+    hidden0 = synth.make_hidden(cfg)
+    sets = synth.new_token_sets(cfg, synth.generation_orders(cfg))
+    G0, G1 = sets[0].astype(np.int32), sets[1].astype(np.int32)
+    rows = synth.replacement_rows(cfg, 0, G0.shape[1])
+    ws, most = m.alloc_workspace(S), max(G0.shape[1], G1.shape[1])
+    staging = torch.empty(m.staging_bytes(most), dtype=torch.uint8, device="cuda")
+    pin = lambda a: torch.as_tensor(np.ascontiguousarray(a)).pin_memory()
+    h_G0, h_G1, h_rows = pin(G0), pin(G1), pin(rows)
+    results = []
+    for refresh in (None, torch.empty(B, 0, dtype=torch.int32, device="cuda")):
+        hidden, cache, out = dev(hidden0), m.alloc_cache(), torch.zeros(B, S, D, device="cuda")
+        h_out0, h_out1 = torch.zeros(B, G0.shape[1], D).pin_memory(), torch.zeros(B, G1.shape[1], D).pin_memory()
+        m.init_cache(cache)
+        assert m.step_host(True, hidden, cache, None, None, h_G0, None, None, 0, 0.0, out, refresh, h_out0, None, most, staging, ws) == 0
+        assert m.step_host(False, hidden, cache, h_rows, h_G0, h_G1, None, None, 0, 0.0, out, refresh, h_out1, None, most, staging, ws) == 0
+        torch.cuda.synchronize()
+        results.append((h_out0, h_out1, out))
+    hidden, cache, out = dev(hidden0), m.alloc_cache(), torch.zeros(B, S, D, device="cuda")
+    m.init_cache(cache)
+    m.full_step(hidden, cache, idx_dev(G0), None, 0.0, out, None, ws)
+    m.scatter_rows(dev(rows), idx_dev(G0), hidden)
+    m.step(hidden, cache, idx_dev(np.concatenate([G1, G0], axis=1)), idx_dev(G1), None, 0.0, out, None, ws)
+    for h_out0, h_out1, o in results:
+        assert torch.equal(o, out)
+        for b in range(B):
+            assert torch.equal(h_out1[b], out[b, torch.as_tensor(G1[b], dtype=torch.long, device="cuda")].cpu())
+    for full in (True, False):
+        with pytest.raises(MarcheError) as e:
+            m.step_host(full, hidden, cache, None, None, h_G1, None, None, 0, 0.1, out, None, h_out1, None, most, staging, ws)
+        assert e.value.code == -1
+
+
 def test_argument_errors():
     cfg = synth.CONFIGS["tiny"]
     blocks = synth.make_weights(cfg)

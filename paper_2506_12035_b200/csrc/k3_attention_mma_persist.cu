@@ -131,15 +131,6 @@ attention_mma_persist_kernel(const __grid_constant__ CUtensorMap tmap_kv, const 
       for (int kk = 0; kk < Cfg::KSTEPS; ++kk)
         ldsm_x4(q_tile + tile_off<DH>(warp * 16 + (lane & 15), 2 * kk + (lane >> 4)), qf[kk][0], qf[kk][1], qf[kk][2],
                 qf[kk][3]);
-      // The producer may fetch the next unit's rows, but not before the fragments are here: the arrival's address depends on
-      // them (n >> 24 is zero).  With an arrival merely behind the reads, launches whose tiles of a unit fit the ring (up to
-      // three), so that the next rows are on their way at once, differed from run to run: at 2048 items, S 33 to 192 and 30
-      // rows by as much as one to five wrong 16-row groups of 4096; none in twenty launches of each with the dependence.
-      uint32_t seen = 0u;
-#pragma unroll
-      for (int kk = 0; kk < Cfg::KSTEPS; ++kk) seen |= (qf[kk][0] | qf[kk][1]) | (qf[kk][2] | qf[kk][3]);
-      __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(q_empty + (seen & ((uint32_t)n >> 24)));
       float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};   // running max of the RAW logits, sum
 #pragma unroll
       for (int j = 0; j < Cfg::ONT; ++j) oacc[j][0] = oacc[j][1] = oacc[j][2] = oacc[j][3] = 0.f;
@@ -230,9 +221,18 @@ attention_mma_persist_kernel(const __grid_constant__ CUtensorMap tmap_kv, const 
             }
           }
         }
-        // this warp is done with the stage: release it to the producer
+        // This warp is done with the stage: release it to the producer, with a unit's first one the query rows too, whose
+        // fragments that tile's products have used.  Released right behind the reads, which nothing made wait for their
+        // results, launches whose tiles of a unit fit the ring (up to three), so that the next rows come at once, differed
+        // from run to run: at 2048 items, S 33 to 192 and 30 rows by as much as one to five wrong 16-row groups of 4096;
+        // none in twenty launches of each since.  No later than the ring's next free slot with four tiles or more: S 320,
+        // 2048 items, 24 rows 28.5 us either way; one tile 10.2 -> 11.2 us.  An arrival that depends on the fragments' values
+        // instead cost 0.4 us per unit.
         __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(empty_bar(s));
+        if (lane == 0) {
+          ptx::mbar_arrive(empty_bar(s));
+          if (kt == 0) ptx::mbar_arrive(q_empty);
+        }
         if (++s == NSTAGE) { s = 0; ring_phase ^= 1u; }
       }
       if (!ok) break;

@@ -4,7 +4,7 @@
 //
 // Persistent CTAs (one per SM).  The work of a CTA is a list of units, one unit = one 128-row query
 // tile of one (sample, head) item against all S keys; FOUR independent streams (three at head_dim 80, whose buffers are
-// larger) inside the CTA take the units in turn.  A unit is a latency chain (Q K^T -> read logits -> exponentials -> write weights
+// larger; one where a CTA has a single unit) inside the CTA take the units in turn.  A unit is a latency chain (Q K^T -> read logits -> exponentials -> write weights
 // -> P V -> next Q K^T ...), and the exponentials - 16 per clock and SM - are the scarce resource once the active set
 // is large; four chains in flight per SM partition keep those units busy while each chain waits on its hand-overs.
 // Each stream owns a query buffer, TMA rings of 64-key tiles (three of K, two of V: a K tile is used up a step earlier)
@@ -52,8 +52,8 @@ enum { ST_ATT_STREAM = 0x51 };
 enum { B_K_FULL = 0, B_K_EMPTY = B_K_FULL + NK, B_V_FULL = B_K_EMPTY + NK, B_V_EMPTY = B_V_FULL + NV, B_Q_FULL = B_V_EMPTY + NV,
        B_Q_EMPTY, B_S_FULL, B_P_FULL, B_O_FULL, NB };
 
-template <int DH> struct Cfg {
-  static constexpr int NS = DH == 64 ? 4 : 3;                // streams per CTA
+template <int DH> struct Streams { static constexpr int N = DH == 64 ? 4 : 3; };   // per CTA
+template <int DH, int NS> struct Cfg {
   static constexpr int THREADS = NS * 6 * 32;                // per stream four softmax warps, a producer, an MMA issuer
   static constexpr int W_PROD = NS * 4, W_MMA = NS * 5;
   static constexpr int T_MAIN = KT * 128, T_BYTES = KT * DH * 2;   // a K or V tile; its columns 0-63
@@ -177,12 +177,12 @@ MARCHE_DEVINL Unit unit_of(int j, int u, bool deal_units, int n_qt, int n, int H
 }
 
 // tmap_kv, tmap_q: columns 0-63 of a head; the tails: columns 64-79 (unused at head_dim 64).
-template <int DH>
-__global__ void __launch_bounds__(Cfg<DH>::THREADS, 1)
+template <int DH, int NS>
+__global__ void __launch_bounds__(Cfg<DH, NS>::THREADS, 1)
 attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid_constant__ CUtensorMap tmap_q,
                            const __grid_constant__ CUtensorMap tmap_kv_tail, const __grid_constant__ CUtensorMap tmap_q_tail, int n, int S, int H, int B, uint16_t* __restrict__ o, int o_bf16, int* __restrict__ status) {
-  using C = Cfg<DH>;
-  constexpr int NS = C::NS;
+  using C = Cfg<DH, NS>;
+  constexpr bool ROOM = NS == 1;                           // registers hold a row's logits and its weights
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = ptx::smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -376,7 +376,7 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
               if (c + KT / 2 < lim) mx[2 + (c & 1)] = fmaxf(mx[2 + (c & 1)], __uint_as_float(vb[c]));
             }
           }
-          ptx::tmem_ld_32x32(t_s, va);                     // again, for the exponentials
+          if (!ROOM) ptx::tmem_ld_32x32(t_s, va);          // again, for the exponentials
           const float tmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
           // lazy reference maximum: move it only when this tile exceeds it by more than 2^8
           const bool move = (tmax - m_ref) * c_log2 > 8.0f;   // also true for a unit's first tile (m_ref = -inf)
@@ -409,7 +409,7 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
             }
           };
           weights(vb, lim - KT / 2);
-          ptx::tmem_ld_wait(va);
+          if (!ROOM) ptx::tmem_ld_wait(va);
           tmem_st_32x16(t_s + KT / 4, vb);                 // over logits that have been read
           weights(va, lim);
           tmem_st_32x16(t_s, va);
@@ -483,10 +483,10 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
   }
 }
 
-template <int DH>
+template <int DH, int NS>
 cudaError_t launch_stream(const void* q, int ld_q, int B, int n, int S, int H, const void* cache_layer, void* o, bool o_bf16,
                           int* status, cudaStream_t st) {
-  using C = Cfg<DH>;
+  using C = Cfg<DH, NS>;
   const int D = H * DH;
   // columns 0-63 of a head as 128-byte rows, columns 64-79 as 32-byte rows, both swizzled
   CUtensorMap tkv, tq, tkv_tail, tq_tail;
@@ -502,12 +502,12 @@ cudaError_t launch_stream(const void* q, int ld_q, int B, int n, int S, int H, c
   if (DH > 64 && (!make(&tkv_tail, cache_layer, D, S, 2 * B, KT, true) || !make(&tq_tail, q, ld_q, n, B, QT, true)))
     return cudaErrorInvalidValue;
   static size_t smem_set[kMaxDevices] = {};
-  cudaError_t e = ensure_dynamic_smem(attention_tc_stream_kernel<DH>, (size_t)C::SMEM_BYTES, smem_set);
+  cudaError_t e = ensure_dynamic_smem(attention_tc_stream_kernel<DH, NS>, (size_t)C::SMEM_BYTES, smem_set);
   if (e != cudaSuccess) return e;
   const int sms = device_sm_count();
   const long units = (long)B * H * ((n + QT - 1) / QT);
   const int grid = units < sms ? (int)units : sms;
-  return launch_pdl(attention_tc_stream_kernel<DH>, dim3(grid), dim3(C::THREADS), (size_t)C::SMEM_BYTES, st, tkv, tq, tkv_tail,
+  return launch_pdl(attention_tc_stream_kernel<DH, NS>, dim3(grid), dim3(C::THREADS), (size_t)C::SMEM_BYTES, st, tkv, tq, tkv_tail,
                     tq_tail, n, S, H, B, (uint16_t*)o, o_bf16 ? 1 : 0, status);
 }
 
@@ -522,7 +522,7 @@ bool attention_tc_stream_wins(int n, int S, int dh, int items, int min_rows) {
   if (n > min_rows) return true;
   if (3 * n <= 2 * min_rows) return false;
   if (dh == 64) return S >= 512;
-  const int streams = Cfg<80>::NS * device_sm_count(), rounds = (items + streams - 1) / streams;
+  const int streams = Streams<80>::N * device_sm_count(), rounds = (items + streams - 1) / streams;
   return S > 4 * KT && (rounds == 1 || 4 * items >= 3 * rounds * streams);
 }
 
@@ -531,8 +531,14 @@ cudaError_t launch_attention_tc_stream(const void* q, int ld_q, int B, int n, in
   if (n == 0) return cudaSuccess;
   if ((dh != 64 && dh != 80) || ld_q % 8 || ((uintptr_t)q & 15) || ((uintptr_t)cache_layer & 15) || ((uintptr_t)o & 15) || S > 2048)
     return cudaErrorInvalidValue;
-  return dh == 64 ? launch_stream<64>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st)
-                  : launch_stream<80>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
+  // No more units than SMs: a CTA has one, and a CTA of one stream, with registers for a row's logits beside its weights (104 a
+  // thread where four streams leave 80), takes it through its tiles faster.  One stream against four, us: 16 items, S 640, 80
+  // rows 12.2 and 13.2; 144 items, S 1088, 116 rows 19.4 and 21.4; S 2048, 96 rows 33.6 and 36.8; 64 items, S 1088, 200 rows
+  // 19.1 and 21.3.
+  if (dh == 64 && (long)B * H * ((n + QT - 1) / QT) <= device_sm_count())
+    return launch_stream<64, 1>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
+  return dh == 64 ? launch_stream<64, Streams<64>::N>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st)
+                  : launch_stream<80, Streams<80>::N>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
 }
 
 }  // namespace marche

@@ -793,3 +793,27 @@ def test_attention_single_pass_streams(dh, H, B, S, n):
                 c = slice(h * dh, (h + 1) * dh)
                 want[:, c], _ = orc.softmax_attention(qq[b][:, c], cc[0, b][:, c], cc[1, b][:, c])
             assert rel_l2(got[b], want) <= 8e-3 and max_abs(got[b], want) <= 3e-2
+
+
+@pytest.mark.parametrize("dh,H", [(64, 4), (80, 8)])
+@pytest.mark.parametrize("B,S,n", [(40, 64, 20), (40, 65, 33), (38, 320, 70), (75, 130, 97), (40, 577, 128), (38, 200, 150)])
+def test_attention_single_pass_streams_of_many_units(dh, H, B, S, n):
+    """More units than SMs (152 to 600): the streams of a CTA work side by side, with query tiles on one to four lane quarters.
+    (With fewer units head_dim 64 runs CTAs of one stream.)  Bounds as in the test above."""
+    from paper_2506_12035_b200 import binding
+    D = H * dh
+    cfg, blocks, m = model_for("bf16", D, H, 128, S, B)
+    m.set_tuning(attention_kernel=binding.ATTENTION_TCGEN05)
+    gen = torch.Generator(device="cuda").manual_seed(B + S + n + dh)
+    cache = torch.randn(2, B, S, D, generator=gen, device="cuda")
+    q = torch.randn(B * n, D, generator=gen, device="cuda") * 3.0
+    ramp, q_ramp = cache.clone(), q.clone()
+    ramp[0, :, :, dh - 1::dh] = torch.linspace(0.0, 40.0, S, device="cuda")[None, :, None]
+    q_ramp[:, dh - 1::dh] = 16.0
+    heads = lambda t: t.view(B, -1, H, dh).transpose(1, 2).double()
+    for qq, cc in ((q.to(torch.bfloat16), cache.to(torch.bfloat16)), (q_ramp.to(torch.bfloat16), ramp.to(torch.bfloat16))):
+        o = torch.zeros(B * n, D, dtype=torch.float16, device="cuda")
+        m.attention(qq, D, n, cc, None, None, o)
+        assert m.device_status() == 0
+        want = torch.softmax(heads(qq) @ heads(cc[0]).transpose(2, 3) / math.sqrt(dh), -1) @ heads(cc[1])
+        assert (heads(o) - want).norm() <= 8e-3 * want.norm() and (heads(o) - want).abs().max() <= 3e-2

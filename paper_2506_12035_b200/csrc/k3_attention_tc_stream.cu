@@ -518,7 +518,11 @@ cudaError_t launch_stream(const void* q, int ld_q, int B, int n, int S, int H, c
 // rows 46 and 98, 320 rows 134 and 350.  33 to 48 rows: over long sequences at head_dim 64 (S 1088, 41 rows: 57 and 62; S 320:
 // 41 and 42, nothing in a whole step); at head_dim 80 over five key tiles or more (S 320: 45 and 49), unless the last
 // round of units leaves the streams (three per SM) idle: 576 items on 444 streams 19 and 16, 1024 items 29 either way.
+// One item per SM or fewer: nothing fills the gaps of a unit's chain, and the mma.sync kernel's warps take an item faster up to
+// 64 rows (head_dim 64: 128 items, S 1088, 41 rows 17.8 and 20.6, 64 rows 16.5 and 20.8; head_dim 80: 64 rows 18.1 and 20.5, but
+// 48 rows, whose three-warp variant is built for four CTAs per SM, 23.1 and 20.5).
 bool attention_tc_stream_wins(int n, int S, int dh, int items, int min_rows) {
+  if (items <= device_sm_count() && 3 * n <= 4 * min_rows && (dh == 64 || n > min_rows)) return false;
   if (n > min_rows) return true;
   if (3 * n <= 2 * min_rows) return false;
   if (dh == 64) return S >= 512;

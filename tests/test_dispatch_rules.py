@@ -1,0 +1,25 @@
+"""The choice between the attention kernels, as the library's own functions make it (no GPU needed: 148 SMs are assumed without
+one).  The cases stand on both sides of a rule's line, at sizes where the other kernel was measured to be slower."""
+import ctypes
+
+import pytest
+
+
+@pytest.fixture(scope="module")
+def lib():
+    from paper_2506_12035_b200 import build
+    return ctypes.CDLL(build.build())
+
+
+@pytest.mark.parametrize("n,S,dh,items,want", [
+    # one item per SM or fewer: mma.sync up to 64 rows, but for three query warps at head_dim 80
+    (36, 2048, 64, 64, False), (48, 1088, 64, 144, False), (64, 1088, 64, 148, False), (65, 1088, 64, 148, True),
+    (64, 1088, 80, 144, False), (56, 640, 80, 96, False), (48, 1088, 80, 144, True), (65, 1088, 80, 144, True),
+    # more items: the streams fill one another's gaps
+    (48, 1088, 64, 149, True), (41, 1088, 64, 1024, True), (49, 320, 64, 2048, True), (64, 1088, 80, 149, True),
+    (41, 320, 64, 2048, False), (32, 2048, 64, 2048, False)])
+def test_streams_or_mma_sync(lib, n, S, dh, items, want):
+    wins = lib._ZN6marche24attention_tc_stream_winsEiiiii
+    wins.restype = ctypes.c_bool
+    assert wins(n, S, dh, items, 48) is want
+    assert wins(n, S, dh, items, 0) is (n > 0)                      # min_rows 0: wherever the caller asks for them

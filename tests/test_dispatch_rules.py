@@ -23,3 +23,22 @@ def test_streams_or_mma_sync(lib, n, S, dh, items, want):
     wins.restype = ctypes.c_bool
     assert wins(n, S, dh, items, 48) is want
     assert wins(n, S, dh, items, 0) is (n > 0)                      # min_rows 0: wherever the caller asks for them
+
+
+@pytest.mark.parametrize("n,S,dh,items,want", [
+    (24, 128, 64, 288, True), (24, 128, 64, 384, False), (8, 100, 64, 592, False),       # two tiles, up to 32 rows
+    (24, 64, 64, 592, True), (24, 192, 64, 592, True), (40, 128, 64, 2048, True),
+    (8, 164, 80, 192, True), (8, 164, 80, 256, False), (24, 164, 80, 256, True), (8, 320, 80, 288, True)])
+def test_keys_split_or_not(lib, n, S, dh, items, want):
+    wins = lib._ZN6marche20attention_split_winsEiiii
+    wins.restype = ctypes.c_bool
+    assert wins(n, S, dh, items) is want
+
+
+@pytest.mark.parametrize("n,S,dh,items,cs", [(64, 320, 80, 64, 1), (64, 320, 80, 32, 1), (64, 320, 80, 16, 4), (64, 320, 64, 64, 2), (48, 320, 80, 64, 2),
+                                             (64, 448, 80, 64, 2)])
+def test_ctas_per_item_of_the_split(lib, n, S, dh, items, cs):
+    got_cs, got_nk = ctypes.c_int(), ctypes.c_int()
+    plan = lib._ZN6marche20attention_split_planEiiiiPiS0_
+    plan.restype = ctypes.c_bool
+    assert plan(n, S, dh, items, ctypes.byref(got_cs), ctypes.byref(got_nk)) and got_cs.value == cs

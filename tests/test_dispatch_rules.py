@@ -42,3 +42,23 @@ def test_ctas_per_item_of_the_split(lib, n, S, dh, items, cs):
     plan = lib._ZN6marche20attention_split_planEiiiiPiS0_
     plan.restype = ctypes.c_bool
     assert plan(n, S, dh, items, ctypes.byref(got_cs), ctypes.byref(got_nk)) and got_cs.value == cs
+
+
+@pytest.mark.parametrize("n,n_new,S,dh,items,want", [
+    (0, 0, 320, 64, 8, False), (8, 33, 320, 64, 8, False), (300, 33, 1088, 64, 1024, False), (400, 1, 2048, 64, 2048, False),
+    # one item per SM or fewer: the sequence has to be long enough for the launch to pay
+    (16, 1, 128, 64, 128, False), (16, 1, 129, 64, 128, True), (64, 17, 192, 64, 16, False), (64, 17, 193, 64, 16, True),
+    (16, 1, 100, 80, 128, False), (48, 1, 192, 80, 64, True), (96, 17, 192, 80, 32, False), (96, 16, 192, 80, 32, True),
+    (100, 4, 320, 64, 128, False), (100, 4, 1088, 64, 128, False), (150, 20, 320, 64, 32, True), (97, 20, 128, 80, 16, True),
+    # up to two per SM
+    (41, 4, 192, 64, 288, False), (41, 4, 256, 64, 288, True), (16, 2, 192, 64, 288, True), (64, 9, 256, 64, 288, False),
+    (64, 9, 320, 64, 288, True), (64, 18, 1088, 64, 288, False), (100, 9, 640, 64, 256, False), (100, 9, 1088, 64, 256, True),
+    (151, 9, 320, 64, 256, False), (151, 9, 640, 64, 256, True), (320, 2, 320, 64, 192, True), (41, 9, 192, 80, 256, False),
+    (56, 9, 128, 80, 256, True), (80, 26, 128, 80, 256, True),
+    # more: the plain kernel has to be far from the scoring one
+    (64, 9, 1088, 64, 1024, False), (41, 5, 320, 80, 2048, False), (72, 10, 320, 64, 2048, True), (72, 24, 320, 64, 2048, False),
+    (116, 24, 1088, 64, 1024, True), (320, 2, 320, 64, 2048, True), (320, 32, 320, 80, 2048, True)])
+def test_scores_in_a_launch_of_their_own(lib, n, n_new, S, dh, items, want):
+    wins = lib._ZN6marche21attention_scores_winsEiiiii
+    wins.restype = ctypes.c_bool
+    assert wins(n, n_new, S, dh, items) is want

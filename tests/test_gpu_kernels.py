@@ -817,3 +817,45 @@ def test_attention_single_pass_streams_of_many_units(dh, H, B, S, n):
         assert m.device_status() == 0
         want = torch.softmax(heads(qq) @ heads(cc[0]).transpose(2, 3) / math.sqrt(dh), -1) @ heads(cc[1])
         assert (heads(o) - want).norm() <= 8e-3 * want.norm() and (heads(o) - want).abs().max() <= 3e-2
+
+
+@pytest.mark.parametrize("dh,H", [(64, 4), (80, 8)])
+@pytest.mark.parametrize("B,S,n,nG", [(2, 129, 16, 1), (3, 192, 7, 7), (2, 320, 48, 16), (2, 1088, 151, 21), (3, 577, 130, 32), (2, 320, 320, 2),
+                                      (1, 2048, 40, 3), (40, 200, 300, 17)])
+def test_scores_of_a_few_among_many_rows(dh, H, B, S, n, nG):
+    """The scoring block of a one-block step, whose generating rows (one or two groups of 16) lie anywhere among the active
+    ones, in the kernel that scores them alone where the rule takes it, and in the attention itself: against the oracle on the
+    step's own q and keys.  Per head as in the test above; the scores are sums over the heads."""
+    from paper_2506_12035_b200 import binding
+    D = H * dh
+    if n > S:
+        n = S
+    cfg, blocks, m = model_for("bf16", D, H, 128, S, B)
+    rng = np.random.default_rng(B + S + n + dh)
+    hidden = dev(rng.standard_normal((B, S, D)).astype(np.float32))
+    act = np.stack([rng.permutation(S)[:n] for _ in range(B)]).astype(np.int32)
+    new = np.stack([a[rng.permutation(n)[:nG]] for a in act]).astype(np.int32)
+    cache, ws, out = m.alloc_cache(), m.alloc_workspace(S), torch.zeros(B, S, D, device="cuda")
+    scores = torch.zeros(B, S, device="cuda")
+    m.init_cache(cache)
+    m.full_step(hidden, cache, idx_dev(new), None, 0.0, out, None, ws)
+    # q of the active rows, by the calls the step makes
+    u = torch.zeros(B * n, D, dtype=torch.float16, device="cuda")
+    qkv = torch.zeros(B * n, 3 * D, dtype=torch.bfloat16, device="cuda")
+    w = m.weights[0]
+    m.gather_layernorm(hidden, idx_dev(act), n, w["ln1_g"], w["ln1_b"], None, u)
+    m.linear(u, w["w_qkv"], w["b_qkv"], 0, qkv)
+    for kernel in (binding.ATTENTION_AUTO, binding.ATTENTION_TCGEN05_TWO_PASS):
+        m.set_tuning(attention_kernel=kernel)
+        m.step(hidden, cache, idx_dev(act), idx_dev(new), None, 0.0, out, None, ws)
+        m.get_scores(ws, scores)
+        got, q, k = host(scores), host(qkv).reshape(B, n, 3 * D), host(cache[0, 0])
+        for b in sorted({0, B // 2, B - 1}):
+            rows = np.isin(act[b], new[b])
+            want = np.zeros(S)
+            for h in range(H):
+                c = slice(h * dh, (h + 1) * dh)
+                _, p = orc.softmax_attention(q[b][rows][:, c], k[b][:, c], k[b][:, c])
+                want += p.sum(axis=0)
+            assert max_abs(got[b], want) <= 2e-4 * H * nG and abs(got[b].sum() - H * nG) <= 1e-4 * H * nG
+    assert m.device_status() == 0

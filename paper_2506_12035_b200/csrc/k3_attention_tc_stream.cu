@@ -45,7 +45,6 @@ namespace {
 constexpr int QT = 128;                    // query rows per unit (= TMEM lanes)
 constexpr int KT = 64;                     // keys per tile
 constexpr int NK = 3, NV = 2;              // K and V tiles in flight per stream
-constexpr int TMEM_COLS = 512;
 constexpr uint32_t COL_O = KT;             // O_j's first column in its stream's share: behind S_j (and P_j over it)
 enum { ST_ATT_STREAM = 0x51 };
 // barriers of one stream (8 bytes each); stream j's block starts at j * NB
@@ -59,13 +58,16 @@ template <int DH, int NS> struct Cfg {
   static constexpr int T_MAIN = KT * 128, T_BYTES = KT * DH * 2;   // a K or V tile; its columns 0-63
   static constexpr int Q_MAIN = QT * 128, Q_BYTES = QT * DH * 2;
   static constexpr uint32_t COL_STREAM = DH == 64 ? 128 : 160;
+  static constexpr int TMEM_COLS = NS > 1 ? 512 : (DH == 64 ? 128 : 256);
   // shared memory (from a 1024-byte aligned base)
   static constexpr int OFF_Q = 0;                            // [stream]
   static constexpr int OFF_K = OFF_Q + NS * Q_BYTES;         // [stream][slot]
   static constexpr int OFF_V = OFF_K + NS * NK * T_BYTES;    // [stream][slot]
   static constexpr int OFF_BAR = OFF_V + NS * NV * T_BYTES;
   static constexpr int OFF_MISC = OFF_BAR + 8 * NS * NB;     // tmem slot (4), abort flags (8)
-  static constexpr int SMEM_BYTES = OFF_MISC + 32 + 1024;
+  // (A CTA of one stream asks for more than it uses: two of them on an SM, where the kernel before has left room on one and
+  // none yet on another, would share its exponential units; in the step 20 us became 37.)
+  static constexpr int USED_BYTES = OFF_MISC + 32 + 1024, SMEM_BYTES = USED_BYTES > 120 * 1024 ? USED_BYTES : 120 * 1024;
   static_assert(NS * COL_STREAM <= TMEM_COLS && COL_O + DH <= COL_STREAM, "tensor memory budget");
   static_assert(SMEM_BYTES <= 227 * 1024 && T_BYTES % 1024 == 0 && Q_BYTES % 1024 == 0, "shared memory of one CTA");
 };
@@ -209,7 +211,7 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
     ptx::fence_proxy_async();
   }
   if (warp == C::W_MMA + NS - 1) {
-    ptx::tmem_alloc(ptx::smem_u32((const void*)tmem_slot), TMEM_COLS);
+    ptx::tmem_alloc(ptx::smem_u32((const void*)tmem_slot), C::TMEM_COLS);
     ptx::tmem_relinquish();
   }
   ptx::tc_fence_before();
@@ -479,7 +481,7 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
   __syncthreads();
   if (warp == C::W_MMA + NS - 1) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem_base, TMEM_COLS);
+    ptx::tmem_dealloc(tmem_base, C::TMEM_COLS);
   }
 }
 
@@ -518,11 +520,13 @@ cudaError_t launch_stream(const void* q, int ld_q, int B, int n, int S, int H, c
 // rows 46 and 98, 320 rows 134 and 350.  33 to 48 rows: over long sequences at head_dim 64 (S 1088, 41 rows: 57 and 62; S 320:
 // 41 and 42, nothing in a whole step); at head_dim 80 over five key tiles or more (S 320: 45 and 49), unless the last
 // round of units leaves the streams (three per SM) idle: 576 items on 444 streams 19 and 16, 1024 items 29 either way.
-// One item per SM or fewer: nothing fills the gaps of a unit's chain, and the mma.sync kernel's warps take an item faster up to
-// 64 rows (head_dim 64: 128 items, S 1088, 41 rows 17.8 and 20.6, 64 rows 16.5 and 20.8; head_dim 80: 64 rows 18.1 and 20.5, but
-// 48 rows, whose three-warp variant is built for four CTAs per SM, 23.1 and 20.5).
+// One item per SM or fewer at head_dim 80, 49 to 64 rows: the mma.sync kernel's four warps take an item faster than a stream that
+// nothing overlaps with (S 1088, 128 items, 60 rows, back to back 18.1 and 20.5, eight blocks of a step 465 and 503; 41 rows, on three
+// warps, 530 and 481).  At head_dim 64 the one-stream CTAs do as well back to back (S 1088, 128 items, 41 rows 18.6 and 17.8, 64 rows
+// 18.7 and 16.5) and better in a step, where the mma.sync kernel's small CTAs crowd on the SMs that are free first (eight blocks, 41
+// rows 404 and 431, 64 rows 442 and 472).
 bool attention_tc_stream_wins(int n, int S, int dh, int items, int min_rows) {
-  if (items <= device_sm_count() && 3 * n <= 4 * min_rows && (dh == 64 || n > min_rows)) return false;
+  if (dh == 80 && items <= device_sm_count() && n > min_rows && 3 * n <= 4 * min_rows) return false;
   if (n > min_rows) return true;
   if (3 * n <= 2 * min_rows) return false;
   if (dh == 64) return S >= 512;
@@ -539,8 +543,10 @@ cudaError_t launch_attention_tc_stream(const void* q, int ld_q, int B, int n, in
   // thread where four streams leave 80), takes it through its tiles faster.  One stream against four, us: 16 items, S 640, 80
   // rows 12.2 and 13.2; 144 items, S 1088, 116 rows 19.4 and 21.4; S 2048, 96 rows 33.6 and 36.8; 64 items, S 1088, 200 rows
   // 19.1 and 21.3.
-  if (dh == 64 && (long)B * H * ((n + QT - 1) / QT) <= device_sm_count())
-    return launch_stream<64, 1>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
+  // Head_dim 80: 144 items, S 100, 80 rows 5.45 and 5.8; nothing over longer sequences.
+  if ((long)B * H * ((n + QT - 1) / QT) <= device_sm_count() && (dh == 64 || S <= 2 * KT))
+    return dh == 64 ? launch_stream<64, 1>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st)
+                    : launch_stream<80, 1>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
   return dh == 64 ? launch_stream<64, Streams<64>::N>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st)
                   : launch_stream<80, Streams<80>::N>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
 }

@@ -295,8 +295,8 @@ bool attention_split_plan(int n, int S, int dh, int items, int* cs, int* nk) {
   if (n_kv > (nq == 1 ? 5 : 3))
     while (c < 4 && 2 * c * items <= device_sm_count()) c *= 2;
   // (... four query warps at head_dim 80 over five tiles or fewer: where clusters would take more than half of the SMs, single
-  // CTAs do better.  64 rows, S 320: 64 items 7.6 us on pairs, 32 items 7.4 on four CTAs, both 6.7 on one, mma.sync kernel 7.2; 16
-  // items on four CTAs 6.4.)
+  // CTAs do better.  64 rows, S 320, eight blocks of a step: 64 items 342 us on pairs, 315 on one, mma.sync kernel 320; 32 items
+  // 295 either way; 16 items on four CTAs 6.4 us against 6.7 back to back.)
   if (dh == 80 && nq == 4 && n_kv <= 5 && 2 * c * items > device_sm_count()) c = 1;
   while (c < 8 && (n_kv + c - 1) / c > (dh == 64 ? 10 : 8)) c *= 2;
   const int tiles = (n_kv + c - 1) / c;
@@ -315,17 +315,19 @@ bool attention_split_plan(int n, int S, int dh, int items, int* cs, int* nk) {
 // S 1088: 17.8 -> 6.8); up to two per SM for five key tiles (288 items: 9.6 -> 8.2; 384 items, 60 rows: 13.5 against 12.5 of
 // the tcgen05 kernel); for three tiles, which leave room for four CTAs, up to four per SM (512 items, 20 rows: 7.8 -> 7.0; 576
 // items, 60 rows: 11.2 either way) and with three groups of queries at head_dim 64 without limit (2048 items: 29.7 -> 26.6).
-// With two tiles and up to 32 rows the persistent kernel is level from two items per SM on (384 items, 30 rows 5.1 against 5.45,
-// 592 items, 24 rows 5.0 and 5.7).  At head_dim 80 up to one and a half items per SM with 33 rows or more (S 320: 192 items 9.6
-// against 9.9, 288 items 11.5 and 10.4) and with up to 16 rows of three tiles (192 items 4.9 and 5.1, 256 items 5.7 and 5.3).
+// With two tiles and up to 32 rows up to three and a half items per SM (eight blocks of a step, 24 rows: 384 items 301 and 309 with
+// the persistent kernel, 512 items 350 and 355, 576 items 386 and 372).  At head_dim 80 up to one and a half items per SM with 33
+// rows or more (S 320: 192 items 9.6 against 9.9, 288 items 11.5 and 10.4), and up to one and three quarters with up to 16 rows of
+// three tiles (eight blocks: 256 items, 8 rows 285 and 298, 288 items, 12 rows 325 and 322).
 bool attention_split_wins(int n, int S, int dh, int items) {
   int cs, nk;
   if (!attention_split_plan(n, S, dh, items, &cs, &nk)) return false;
   const int n_kv = (S + KT - 1) / KT, nq = (n + 15) / 16, sms = device_sm_count();
   if (items * cs <= sms) return true;
   if (cs > 1 || n_kv > 5) return false;
-  if (dh == 80 && (nq >= 3 || (nq == 1 && n_kv == 3))) return 2 * items <= 3 * sms;
-  if (dh == 64 && n_kv <= 3 && (n_kv != 2 || nq > 2)) return nq == 3 || items <= 4 * sms;
+  if (dh == 80 && nq >= 3) return 2 * items <= 3 * sms;
+  if (dh == 80 && nq == 1 && n_kv == 3) return 4 * items <= 7 * sms;
+  if (dh == 64 && n_kv <= 3) return nq == 3 || 2 * items <= (n_kv == 2 && nq <= 2 ? 7 : 8) * sms;
   return items <= 2 * sms;
 }
 

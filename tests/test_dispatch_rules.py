@@ -26,9 +26,9 @@ def test_streams_or_mma_sync(lib, n, S, dh, items, want):
 
 
 @pytest.mark.parametrize("n,S,dh,items,want", [
-    (24, 128, 64, 288, True), (24, 128, 64, 384, False), (8, 100, 64, 592, False),       # two tiles, up to 32 rows
+    (24, 128, 64, 512, True), (24, 128, 64, 576, False), (8, 100, 64, 592, False),       # two tiles, up to 32 rows
     (24, 64, 64, 592, True), (24, 192, 64, 592, True), (40, 128, 64, 2048, True),
-    (8, 164, 80, 192, True), (8, 164, 80, 256, False), (24, 164, 80, 256, True), (8, 320, 80, 288, True)])
+    (8, 164, 80, 256, True), (8, 164, 80, 288, False), (24, 164, 80, 288, True), (8, 320, 80, 288, True)])
 def test_keys_split_or_not(lib, n, S, dh, items, want):
     wins = lib._ZN6marche20attention_split_winsEiiii
     wins.restype = ctypes.c_bool

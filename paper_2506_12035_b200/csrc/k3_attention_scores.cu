@@ -233,27 +233,29 @@ cudaError_t launch_scores(const CUtensorMap& tm, const CUtensorMap& tail, const 
 
 // A launch of its own costs 2 to 4 us (rows listed, K tiles loaded, two passes over them; twice that with a second group of 16
 // generating rows), and saves what the one-kernel flavour costs over the plain one.  Difference of a one-block step, us, one group
-// unless stated (few: one item per SM or less; many: more than two):
+// unless stated (few: one item per SM or less; many: more than two; beyond 13 tiles, at head_dim 80 11, an SM holds one CTA of it):
 //   head_dim 64  up to 64 rows   few: one tile +2.4, two +0.4, three -2, five -4, 17 -30; 256 items: three 0, five -2 to -4; 64 rows
-//                                three +2, four +1, five -2, with two groups +2 and at 17 tiles +7
+//                                three +2, four +1, five -2, with two groups five +1.5, ten -4.5, 17 +7
 //                65 to 128 rows  (the two-pass tcgen05 kernel is close to the plain one) few +2 to +5, 256 items +5, at 17 tiles -11;
 //                                many -0 to -58, with two groups -3 to +10, at 17 tiles -4
 //                more            few: three tiles -1, ten -11; 256 items: three +3, five +1, ten -7; many -7 to -270
-//   head_dim 80  up to 64 rows   few: as head_dim 64; 256 items: three tiles +1, four -1 to -6, from 49 rows two -4, five -14
+//   head_dim 80  up to 64 rows   few: as head_dim 64; 256 items: up to 16 rows three tiles +0.4, five -3, 17 +4; 17 to 32 rows two -1.3,
+//                                three -3.4; 33 to 48 three +1.4, five -4.5; more two -4, five -14
 //                more            few: two tiles +1, three -1, with two groups four -1; else -5 to -720 (no tcgen05 two-pass kernel)
 bool attention_scores_wins(int n, int n_new, int S, int dh, int items) {
-  if (n < 1 || (dh != 64 && dh != 80) || S > kMaxTiles * KT || scores_smem(n, S, dh) > 224 * 1024 || n_new > 16 * kGroups)
-    return false;
+  const size_t smem = scores_smem(n, S, dh);
+  if (n < 1 || (dh != 64 && dh != 80) || S > kMaxTiles * KT || smem > 224 * 1024 || n_new > 16 * kGroups) return false;
   const int n_kv = (S + KT - 1) / KT, sms = device_sm_count();
-  const bool two = n_new > 16, few = items <= sms, many = items > 2 * sms;
+  const bool two = n_new > 16, few = items <= sms, many = items > 2 * sms, pair = smem <= 113 * 1024;   // two CTAs per SM
   const bool long_enough = n_kv >= (two ? 4 : 3);
   if (dh == 80 && (n > 96 || (n > 64 && !few))) return true;
   if (dh == 64 && n > 128) return many || (few ? long_enough : n_kv >= 10 || n > 256);
   if (dh == 64 && n > 64) return n_kv >= 16 ? many || (!two && !few) : many && !two;
   if (many) return false;
   if (few) return long_enough;
-  if (dh == 80) return n_kv >= (n > 48 ? 2 : 4);
-  return n > 48 ? n_kv >= 5 && !two : n_kv >= (n > 16 ? 4 : 3);
+  if (dh == 80) return n <= 16 ? n_kv >= 4 && pair : n_kv >= (n > 32 && n <= 48 ? 4 : 2);
+  if (n > 48) return two ? n_kv >= 8 && pair : n_kv >= 5;
+  return n_kv >= (n > 16 ? 4 : 3);
 }
 
 cudaError_t launch_attention_scores(const void* q, int ld_q, int B, int n, int S, int H, int dh, const void* cache_layer,

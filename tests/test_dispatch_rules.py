@@ -54,7 +54,8 @@ def test_ctas_per_item_of_the_split(lib, n, S, dh, items, cs):
     (41, 4, 192, 64, 288, False), (41, 4, 256, 64, 288, True), (16, 2, 192, 64, 288, True), (64, 9, 256, 64, 288, False),
     (64, 9, 320, 64, 288, True), (64, 18, 1088, 64, 288, False), (100, 9, 640, 64, 256, False), (100, 9, 1088, 64, 256, True),
     (151, 9, 320, 64, 256, False), (151, 9, 640, 64, 256, True), (320, 2, 320, 64, 192, True), (41, 9, 192, 80, 256, False),
-    (56, 9, 128, 80, 256, True), (80, 26, 128, 80, 256, True),
+    (56, 9, 128, 80, 256, True), (80, 26, 128, 80, 256, True), (24, 3, 128, 80, 256, True), (24, 3, 64, 80, 256, False),
+    (16, 3, 640, 80, 256, True), (16, 3, 1088, 80, 256, False), (64, 20, 640, 64, 288, True), (64, 20, 320, 64, 288, False),
     # more: the plain kernel has to be far from the scoring one
     (64, 9, 1088, 64, 1024, False), (41, 5, 320, 80, 2048, False), (72, 10, 320, 64, 2048, True), (72, 24, 320, 64, 2048, False),
     (116, 24, 1088, 64, 1024, True), (320, 2, 320, 64, 2048, True), (320, 32, 320, 80, 2048, True)])

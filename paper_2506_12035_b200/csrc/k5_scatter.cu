@@ -13,8 +13,21 @@
 #include "common.cuh"
 #include "kernels.h"
 #include "launch_pdl.h"
+#include "tma_host.h"
 
 namespace marche {
+
+// Up to four rows per SM, as in the LayerNorm, a row kernel asks for the projections' division of L1 and shared memory; with
+// more it is the bandwidth that counts, for which it wants its L1: 40 960 rows of 4 KB 57.8 us with the preference, 51.4 without.
+// The preference belongs to the kernel, hence an instantiation for each.
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_rows(void (*few_rows)(KArgs...), void (*many_rows)(KArgs...), bool (&carved)[kMaxDevices], long rows,
+                               cudaStream_t st, Args... args) {
+  const bool few = rows <= 4L * device_sm_count();
+  const cudaError_t e = few ? prefer_shared_memory(few_rows, carved) : cudaSuccess;
+  if (e != cudaSuccess) return e;
+  return launch_pdl(few ? few_rows : many_rows, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, args...);
+}
 
 // One warp per (row, K|V) pair; 16-byte vectors, row_vecs = D*sizeof(T)/16 per row.
 __global__ void __launch_bounds__(256)
@@ -34,6 +47,7 @@ scatter_kv_kernel(const uint4* __restrict__ k, const uint4* __restrict__ v, long
   for (int c = lane; c < row_vecs; c += 32) dst[c] = __ldg(src + c);
 }
 
+template <bool FEW>
 __global__ void __launch_bounds__(256)
 scatter_rows_kernel(const float4* __restrict__ rows, const int32_t* __restrict__ idx, int n, int S,
                     int row_vecs, long total_rows, float4* __restrict__ dst) {
@@ -48,6 +62,7 @@ scatter_rows_kernel(const float4* __restrict__ rows, const int32_t* __restrict__
   for (int c = lane; c < row_vecs; c += 32) d[c] = __ldg(src + c);
 }
 
+template <bool FEW>
 __global__ void __launch_bounds__(256)
 gather_rows_kernel(const float4* __restrict__ src, const int32_t* __restrict__ idx, int n, int S, int row_vecs,
                    long total_rows, float4* __restrict__ out) {
@@ -62,6 +77,7 @@ gather_rows_kernel(const float4* __restrict__ src, const int32_t* __restrict__ i
 }
 
 // out[r] = table[idx[r]]: rows of a table shared by all samples (positional embedding), one warp per row.
+template <bool FEW>
 __global__ void __launch_bounds__(256)
 gather_table_rows_kernel(const float4* __restrict__ table, const int32_t* __restrict__ idx, int row_vecs,
                          long total_rows, float4* __restrict__ out) {
@@ -76,6 +92,7 @@ gather_table_rows_kernel(const float4* __restrict__ table, const int32_t* __rest
 
 // out[b][s] = mask_token + pos[s] for every token of every sample (Eq. 2: the decoder's input at a
 // masked position); the rows of known tokens are overwritten afterwards.
+template <bool FEW>
 __global__ void __launch_bounds__(256)
 fill_mask_rows_kernel(const float4* __restrict__ mask_token, const float4* __restrict__ pos, int S, int row_vecs,
                       long total_rows, float4* __restrict__ out) {
@@ -171,9 +188,7 @@ cudaError_t launch_scatter_rows(const float* rows, const int32_t* idx, int B, in
   const long total = (long)B * n;
   if (total == 0) return cudaSuccess;
   static bool carved[kMaxDevices] = {};
-  const cudaError_t e = prefer_shared_memory(scatter_rows_kernel, carved);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(scatter_rows_kernel, dim3((unsigned)((total + 7) / 8)), dim3(256), 0, st, (const float4*)rows, idx,
+  return launch_rows(scatter_rows_kernel<true>, scatter_rows_kernel<false>, carved, total, st, (const float4*)rows, idx,
                     n, S, D / 4, total, (float4*)dst);
 }
 
@@ -183,9 +198,7 @@ cudaError_t launch_gather_rows(const float* src, const int32_t* idx, int B, int 
   const long total = (long)B * n;
   if (total == 0) return cudaSuccess;
   static bool carved[kMaxDevices] = {};
-  const cudaError_t e = prefer_shared_memory(gather_rows_kernel, carved);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(gather_rows_kernel, dim3((unsigned)((total + 7) / 8)), dim3(256), 0, st, (const float4*)src, idx, n,
+  return launch_rows(gather_rows_kernel<true>, gather_rows_kernel<false>, carved, total, st, (const float4*)src, idx, n,
                     S, D / 4, total, (float4*)out);
 }
 
@@ -194,9 +207,7 @@ cudaError_t launch_gather_table_rows(const float* table, const int32_t* idx, lon
   if (D % 4) return cudaErrorInvalidValue;
   if (total_rows == 0) return cudaSuccess;
   static bool carved[kMaxDevices] = {};
-  const cudaError_t e = prefer_shared_memory(gather_table_rows_kernel, carved);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(gather_table_rows_kernel, dim3((unsigned)((total_rows + 7) / 8)), dim3(256), 0, st,
+  return launch_rows(gather_table_rows_kernel<true>, gather_table_rows_kernel<false>, carved, total_rows, st,
                     (const float4*)table, idx, D / 4, total_rows, (float4*)out);
 }
 
@@ -205,9 +216,7 @@ cudaError_t launch_fill_mask_rows(const float* mask_token, const float* pos, int
   if (D % 4) return cudaErrorInvalidValue;
   const long total = (long)B * S;
   static bool carved[kMaxDevices] = {};
-  const cudaError_t e = prefer_shared_memory(fill_mask_rows_kernel, carved);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(fill_mask_rows_kernel, dim3((unsigned)((total + 7) / 8)), dim3(256), 0, st,
+  return launch_rows(fill_mask_rows_kernel<true>, fill_mask_rows_kernel<false>, carved, total, st,
                     (const float4*)mask_token, (const float4*)pos, S, D / 4, total, (float4*)out);
 }
 

@@ -195,14 +195,10 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid
       }
     }
   }
-  ok = __all_sync(0xffffffffu, ok);
-  if (!ok) {
-    if (lane == 0) {
-      *(volatile int*)status = ST_ATTENTION_SPLIT;
-      // let copies already issued land before the CTA's shared memory is released
-      for (int i = 0; i < n_tiles; ++i) ptx::mbar_wait(full0 + 8u * i, 0, abort_flag + 1, 20000000LL);
-    }
-    __syncwarp();
+  if (!ok && lane == 0) {
+    *(volatile int*)status = ST_ATTENTION_SPLIT;
+    // let copies already issued land before the CTA's shared memory is released
+    for (int i = 0; i < n_tiles; ++i) ptx::mbar_wait(full0 + 8u * i, 0, abort_flag + 1, 20000000LL);
   }
 
   if (n_parts == 1) {
@@ -219,9 +215,13 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid
     }
   } else {
     // ---- partial results to the owners of the rows
-    if (cs > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // every CTA of the cluster has started
-    else __syncthreads();                                // the tiles are used up
-    if (cs > 1 && !ok) ptx::cluster_raise(ptx::smem_u32(abort_flags), cs, lane);         // nobody merges what is missing
+    if (cs > 1) {
+      __syncwarp();                                      // (lane 0 may have been waiting for copies)
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");                // every CTA of the cluster has started
+      if (!ok) ptx::cluster_raise(ptx::smem_u32(abort_flags), cs);                       // nobody merges what is missing
+    } else {
+      __syncthreads();                                   // the tiles are used up
+    }
     if (warp_active && ok) {
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
@@ -240,8 +240,12 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid
         }
       }
     }
-    if (cs > 1) ptx::cluster_sync_all();
-    else __syncthreads();
+    if (cs > 1) {
+      __syncwarp();
+      ptx::cluster_sync_all();
+    } else {
+      __syncthreads();
+    }
     // ---- merge, in rank order: one thread per four columns of a row this CTA owns
     if (!*abort_flag) {
       for (int e = threadIdx.x; e < own * (DH / 4); e += (int)blockDim.x) {

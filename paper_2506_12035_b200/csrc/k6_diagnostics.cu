@@ -1,7 +1,7 @@
 // Diagnostic kernel behind marche_debug_bounded_wait: exercises the give-up path of the bounded
 // mbarrier wait that every TMA / tcgen05 kernel of the library relies on (sm100_ptx.cuh, mbar_wait), and of a cluster one
 // of whose CTAs gave up (cluster_raise).  One thread of a cluster of two CTAs waits on a barrier that nothing ever arrives
-// on; once the cycle limit has passed the wait returns false and its warp raises the cluster's flags; behind the cluster
+// on; once the cycle limit has passed the wait returns false and the thread raises the cluster's flags; behind the cluster
 // barrier the OTHER CTA, which finds its flag raised, writes the code into the status word and the kernel ends normally.
 // Nothing traps, faults or spins without a bound; the context stays usable.
 #include "kernels.h"
@@ -30,8 +30,8 @@ bounded_wait_probe_kernel(long long limit_cycles, int* __restrict__ status) {
   pdl_sync();
   bool ok = true;
   if (waiter && lane == 0) ok = ptx::mbar_wait(ptx::smem_u32(&bar), 0u, &abort_flag, limit_cycles);
-  ok = __all_sync(0xffffffffu, ok);
-  if (!ok) ptx::cluster_raise(ptx::smem_u32(&abort_flag), 2, lane);
+  if (!ok) ptx::cluster_raise(ptx::smem_u32(&abort_flag), 2);
+  __syncwarp();
   ptx::cluster_sync_all();
   if (!waiter && lane == 0 && *(volatile int*)&abort_flag) *(volatile int*)status = ST_PROBE;
 }

@@ -217,11 +217,11 @@ MARCHE_DEVINL uint32_t mapa(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-// Raises a flag (a word at the same shared address in every CTA) in all CTAs of a cluster of `n`, by the lanes of one warp.
-// Those see it after the next cluster barrier, or earlier.
-MARCHE_DEVINL void cluster_raise(uint32_t flag, int n, int lane) {
-  if (lane < n) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(mapa(flag, (uint32_t)lane)), "r"(1) : "memory");
-  __syncwarp();
+// Raises a flag (a word at the same shared address in every CTA) in all CTAs of a cluster of `n`, which see it after the next
+// cluster barrier, or earlier.
+MARCHE_DEVINL void cluster_raise(uint32_t flag, int n) {
+  for (int r = 0; r < n; ++r)
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(mapa(flag, (uint32_t)r)), "r"(1) : "memory");
 }
 MARCHE_DEVINL void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");

@@ -14,6 +14,7 @@
 #include "common.cuh"
 #include "kernels.h"
 #include "launch_pdl.h"
+#include "tma_host.h"
 
 namespace marche {
 
@@ -46,8 +47,11 @@ MARCHE_DEVINL uint32_t mix32(uint32_t seed, uint32_t b, uint32_t t) {
 constexpr int kIdxBits = 11, kBinBits = 9, kBins = 1 << kBinBits, kMaxPasses = (32 + kIdxBits + kBinBits - 1) / kBinBits;
 constexpr int kPerThread = 2048 / kTopkThreads, kTopkWarps = kTopkThreads / 32;
 
-// (48 registers, five CTAs per SM: left alone the compiler takes 64 and four, 158 -> 169 us for those samples with distinct scores)
-__global__ void __launch_bounds__(kTopkThreads, 5)
+// MANY: more samples than run at once, where what a sample costs counts beside its latency: a crowded bin is looked at (64
+// samples of 1088 tokens 5.4 us without that, 5.6 with it).  48 registers, five CTAs per SM: left alone the compiler takes 64
+// and four, 16 384 samples of 320 tokens 158 -> 169 us.
+template <bool MANY>
+__global__ void __launch_bounds__(kTopkThreads, MANY ? 5 : 0)
 topk_kernel(const float* __restrict__ partial, int H, float* __restrict__ scores, const int32_t* __restrict__ new_idx,
             int n_new, const int32_t* __restrict__ excl_idx, int n_excl, int S, int k, int policy, uint32_t seed,
             int32_t* __restrict__ refresh_idx) {
@@ -59,7 +63,7 @@ topk_kernel(const float* __restrict__ partial, int H, float* __restrict__ scores
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int i = tid; i < kMaxPasses * kBins / 4; i += kTopkThreads) (&hist[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
   for (int i = tid; i < 2048 / 4; i += kTopkThreads) taken[i] = 0u;
-  if (tid < kMaxPasses) least[tid] = 0xffffffffu;
+  if (MANY && tid < kMaxPasses) least[tid] = 0xffffffffu;
   __syncthreads();
   pdl_sync();
 
@@ -154,7 +158,7 @@ topk_kernel(const float* __restrict__ partial, int H, float* __restrict__ scores
 #pragma unroll
     for (int i = 0; i < kPerThread; ++i)
       if ((in_range & (1u << i)) && (composite(i) < lo || composite(i) - lo > range)) in_range &= ~(1u << i);
-    if (held > 32u) {
+    if (MANY && held > 32u) {
       // A crowded bin, most likely one score: then only the indices are left to compare, where up to three passes over bits in
       // common would follow.  Scores of three values, 16 384 samples of 320 tokens: 324 -> 206 us.
 #pragma unroll
@@ -196,10 +200,12 @@ cudaError_t launch_topk(const float* partial, int H, float* scores, const int32_
                         const int32_t* excl_idx, int n_excl, int B, int S, int k, int32_t* refresh_idx, cudaStream_t st,
                         int policy, uint32_t seed) {
   if (S > 2048) return cudaErrorInvalidValue;
-  static bool carved[kMaxDevices] = {};
-  const cudaError_t e = prefer_shared_memory(topk_kernel, carved);
+  static bool carved[2][kMaxDevices] = {};
+  const bool many = B > 512 && B > 5 * device_sm_count();   // (the first test saves the usual call the query of its device)
+  auto* kernel = many ? topk_kernel<true> : topk_kernel<false>;
+  const cudaError_t e = prefer_shared_memory(kernel, carved[many]);
   if (e != cudaSuccess) return e;
-  return launch_pdl(topk_kernel, dim3(B), dim3(kTopkThreads), 0, st, partial, H, scores, new_idx, n_new, excl_idx, n_excl, S,
+  return launch_pdl(kernel, dim3(B), dim3(kTopkThreads), 0, st, partial, H, scores, new_idx, n_new, excl_idx, n_excl, S,
                     k, policy, seed, refresh_idx);
 }
 

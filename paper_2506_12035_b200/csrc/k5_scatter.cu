@@ -23,7 +23,7 @@ namespace marche {
 template <typename... KArgs, typename... Args>
 static cudaError_t launch_rows(void (*few_rows)(KArgs...), void (*many_rows)(KArgs...), bool (&carved)[kMaxDevices], long rows,
                                cudaStream_t st, Args... args) {
-  const bool few = rows <= 4L * device_sm_count();
+  const bool few = rows <= 512 || rows <= 4L * device_sm_count();   // (the first test saves a small call the query of its device)
   const cudaError_t e = few ? prefer_shared_memory(few_rows, carved) : cudaSuccess;
   if (e != cudaSuccess) return e;
   return launch_pdl(few ? few_rows : many_rows, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, args...);

@@ -384,6 +384,25 @@ def test_select_refresh_policies_bit_exact(policy, name):
         assert np.array_equal(out.cpu().numpy(), orc.select_refresh(sc, new, excl, k, policy=name, seed=1234))
 
 
+@pytest.mark.parametrize("S,k", [(33, 9), (320, 32), (1088, 700)])
+def test_select_refresh_many_samples_bit_exact(S, k):
+    """More samples than run at once (a crowded bin of one score goes straight to the indices): scores of few values, of one, and
+    of a few spread ones in one crowded bin; distinct ones."""
+    B = 800
+    cfg, blocks, m = model_for("f32", 128, 2, 128, S, B)
+    rng = np.random.default_rng(S + k)
+    mask = torch.empty(B * S, dtype=torch.uint8, device="cuda")
+    perm = np.stack([rng.permutation(S) for _ in range(B)]).astype(np.int32)
+    new, excl = perm[:, :3], perm[:, 3:7]
+    near = 1.0 + rng.integers(0, 40, (B, S)) * 2.0 ** -23
+    near[:, 0], near[:, 1] = 1e-30, 1e30
+    for sc in (rng.integers(0, 3, (B, S)), np.ones((B, S)), near, rng.random((B, S))):
+        sc = sc.astype(np.float32)
+        out = torch.full((B, k), -1, dtype=torch.int32, device="cuda")
+        m.select_refresh(dev(sc), idx_dev(new), idx_dev(excl), k, out, mask)
+        assert np.array_equal(out.cpu().numpy(), orc.select_refresh(sc, new, excl, k))
+
+
 @pytest.mark.parametrize("F,S,B", [(2048, 300, 64), (4096, 320, 64), (3072, 330, 100)])
 def test_fc2_shared_tiles_equal_whole_tiles(F, S, B):
     """75, 80 and 129 tiles of 256 x 256 dealt to the CTA pairs in whole tiles or in ranges of 5/4, 9/8 and 7/4 tiles (74
@@ -525,8 +544,8 @@ def test_projection_shapes_of_the_configs(D, F, M):
 @pytest.mark.parametrize("dh,H", [(64, 4), (80, 8)])
 @pytest.mark.parametrize("n,nG", [(159, 25), (320, 320), (97, 1)])
 def test_attention_many_rows(S, dh, H, n, nG):
-    """Active sets beyond one query tile (both tensor-core kernels are reached: tcgen05 for head_dim 64,
-    mma.sync with seven consumer warps for head_dim 80), every query scoring in one case."""
+    """Active sets beyond one query tile, every query scoring in one case.  With scores: the two-pass tcgen05 kernel
+    (head_dim 64) and mma.sync with seven consumer warps (80); without: the single-pass tcgen05 kernel for both."""
     dtype = "bf16"
     B, D = 2, dh * H
     cfg, blocks, m = model_for(dtype, D, H, 128, S, B)
@@ -563,15 +582,18 @@ def test_attention_many_rows(S, dh, H, n, nG):
 @pytest.mark.parametrize("B,H,S,n", [(2, 4, 68, 1), (3, 4, 257, 7), (2, 8, 320, 16), (2, 8, 320, 17), (5, 4, 64, 32),
                                      (80, 16, 200, 5), (140, 8, 130, 20)])
 def test_attention_small_sets_persistent(operand, dh, B, H, S, n):
-    """Plain attention at up to 32 query rows takes the persistent mma.sync launch: one and two consumer warps,
-    both head sizes, ragged key tiles, fewer items than resident CTAs and several items per CTA (1280 and 1120
-    items), where a CTA's loads run ahead into its next item."""
+    """The persistent mma.sync launch, which the plain attention takes at up to 32 query rows where the keys are not split (it
+    is asked for here, since few items would be): one and two consumer warps, both head sizes, ragged key tiles, fewer
+    items than resident CTAs and several items per CTA (1280 and 1120 items), where a CTA's loads run ahead into its next
+    item."""
+    from paper_2506_12035_b200 import binding
     if dh == 80:
         H = (H + 7) // 8 * 8                                # the model width must be a multiple of 128
     D = H * dh
     if operand == "bf16b" and B > 5:
         pytest.skip("one operand type is enough for the large shapes")
     cfg, blocks, m = model_for(operand, D, H, 128, S, B)
+    m.set_tuning(attention_kernel=binding.ATTENTION_MMA)
     rng = np.random.default_rng(7 * B + H + S + n + dh)
     cache = rng.standard_normal((2, B, S, D)).astype(np.float32)
     q = (rng.standard_normal((B * n, D)) * 2.0).astype(np.float32)
@@ -614,6 +636,40 @@ def test_attention_persistent_rows_of_every_item(dh, S, n):
         assert first is None or torch.equal(o, first)
         first = o
     assert (heads(first) - want).abs().max() <= 3e-2 and m.device_status() == 0
+
+
+@pytest.mark.parametrize("operand", ["bf16", "bf16b"])
+@pytest.mark.parametrize("dh,H", [(64, 4), (80, 8)])
+@pytest.mark.parametrize("B,S,n,nG", [(2, 68, 33, 33), (3, 257, 41, 5), (30, 320, 48, 9), (2, 320, 49, 0), (2, 1088, 64, 20), (2, 130, 97, 97),
+                                      (2, 320, 120, 3)])
+def test_attention_mma_sync_one_cta_per_item(operand, dh, H, B, S, n, nG):
+    """The mma.sync kernel with one CTA per item, asked for by name: three to seven consumer warps and a second query tile, ragged
+    keys, plain and with scores.  Bounds as in the tests above."""
+    from paper_2506_12035_b200 import binding
+    D = H * dh
+    cfg, blocks, m = model_for(operand, D, H, 128, S, B)
+    m.set_tuning(attention_kernel=binding.ATTENTION_MMA)
+    rng = np.random.default_rng(B + S + n + dh)
+    cache, q = rng.standard_normal((2, B, S, D)).astype(np.float32), (rng.standard_normal((B * n, D)) * 3.0).astype(np.float32)
+    flags = np.zeros((B, n), dtype=np.uint8)
+    for b in range(B):
+        flags[b, rng.permutation(n)[:nG]] = 1
+    partial = torch.full((B, H, S), -1.0, device="cuda")
+    outs = []
+    for f in (flags, None):
+        outs.append(torch.zeros(B * n, D, dtype=adt(operand), device="cuda"))
+        m.attention(dev(q, torch.bfloat16), D, n, dev(cache, torch.bfloat16), None if f is None else dev(f), partial, outs[-1])
+    assert m.device_status() == 0
+    qq, cc, got_p = quant(q, "bf16").reshape(B, n, D), quant(cache, "bf16"), host(partial)
+    for b in sorted({0, B // 2, B - 1}):
+        want = np.zeros((n, D))
+        for h in range(H):
+            c = slice(h * dh, (h + 1) * dh)
+            want[:, c], p = orc.softmax_attention(qq[b][:, c], cc[0, b][:, c], cc[1, b][:, c])
+            assert max_abs(got_p[b, h], p[flags[b].astype(bool)].sum(axis=0)) <= 2e-2 * max(1, nG) / 8 + 1e-6
+        for o in outs:
+            got = host(o).reshape(B, n, D)[b]
+            assert rel_l2(got, want) <= 8e-3 and max_abs(got, want) <= 3e-2
 
 
 @pytest.mark.parametrize("operand", ["bf16", "bf16b"])

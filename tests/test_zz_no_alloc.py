@@ -2,11 +2,11 @@
 
 Some users of the library run where asking the device allocator for a scratch buffer is off
 limits (memory planned up front, a serving loop that must not touch the allocator, a plug-in
-that only receives its tensors).  For them the candidate mask sits in a fixed array inside the
-library.  This file checks, through the C ABI, that the variant returns exactly what the
-ordinary entry point returns (index work: bit-exact) on two calls in a row that use different
-token sets, so that bytes left in the shared array by the first call would show up in the
-second if they mattered; and that shapes beyond the built-in array are refused.
+that only receives its tensors).  For them there is a call that needs no scratch; it keeps a limit on
+batch x tokens as part of its interface.  This file checks, through the C ABI, that the variant returns
+exactly what the ordinary entry point returns (index work: bit-exact) on two calls in a row that use
+different token sets, so that anything kept from the first call would show up in the second; and that
+shapes beyond the limit are refused.
 
 Collected last on purpose: a failure here cannot hide the result of any other test.
 """
@@ -49,7 +49,7 @@ def test_static_scratch_selection_matches_ordinary_entry_point():
 
 
 def test_static_scratch_rejects_shapes_beyond_its_size():
-    B, S = 900, 320                                   # 288000 bytes of mask > 256 KiB
+    B, S = 900, 320                                   # 288000 > 256 Ki
     m = _model(B, S)
     sc = torch.zeros(B, S, device="cuda")
     out = torch.full((B, 4), -7, dtype=torch.int32, device="cuda")
@@ -61,7 +61,7 @@ def test_static_scratch_rejects_shapes_beyond_its_size():
 
 
 def test_static_scratch_accepts_the_largest_shape_it_holds():
-    B, S = 128, 2048                                  # exactly 262144 bytes of mask: the limit itself
+    B, S = 128, 2048                                  # exactly 262144: the limit itself
     m = _model(B, S)
     rng = np.random.default_rng(7)
     scores = rng.integers(0, 50, (B, S)).astype(np.float32)

@@ -88,7 +88,8 @@ enum {
   MARCHE_EPI_BIAS_GELU = 2      /* out A[M][N]      = GELU_erf(acc + bias)                */
 };
 
-/* Kernel classes of marche_profile_end / marche_kernel_class_name. */
+/* Kernel classes of marche_profile_end / marche_kernel_class_name.  The attention class is one launch per block; where the
+ * scoring block's relevance scores have a launch of their own, that one is charged to MARCHE_KC_OTHER. */
 enum {
   MARCHE_KC_FLAGS = 0, MARCHE_KC_GATHER_LN = 1, MARCHE_KC_GEMM_QKV = 2, MARCHE_KC_SCATTER_KV = 3,
   MARCHE_KC_ATTENTION = 4, MARCHE_KC_GEMM_O = 5, MARCHE_KC_GEMM_FC1 = 6, MARCHE_KC_GEMM_FC2 = 7,
@@ -293,8 +294,9 @@ int marche_select_refresh_policy(marche_ctx* ctx, const float* scores,
  * whose memory was sized up front, a latency-critical serving loop that must never touch the
  * allocator, a plug-in that is handed only its input and output tensors).  The paper has no
  * counterpart; this is a packaging variant of the same kernels.
- *   - batch*seq_len must not exceed MARCHE_STATIC_SCRATCH_BYTES (256 Ki); otherwise MARCHE_EWORKSPACE is
- *     returned, nothing is enqueued and marche_last_error() names both numbers.
+ *   - batch*seq_len must not exceed MARCHE_STATIC_SCRATCH_BYTES (256 Ki), a limit kept as part of the interface (the
+ *     selection needs no scratch); otherwise MARCHE_EWORKSPACE is returned, nothing is enqueued and
+ *     marche_last_error() names both numbers.
  *   - No device memory is allocated or freed by this call, now or later, and none is shared between calls.
  * Arguments, result and errors otherwise exactly as marche_select_refresh without mask_scratch. */
 #define MARCHE_STATIC_SCRATCH_BYTES (256 * 1024)
@@ -313,8 +315,8 @@ int marche_get_scores(marche_ctx* ctx, const void* workspace, float* scores_out,
  * accumulate scores in addition to score_layer (which alone drives the selection); it changes the
  * workspace size, so call it before marche_workspace_bytes.  n = 0 clears the list.  The extra
  * blocks are honoured by marche_step and marche_full_step, and by the every-token phase of
- * marche_step_in_step_selection / marche_mar_step (full decoder only); each costs the two-pass
- * scoring variant of the attention kernel.  marche_get_layer_scores sums the per-head partials of
+ * marche_step_in_step_selection / marche_mar_step (full decoder only); each costs what a scoring block
+ * costs: the two-pass variant of the attention kernel, or a launch for the generating rows beside the plain one.  marche_get_layer_scores sums the per-head partials of
  * one registered block (or of score_layer) left in `workspace` by the last step, in head order,
  * into scores_out, device float [B][S].  MARCHE_EINVAL for a block that is not registered. */
 int marche_set_score_layers(marche_ctx* ctx, const int32_t* layers /* host */, int n);
@@ -440,12 +442,16 @@ int marche_attention_two_segment(marche_ctx* ctx, const void* qkv, int ld, int n
  * `pdl` is process-wide (it is a property of how kernels are launched). */
 enum { MARCHE_ATTENTION_AUTO = 0, MARCHE_ATTENTION_MMA = 1, MARCHE_ATTENTION_TCGEN05 = 2,
        MARCHE_ATTENTION_TCGEN05_TWO_PASS = 3 /* the two-pass tcgen05 kernel also where no scores are taken */ };
-enum { MARCHE_GEMM_AUTO = 0, MARCHE_GEMM_SINGLE = 1, MARCHE_GEMM_PAIR = 2 };
+enum { MARCHE_GEMM_AUTO = 0, MARCHE_GEMM_SINGLE = 1 /* split-K: one CTA, or a cluster that shares K, per tile */,
+       MARCHE_GEMM_PAIR = 2 /* CTA pairs on 256-row tiles */ };
 typedef struct {
   int32_t stream_k;              /* 1: fc2-sized residual projections use stream-K with ordered reduce-adds   */
   int32_t fuse_qkv_scatter;      /* 1: the QKV projection's epilogue writes K, V into the cache (no K5 launch)*/
-  int32_t attention_kernel;      /* MARCHE_ATTENTION_*: AUTO picks by active rows and head_dim                 */
-  int32_t attention_tc_min_rows; /* AUTO: tcgen05 attention above this many active rows (head_dim 64; 48)      */
+  int32_t attention_kernel;      /* MARCHE_ATTENTION_*: AUTO picks by query rows, keys, head_dim and items     */
+  int32_t attention_tc_min_rows; /* AUTO, both head sizes, after the kernel that splits few items' keys: tcgen05
+                                    streams above this many active rows (48); from above two thirds of it
+                                    where long sequences or head_dim 80 make them faster; at head_dim 80 up to
+                                    four thirds of it not with one item per SM or fewer                        */
   int32_t two_segment_attention; /* 1: the step uses marche_attention_two_segment instead of K5 + K3           */
   int32_t gemm_kernel;           /* MARCHE_GEMM_*: AUTO = the kernel with the shorter estimated time           */
   int32_t tail_split;            /* 0 off, 1 cost model, 2 / 4 forced: column slices in a partial last round   */

@@ -1,10 +1,11 @@
 // C ABI of libmarche (see include/marche.h) and the per-step kernel sequence.
 //
 // The step is a fixed chain of launches on the caller's stream, per block:
-//   K1 LayerNorm (with the row gather at block 0) -> K2 QKV projection -> K5 K/V
-//   write-back -> K3 attention over the whole cache (+ score partials at the scoring
-//   block) -> K2 output projection (+residual) -> K1 LayerNorm -> K2 fc1 (+GELU) ->
-//   K2 fc2 (+residual);
+//   K1 LayerNorm (with the row gather at block 0) -> K2 QKV projection, whose epilogue
+//   writes K and V into the cache (a K5 launch of its own where that is switched off) ->
+//   K3 attention over the whole cache (+ score partials at the scoring block, in the same
+//   kernel or in one of their own before it) -> K2 output projection (+residual) -> K1
+//   LayerNorm -> K2 fc1 (+GELU) -> K2 fc2 (+residual);
 // then once per step the fp32 row scatter into hidden_out and K4 (score reduction +
 // top-K).  Nothing here allocates device memory or synchronises, except where the
 // header says a call is synchronous.
@@ -242,7 +243,7 @@ int do_attention(marche_ctx* ctx, const void* q, int ld_q, int n, const void* ca
   // The plain attention has four tensor-core kernels; which one runs is a matter of query rows, keys, head_dim and items, by
   // rules that stand beside the kernels with both sides measured:
   //   few items (or few key tiles)      all tiles in flight, split over a cluster and over warps (attention_split_wins)
-  //   more than 48 rows, or nearly so   four tcgen05 streams per SM (attention_tc_stream_wins)
+  //   more than 48 rows, or nearly so   tcgen05 streams, up to four per SM (attention_tc_stream_wins)
   //   32 rows or fewer                  the persistent mma.sync launch (31 vs 34 us at n = 8, 32 vs 36 us at n = 24..32, S 320)
   //   else                              mma.sync with one CTA per item
   // Where relevance scores are taken in the same kernel their final weights take two passes: on tcgen05 above 64 rows (head_dim
@@ -951,7 +952,7 @@ int marche_select_refresh_static(marche_ctx* ctx, const float* scores, const int
   if (!refresh_idx) return MARCHE_EINVAL;
   if ((size_t)B * (size_t)S > (size_t)MARCHE_STATIC_SCRATCH_BYTES) {
     char msg[160];
-    snprintf(msg, sizeof msg, "marche_select_refresh_static: batch*seq_len = %zu exceeds the built-in scratch of %d bytes",
+    snprintf(msg, sizeof msg, "marche_select_refresh_static: batch*seq_len = %zu exceeds the call's limit of %d",
              (size_t)B * (size_t)S, (int)MARCHE_STATIC_SCRATCH_BYTES);
     ctx->last_error = msg;
     return MARCHE_EWORKSPACE;

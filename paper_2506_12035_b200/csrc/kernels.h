@@ -58,9 +58,8 @@ cudaError_t launch_topk(const float* partial, int H, float* scores, const int32_
 
 // Where the K and V columns of a fused QKV projection go (Algorithm 1 line 11 done by the projection's
 // epilogue, epilogue code 4): row r of the GEMM is active token j = r % n of sample b = r / n, its cache row is
-// idx[r] (identity when idx is NULL).  cache is one block's [2][B][S][D] slice (bf16, or fp32
-// in an fp32 context).  Needs N == 3 D,
-// D a multiple of 256 and 2 B S D < 2^31.
+// idx[r] (identity when idx is NULL).  cache is one block's [2][B][S][D] slice (bf16, or fp32 in an fp32 context), 16-byte
+// aligned.  Needs N == 3 D and D a multiple of the kernel's tile width (128 always is); cache offsets are 64-bit.
 struct KvScatter {
   const int32_t* idx;
   void* cache;

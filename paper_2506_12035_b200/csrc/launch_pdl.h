@@ -5,8 +5,10 @@
 // pdl_launch_dependents(), and every launch carries the programmatic-stream-serialization
 // attribute.  The next kernel's CTAs may therefore become resident, and run their private
 // set-up (barrier init, TMEM allocation, tensor-map prefetch), while the current kernel is
-// still draining; they touch global memory only after the wait.  Because each kernel releases
-// its dependents only after its own wait has returned, at most one kernel runs ahead.
+// still draining.  Of global memory they read before the wait only what was complete before the
+// current kernel began (weights, biases, a stack's LayerNorm parameters) and prefetch into L2;
+// they write nothing.  Because each kernel releases its dependents only after its own wait has
+// returned, at most one kernel runs ahead.
 // pdl_switch() holds the process-wide on/off state (marche_set_tuning; on by default).
 #pragma once
 

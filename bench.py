@@ -77,8 +77,8 @@ def write_ncu_traffic(csv_paths):
             b = float(r[i_rd].replace(",", "")) * scale[units[i_rd]] + float(r[i_wr].replace(",", "")) * scale[units[i_wr]]
             acc.setdefault(cls, []).append(b)
     with open(TRAFFIC_FILE, "w") as f:
-        f.write("# mean dram__bytes_read.sum + dram__bytes_write.sum per launch, from ncu --set full captures of\n"
-                "# 4-block slices of the benchmark workloads (see the *.md summaries beside this file for the commands)\n")
+        f.write("# mean dram__bytes_read.sum + dram__bytes_write.sum per launch, from ncu captures of single launches\n"
+                "# at the benchmark workloads' shapes (see attention_kernels.md beside this file for shapes and commands)\n")
         f.write("# class bytes_per_launch launches\n")
         for cls, v in sorted(acc.items()):
             f.write("%s %.0f %d\n" % (cls, float(np.mean(v)), len(v)))

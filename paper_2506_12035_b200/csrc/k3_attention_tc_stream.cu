@@ -522,9 +522,9 @@ cudaError_t launch_stream(const void* q, int ld_q, int B, int n, int S, int H, c
 // round of units leaves the streams (three per SM) idle: 576 items on 444 streams 19 and 16, 1024 items 29 either way.
 // One item per SM or fewer at head_dim 80, 49 to 64 rows: the mma.sync kernel's four warps take an item faster than a stream that
 // nothing overlaps with (S 1088, 128 items, 60 rows, back to back 18.1 and 20.5, eight blocks of a step 465 and 503; 41 rows, on three
-// warps, 530 and 481).  At head_dim 64 the one-stream CTAs do as well back to back (S 1088, 128 items, 41 rows 18.6 and 17.8, 64 rows
-// 18.7 and 16.5) and better in a step, where the mma.sync kernel's small CTAs crowd on the SMs that are free first (eight blocks, 41
-// rows 404 and 431, 64 rows 442 and 472).
+// warps, 530 and 481).  At head_dim 64 the one-stream CTAs are slower back to back (S 1088, 128 items, 41 rows 18.6 and 17.8, 64 rows
+// 18.7 and 16.5) but faster in a step, in which up to four of the mma.sync kernel's small CTAs fit an SM that is free early (eight
+// blocks, 41 rows 404 and 431, 64 rows 442 and 472).
 bool attention_tc_stream_wins(int n, int S, int dh, int items, int min_rows) {
   if (dh == 80 && items <= device_sm_count() && n > min_rows && 3 * n <= 4 * min_rows) return false;
   if (n > min_rows) return true;

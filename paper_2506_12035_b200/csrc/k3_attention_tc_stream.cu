@@ -3,24 +3,28 @@
 // Appendix A), with the running-maximum / running-sum merge of Eq. 6-10 applied tile by tile.
 //
 // Persistent CTAs (one per SM).  The work of a CTA is a list of units, one unit = one 128-row query
-// tile of one (sample, head) item against all S keys; FOUR independent streams (three at head_dim 80, whose buffers are
-// larger; one where a CTA has a single unit) inside the CTA take the units in turn.  A unit is a latency chain (Q K^T -> read logits -> exponentials -> write weights
-// -> P V -> next Q K^T ...), and the exponentials - 16 per clock and SM - are the scarce resource once the active set
-// is large; four chains in flight per SM partition keep those units busy while each chain waits on its hand-overs.
+// tile of one (sample, head) item against all S keys; three independent streams inside the CTA (one where a CTA has a single unit,
+// four where that saves a round) take the units in turn.  A unit is a latency chain (Q K^T -> read logits -> exponentials -> write
+// weights -> P V), and the exponentials - 16 per clock and SM - are the scarce resource once the active set
+// is large; the chains in flight per SM partition keep those units busy while each waits on its hand-overs.
 // Each stream owns a query buffer, TMA rings of 64-key tiles (three of K, two of V: a K tile is used up a step earlier)
-// that run ahead across units and 128 (144) columns of tensor memory: S_j 64 columns (fp32 logits), whose first 32 the
-// weights P_j (packed bf16) overwrite, and O_j.  So P V of a tile and Q K^T of the next are issued together,
-// in the order in which the tensor core executes them, and one barrier per tile tells the softmax that both are done:
-// its weights may be overwritten, its accumulator rescaled, its logits read.
-// Roles, for four streams (24 warps of 80 registers a thread):
-//   warps 0-15    softmax: warps 4j .. 4j+3 serve stream j, one thread per query row.  A thread pulls its
-//                 S row into registers (tcgen05.ld; the first half again for its exponentials, since 80 registers do
-//                 not hold a row and its weights) and writes the weights to tensor memory
+// that run ahead across units and 160 columns of tensor memory: S_j 64 columns (fp32 logits), P_j 32 (the weights, packed bf16),
+// O_j 64.  The logits are free as soon as they have been read, so Q K^T of the next tile runs under the
+// exponentials of this one and only the softmax itself is left of the chain.  Four streams, and three at head_dim 80 (O_j 80
+// columns), have no columns to spare: there P_j overwrites S_j, P V of a tile and Q K^T of the next are issued together, in the
+// order in which the tensor core executes them, and both are part of the chain.  Three streams with columns for P_j against four
+// without, 128 x 16 items, S 320, us: 320 rows 107 and 122, 128 rows 42.5 and 50.5, 60 rows 36 and 40; 64 x 16 items, S 1088: 151
+// rows 98 and 104, 1088 rows 528 and 590; one stream, with and without: S 1088, 144 items, 116 rows 17.1 and 19.5, S 2048, 64
+// items, 200 rows 28.2 and 33.0.
+// Roles, for three streams (18 warps of 112 registers a thread; numbers for four in brackets):
+//   warps 0-11    [0-15] softmax: warps 4j .. 4j+3 serve stream j, one thread per query row.  A thread pulls its
+//                 S row into registers (tcgen05.ld; without columns for P_j the first half again for its exponentials, since 80
+//                 registers do not hold a row and its weights) and writes the weights to tensor memory
 //                 (tcgen05.st), from where the tensor core reads them as the A operand of P V
-//   warps 16-19   TMA producer of stream 0 .. 3: Q tile per unit, K and V rings
-//   warps 20-23   issue tcgen05.mma for stream 0 .. 3: O_j += P_j V (M128 x N64 x K64, V as an MN-major operand from
-//                 shared memory) as soon as the weights are there, then S_j = Q_j K^T (M128 x N64 x K64) of the next
-//                 tile; warp 23 also allocates / frees tensor memory
+//   warps 12-14   [16-19] TMA producer of stream 0, 1, ..: Q tile per unit, K and V rings
+//   warps 15-17   [20-23] issue tcgen05.mma for stream 0, 1, ..: S_j = Q_j K^T (M128 x N64 x K64) of the next tile as soon as the
+//                 last one has been read, O_j += P_j V (M128 x N64 x K64, V as an MN-major operand from
+//                 shared memory) as soon as the weights are there; the last warp also allocates / frees tensor memory
 // A warp can only reach the tensor-memory lanes of its quarter, and a quarter is one SM partition.  A query tile of
 // fewer than 97 rows is therefore placed on other lanes by other streams, so that the partitions share the work.
 // head_dim 80: a tile arrives as two boxes, columns 0-63 in rows of 128 bytes under the 128-byte swizzle and columns 64-79
@@ -45,20 +49,23 @@ namespace {
 constexpr int QT = 128;                    // query rows per unit (= TMEM lanes)
 constexpr int KT = 64;                     // keys per tile
 constexpr int NK = 3, NV = 2;              // K and V tiles in flight per stream
-constexpr uint32_t COL_O = KT;             // O_j's first column in its stream's share: behind S_j (and P_j over it)
 enum { ST_ATT_STREAM = 0x51 };
 // barriers of one stream (8 bytes each); stream j's block starts at j * NB
 enum { B_K_FULL = 0, B_K_EMPTY = B_K_FULL + NK, B_V_FULL = B_K_EMPTY + NK, B_V_EMPTY = B_V_FULL + NV, B_Q_FULL = B_V_EMPTY + NV,
-       B_Q_EMPTY, B_S_FULL, B_P_FULL, B_O_FULL, NB };
+       B_Q_EMPTY, B_S_FULL, B_S_FREE, B_P_FULL, B_O_FULL, NB };
 
-template <int DH> struct Streams { static constexpr int N = DH == 64 ? 4 : 3; };   // per CTA
+constexpr int kStreams = 3;                // per CTA, but for launches of few units
 template <int DH, int NS> struct Cfg {
+  // The weights P_j have columns of their own where a stream's share leaves room: then Q K^T of the next tile runs under the
+  // exponentials of this one.  Else they overwrite the logits, and P V and Q K^T are both part of the chain.
+  static constexpr bool OWN_P = NS < (DH == 64 ? 4 : 3);
+  static constexpr uint32_t COL_P = OWN_P ? KT : 0, COL_O = OWN_P ? KT + KT / 2 : KT;
   static constexpr int THREADS = NS * 6 * 32;                // per stream four softmax warps, a producer, an MMA issuer
   static constexpr int W_PROD = NS * 4, W_MMA = NS * 5;
   static constexpr int T_MAIN = KT * 128, T_BYTES = KT * DH * 2;   // a K or V tile; its columns 0-63
   static constexpr int Q_MAIN = QT * 128, Q_BYTES = QT * DH * 2;
-  static constexpr uint32_t COL_STREAM = DH == 64 ? 128 : 160;
-  static constexpr int TMEM_COLS = NS > 1 ? 512 : (DH == 64 ? 128 : 256);
+  static constexpr uint32_t COL_STREAM = DH == 64 ? (OWN_P ? 160 : 128) : (OWN_P ? 192 : 160);
+  static constexpr int TMEM_COLS = NS > 1 ? 512 : 256;
   // shared memory (from a 1024-byte aligned base)
   static constexpr int OFF_Q = 0;                            // [stream]
   static constexpr int OFF_K = OFF_Q + NS * Q_BYTES;         // [stream][slot]
@@ -150,24 +157,24 @@ MARCHE_DEVINL float ex2_approx(float x) {
   return y;
 }
 
-// Unit k of a CTA: query tile (k % n_qt) of its (k / n_qt)-th item; stream j takes k = j, j + NS, ...  Items are dealt to the
-// CTAs in turn, so that CTAs that run at the same time read neighbouring heads of the same cache rows (consecutive
-// ranges per CTA: 59 -> 65 us at S 1088, 41 rows).  Where all units of the launch can run at once the units are dealt
-// instead: with more items than SMs but less than four units per SM some CTAs would get a second round of units (192 items
-// of three tiles, S 320: 25.7 -> 17.5 us).
+// Units are dealt to the CTAs in turn: the k-th of a CTA is one of units k * grid .. k * grid + grid - 1, and unit i is query tile
+// i % n_qt of item i / n_qt, so that CTAs that run at the same time read the same or neighbouring heads of the same cache rows.
+// (Whole items dealt instead leave CTAs without work where items are few, S 1088, 512 items, 151 rows 70 us and 61; S 900, 320
+// items, 300 rows 62 and 55; S 320, 512 items, 230 rows 25.4 and 24.1; level with many.)  Stream j of a CTA takes k = j, j + NS, ...
+// An item's last tile can be much shorter than the others, and no CTA or stream should get the short ones only, or none: where
+// there is more than one turn, a CTA's place in the row of CTAs moves on by `rotate` with every k and by `rotate_turn` with
+// every turn of its streams (chosen by the launch so that the tile number changes along both).
+struct Deal {
+  int units, grid, rotate, rotate_turn;
+  template <int NS> MARCHE_DEVINL int place(int k) const {
+    return ((int)blockIdx.x + k * rotate + k / NS * rotate_turn) % grid;
+  }
+};
 struct Unit { int b, h, start, row0; };    // the tile's first query row; the row on lane 0 (up to 96 before it)
 template <int NS>
-MARCHE_DEVINL Unit unit_of(int j, int u, bool deal_units, int n_qt, int n, int H) {
-  int k = NS * u + j, item, qt;
-  if (deal_units) {
-    k = (int)blockIdx.x + k * (int)gridDim.x;
-    item = k / n_qt;
-    qt = k - item * n_qt;
-  } else {
-    item = k / n_qt;
-    qt = k - item * n_qt;
-    item = (int)blockIdx.x + item * (int)gridDim.x;
-  }
+MARCHE_DEVINL Unit unit_of(int j, int u, const Deal& deal, int n_qt, int n, int H) {
+  const int k = NS * u + j, i = k * deal.grid + deal.place<NS>(k);
+  const int item = i / n_qt, qt = i - item * n_qt;
   Unit r;
   r.b = item / H;
   r.h = item - r.b * H;
@@ -182,9 +189,10 @@ MARCHE_DEVINL Unit unit_of(int j, int u, bool deal_units, int n_qt, int n, int H
 template <int DH, int NS>
 __global__ void __launch_bounds__(Cfg<DH, NS>::THREADS, 1)
 attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid_constant__ CUtensorMap tmap_q,
-                           const __grid_constant__ CUtensorMap tmap_kv_tail, const __grid_constant__ CUtensorMap tmap_q_tail, int n, int S, int H, int B, uint16_t* __restrict__ o, int o_bf16, int* __restrict__ status) {
+                           const __grid_constant__ CUtensorMap tmap_kv_tail, const __grid_constant__ CUtensorMap tmap_q_tail, int n, int S, int H, int B, uint16_t* __restrict__ o, int o_bf16, int* __restrict__ status, int rotate,
+                           int rotate_turn) {
   using C = Cfg<DH, NS>;
-  constexpr bool ROOM = NS == 1;                           // registers hold a row's logits and its weights
+  constexpr bool OWN_P = C::OWN_P;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = ptx::smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -196,14 +204,14 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int D = H * DH;
   const int n_kv = (S + KT - 1) / KT, n_qt = (n + QT - 1) / QT;
-  const bool deal_units = B * H * n_qt <= NS * (int)gridDim.x;
-  const int dealt = deal_units ? B * H * n_qt : B * H;     // units or items over the CTAs
-  const int units_cta = (dealt - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x * (deal_units ? 1 : n_qt);
+  const Deal deal = {B * H * n_qt, (int)gridDim.x, rotate, rotate_turn};
+  const int units_cta = deal.units / deal.grid +           // (the last turn over the CTAs may not reach this one)
+                        (deal.place<NS>(deal.units / deal.grid) < deal.units % deal.grid ? 1 : 0);
   constexpr float c_log2 = (DH == 64 ? 0.125f : 0.111803399f) * 1.4426950408889634f;   // log2(e) / sqrt(head_dim)
 
   if (threadIdx.x == 0) {
     for (int j = 0; j < NS; ++j) {
-      for (int i = 0; i < NB; ++i) ptx::mbar_init(bar(j, i), i == B_P_FULL ? 4 : 1);
+      for (int i = 0; i < NB; ++i) ptx::mbar_init(bar(j, i), i == B_P_FULL || i == B_S_FREE ? 4 : 1);
     }
     abort_flag[0] = 0;
     abort_flag[1] = 0;
@@ -232,7 +240,7 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
       uint32_t k_phase = 1, v_phase = 1;                   // an empty slot's first wait passes at once
       bool ok = true;
       for (int u = 0; u < n_units && ok; ++u) {
-        const Unit un = unit_of<NS>(j, u, deal_units, n_qt, n, H);
+        const Unit un = unit_of<NS>(j, u, deal, n_qt, n, H);
         if (!ptx::mbar_wait(bar(j, B_Q_EMPTY), ((uint32_t)u & 1u) ^ 1u, abort_flag)) { ok = false; break; }
         ptx::mbar_expect_tx(bar(j, B_Q_FULL), C::Q_BYTES);
         ptx::tma_load_3d(base + C::OFF_Q + j * C::Q_BYTES, &tmap_q, un.h * DH, un.row0, un.b, bar(j, B_Q_FULL));
@@ -276,7 +284,7 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
       constexpr uint32_t idesc_s = idesc_bf16(QT, KT, false);
       constexpr uint32_t idesc_o = idesc_bf16(QT, 64, true), idesc_tail = idesc_bf16(QT, 16, true);
       const int total = n_units * n_kv;
-      const uint32_t d_s = tmem_base + (uint32_t)j * C::COL_STREAM, d_o = d_s + COL_O;
+      const uint32_t d_s = tmem_base + (uint32_t)j * C::COL_STREAM, d_p = d_s + C::COL_P, d_o = d_s + C::COL_O;
       const uint64_t dq = ptx::smem_desc_k_sw128(base + C::OFF_Q + j * C::Q_BYTES),
                      dk0 = ptx::smem_desc_k_sw128(base + C::OFF_K + j * NK * C::T_BYTES),
                      dv0 = smem_desc_mn_sw128(base + C::OFF_V + j * NV * C::T_BYTES),
@@ -299,7 +307,7 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
 #pragma unroll
         for (int k = 0; k < 4; ++k) ptx::umma_f16(d_s, dq + 2 * k, dk + 2 * k, idesc_s, k ? 1u : 0u);
         if (DH > 64) ptx::umma_f16(d_s, dq_tail, dk_tail0 + (uint32_t)(s_slot * (C::T_BYTES >> 4)), idesc_s, 1u);
-        ptx::umma_commit(bar(j, B_S_FULL));                // covers the P V before it, too
+        ptx::umma_commit(bar(j, B_S_FULL));                // (covers the P V before it, too, where they are issued together)
         ptx::umma_commit(bar(j, B_K_EMPTY + s_slot));
         if (++s_i == n_kv) {                               // the unit's last Q K^T: Q_j may be overwritten
           s_i = 0;
@@ -314,24 +322,28 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
       }
       for (int t = 0; t < total && ok; ++t) {
         // a wait costs 110 cycles even if nothing is waited for, so those for the tiles come before the one for the weights
-        if ((t + 1 < total && !wait_s()) || !ptx::mbar_wait(bar(j, B_V_FULL + o_slot), v_phase, abort_flag) ||
+        if (t + 1 < total && !wait_s()) { ok = false; break; }
+        if (OWN_P && t + 1 < total) {                      // the logits are in registers: the next ones may come
+          if (!ptx::mbar_wait(bar(j, B_S_FREE), (uint32_t)t & 1u, abort_flag)) { ok = false; break; }
+          ptx::tc_fence_after();
+          issue_s();
+        }
+        if (!ptx::mbar_wait(bar(j, B_V_FULL + o_slot), v_phase, abort_flag) ||
             // (for a unit's first tile the previous output has been read out: every softmax warp did so before it wrote)
             !ptx::mbar_wait(bar(j, B_P_FULL), (uint32_t)t & 1u, abort_flag)) { ok = false; break; }
         ptx::tc_fence_after();
         const uint64_t dv = dv0 + (uint32_t)(o_slot * (C::T_BYTES >> 4));
 #pragma unroll
         for (int k = 0; k < KT / 16; ++k) {
-          umma_f16_ts(d_o, d_s + 8u * k, dv + 128 * k, idesc_o, (o_i | k) ? 1u : 0u);
+          umma_f16_ts(d_o, d_p + 8u * k, dv + 128 * k, idesc_o, (o_i | k) ? 1u : 0u);
           if (DH > 64)
-            umma_f16_ts(d_o + 64u, d_s + 8u * k, dv_tail0 + (uint32_t)(o_slot * (C::T_BYTES >> 4)) + 32 * k, idesc_tail,
+            umma_f16_ts(d_o + 64u, d_p + 8u * k, dv_tail0 + (uint32_t)(o_slot * (C::T_BYTES >> 4)) + 32 * k, idesc_tail,
                         (o_i | k) ? 1u : 0u);
         }
-        if (++o_i == n_kv) {
-          o_i = 0;
-          ptx::umma_commit(bar(j, B_O_FULL));
-        }
+        if (++o_i == n_kv) o_i = 0;
+        if (OWN_P || o_i == 0) ptx::umma_commit(bar(j, B_O_FULL));
         // behind it, in the order of execution, the next logits over these weights
-        if (t + 1 < total) issue_s();
+        if (!OWN_P && t + 1 < total) issue_s();
         ptx::umma_commit(bar(j, B_V_EMPTY + o_slot));
         if (++o_slot == NV) { o_slot = 0; v_phase ^= 1u; }
       }
@@ -345,25 +357,33 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
     const int quarter = warp & 3;
     const int r = quarter * 32 + lane;                     // row inside the query tile = TMEM lane
     const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16);
-    const uint32_t t_s = t_lane + (uint32_t)j * C::COL_STREAM, t_o = t_s + COL_O;   // (the weights go to t_s, too)
+    const uint32_t t_s = t_lane + (uint32_t)j * C::COL_STREAM, t_p = t_s + C::COL_P, t_o = t_s + C::COL_O;
     bool ok = true;
     int t = 0;                                             // tiles of this stream so far
     for (int u = 0; u < n_units && ok; ++u) {
-      const Unit un = unit_of<NS>(j, u, deal_units, n_qt, n, H);
+      const Unit un = unit_of<NS>(j, u, deal, n_qt, n, H);
       const int row = un.row0 + r, row_w = un.row0 + quarter * 32;   // this thread's query row, the warp's first one
       const bool warp_valid = row_w >= un.start && row_w < n;
       float m_ref = -INFINITY, l = 0.f;                    // exponent reference (raw logit units), running sum
       for (int i = 0; i < n_kv; ++i, ++t) {
-        // S_j of this tile is there, and the previous P V is done: it has read the weights and added to O_j
+        // S_j of this tile is there (and without columns for P_j the previous P V is done)
         if (!ptx::mbar_wait(bar(j, B_S_FULL), (uint32_t)t & 1u, abort_flag)) { ok = false; break; }
         ptx::tc_fence_after();
         const int lim = S - i * KT;                        // keys of this tile that exist
+        // The previous P V of this unit has read its weights and added to O_j.  (Without it no warp may announce this tile's
+        // weights, not even one without rows: its arrival would count for the tile before.)
+        auto previous_done = [&]() { return i == 0 || ptx::mbar_wait(bar(j, B_O_FULL), (uint32_t)(t - 1) & 1u, abort_flag); };
         if (warp_valid) {
           uint32_t va[KT / 2], vb[KT / 2];                 // logits of the first and second 32 keys
           ptx::tmem_ld_32x32(t_s, va);
           ptx::tmem_ld_32x32(t_s + KT / 2, vb);
           ptx::tmem_ld_wait(va);
           ptx::tmem_ld_wait(vb);
+          if (OWN_P) {
+            ptx::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(bar(j, B_S_FREE));
+          }
           float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
           if (lim >= KT) {
 #pragma unroll
@@ -378,7 +398,7 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
               if (c + KT / 2 < lim) mx[2 + (c & 1)] = fmaxf(mx[2 + (c & 1)], __uint_as_float(vb[c]));
             }
           }
-          if (!ROOM) ptx::tmem_ld_32x32(t_s, va);          // again, for the exponentials
+          if (!OWN_P) ptx::tmem_ld_32x32(t_s, va);         // again, for the exponentials
           const float tmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
           // lazy reference maximum: move it only when this tile exceeds it by more than 2^8
           const bool move = (tmax - m_ref) * c_log2 > 8.0f;   // also true for a unit's first tile (m_ref = -inf)
@@ -411,10 +431,15 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
             }
           };
           weights(vb, lim - KT / 2);
-          if (!ROOM) ptx::tmem_ld_wait(va);
-          tmem_st_32x16(t_s + KT / 4, vb);                 // over logits that have been read
+          if (OWN_P) {
+            ok = previous_done();
+            ptx::tc_fence_after();
+          } else {
+            ptx::tmem_ld_wait(va);
+          }
+          tmem_st_32x16(t_p + KT / 4, vb);                 // (without columns of their own: over logits that have been read)
           weights(va, lim);
-          tmem_st_32x16(t_s, va);
+          tmem_st_32x16(t_p, va);
           if (rescale) {
             // this row's accumulator in tensor memory moves to the new reference
 #pragma unroll 1
@@ -430,14 +455,18 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
           }
           l += (ls[0] + ls[1]) + (ls[2] + ls[3]);
           tmem_st_wait();
+        } else if (OWN_P) {
+          if (lane == 0) ptx::mbar_arrive(bar(j, B_S_FREE));
+          ok = previous_done();
         }
+        if (!ok) break;
         ptx::tc_fence_before();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(bar(j, B_P_FULL));
       }
       if (!ok) break;
       // ---- end of the unit: O / l -> output rows
-      if (!ptx::mbar_wait(bar(j, B_O_FULL), (uint32_t)u & 1u, abort_flag)) { ok = false; break; }
+      if (!ptx::mbar_wait(bar(j, B_O_FULL), (uint32_t)(OWN_P ? t - 1 : u) & 1u, abort_flag)) { ok = false; break; }
       ptx::tc_fence_after();
       if (warp_valid) {
         const float inv = 1.0f / l;
@@ -508,9 +537,13 @@ cudaError_t launch_stream(const void* q, int ld_q, int B, int n, int S, int H, c
   if (e != cudaSuccess) return e;
   const int sms = device_sm_count();
   const long units = (long)B * H * ((n + QT - 1) / QT);
-  const int grid = units < sms ? (int)units : sms;
+  const int grid = units < sms ? (int)units : sms, n_qt = (n + QT - 1) / QT;
+  // a CTA's next unit is grid + rotate units on, a stream's NS (grid + rotate) + rotate_turn: neither a multiple of an item's tiles
+  const bool turns = units > (long)NS * grid;
+  const int rotate = turns ? (n_qt > 1 && (grid + 1) % n_qt == 0 ? 2 : 1) : 0;
+  const int rotate_turn = turns && n_qt > 1 && NS * (grid + rotate) % n_qt == 0 ? 1 : 0;
   return launch_pdl(attention_tc_stream_kernel<DH, NS>, dim3(grid), dim3(C::THREADS), (size_t)C::SMEM_BYTES, st, tkv, tq, tkv_tail,
-                    tq_tail, n, S, H, B, (uint16_t*)o, o_bf16 ? 1 : 0, status);
+                    tq_tail, n, S, H, B, (uint16_t*)o, o_bf16 ? 1 : 0, status, rotate, rotate_turn);
 }
 
 }  // namespace
@@ -530,7 +563,7 @@ bool attention_tc_stream_wins(int n, int S, int dh, int items, int min_rows) {
   if (n > min_rows) return true;
   if (3 * n <= 2 * min_rows) return false;
   if (dh == 64) return S >= 512;
-  const int streams = Streams<80>::N * device_sm_count(), rounds = (items + streams - 1) / streams;
+  const int streams = kStreams * device_sm_count(), rounds = (items + streams - 1) / streams;
   return S > 4 * KT && (rounds == 1 || 4 * items >= 3 * rounds * streams);
 }
 
@@ -539,16 +572,19 @@ cudaError_t launch_attention_tc_stream(const void* q, int ld_q, int B, int n, in
   if (n == 0) return cudaSuccess;
   if ((dh != 64 && dh != 80) || ld_q % 8 || ((uintptr_t)q & 15) || ((uintptr_t)cache_layer & 15) || ((uintptr_t)o & 15) || S > 2048)
     return cudaErrorInvalidValue;
-  // No more units than SMs: a CTA has one, and a CTA of one stream, with registers for a row's logits beside its weights (104 a
-  // thread where four streams leave 80), takes it through its tiles faster.  One stream against four, us: 16 items, S 640, 80
-  // rows 12.2 and 13.2; 144 items, S 1088, 116 rows 19.4 and 21.4; S 2048, 96 rows 33.6 and 36.8; 64 items, S 1088, 200 rows
-  // 19.1 and 21.3.
-  // Head_dim 80: 144 items, S 100, 80 rows 5.45 and 5.8; nothing over longer sequences.
-  if ((long)B * H * ((n + QT - 1) / QT) <= device_sm_count() && (dh == 64 || S <= 2 * KT))
+  const long units = (long)B * H * ((n + QT - 1) / QT);
+  const int sms = device_sm_count();
+  // No more units than SMs: a CTA has one, and a CTA of one stream is smaller and starts sooner.  Head_dim 80: 144 items, S 100,
+  // 80 rows 5.4 and 5.8 us; not over longer sequences.
+  if (units <= sms && (dh == 64 || S <= 2 * KT))
     return dh == 64 ? launch_stream<64, 1>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st)
                     : launch_stream<80, 1>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
-  return dh == 64 ? launch_stream<64, Streams<64>::N>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st)
-                  : launch_stream<80, Streams<80>::N>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
+  // Head_dim 64: four streams take more units at a time than three, each more slowly; where all units run at once that counts
+  // (192 items, S 320, 320 rows: 576 units on 444 or 592 streams 16.0 and 14.4 us).
+  if (dh == 64 && units > (long)kStreams * sms && units <= 4L * sms)
+    return launch_stream<64, 4>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
+  return dh == 64 ? launch_stream<64, kStreams>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st)
+                  : launch_stream<80, kStreams>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
 }
 
 }  // namespace marche

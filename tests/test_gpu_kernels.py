@@ -915,3 +915,24 @@ def test_scores_of_a_few_among_many_rows(dh, H, B, S, n, nG):
                 want += p.sum(axis=0)
             assert max_abs(got[b], want) <= 2e-4 * H * nG and abs(got[b].sum() - H * nG) <= 1e-4 * H * nG
     assert m.device_status() == 0
+
+
+@pytest.mark.parametrize("dh,H", [(64, 4), (80, 8)])
+@pytest.mark.parametrize("B,S,n", [(111, 128, 128), (112, 100, 65), (148, 130, 128), (149, 33, 33), (75, 257, 257), (50, 300, 300), (23, 577, 577),
+                                   (16, 1100, 1100)])
+def test_attention_single_pass_streams_deal_units(dh, H, B, S, n):
+    """Around one unit per stream (444 units of three streams, 592 of four) and over several turns, with 1 to 9 query tiles per
+    item: every unit is taken once, whole and by one stream.  Bounds as in the two tests of these streams above."""
+    from paper_2506_12035_b200 import binding
+    D = H * dh
+    cfg, blocks, m = model_for("bf16", D, H, 128, S, B)
+    m.set_tuning(attention_kernel=binding.ATTENTION_TCGEN05)
+    gen = torch.Generator(device="cuda").manual_seed(B + S + n + dh)
+    cache = torch.randn(2, B, S, D, generator=gen, device="cuda").to(torch.bfloat16)
+    q = (torch.randn(B * n, D, generator=gen, device="cuda") * 3.0).to(torch.bfloat16)
+    o = torch.full((B * n + 1, D), 7.0, dtype=torch.float16, device="cuda")
+    m.attention(q, D, n, cache, None, None, o[:-1])
+    assert m.device_status() == 0 and (o[-1] == 7.0).all()
+    heads = lambda t: t.view(B, -1, H, dh).transpose(1, 2).float()
+    want = torch.softmax(heads(q) @ heads(cache[0]).transpose(2, 3) / math.sqrt(dh), -1) @ heads(cache[1])
+    assert (heads(o[:-1]) - want).norm() <= 8e-3 * want.norm() and (heads(o[:-1]) - want).abs().max() <= 3e-2

@@ -180,6 +180,17 @@ bool use_pair(const marche_ctx* ctx, int M, int N, int K) {
   return gemm_splitk_cost(M, N, K, gemm_splitk_pick(M, N, K)) > (wide < narrow ? wide : narrow);
 }
 
+// A handful of rows: the mma.sync kernel (use_pair is not asked then).
+bool use_few(const marche_ctx* ctx, int M, int N, int K, bool norm = false) {
+  return ctx->bf16 && ctx->tune.gemm_kernel == MARCHE_GEMM_AUTO && gemm_few_wins(M, N, K, norm);
+}
+
+// The M x N x D projection takes the residual rows themselves and normalises them: no LayerNorm launch before it.
+bool use_few_norm(const marche_ctx* ctx, int M, int N) {
+  const unsigned ln = 1u << MARCHE_KC_GATHER_LN;           // (the measurement hooks mean a launch of its own)
+  return use_few(ctx, M, N, ctx->cfg.width, true) && !((ctx->skip_mask | ctx->repeat_mask) & ln);
+}
+
 // True when a projection of a step on M rows may run stream-K, whose turn flags in the workspace have to start at zero.
 // (Clearing them costs a few microseconds of a step on few rows: the kernels on either side of a memset do not overlap.)
 bool needs_turn(const marche_ctx* ctx, int M) {
@@ -192,8 +203,10 @@ bool qkv_scatter_fused(const marche_ctx* ctx) {
   return ctx->tune.fuse_qkv_scatter && !(ctx->bf16 && ctx->tune.two_segment_attention);
 }
 
+// gamma, beta given (use_few_norm): a holds fp32 rows that are normalised first.
 int do_linear(marche_ctx* ctx, int cls, const void* a, int lda, int M, const void* w, const float* bias, int N, int K,
-              int epi, void* out, cudaStream_t st, int* turn = nullptr, const KvScatter* kv = nullptr) {
+              int epi, void* out, cudaStream_t st, int* turn = nullptr, const KvScatter* kv = nullptr,
+              const float* gamma = nullptr, const float* beta = nullptr) {
   if (skipped(ctx, cls)) return MARCHE_OK;
   if (!ctx->bf16) {
     if (M > 0) mark(ctx, cls, st);
@@ -204,10 +217,12 @@ int do_linear(marche_ctx* ctx, int cls, const void* a, int lda, int M, const voi
   if (N % 128 || K % 64) return MARCHE_ESHAPE;
   if (lda % 8 || (((uintptr_t)a | (uintptr_t)w | (uintptr_t)out) & 15)) return misaligned(ctx, "projection");
   if (M == 0) return MARCHE_OK;                         // no rows: no estimate of a kernel's time either
-  const bool pair = use_pair(ctx, M, N, K);
+  const bool few = use_few(ctx, M, N, K, gamma != nullptr), pair = !few && use_pair(ctx, M, N, K);
   for (int r = 0; r < launches_of(ctx, cls); ++r) {
     if (M > 0) mark(ctx, cls, st);
-    if (pair)
+    if (few)
+      MARCHE_TRY(launch_gemm_few(a, lda, M, w, bias, N, K, epi, out, ctx->a_bf16, ctx->status_dev, st, kv, gamma, beta, ctx->eps), "gemm_few");
+    else if (pair)
       MARCHE_TRY(launch_gemm_tcgen05_2cta(a, lda, M, w, bias, N, K, epi, out, ctx->a_bf16, ctx->status_dev, st,
                                           gemm_tuning(ctx), turn, kv), "gemm_tcgen05_2cta");
     else
@@ -319,11 +334,12 @@ int run_blocks(marche_ctx* ctx, int l_begin, int l_end, const float* gather_src,
     const int slot = is_new ? score_slot(ctx, l) : -1;
     const uint8_t* flags_l = slot >= 0 ? is_new : nullptr;
     float* partial_l = bf.partial + (size_t)(slot > 0 ? slot : 0) * B * c.n_heads * c.seq_len;
-    const bool skip_ln = skipped(ctx, MARCHE_KC_GATHER_LN);
-    if (!skip_ln) mark(ctx, MARCHE_KC_GATHER_LN, st);
-    for (int r = 0; r < (skip_ln ? 0 : launches_of(ctx, MARCHE_KC_GATHER_LN)); ++r) {
+    const bool skip_ln = skipped(ctx, MARCHE_KC_GATHER_LN), gather = l == l_begin && gather_src;
+    const bool norm1 = !gather && use_few_norm(ctx, M, 3 * D), norm2 = use_few_norm(ctx, M, F);
+    if (!skip_ln && !norm1) mark(ctx, MARCHE_KC_GATHER_LN, st);
+    for (int r = 0; r < (skip_ln || norm1 ? 0 : launches_of(ctx, MARCHE_KC_GATHER_LN)); ++r) {
       if (r) mark(ctx, MARCHE_KC_GATHER_LN, st);
-      if (l == l_begin && gather_src)
+      if (gather)
         MARCHE_TRY(launch_gather_layernorm(ctx->a_kind, gather_src, src_rows, idx, B, nA, D, bw.ln1_g, bw.ln1_b, ctx->eps,
                                            x, bf.u, st), "gather_layernorm");
       else
@@ -332,8 +348,9 @@ int run_blocks(marche_ctx* ctx, int l_begin, int l_end, const float* gather_src,
     }
     const bool fused_kv = qkv_scatter_fused(ctx);
     const KvScatter kvs = {kv_idx, cache_l, nA, S, B, D};
-    int rc = do_linear(ctx, MARCHE_KC_GEMM_QKV, bf.u, D, M, bw.w_qkv, bw.b_qkv, 3 * D, D, fused_kv ? 4 : MARCHE_EPI_BIAS,
-                       bf.qkv, st, nullptr, fused_kv ? &kvs : nullptr);
+    int rc = do_linear(ctx, MARCHE_KC_GEMM_QKV, norm1 ? (const void*)x : bf.u, D, M, bw.w_qkv, bw.b_qkv, 3 * D, D,
+                       fused_kv ? 4 : MARCHE_EPI_BIAS, bf.qkv, st, nullptr, fused_kv ? &kvs : nullptr,
+                       norm1 ? bw.ln1_g : nullptr, norm1 ? bw.ln1_b : nullptr);
     if (rc) return rc;
     if (fused_kv) {
       // the projection's epilogue has written K and V into the cache (Algorithm 1 line 11)
@@ -355,12 +372,13 @@ int run_blocks(marche_ctx* ctx, int l_begin, int l_end, const float* gather_src,
     }
     rc = do_linear(ctx, MARCHE_KC_GEMM_O, bf.o, D, M, bw.w_o, bw.b_o, D, D, MARCHE_EPI_BIAS_RESIDUAL, x, st, bf.turn);
     if (rc) return rc;
-    for (int r = 0; r < (skip_ln ? 0 : launches_of(ctx, MARCHE_KC_GATHER_LN)); ++r) {
+    for (int r = 0; r < (skip_ln || norm2 ? 0 : launches_of(ctx, MARCHE_KC_GATHER_LN)); ++r) {
       mark(ctx, MARCHE_KC_GATHER_LN, st);
       MARCHE_TRY(launch_gather_layernorm(ctx->a_kind, x, nA, nullptr, B, nA, D, bw.ln2_g, bw.ln2_b, ctx->eps, nullptr,
                                          bf.u, st), "layernorm2");
     }
-    rc = do_linear(ctx, MARCHE_KC_GEMM_FC1, bf.u, D, M, bw.w_fc1, bw.b_fc1, F, D, MARCHE_EPI_BIAS_GELU, bf.g, st);
+    rc = do_linear(ctx, MARCHE_KC_GEMM_FC1, norm2 ? (const void*)x : bf.u, D, M, bw.w_fc1, bw.b_fc1, F, D, MARCHE_EPI_BIAS_GELU,
+                   bf.g, st, nullptr, nullptr, norm2 ? bw.ln2_g : nullptr, norm2 ? bw.ln2_b : nullptr);
     if (rc) return rc;
     rc = do_linear(ctx, MARCHE_KC_GEMM_FC2, bf.g, F, M, bw.w_fc2, bw.b_fc2, D, F, MARCHE_EPI_BIAS_RESIDUAL, x, st, bf.turn);
     if (rc) return rc;

@@ -99,6 +99,14 @@ cudaError_t launch_gemm_splitk(const void* a, int lda, int M, const void* w, con
                                void* out, bool a_bf16, int* status, cudaStream_t st, SplitKShape shape,
                                const KvScatter* kv_scatter = nullptr);
 
+// K2 for up to 32 rows on mma.sync.  Same operand rules.  gamma (and beta) given: a is fp32 [M][lda] and its rows are normalised
+// first (epilogues 0, 2 and 4).  Weights, bias, gamma, beta and the scatter's token indices are read ahead of the dependency wait: they
+// were complete before the preceding launch.
+bool gemm_few_wins(int M, int N, int K, bool norm);
+cudaError_t launch_gemm_few(const void* a, int lda, int M, const void* w, const float* bias, int N, int K, int epilogue, void* out,
+                            bool a_bf16, int* status, cudaStream_t st, const KvScatter* kv_scatter = nullptr, const float* gamma = nullptr,
+                            const float* beta = nullptr, float eps = 0.f);
+
 // K3 of the fp32 configuration (SIMT): attention of n queries per sample over all S cache rows.
 cudaError_t launch_attention_simt(const float* q, int ld_q, int B, int n, int S, int H, int dh,
                                   const float* cache_layer, const uint8_t* is_new, float* score_partial,

@@ -936,3 +936,67 @@ def test_attention_single_pass_streams_deal_units(dh, H, B, S, n):
     heads = lambda t: t.view(B, -1, H, dh).transpose(1, 2).float()
     want = torch.softmax(heads(q) @ heads(cache[0]).transpose(2, 3) / math.sqrt(dh), -1) @ heads(cache[1])
     assert (heads(o[:-1]) - want).norm() <= 8e-3 * want.norm() and (heads(o[:-1]) - want).abs().max() <= 3e-2
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "bf16b"])
+@pytest.mark.parametrize("M,N,K", [(1, 128, 64), (3, 384, 128), (7, 2304, 768), (15, 128, 2048), (16, 640, 2112), (16, 1024, 4096), (17, 768, 768),
+                                   (31, 384, 1088), (32, 768, 3072)])
+def test_linear_of_a_handful_of_rows(dtype, M, N, K):
+    """Up to 32 rows, whole K per CTA and K split over pairs of CTAs, K blocks that do not divide evenly among warps and CTAs:
+    against the oracle's product, rows beyond M untouched, and the same bits every time.  (fp32 sums of K products of unit
+    scale, then one rounding of the output; residual outputs stay fp32.)"""
+    cfg, blocks, m = model_for(dtype, 256, 4, 1024, 68, 2)
+    rng = np.random.default_rng(M + N + K)
+    a = rng.standard_normal((M, K)).astype(np.float32)
+    w = (rng.standard_normal((N, K)) * 0.05).astype(np.float32)
+    bias = rng.standard_normal(N).astype(np.float32)
+    acc = orc.linear(quant_a(a, dtype), quant_a(w, dtype), bias.astype(np.float64))
+    a_d, w_d, b_d = dev(a, adt(dtype)), dev(w, adt(dtype)), dev(bias)
+    scale = math.sqrt(K / 256)
+    out = torch.full((M + 2, N), 5.0, dtype=tdt(dtype), device="cuda")
+    m.linear(a_d, w_d, b_d, 0, out, M=M)
+    assert max_abs(host(out[:M]), acc) <= 3e-2 * max(1.0, scale) and rel_l2(host(out[:M]), acc) <= 4e-3
+    assert (host(out[M:]) == 5.0).all()
+    res = rng.standard_normal((M, N)).astype(np.float32)
+    first = None
+    for _ in range(3):
+        out = dev(res)
+        m.linear(a_d, w_d, b_d, 1, out)
+        assert max_abs(host(out), acc + res) <= 2e-5 * max(1.0, scale)
+        assert first is None or torch.equal(out, first)
+        first = out
+    out = torch.zeros(M, N, dtype=adt(dtype), device="cuda")
+    m.linear(a_d, w_d, b_d, 2, out)
+    want = orc.gelu(acc)
+    assert max_abs(host(out), want) <= 3e-2 * max(1.0, scale) and rel_l2(host(out), want) <= 4e-3
+    assert m.device_status() == 0
+
+
+@pytest.mark.parametrize("operand", ["f16", "bf16"])
+@pytest.mark.parametrize("D,H,F,B,n", [(256, 4, 1024, 1, 1), (768, 12, 3072, 2, 8), (768, 12, 3072, 3, 9), (1024, 16, 4096, 1, 15), (1280, 16, 2560, 2, 7),
+                                       (2048, 32, 2048, 1, 16)])
+def test_few_rows_normalise_in_the_projection(operand, D, H, F, B, n):
+    """A step on up to 32 rows whose projections normalise their rows, against the same step with LayerNorm launches (which a
+    measurement hook asks for): rows with a mean of ten deviations.  The two statistics differ by fp32 rounding, so what
+    differs are single 16-bit roundings of the operands (2^-11 and 2^-8 of a value) on a part of the values."""
+    import synth
+    from helpers import make_model
+    cfg = synth.CONFIGS["mar_b"].replace(L=3, E=0, D=D, H=H, F=F, B=B, S=40, n_buffer=8)
+    m = make_model(cfg, synth.make_weights(cfg), operand=operand)
+    rng = np.random.default_rng(D + n)
+    hidden = dev((rng.standard_normal((B, cfg.S, D)) + 10.0 * rng.standard_normal((B, cfg.S, 1))).astype(np.float32))
+    act = idx_dev(np.stack([rng.permutation(cfg.S)[:n] for _ in range(B)]))
+    got = []
+    for hook in ((), ("gather_layernorm",)):
+        m.debug_repeat_classes(hook)
+        cache, out, ws = m.alloc_cache(), torch.zeros(B, cfg.S, D, device="cuda"), m.alloc_workspace(cfg.S)
+        m.init_cache(cache)
+        m.full_step(hidden, cache, act, None, 0.0, out, None, ws)
+        before = m.launch_count()
+        m.step(hidden, cache, act, act, None, 0.0, out, None, ws)
+        got.append((host(out), host(cache), m.launch_count() - before))
+    m.debug_repeat_classes(())
+    assert got[1][2] - got[0][2] == 2 * cfg.L + 2 * cfg.L - 1              # all but the first are gone, and the hook doubles them
+    rel = 2e-4 if operand == "f16" else 1.6e-3
+    assert rel_l2(got[0][0], got[1][0]) <= rel and rel_l2(got[0][1], got[1][1]) <= 8 * rel
+    assert m.device_status() == 0

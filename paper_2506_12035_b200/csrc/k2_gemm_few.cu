@@ -384,12 +384,13 @@ cudaError_t launch_any(const Plan& p, bool norm, Args... args) {
 
 }  // namespace
 
-// One group of rows always (a block of a step at 16 rows: widths 768, 1024, 1280 22.8 -> 17.3, 25.6 -> 19.7, 30.1 -> 26.0 us against the
-// split-K kernel with LayerNorm launches), two where the launch is one and a half CTAs per SM at most (32 rows: width 768, 192 CTAs
-// 23.9 -> 21.2; width 1024, 256 CTAs 27.1 -> 27.0; width 1280, 640 CTAs 31.8 -> 43.6), three never (48 rows, width 768 25.5 -> 26.2).
+// One group of rows always (a block of a step at 16 rows: widths 768, 1024, 1280 22.8 -> 17.3, 25.6 -> 20.0, 30.1 -> 26.4 us against the
+// split-K kernel with LayerNorm launches), two where the launch has no more warps than one CTA of 16 per SM (32 rows: width 768, 192
+// CTAs of 12 warps 23.9 -> 20.4; width 1024, 192 CTAs of 16 26.6 -> 27.0; width 1280, 640 CTAs 31.8 -> 43.6), three never (48 rows, width
+// 768 25.5 -> 26.2).
 bool gemm_few_wins(int M, int N, int K, bool norm) {
   Plan p;
-  return M <= 2 * kRows && make_plan(M, N, K, norm, &p) && (M <= kRows || 2 * p.ctas <= 3 * device_sm_count());
+  return M <= 2 * kRows && make_plan(M, N, K, norm, &p) && (M <= kRows || p.ctas * p.warps <= kMaxWarps * device_sm_count());
 }
 
 cudaError_t launch_gemm_few(const void* a, int lda, int M, const void* w, const float* bias, int N, int K, int epilogue, void* out,

@@ -29,14 +29,20 @@ using namespace att;
 
 constexpr int kMaxTiles = 12;                            // per CTA
 constexpr int kMaxThreads = 512;
+constexpr int kFewParts = 5;                             // partial results of a row that are merged without a loop
 enum { ST_ATTENTION_SPLIT = 0x24 };
+
+template <bool Q_TMA> struct QueryMaps { CUtensorMap main, tail; };   // columns 0-63 and 64-79 of a head
+template <> struct QueryMaps<false> {};
 
 // NQ * nk consumer warps (NQ groups of 16 query rows, nk shares of the CTA's tiles) and a producer warp.  Grid: cs * B * H
 // CTAs in clusters of cs.
-template <int DH, int NQ>
+// Q_TMA: the query rows come by TMA (16-byte aligned rows), for many groups of warps (see the launch).
+template <int DH, int NQ, bool Q_TMA>
 __global__ void __launch_bounds__(kMaxThreads)
 attention_split_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid_constant__ CUtensorMap tmap_tail,
-                       const bf16* __restrict__ q, int ld_q, int n, int S, int H, int B, int cs, int nk, int tiles_max,
+                       const __grid_constant__ QueryMaps<Q_TMA> tmap_q,
+                       const bf16* __restrict__ q, int ld_q, int n, int S, int H, int B, int cs, int nk, int tiles_max, int q_off,
                        uint16_t* __restrict__ o, bool o_bf16, int* __restrict__ status) {
   using Cfg = AttCfg<DH>;
   constexpr int ROW = DH + 4;                            // a row's partial result: DH sums, maximum, sum of weights
@@ -46,9 +52,11 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid
   const int own = (NQ * 16 + cs - 1) / cs;               // query rows merged per CTA
   const int n_parts = cs * nk;                           // partial results of a row
   // [n_parts][own][ROW] floats: over the tiles once they are used up, or behind them where other CTAs may be earlier
+  // (a query tile, where TMA can address the rows, behind both)
   const uint32_t recv = cs > 1 ? base + (uint32_t)tiles_max * Cfg::STAGE_BYTES : base;
+  const uint32_t q_tile = base + (uint32_t)q_off;
   const float* recv_gen = reinterpret_cast<const float*>(smem_raw + (recv - raw));
-  __shared__ __align__(8) uint64_t full_bars[kMaxTiles];
+  __shared__ __align__(8) uint64_t full_bars[kMaxTiles + 1];   // the tiles', the queries'
   __shared__ int abort_flags[2];
   const uint32_t full0 = ptx::smem_u32(full_bars);
   volatile int* abort_flag = abort_flags;
@@ -63,7 +71,7 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid
   const float scale_log2 = rsqrtf((float)DH) * 1.4426950408889634f;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kMaxTiles; ++s) ptx::mbar_init(full0 + 8u * s, 1);
+    for (int s = 0; s <= kMaxTiles; ++s) ptx::mbar_init(full0 + 8u * s, 1);
     abort_flags[0] = abort_flags[1] = 0;
     ptx::fence_barrier_init();
     ptx::fence_proxy_async();
@@ -88,6 +96,12 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid
   const bool warp_active = warp < n_cons && wq * 16 < n;
   if (warp == n_cons) {
     if (lane == 0) {
+      if constexpr (Q_TMA) {
+        const uint32_t bar = full0 + 8u * kMaxTiles;
+        ptx::mbar_expect_tx(bar, (uint32_t)(NQ * 16 * DH * 2));
+        ptx::tma_load_3d(q_tile, &tmap_q.main, h * DH, 0, b, bar);
+        if (DH > 64) ptx::tma_load_3d(q_tile + KT * 128, &tmap_q.tail, h * DH + 64, 0, b, bar);
+      }
       for (int i = 0; i < n_tiles; ++i) {
         const uint32_t dst = base + i * Cfg::STAGE_BYTES, bar = full0 + 8u * i;
         ptx::mbar_expect_tx(bar, Cfg::STAGE_BYTES);
@@ -100,7 +114,12 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid
     __syncwarp();
   } else if (warp_active) {
     uint32_t qf[Cfg::KSTEPS][4];                         // this warp's 16 query rows as A fragments
-    {
+    if constexpr (Q_TMA) {
+      ok = ptx::mbar_wait(full0 + 8u * kMaxTiles, 0, abort_flag);
+#pragma unroll
+      for (int kk = 0; kk < Cfg::KSTEPS; ++kk)
+        ldsm_x4(q_tile + kv_off<DH>(wq * 16 + (lane & 15), 2 * kk + (lane >> 4)), qf[kk][0], qf[kk][1], qf[kk][2], qf[kk][3]);
+    } else {
       const int r0 = wq * 16 + g, r1 = r0 + 8;
       const bf16* q0 = q + ((size_t)b * n + r0) * ld_q + h * DH;
       const bf16* q1 = q + ((size_t)b * n + r1) * ld_q + h * DH;
@@ -112,7 +131,7 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid
         qf[kk][3] = r1 < n ? *reinterpret_cast<const uint32_t*>(q1 + kk * 16 + 8 + 2 * tg) : 0u;
       }
     }
-    for (int i = wk; i < n_tiles; i += nk) {
+    for (int i = wk; i < n_tiles && ok; i += nk) {
       if (!ptx::mbar_wait(full0 + 8u * i, 0, abort_flag)) { ok = false; break; }
       const uint32_t k_tile = base + i * Cfg::STAGE_BYTES, v_tile = k_tile + Cfg::TILE_BYTES;
       // ---- raw logits of 16 rows x 64 keys
@@ -199,6 +218,7 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid
     *(volatile int*)status = ST_ATTENTION_SPLIT;
     // let copies already issued land before the CTA's shared memory is released
     for (int i = 0; i < n_tiles; ++i) ptx::mbar_wait(full0 + 8u * i, 0, abort_flag + 1, 20000000LL);
+    if (Q_TMA) ptx::mbar_wait(full0 + 8u * kMaxTiles, 0, abort_flag + 1, 20000000LL);
   }
 
   if (n_parts == 1) {
@@ -227,7 +247,7 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid
       for (int r = 0; r < 2; ++r) {
         const int row = wq * 16 + g + 8 * r;
         if (row < n) {
-          const int owner = row / own;
+          const int owner = cs > 1 ? row / own : 0;
           uint32_t dst = recv + 4u * (uint32_t)(((rank * nk + wk) * own + row - owner * own) * ROW);
           if (cs > 1) dst = ptx::mapa(dst, (uint32_t)owner);
 #pragma unroll
@@ -248,19 +268,33 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid
     }
     // ---- merge, in rank order: one thread per four columns of a row this CTA owns
     if (!*abort_flag) {
+      const int stride = own * ROW;
       for (int e = threadIdx.x; e < own * (DH / 4); e += (int)blockDim.x) {
         const int j = e / (DH / 4), c = e % (DH / 4) * 4, row = rank * own + j;
         if (row >= n) continue;
+        const float* p = recv_gen + j * ROW;
         float m = -INFINITY, l = 0.f;
-        for (int s = 0; s < n_parts; ++s) m = fmaxf(m, recv_gen[(s * own + j) * ROW + DH]);
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int s = 0; s < n_parts; ++s) {
-          const float* p = recv_gen + (s * own + j) * ROW;
-          const float w = ex2_approx((p[DH] - m) * scale_log2);
-          const float4 v = *reinterpret_cast<const float4*>(p + c);
-          l = fmaf(w, p[DH + 1], l);
+        auto add = [&](float w, float l_s, const float4& v) {
+          l = fmaf(w, l_s, l);
           acc.x = fmaf(w, v.x, acc.x); acc.y = fmaf(w, v.y, acc.y);
           acc.z = fmaf(w, v.z, acc.z); acc.w = fmaf(w, v.w, acc.w);
+        };
+        if constexpr (Q_TMA) {                        // all loads at once (a loop of loads took 2500 cycles for five parts)
+          float2 ml[kFewParts];
+          float4 v[kFewParts];
+#pragma unroll
+          for (int s = 0; s < kFewParts; ++s) {
+            ml[s] = s < n_parts ? *reinterpret_cast<const float2*>(p + s * stride + DH) : make_float2(-INFINITY, 0.f);
+            v[s] = s < n_parts ? *reinterpret_cast<const float4*>(p + s * stride + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+            m = fmaxf(m, ml[s].x);
+          }
+#pragma unroll
+          for (int s = 0; s < kFewParts; ++s) add(ex2_approx((ml[s].x - m) * scale_log2), ml[s].y, v[s]);
+        } else {
+          for (int s = 0; s < n_parts; ++s) m = fmaxf(m, p[s * stride + DH]);
+          for (int s = 0; s < n_parts; ++s)
+            add(ex2_approx((p[s * stride + DH] - m) * scale_log2), p[s * stride + DH + 1], *reinterpret_cast<const float4*>(p + s * stride + c));
         }
         const float f = 1.0f / l;
         uint2 u;
@@ -272,18 +306,27 @@ attention_split_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __grid
   }
 }
 
-template <int DH, int NQ>
+template <int DH, int NQ, bool Q_TMA>
 cudaError_t launch_split(const CUtensorMap& tm, const CUtensorMap& tail, const bf16* q, int ld_q, int B, int n, int S, int H,
                          int cs, int nk, uint16_t* o, bool o_bf16, int* status, cudaStream_t st) {
   const int n_kv = (S + KT - 1) / KT, tiles = (n_kv + cs - 1) / cs, own = (NQ * 16 + cs - 1) / cs, threads = (NQ * nk + 1) * 32;
   const size_t ring = (size_t)tiles * AttCfg<DH>::STAGE_BYTES, recv = cs * nk > 1 ? (size_t)cs * nk * own * (DH + 4) * 4 : 0;
-  const size_t smem = 1024 + (cs > 1 ? ring + recv : (ring > recv ? ring : recv));
+  const size_t used = cs > 1 ? ring + recv : (ring > recv ? ring : recv);
+  const size_t q_off = (used + 1023) / 1024 * 1024, smem = 1024 + (Q_TMA ? q_off + AttCfg<DH>::TILE_BYTES : used);
+  QueryMaps<Q_TMA> tq;
+  if constexpr (Q_TMA) {
+    const uint64_t dims[3] = {(uint64_t)ld_q, (uint64_t)n, (uint64_t)B};
+    const uint64_t strides[2] = {(uint64_t)ld_q * 2, (uint64_t)n * ld_q * 2};
+    const uint32_t box[3] = {64, NQ * 16, 1}, box_tail[3] = {16, NQ * 16, 1};
+    if (!tma_make_map_bf16(&tq.main, q, 3, dims, strides, box, true)) return cudaErrorInvalidValue;
+    tq.tail = tq.main;
+    if (DH > 64 && !tma_make_map_bf16(&tq.tail, q, 3, dims, strides, box_tail, false, false, true)) return cudaErrorInvalidValue;
+  }
   if (tiles > kMaxTiles || threads > kMaxThreads || smem > 226 * 1024) return cudaErrorInvalidValue;
   static size_t smem_set[kMaxDevices] = {};
-  cudaError_t e = ensure_dynamic_smem(attention_split_kernel<DH, NQ>, smem, smem_set);
+  cudaError_t e = ensure_dynamic_smem(attention_split_kernel<DH, NQ, Q_TMA>, smem, smem_set);
   if (e != cudaSuccess) return e;
-  return launch_pdl_cluster(attention_split_kernel<DH, NQ>, dim3(cs * B * H), dim3(threads), smem, cs, st, tm, tail, q, ld_q, n,
-                            S, H, B, cs, nk, tiles, o, o_bf16, status);
+  return launch_pdl_cluster(attention_split_kernel<DH, NQ, Q_TMA>, dim3(cs * B * H), dim3(threads), smem, cs, st, tm, tail, tq, q, ld_q, n, S, H, B, cs, nk, tiles, (int)q_off, o, o_bf16, status);
 }
 
 }  // namespace
@@ -302,6 +345,16 @@ bool attention_split_plan(int n, int S, int dh, int items, int* cs, int* nk) {
   // CTAs do better.  64 rows, S 320, eight blocks of a step: 64 items 342 us on pairs, 315 on one, mma.sync kernel 320; 32 items
   // 295 either way; 16 items on four CTAs 6.4 us against 6.7 back to back.)
   if (dh == 80 && nq == 4 && n_kv <= 5 && 2 * c * items > device_sm_count()) c = 1;
+  // Two or three groups of query rows over four or five tiles: a single CTA whose groups of warps take a tile each, where there are
+  // enough items that pairs of CTAs would be the alternative (a block of a step, us, five tiles: 43 rows, 32 items 30.8 -> 29.8, 48 items
+  // 30.3 -> 29.0; 20 rows, 64 items 32.1 -> 29.6, 72 items 30.4 -> 28.9; head_dim 80, 32 items 37.9 -> 35.7, 20 rows, 64 items 35.8 -> 34.5;
+  // with fewer items clusters of four do better: 43 rows, 24 items 26.6 and 27.2).  At head_dim 80 three groups from 49 items on stay on
+  // pairs of CTAs.
+  if ((nq == 2 || nq == 3) && (n_kv == 4 || n_kv == 5) && items > 28 && 2 * items <= device_sm_count() && !(dh == 80 && nq == 3 && items > 48)) {
+    *cs = 1;
+    *nk = n_kv;
+    return true;
+  }
   while (c < 8 && (n_kv + c - 1) / c > (dh == 64 ? 10 : 8)) c *= 2;
   const int tiles = (n_kv + c - 1) / c;
   if (tiles > kMaxTiles || tiles * stage > 160 * 1024) return false;
@@ -353,9 +406,19 @@ cudaError_t launch_attention_split(const void* q, int ld_q, int B, int n, int S,
     if (!tma_make_map_bf16(&tail, cache_layer, 3, dims, strides, box_tail, false, false, true)) return cudaErrorInvalidValue;
   }
   const int nq = (n + 15) / 16;
+  // Groups of warps for every tile: the queries by TMA, 700 cycles earlier in registers than by loads of four bytes, and a merge without
+  // loops (up to five partial results).  With fewer groups the loads overlap the wait for the tiles and the larger kernel costs
+  // (120 items, 43 rows on single CTAs: a block 36.4 -> 37.1 us).
+  if (cs == 1 && nk > 2 && nk <= kFewParts && (nq == 2 || nq == 3) && ld_q % 8 == 0 && ((uintptr_t)q & 15) == 0) {
+    if (dh == 64)
+      return nq == 2 ? launch_split<64, 2, true>(tm, tail, (const bf16*)q, ld_q, B, n, S, H, cs, nk, (uint16_t*)o, o_bf16, status, st)
+                     : launch_split<64, 3, true>(tm, tail, (const bf16*)q, ld_q, B, n, S, H, cs, nk, (uint16_t*)o, o_bf16, status, st);
+    return nq == 2 ? launch_split<80, 2, true>(tm, tail, (const bf16*)q, ld_q, B, n, S, H, cs, nk, (uint16_t*)o, o_bf16, status, st)
+                   : launch_split<80, 3, true>(tm, tail, (const bf16*)q, ld_q, B, n, S, H, cs, nk, (uint16_t*)o, o_bf16, status, st);
+  }
 #define MARCHE_SPLIT_CASE(DH_, NW_) \
   if (dh == DH_ && nq == NW_)       \
-    return launch_split<DH_, NW_>(tm, tail, (const bf16*)q, ld_q, B, n, S, H, cs, nk, (uint16_t*)o, o_bf16, status, st);
+    return launch_split<DH_, NW_, false>(tm, tail, (const bf16*)q, ld_q, B, n, S, H, cs, nk, (uint16_t*)o, o_bf16, status, st);
   MARCHE_SPLIT_CASE(64, 1) MARCHE_SPLIT_CASE(64, 2) MARCHE_SPLIT_CASE(64, 3) MARCHE_SPLIT_CASE(64, 4)
   MARCHE_SPLIT_CASE(80, 1) MARCHE_SPLIT_CASE(80, 2) MARCHE_SPLIT_CASE(80, 3) MARCHE_SPLIT_CASE(80, 4)
 #undef MARCHE_SPLIT_CASE

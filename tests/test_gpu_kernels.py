@@ -1000,3 +1000,27 @@ def test_few_rows_normalise_in_the_projection(operand, D, H, F, B, n):
     rel = 2e-4 if operand == "f16" else 1.6e-3
     assert rel_l2(got[0][0], got[1][0]) <= rel and rel_l2(got[0][1], got[1][1]) <= 8 * rel
     assert m.device_status() == 0
+
+
+@pytest.mark.parametrize("dh", [64, 80])
+@pytest.mark.parametrize("S", [193, 256, 257, 320])
+@pytest.mark.parametrize("n,ld_pad", [(17, 0), (32, 8), (33, 0), (48, 0), (43, 2)])
+def test_attention_a_group_of_warps_per_tile(dh, S, n, ld_pad):
+    """32 items, two or three groups of query rows over four or five key tiles: one CTA per item, a group of warps per tile, queries by TMA
+    (with a row stride of 2 elements more, by loads).  Bounds as in the test of the split over a cluster."""
+    H, B = 16, 2
+    D = H * dh
+    cfg, blocks, m = model_for("bf16", D, H, 128, S, B)
+    gen = torch.Generator(device="cuda").manual_seed(S + n + dh)
+    cache = torch.randn(2, B, S, D, generator=gen, device="cuda").to(torch.bfloat16)
+    ld = D + ld_pad
+    q = (torch.randn(B * n, ld, generator=gen, device="cuda") * 3.0).to(torch.bfloat16)
+    o = torch.full((B * n + 1, D), 7.0, dtype=torch.float16, device="cuda")
+    m.attention(q, ld, n, cache, None, None, o[:-1])
+    assert m.device_status() == 0 and (o[-1] == 7.0).all()
+    heads = lambda t: t.reshape(B, -1, H, dh).transpose(1, 2).float()
+    want = torch.softmax(heads(q[:, :D]) @ heads(cache[0]).transpose(2, 3) / math.sqrt(dh), -1) @ heads(cache[1])
+    assert (heads(o[:-1]) - want).norm() <= 8e-3 * want.norm() and (heads(o[:-1]) - want).abs().max() <= 3e-2
+    again = torch.zeros_like(o)
+    m.attention(q, ld, n, cache, None, None, again[:-1])
+    assert torch.equal(again[:-1], o[:-1])

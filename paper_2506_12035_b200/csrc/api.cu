@@ -6,6 +6,7 @@
 //   K3 attention over the whole cache (+ score partials at the scoring block, in the same
 //   kernel or in one of their own before it) -> K2 output projection (+residual) -> K1
 //   LayerNorm -> K2 fc1 (+GELU) -> K2 fc2 (+residual);
+// on up to 32 rows the projections after a LayerNorm do it themselves (K1 remains at block 0);
 // then once per step the fp32 row scatter into hidden_out and K4 (score reduction +
 // top-K).  Nothing here allocates device memory or synchronises, except where the
 // header says a call is synchronous.

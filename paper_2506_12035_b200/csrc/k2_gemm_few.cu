@@ -58,8 +58,8 @@ MARCHE_DEVINL void mma_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// Columns of a row and of a CTA's slice of it (LayerNorm), and the reciprocals that the statistics' merges need.
-struct NormShape { float cols, inv_cols, cols_cta, inv_warps; };
+// Columns of a CTA's slice of a row (LayerNorm), and the reciprocals that the statistics' merges need.
+struct NormShape { float inv_cols, cols_cta, inv_warps; };
 enum { ST_GEMM_FEW = 0x64 };
 
 // Grid: CS * N / (8 NT) * n_m CTAs (n_m groups of 16 rows); the CS CTAs of a cluster share a tile.  NORM: a is fp32 [M][lda], to be
@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 2)
 gemm_few_kernel(const void* __restrict__ a, int lda, int M, const uint16_t* __restrict__ w, const float* __restrict__ bias, int N,
                 int K, int epi, void* __restrict__ out, const KvScatter kv, const float* __restrict__ gamma,
                 const float* __restrict__ beta, float eps, const NormShape sh, int kbw, int n_m, int* __restrict__ status) {
-  static_assert(!NORM || CS > 1, "the statistics go through the cluster");
+  static_assert(!NORM || CS % 2 == 0, "the statistics go through the cluster");
   constexpr int cs = CS, pairs = NT * 64, own = pairs / cs;  // output pairs of the cluster's tile, of this CTA
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ __align__(8) uint64_t bars[2];                // statistics there, partial sums there
@@ -211,22 +211,30 @@ gemm_few_kernel(const void* __restrict__ a, int lda, int M, const uint16_t* __re
     asm volatile("cp.async.wait_group 1;" ::: "memory");   // gamma and beta (W is another group)
     __syncthreads();                                       // the warps' statistics, and everybody's gamma and beta
     cluster_wait();                                        // every CTA of the cluster has started
-    if (tid < kRows) {                                     // the CTA's share of a row, to all CTAs of the cluster
-      const float pivot = s_warp[tid].x;                   // (all counts are equal: sums around one of the means)
-      float s1 = 0.f, s2 = 0.f;
+    if (warp == 0) {                                       // the CTA's share of a row, to all CTAs of the cluster
+      // Two lanes a row, every other warp's part each.  Squared deviations are summed around the merged mean and not as a
+      // difference of sums: nothing cancels, and a deviation whose square overflows leaves infinity, i.e. a row of beta, as in
+      // the LayerNorm launch.
+      const int row = lane & 15, odd = lane >> 4;
+      const float pivot = s_warp[row].x;                   // (all counts are equal: the mean, around one of the means)
+      float s1 = 0.f, dev = 0.f;
 #pragma unroll
-      for (int v = 0; v < kMaxWarps; ++v)
-        if (v < warps) {
-          const float2 p = s_warp[v * kRows + tid];
-          const float d = p.x - pivot;
-          s1 += d;
-          s2 += fmaf(d * d, (float)kBlockK, p.y);
+      for (int v = 0; v < kMaxWarps; v += 2)
+        if (v + odd < warps) s1 += s_warp[(v + odd) * kRows + row].x - pivot;
+      s1 += __shfl_xor_sync(0xffffffffu, s1, 16);
+      const float mean = fmaf(s1, sh.inv_warps, pivot);
+#pragma unroll
+      for (int v = 0; v < kMaxWarps; v += 2)
+        if (v + odd < warps) {
+          const float2 p = s_warp[(v + odd) * kRows + row];
+          const float d = p.x - mean;
+          dev += fmaf(d * d, (float)kBlockK, p.y);
         }
-      s1 *= sh.inv_warps;
-      const float mean = pivot + s1, dev = fmaxf(fmaf(-s1 * s1, sh.cols_cta, s2), 0.f);
-      const uint32_t dst = ptx::smem_u32(s_cta + rank * kRows + tid);
+      dev += __shfl_xor_sync(0xffffffffu, dev, 16);
+      const uint32_t dst = ptx::smem_u32(s_cta + rank * kRows + row);
 #pragma unroll
-      for (int c = 0; c < cs; ++c) st_async_v2(ptx::mapa(dst, (uint32_t)c), mean, dev, ptx::mapa(bar_stats, (uint32_t)c));
+      for (int c = 0; c < cs; c += 2)
+        st_async_v2(ptx::mapa(dst, (uint32_t)(c + odd)), mean, dev, ptx::mapa(bar_stats, (uint32_t)(c + odd)));
     }
     __syncwarp();                                          // (lanes that wait must not keep those that send from running)
     const float* gm = s_gamma + warp * kBlockK + t4 * 8;
@@ -237,18 +245,18 @@ gemm_few_kernel(const void* __restrict__ a, int lda, int M, const uint16_t* __re
     uint32_t u[2][4];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const float2* p = s_cta + 8 * h + g;
-      const float pivot = p[0].x;
-      float s1 = 0.f, s2 = 0.f;
+      float2 q[cs];                                        // the CTAs' slices, merged in pairs
 #pragma unroll
-      for (int c = 0; c < cs; ++c) {
-        const float2 q = p[c * kRows];
-        const float d = q.x - pivot;
-        s1 += d;
-        s2 += fmaf(d * d, sh.cols_cta, q.y);
-      }
-      s1 *= 1.0f / cs;
-      const float mean = pivot + s1, rstd = rsqrtf(fmaxf(fmaf(-s1 * s1, sh.cols, s2), 0.f) * sh.inv_cols + eps);
+      for (int c = 0; c < cs; ++c) q[c] = s_cta[c * kRows + 8 * h + g];
+#pragma unroll
+      for (int n = 1; n < cs; n *= 2)
+#pragma unroll
+        for (int c = 0; c + n < cs; c += 2 * n) {
+          const float d = q[c + n].x - q[c].x;
+          q[c].x = fmaf(d, 0.5f, q[c].x);
+          q[c].y = fmaf(d * d, 0.5f * n * sh.cols_cta, q[c].y + q[c + n].y);
+        }
+      const float mean = q[0].x, rstd = rsqrtf(q[0].y * sh.inv_cols + eps);
       const float* y = x[h];
       u[h][0] = pack_a16x2((y[0] - mean) * rstd * g0.x + b0.x, (y[1] - mean) * rstd * g0.y + b0.y, BF);
       u[h][1] = pack_a16x2((y[2] - mean) * rstd * g0.z + b0.z, (y[3] - mean) * rstd * g0.w + b0.w, BF);
@@ -370,7 +378,7 @@ cudaError_t launch_one(const Plan& p, const void* a, int lda, int M, const void*
   if (e == cudaSuccess) e = prefer_shared_memory(kernel, carved);
   if (e != cudaSuccess) return e;
   const float cta_cols = (float)(p.warps * kBlockK);
-  const NormShape sh = {(float)K, 1.0f / K, cta_cols, 1.0f / p.warps};
+  const NormShape sh = {1.0f / K, cta_cols, 1.0f / p.warps};
   return launch_pdl_cluster(kernel, dim3(p.ctas), dim3(p.warps * 32), p.smem, CS, st,
                             a, lda, M, (const uint16_t*)w, bias, N, K, epi, out, kv, gamma, beta, eps, sh, p.kbw, p.n_m, status);
 }

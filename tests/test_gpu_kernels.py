@@ -1024,3 +1024,38 @@ def test_attention_a_group_of_warps_per_tile(dh, S, n, ld_pad):
     again = torch.zeros_like(o)
     m.attention(q, ld, n, cache, None, None, again[:-1])
     assert torch.equal(again[:-1], o[:-1])
+
+
+@pytest.mark.parametrize("value", [1e20, -3e24])
+@pytest.mark.parametrize("D,H,F", [(256, 4, 512), (768, 12, 768), (1280, 16, 1280)])
+def test_few_rows_whose_squares_overflow(value, D, H, F):
+    """Rows with one value whose squared deviation is beyond fp32: the variance is infinite, the normalised row is beta, in the
+    projection as in the LayerNorm launch.  The value stands in another warp's columns for every row (first, last, both sides of a
+    slice's end).  Bounds on the later blocks' K and V: beta of unit size rounds the same way on both sides, weights of 0.02."""
+    import synth
+    from helpers import make_model
+    cfg = synth.CONFIGS["mar_b"].replace(L=2, E=0, D=D, H=H, F=F, B=2, S=40, n_buffer=8)
+    blocks = synth.make_weights(cfg)
+    rng = np.random.default_rng(D)
+    for blk in blocks:
+        blk["ln1_b"], blk["ln2_b"] = (rng.standard_normal(D).astype(np.float32) for _ in range(2))
+    m = make_model(cfg, blocks)
+    hidden_np = rng.standard_normal((cfg.B, cfg.S, D)).astype(np.float32)
+    cols = [0, 31, 32, D // 2 - 1, D // 2, D - 33, D - 32, D - 1]
+    act = np.stack([rng.permutation(cfg.S)[:8] for _ in range(cfg.B)])
+    for b in range(cfg.B):
+        hidden_np[b, act[b], cols] = value
+    hidden, act_d = dev(hidden_np), idx_dev(act)
+    got = []
+    for hook in ((), ("gather_layernorm",)):
+        m.debug_repeat_classes(hook)
+        cache, out, ws = m.alloc_cache(), torch.zeros(cfg.B, cfg.S, D, device="cuda"), m.alloc_workspace(cfg.S)
+        m.init_cache(cache)
+        m.full_step(hidden, cache, act_d, None, 0.0, out, None, ws)
+        m.step(hidden, cache, act_d, act_d, None, 0.0, out, None, ws)
+        kv = host(cache[1])                                              # [2][B][S][D] of the block behind a normalising projection
+        got.append(np.stack([kv[:, b, act[b]] for b in range(cfg.B)]))
+    m.debug_repeat_classes(())
+    assert np.isfinite(got[1]).all() and np.abs(got[1]).max() > 0.1
+    assert max_abs(got[0], got[1]) <= 2.0 ** -7 * np.abs(got[1]).max()   # one bf16 step
+    assert m.device_status() == 0

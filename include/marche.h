@@ -478,8 +478,9 @@ int marche_device_status(const marche_ctx* ctx);
 int marche_check_status(marche_ctx* ctx, marche_stream stream);
 /* Test hook for that path: enqueues a kernel of two one-warp CTAs (a cluster) in which one thread uses the
  * library's bounded wait on a barrier that nothing arrives on.  After `limit_cycles` SM clock cycles (1 ..
- * 2e9; a million is about half a millisecond) the wait gives up, the cluster is told, the other CTA sets the
- * status word and the kernel returns; nothing traps and the context stays usable.  Asynchronous. */
+ * 2e9; a million is about half a millisecond) the wait gives up and the cluster is told; that ends the wait of the other
+ * CTA (for bytes that now are not sent, 2e8 cycles longer), which sets the status word; the kernel returns, nothing traps and
+ * the context stays usable.  Asynchronous. */
 int marche_debug_bounded_wait(marche_ctx* ctx, long long limit_cycles, marche_stream stream);
 /* Number of kernels this context has launched so far. */
 unsigned long long marche_launch_count(const marche_ctx* ctx);

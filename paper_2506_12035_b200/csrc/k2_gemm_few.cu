@@ -34,11 +34,6 @@ constexpr int kSmemMax = 110 * 1024;       // two CTAs per SM, this launch's and
 
 MARCHE_DEVINL void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 MARCHE_DEVINL void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
-// To another CTA's shared memory, the bytes counted by a barrier there: no fence and no barrier of the cluster.
-MARCHE_DEVINL void st_async_v2(uint32_t addr, float a, float b, uint32_t bar) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(a), "f"(b), "r"(bar)
-               : "memory");
-}
 MARCHE_DEVINL void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
@@ -234,7 +229,7 @@ gemm_few_kernel(const void* __restrict__ a, int lda, int M, const uint16_t* __re
       const uint32_t dst = ptx::smem_u32(s_cta + rank * kRows + row);
 #pragma unroll
       for (int c = 0; c < cs; c += 2)
-        st_async_v2(ptx::mapa(dst, (uint32_t)(c + odd)), mean, dev, ptx::mapa(bar_stats, (uint32_t)(c + odd)));
+        ptx::st_async_v2(ptx::mapa(dst, (uint32_t)(c + odd)), mean, dev, ptx::mapa(bar_stats, (uint32_t)(c + odd)));
     }
     __syncwarp();                                          // (lanes that wait must not keep those that send from running)
     const float* gm = s_gamma + warp * kBlockK + t4 * 8;
@@ -282,6 +277,9 @@ gemm_few_kernel(const void* __restrict__ a, int lda, int M, const uint16_t* __re
       dst[nt * 64 + 32] = make_float2(acc[nt][2], acc[nt][3]);
     }
   }
+  // A CTA whose statistics did not come sends no sums and tells the cluster, all of which waits for them: nobody stores anything.
+  // (The others are still there for the same reason.)
+  if (NORM && !ok) ptx::cluster_raise(ptx::smem_u32(abort_flags), cs);
   __syncthreads();
   auto sum_warps = [&](int q) {
     const uint8_t* p = smem + q * 8;
@@ -298,10 +296,10 @@ gemm_few_kernel(const void* __restrict__ a, int lda, int M, const uint16_t* __re
   if (cs > 1) {
     if (!NORM) cluster_wait();                             // every CTA of the cluster has started
     const uint32_t dst = ptx::smem_u32(recv + rank * own);
-    for (int q = tid; q < pairs; q += threads) {
+    for (int q = NORM && *abort_flag ? pairs : tid; q < pairs; q += threads) {
       const float2 f = sum_warps(q);
       const uint32_t o = (uint32_t)q / own;
-      st_async_v2(ptx::mapa(dst + (uint32_t)q % own * 8u, o), f.x, f.y, ptx::mapa(bar_sums, o));
+      ptx::st_async_v2(ptx::mapa(dst + (uint32_t)q % own * 8u, o), f.x, f.y, ptx::mapa(bar_sums, o));
     }
     __syncwarp();
     ok = ptx::mbar_wait_cluster(bar_sums, 0, abort_flag) && ok;

@@ -217,6 +217,11 @@ MARCHE_DEVINL uint32_t mapa(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
+// To another CTA's shared memory, the bytes counted by a barrier there: no fence and no barrier of the cluster.
+MARCHE_DEVINL void st_async_v2(uint32_t addr, float a, float b, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(a), "f"(b), "r"(bar)
+               : "memory");
+}
 // Raises a flag (a word at the same shared address in every CTA) in all CTAs of a cluster of `n`, which see it after the next
 // cluster barrier, or earlier.
 MARCHE_DEVINL void cluster_raise(uint32_t flag, int n) {

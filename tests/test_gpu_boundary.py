@@ -34,17 +34,22 @@ def _one_step(m, cfg, hidden, A, G, ratio=0.1):
 def test_bounded_wait_runs_out_and_is_reported_as_timeout():
     """A wait on a barrier nothing arrives on gives up after its cycle limit: the kernel returns, the
     status word is set, the synchronous calls answer MARCHE_ETIMEOUT, and after clearing the word the
-    context computes a correct step again (nothing trapped, nothing hung)."""
+    context computes a correct step again (nothing trapped, nothing hung).  The other CTA of the cluster waits for bytes that
+    the one that gave up does not send: it is told, and does not wait for its own limit (a tenth of a second more)."""
     cfg = synth.CONFIGS["tiny"].replace(dtype="bf16", B=4)
     blocks = synth.make_weights(cfg)
     m = make_model(cfg, blocks)
     assert m.device_status() == 0
     m.check_status()                                                   # clean: no exception
+    start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    start.record()
     m.debug_bounded_wait(1_000_000)                                    # about half a millisecond
+    end.record()
     with pytest.raises(MarcheError) as e:
         m.check_status()
     assert e.value.code == -7
-    assert m.device_status() == 0x71                                   # written by the CTA that did not wait: it was told
+    assert m.device_status() == 0x71                                   # written by the CTA that was told
+    assert start.elapsed_time(end) < 50.0                              # its own limit: over 100 ms
     act = np.array([[1, 2, 3, 4]] * cfg.B, np.int32)
     with pytest.raises(MarcheError) as e:                              # the other synchronous calls report it too
         m.validate_indices(idx_dev(act), idx_dev(act[:, :2]), None)

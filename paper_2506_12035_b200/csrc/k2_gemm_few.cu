@@ -31,6 +31,7 @@ constexpr int kBlockK = 32;                // K block of a warp: four lanes of a
 constexpr int kMaxWarps = 16;              // all along K; two CTAs of 64 registers a thread per SM
 constexpr int kRows = 16;                  // of a tile
 constexpr int kSmemMax = 110 * 1024;       // two CTAs per SM, this launch's and the next one's
+constexpr int kSmemSm = 228 * 1024;        // of an SM, 1 KB of it for every CTA
 
 MARCHE_DEVINL void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 MARCHE_DEVINL void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
@@ -390,13 +391,27 @@ cudaError_t launch_any(const Plan& p, bool norm, Args... args) {
 
 }  // namespace
 
-// One group of rows always (a block of a step at 16 rows: widths 768, 1024, 1280 22.8 -> 17.3, 25.6 -> 20.0, 30.1 -> 26.4 us against the
-// split-K kernel with LayerNorm launches), two where the launch has no more warps than one CTA of 16 per SM (32 rows: width 768, 192
-// CTAs of 12 warps 23.9 -> 20.4; width 1024, 192 CTAs of 16 26.6 -> 27.0; width 1280, 640 CTAs 31.8 -> 43.6), three never (48 rows, width
-// 768 25.5 -> 26.2).
+// One group of rows where the whole launch runs at once: 32 warps of 64 registers a thread fit an SM, and their shared memory has to.
+// (Beyond, us, split-K and this kernel: 16 x 5120 x 1280 4.8 and 8.1, 16 x 6144 x 1536 5.5 and 9.7, 16 x 2560 x 4096 6.4 and 10.9; with the
+// LayerNorm, a block of a step of 16 rows: width 1792, MLP 7168, 39.4 with LayerNorm launches, 42.9 without.  CTAs of 16 warps, which fill
+// the SM, may be a third more: the QKV projection of width 2048 is level, 37.2 and 37.8 at MLP 4096, 49.9 and 47.8 in front of fc1 at 8192.)
+// And not where a warp has many K blocks, so that every CTA reads long rows for its 16 columns: 16 x 2048 x 2048 3.7 and 4.3 (8 rows 5 %
+// slower, one row level), 16 x 1536 x 6144 6.1 and 7.2, 1 row 6.1 and 6.3; with few columns the few CTAs are fed anyway (16 x 1024 x 6144
+// 5.3 either way), and with more the split-K kernel's clusters of eight do not all fit (16 x 2048 x 6144 11.1 and 8.0, 16 x 4608 x 2048
+// 9.5 and 6.7).
+// Two groups of rows where the launch has no more warps than one CTA of 16 per SM (a block of a step, 32 rows: width 768, 192 CTAs of 12
+// warps 24.0 -> 22.3; width 1024, 192 CTAs of 16 26.6 -> 27.0; width 1280, 640 CTAs 31.8 -> 43.6), and without the LayerNorm only for up
+// to 1024 columns or a K of up to 1024 (24 rows: width 1280, MLP 2560, 27.9 and 30.6; width 1152, MLP 4608, 29.8 and 30.2; width 1024
+// 25.1 and 25.0 to 25.6, by rows); three never (48 rows, width 768 25.5 -> 26.2).
 bool gemm_few_wins(int M, int N, int K, bool norm) {
   Plan p;
-  return M <= 2 * kRows && make_plan(M, N, K, norm, &p) && (M <= kRows || p.ctas * p.warps <= kMaxWarps * device_sm_count());
+  if (M > 2 * kRows || !make_plan(M, N, K, norm, &p)) return false;
+  if (M > kRows) return p.ctas * p.warps <= kMaxWarps * device_sm_count() && (norm || N <= 1024 || K <= 1024);
+  const int by_smem = kSmemSm / ((int)p.smem + 1024), by_regs = 2 * kMaxWarps / p.warps;
+  const int fit = device_sm_count() * (by_smem < by_regs ? by_smem : by_regs);
+  if (p.ctas > (norm && p.warps == kMaxWarps ? fit * 4 / 3 : fit)) return false;
+  if (norm || N <= 1024) return true;
+  return p.cs == 1 ? p.kbw <= 3 || M <= kRows / 2 || N >= 4096 : p.kbw <= 5 || N >= 2048;
 }
 
 cudaError_t launch_gemm_few(const void* a, int lda, int M, const void* w, const float* bias, int N, int K, int epilogue, void* out,

@@ -63,3 +63,21 @@ def test_scores_in_a_launch_of_their_own(lib, n, n_new, S, dh, items, want):
     wins = lib._ZN6marche21attention_scores_winsEiiiii
     wins.restype = ctypes.c_bool
     assert wins(n, n_new, S, dh, items) is want
+
+
+@pytest.mark.parametrize("M,N,K,norm,want", [
+    # with the LayerNorm: as many CTAs as run at once, a third more of 16 warps
+    (16, 2304, 768, 1, True), (16, 3072, 768, 1, True), (16, 3840, 1280, 1, True), (1, 5120, 1280, 1, True), (16, 4608, 1536, 1, True),
+    (16, 6144, 2048, 1, True), (16, 4992, 1664, 1, False), (16, 5760, 1920, 1, False), (1, 7168, 1792, 1, False), (16, 8192, 2048, 1, False),
+    (16, 4096, 2048, 1, True),
+    # without
+    (16, 4608, 1536, 0, True), (16, 4864, 1536, 0, False), (1, 5120, 1280, 0, False), (1, 8192, 1024, 0, False), (8, 2560, 4096, 0, False),
+    (8, 2048, 2048, 0, True), (9, 2048, 2048, 0, False), (16, 1024, 2048, 0, True), (16, 4608, 2048, 0, True), (16, 1280, 5120, 0, True),
+    (1, 1536, 6144, 0, False), (16, 2048, 6144, 0, True), (16, 1024, 6144, 0, True),
+    # two groups of rows, three
+    (32, 768, 768, 0, True), (32, 3072, 1024, 1, False), (33, 768, 768, 0, False), (24, 1280, 2560, 0, False), (17, 1152, 1152, 0, False),
+    (24, 1280, 768, 0, True), (32, 1024, 2048, 0, True)])
+def test_projections_of_a_handful_of_rows(lib, M, N, K, norm, want):
+    wins = lib._ZN6marche13gemm_few_winsEiiib
+    wins.restype = ctypes.c_bool
+    assert wins(M, N, K, ctypes.c_bool(norm)) is want

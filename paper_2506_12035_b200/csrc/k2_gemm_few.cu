@@ -281,7 +281,9 @@ gemm_few_kernel(const void* __restrict__ a, int lda, int M, const uint16_t* __re
   // A CTA whose statistics did not come sends no sums and tells the cluster, all of which waits for them: nobody stores anything.
   // (The others are still there for the same reason.)
   if (NORM && !ok) ptx::cluster_raise(ptx::smem_u32(abort_flags), cs);
-  __syncthreads();
+  bool silent = false;
+  if (NORM) silent = __syncthreads_or(!ok);
+  else __syncthreads();
   auto sum_warps = [&](int q) {
     const uint8_t* p = smem + q * 8;
     float2 f = *reinterpret_cast<const float2*>(p);
@@ -297,7 +299,7 @@ gemm_few_kernel(const void* __restrict__ a, int lda, int M, const uint16_t* __re
   if (cs > 1) {
     if (!NORM) cluster_wait();                             // every CTA of the cluster has started
     const uint32_t dst = ptx::smem_u32(recv + rank * own);
-    for (int q = NORM && *abort_flag ? pairs : tid; q < pairs; q += threads) {
+    for (int q = silent ? pairs : tid; q < pairs; q += threads) {
       const float2 f = sum_warps(q);
       const uint32_t o = (uint32_t)q / own;
       ptx::st_async_v2(ptx::mapa(dst + (uint32_t)q % own * 8u, o), f.x, f.y, ptx::mapa(bar_sums, o));

@@ -567,24 +567,40 @@ bool attention_tc_stream_wins(int n, int S, int dh, int items, int min_rows) {
   return S > 4 * KT && (rounds == 1 || 4 * items >= 3 * rounds * streams);
 }
 
+// Streams per CTA.  No more units than SMs: a CTA has one, and a CTA of one stream is smaller and starts sooner.  Head_dim 80: 144
+// items, S 100, 80 rows 5.4 and 5.8 us; not over longer sequences.
+// Head_dim 64: four streams take more units at a time than three, each more slowly, since their weights share the logits' columns.  That
+// counts where it saves a round of two (192 items, S 320, 320 rows: 576 units on 444 or 592 streams 16.0 and 14.4 us), and over long
+// sequences, where the tiles come from HBM and a fourth stream's are on their way meanwhile, also a round of three (64 x 16 items, us on
+// three and four: S 640, 48 rows 38.7 and 37.0; S 1088, 64 rows 59.8 and 57.1, 116 rows 66.7 and 63.8; S 2048, 80 rows 110 and 104; 448
+// items, S 1536, 200 rows 83.0 and 78.0; 116 rows over S 448 32.4 and 32.6, S 320 25.7 and 26.4), or of four behind a short last tile
+// (S 1088, 2048 items, 151 rows 205 and 192, 800 items 83.5 and 81.2, with 200 rows 88.4 and 90.0; S 2048, 800 items, 151 rows 150 and 141).
+// One in five costs (S 1088, 1024 items, 151 rows 98 and 104).
+int attention_tc_streams(int n, int S, int dh, int items) {
+  const long units = (long)items * ((n + QT - 1) / QT);
+  const int sms = device_sm_count();
+  if (units <= sms && (dh == 64 || S <= 2 * KT)) return 1;
+  if (dh != 64) return kStreams;
+  const long r3 = (units + kStreams * sms - 1) / (kStreams * sms), r4 = (units + 4L * sms - 1) / (4L * sms);
+  const bool short_tile = n > QT && n % QT > 0 && n % QT <= 32;
+  return r3 >= 2 * r4 || (S >= 8 * KT && 2 * r3 >= 3 * r4) || (S >= 14 * KT && short_tile && 3 * r3 >= 4 * r4) ? 4 : kStreams;
+}
+
 cudaError_t launch_attention_tc_stream(const void* q, int ld_q, int B, int n, int S, int H, int dh,
                                        const void* cache_layer, void* o, bool o_bf16, int* status, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   if ((dh != 64 && dh != 80) || ld_q % 8 || ((uintptr_t)q & 15) || ((uintptr_t)cache_layer & 15) || ((uintptr_t)o & 15) || S > 2048)
     return cudaErrorInvalidValue;
-  const long units = (long)B * H * ((n + QT - 1) / QT);
-  const int sms = device_sm_count();
-  // No more units than SMs: a CTA has one, and a CTA of one stream is smaller and starts sooner.  Head_dim 80: 144 items, S 100,
-  // 80 rows 5.4 and 5.8 us; not over longer sequences.
-  if (units <= sms && (dh == 64 || S <= 2 * KT))
-    return dh == 64 ? launch_stream<64, 1>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st)
-                    : launch_stream<80, 1>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
-  // Head_dim 64: four streams take more units at a time than three, each more slowly; where all units run at once that counts
-  // (192 items, S 320, 320 rows: 576 units on 444 or 592 streams 16.0 and 14.4 us).
-  if (dh == 64 && units > (long)kStreams * sms && units <= 4L * sms)
-    return launch_stream<64, 4>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
-  return dh == 64 ? launch_stream<64, kStreams>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st)
-                  : launch_stream<80, kStreams>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
+  switch (attention_tc_streams(n, S, dh, B * H)) {
+    case 1:
+      return dh == 64 ? launch_stream<64, 1>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st)
+                      : launch_stream<80, 1>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
+    case 4:
+      return launch_stream<64, 4>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
+    default:
+      return dh == 64 ? launch_stream<64, kStreams>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st)
+                      : launch_stream<80, kStreams>(q, ld_q, B, n, S, H, cache_layer, o, o_bf16, status, st);
+  }
 }
 
 }  // namespace marche

@@ -100,8 +100,8 @@ cudaError_t launch_gemm_splitk(const void* a, int lda, int M, const void* w, con
                                const KvScatter* kv_scatter = nullptr);
 
 // K2 for up to 32 rows on mma.sync.  Same operand rules.  gamma (and beta) given: a is fp32 [M][lda] and its rows are normalised
-// first (epilogues 0, 2 and 4).  Weights, bias, gamma, beta and the scatter's token indices are read ahead of the dependency wait: they
-// were complete before the preceding launch.
+// first (epilogues 0, 2 and 4).  Weights, bias, gamma and beta are read ahead of the dependency wait: they were complete before the
+// preceding launch.  (The scatter's token indices, which kernels write, are read behind it.)
 bool gemm_few_wins(int M, int N, int K, bool norm);
 cudaError_t launch_gemm_few(const void* a, int lda, int M, const void* w, const float* bias, int N, int K, int epilogue, void* out,
                             bool a_bf16, int* status, cudaStream_t st, const KvScatter* kv_scatter = nullptr, const float* gamma = nullptr,
@@ -146,6 +146,7 @@ cudaError_t launch_attention_tcgen05(const void* q, int ld_q, int B, int n, int 
 // K3 on tcgen05, single pass with online softmax, persistent over (sample, head) items, P kept in tensor
 // memory (head_dim 64 or 80, no relevance scores).  Same alignment rules as launch_attention_tcgen05, o 16-byte aligned.
 bool attention_tc_stream_wins(int n, int S, int dh, int items, int min_rows);
+int attention_tc_streams(int n, int S, int dh, int items);   // streams per CTA
 cudaError_t launch_attention_tc_stream(const void* q, int ld_q, int B, int n, int S, int H, int dh,
                                        const void* cache_layer, void* o, bool o_bf16, int* status, cudaStream_t st);
 

@@ -81,3 +81,17 @@ def test_projections_of_a_handful_of_rows(lib, M, N, K, norm, want):
     wins = lib._ZN6marche13gemm_few_winsEiiib
     wins.restype = ctypes.c_bool
     assert wins(M, N, K, ctypes.c_bool(norm)) is want
+
+
+@pytest.mark.parametrize("n,S,dh,items,want", [
+    # one unit per CTA; one round of four for two of three
+    (116, 1088, 64, 148, 1), (116, 1088, 64, 149, 3), (80, 100, 80, 144, 1), (80, 129, 80, 144, 3), (64, 100, 64, 444, 3), (64, 100, 64, 445, 4),
+    (320, 320, 64, 192, 4), (64, 100, 64, 593, 3), (320, 320, 80, 192, 3),
+    # two rounds for three over long sequences
+    (116, 511, 64, 1024, 3), (116, 512, 64, 1024, 4), (200, 1088, 64, 448, 4), (128, 2048, 64, 889, 4), (128, 2048, 64, 888, 3), (128, 2048, 64, 1185, 3),
+    # three rounds for four, seven for ten: behind a short last tile
+    (151, 1088, 64, 800, 4), (161, 1088, 64, 800, 3), (160, 1088, 64, 800, 4), (256, 1088, 64, 800, 3), (151, 895, 64, 800, 3), (151, 1088, 64, 2048, 4),
+    (23, 1088, 64, 1600, 3), (151, 1088, 64, 1024, 3)])
+def test_streams_per_cta(lib, n, S, dh, items, want):
+    streams = lib._ZN6marche20attention_tc_streamsEiiii
+    assert streams(n, S, dh, items) == want

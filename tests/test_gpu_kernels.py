@@ -1059,3 +1059,24 @@ def test_few_rows_whose_squares_overflow(value, D, H, F):
     assert np.isfinite(got[1]).all() and np.abs(got[1]).max() > 0.1
     assert max_abs(got[0], got[1]) <= 2.0 ** -7 * np.abs(got[1]).max()   # one bf16 step
     assert m.device_status() == 0
+
+
+@pytest.mark.parametrize("items,S,n", [(1024, 512, 33), (1024, 577, 128), (448, 512, 129), (448, 700, 256), (800, 896, 160), (460, 1088, 260)])
+def test_attention_four_streams_over_several_rounds(items, S, n):
+    """Four streams per CTA, whose weights share the logits' columns, over two rounds and more, one to three query tiles per item, every
+    unit taken once.  Bounds as in the test above."""
+    H, dh = 4, 64
+    B, D = items // H, H * dh
+    cfg, blocks, m = model_for("bf16", D, H, 128, S, B)
+    gen = torch.Generator(device="cuda").manual_seed(B + S + n)
+    cache = torch.randn(2, B, S, D, generator=gen, device="cuda").to(torch.bfloat16)
+    q = (torch.randn(B * n, D, generator=gen, device="cuda") * 3.0).to(torch.bfloat16)
+    o = torch.full((B * n + 1, D), 7.0, dtype=torch.float16, device="cuda")
+    m.attention(q, D, n, cache, None, None, o[:-1])
+    assert m.device_status() == 0 and (o[-1] == 7.0).all()
+    heads = lambda t: t.view(-1, t.shape[-2], H, dh).transpose(1, 2).float()
+    for b in range(0, B, 16):                                            # (the logits of all samples would be gigabytes)
+        q_b, k_b, v_b = q.view(B, n, D)[b:b + 16], cache[0, b:b + 16], cache[1, b:b + 16]
+        want = torch.softmax(heads(q_b) @ heads(k_b).transpose(2, 3) / math.sqrt(dh), -1) @ heads(v_b)
+        got = heads(o[:-1].view(B, n, D)[b:b + 16])
+        assert (got - want).norm() <= 8e-3 * want.norm() and (got - want).abs().max() <= 3e-2

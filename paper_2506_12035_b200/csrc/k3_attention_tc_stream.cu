@@ -514,6 +514,23 @@ attention_tc_stream_kernel(const __grid_constant__ CUtensorMap tmap_kv, const __
   }
 }
 
+}  // namespace
+
+// How the units of a launch are dealt (Deal).  A CTA's next unit is grid + rotate units on, a stream's NS (grid + rotate) + rotate_turn:
+// neither a multiple of an item's tiles.
+// Items of one tile have no tiles to mix: there the units of the last turn should go to the CTAs that started first, as long as there are
+// few turns (head_dim 80, 448 items, 80 rows, S 100 11.6 and 10.9 us, S 320 18.8 and 18.2; head_dim 64, 600 items, 116 rows, S 256 16.8
+// and 15.8); over more than two turns of the streams rotation spreads the CTAs' reads (head_dim 80, 2048 items, 64 rows, S 1088 132 and 137).
+int attention_tc_rotation(long units, int n_qt, int grid, int streams, int* rotate_turn) {
+  *rotate_turn = 0;
+  if (units <= (n_qt > 1 ? 1L : 2L) * streams * grid) return 0;
+  const int rotate = n_qt > 1 && (grid + 1) % n_qt == 0 ? 2 : 1;
+  *rotate_turn = n_qt > 1 && streams * (grid + rotate) % n_qt == 0 ? 1 : 0;
+  return rotate;
+}
+
+namespace {
+
 template <int DH, int NS>
 cudaError_t launch_stream(const void* q, int ld_q, int B, int n, int S, int H, const void* cache_layer, void* o, bool o_bf16,
                           int* status, cudaStream_t st) {
@@ -538,10 +555,8 @@ cudaError_t launch_stream(const void* q, int ld_q, int B, int n, int S, int H, c
   const int sms = device_sm_count();
   const long units = (long)B * H * ((n + QT - 1) / QT);
   const int grid = units < sms ? (int)units : sms, n_qt = (n + QT - 1) / QT;
-  // a CTA's next unit is grid + rotate units on, a stream's NS (grid + rotate) + rotate_turn: neither a multiple of an item's tiles
-  const bool turns = units > (long)NS * grid;
-  const int rotate = turns ? (n_qt > 1 && (grid + 1) % n_qt == 0 ? 2 : 1) : 0;
-  const int rotate_turn = turns && n_qt > 1 && NS * (grid + rotate) % n_qt == 0 ? 1 : 0;
+  int rotate_turn;
+  const int rotate = attention_tc_rotation(units, n_qt, grid, NS, &rotate_turn);
   return launch_pdl(attention_tc_stream_kernel<DH, NS>, dim3(grid), dim3(C::THREADS), (size_t)C::SMEM_BYTES, st, tkv, tq, tkv_tail,
                     tq_tail, n, S, H, B, (uint16_t*)o, o_bf16 ? 1 : 0, status, rotate, rotate_turn);
 }

@@ -147,6 +147,7 @@ cudaError_t launch_attention_tcgen05(const void* q, int ld_q, int B, int n, int 
 // memory (head_dim 64 or 80, no relevance scores).  Same alignment rules as launch_attention_tcgen05, o 16-byte aligned.
 bool attention_tc_stream_wins(int n, int S, int dh, int items, int min_rows);
 int attention_tc_streams(int n, int S, int dh, int items);   // streams per CTA
+int attention_tc_rotation(long units, int n_qt, int grid, int streams, int* rotate_turn);
 cudaError_t launch_attention_tc_stream(const void* q, int ld_q, int B, int n, int S, int H, int dh,
                                        const void* cache_layer, void* o, bool o_bf16, int* status, cudaStream_t st);
 

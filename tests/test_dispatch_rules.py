@@ -95,3 +95,27 @@ def test_projections_of_a_handful_of_rows(lib, M, N, K, norm, want):
 def test_streams_per_cta(lib, n, S, dh, items, want):
     streams = lib._ZN6marche20attention_tc_streamsEiiii
     assert streams(n, S, dh, items) == want
+
+
+@pytest.mark.parametrize("streams", [3, 4])
+@pytest.mark.parametrize("items,n_qt", [(444, 1), (448, 1), (592, 1), (888, 1), (1184, 1), (2048, 1), (300, 3), (448, 2), (1024, 2), (2048, 2), (149, 9), (2048, 3),
+                                        (512, 149)])
+def test_units_are_dealt_once_and_evenly(lib, streams, items, n_qt):
+    """Every unit to one CTA, as many to each but for one; no stream of many units gets tiles of one kind only.  Items of one tile
+    stay in the CTAs' order, the last turn's on the first CTAs, up to two turns of the streams."""
+    grid, units = 148, items * n_qt
+    deal, turn = lib._ZN6marche21attention_tc_rotationEliiiPi, ctypes.c_int()
+    rotate = deal(ctypes.c_long(units), n_qt, grid, streams, ctypes.byref(turn))
+    if n_qt == 1:
+        assert (rotate, turn.value) == ((0, 0) if units <= 2 * streams * grid else (1, 0))
+    taken, kinds = set(), {}
+    for k in range((units + grid - 1) // grid):
+        for cta in range(grid):
+            i = k * grid + (cta + k * rotate + k // streams * turn.value) % grid
+            if i < units:
+                assert i not in taken
+                taken.add(i)
+                kinds.setdefault((cta, k % streams), []).append(i % n_qt)
+    assert len(taken) == units
+    if 1 < n_qt < 9 and units >= 3 * streams * grid:
+        assert all(len(set(v)) > 1 for v in kinds.values())

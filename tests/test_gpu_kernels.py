@@ -451,8 +451,11 @@ def test_validate_indices():
 def test_linear_few_rows_split_k(dtype, M, N, K):
     """Row counts at the edges of the A tile, every tile width and cluster size of the split-K kernel, K ranges that do
     not divide evenly (5, 7, 40 blocks over 4, 4, 8 CTAs).  Products of unit size: |acc + bias| stays below 8, where
-    half a bf16 step is 0.016 (limit 0.02 with the fp32 sum), and an fp32 sum of K terms errs by sqrt(K) 2^-24."""
+    half a bf16 step is 0.016 (limit 0.02 with the fp32 sum), and an fp32 sum of K terms errs by sqrt(K) 2^-24.
+    (Asked for by name: up to 32 rows run on another kernel by themselves.)"""
+    from paper_2506_12035_b200 import binding
     cfg, blocks, m = model_for(dtype, 256, 4, 1024, 68, 2)
+    m.set_tuning(gemm_kernel=binding.GEMM_SINGLE)
     rng = np.random.default_rng(M + N + K)
     a = rng.standard_normal((M, K)).astype(np.float32)
     w = (rng.standard_normal((N, K)) / math.sqrt(K)).astype(np.float32)
@@ -827,7 +830,7 @@ def test_attention_scores_of_the_generating_rows(dh, H, B, S, n, nG):
 @pytest.mark.parametrize("B,S,n", [(1, 1, 1), (2, 65, 33), (3, 320, 70), (2, 128, 128), (60, 130, 129), (2, 1088, 150), (25, 577, 300)])
 def test_attention_single_pass_streams(dh, H, B, S, n):
     """The single-pass tcgen05 kernel at both head sizes: query tiles on one to four lane quarters (alone and behind full
-    ones), units dealt one by one (few) and by items (more than run at once), ragged keys, row maxima that keep growing."""
+    ones), fewer and more units than run at once, ragged keys, row maxima that keep growing."""
     from paper_2506_12035_b200 import binding
     D = H * dh
     cfg, blocks, m = model_for("bf16", D, H, 128, S, B)
@@ -976,29 +979,53 @@ def test_linear_of_a_handful_of_rows(dtype, M, N, K):
 @pytest.mark.parametrize("D,H,F,B,n", [(256, 4, 1024, 1, 1), (768, 12, 3072, 2, 8), (768, 12, 3072, 3, 9), (1024, 16, 4096, 1, 15), (1280, 16, 2560, 2, 7),
                                        (2048, 32, 2048, 1, 16)])
 def test_few_rows_normalise_in_the_projection(operand, D, H, F, B, n):
-    """A step on up to 32 rows whose projections normalise their rows, against the same step with LayerNorm launches (which a
-    measurement hook asks for): rows with a mean of ten deviations.  The two statistics differ by fp32 rounding, so what
-    differs are single 16-bit roundings of the operands (2^-11 and 2^-8 of a value) on a part of the values."""
+    """A step on up to 32 rows whose projections normalise their rows (a mean of ten deviations; gamma 0.5 to 2, beta of unit size):
+    what the blocks add to the active rows, and the active tokens' K and V behind a normalising projection, against the oracle,
+    against the same step with LayerNorm launches (which a measurement hook asks for), and with the K/V write-back in a launch of
+    its own.  Operands are rounded by 2^-11 or 2^-8 of a value, q, k, v by 2^-8: the limits leave a factor of three for what three
+    blocks add up.  The oracle without one of the four parameter arrays is more than five limits away."""
     import synth
     from helpers import make_model
     cfg = synth.CONFIGS["mar_b"].replace(L=3, E=0, D=D, H=H, F=F, B=B, S=40, n_buffer=8)
-    m = make_model(cfg, synth.make_weights(cfg), operand=operand)
     rng = np.random.default_rng(D + n)
-    hidden = dev((rng.standard_normal((B, cfg.S, D)) + 10.0 * rng.standard_normal((B, cfg.S, 1))).astype(np.float32))
-    act = idx_dev(np.stack([rng.permutation(cfg.S)[:n] for _ in range(B)]))
+    blocks = synth.make_weights(cfg)
+    for blk in blocks:
+        for g, b in (("ln1_g", "ln1_b"), ("ln2_g", "ln2_b")):
+            blk[g], blk[b] = rng.uniform(0.5, 2.0, D).astype(np.float32), rng.standard_normal(D).astype(np.float32)
+    m = make_model(cfg, blocks, operand=operand)
+    hidden = (rng.standard_normal((B, cfg.S, D)) + 10.0 * rng.standard_normal((B, cfg.S, 1))).astype(np.float32)
+    act = np.stack([rng.permutation(cfg.S)[:n] for _ in range(B)]).astype(np.int32)
+
+    def of_active_rows(out, K, V):                                       # [L][B][S][D] K and V; block 0 has its LayerNorm launch
+        return (np.stack([out[b, act[b]] - hidden[b, act[b]] for b in range(B)]),
+                np.stack([np.stack([K[1:, b][:, act[b]], V[1:, b][:, act[b]]]) for b in range(B)]))
+
+    def oracle(step_blocks):
+        oc, out = orc.KVCache(cfg.L, B, cfg.S, D), np.zeros((B, cfg.S, D))
+        kw = dict(n_heads=H, score_layer=cfg.score_layer, ln_eps=cfg.ln_eps)
+        orc.full_step(blocks, hidden, oc, act, None, 0.0, out, **kw)
+        orc.marche_step(step_blocks, hidden, oc, act, act, None, 0.0, out, **kw)
+        return of_active_rows(out, oc.K, oc.V)
+
+    want, limit = oracle(blocks), 1e-2 if operand == "f16" else 2e-2
+    for name, neutral, part in (("ln1_g", 1.0, 1), ("ln1_b", 0.0, 1), ("ln2_g", 1.0, 0), ("ln2_b", 0.0, 0)):
+        left_out = oracle([blk if l == 0 and part else {**blk, name: np.full(D, neutral)} for l, blk in enumerate(blocks)])
+        assert rel_l2(left_out[part], want[part]) > 5 * limit
     got = []
-    for hook in ((), ("gather_layernorm",)):
+    for hook, fuse in (((), 1), (("gather_layernorm",), 1), ((), 0)):
         m.debug_repeat_classes(hook)
+        m.set_tuning(fuse_qkv_scatter=fuse)
         cache, out, ws = m.alloc_cache(), torch.zeros(B, cfg.S, D, device="cuda"), m.alloc_workspace(cfg.S)
         m.init_cache(cache)
-        m.full_step(hidden, cache, act, None, 0.0, out, None, ws)
+        m.full_step(dev(hidden), cache, idx_dev(act), None, 0.0, out, None, ws)
         before = m.launch_count()
-        m.step(hidden, cache, act, act, None, 0.0, out, None, ws)
-        got.append((host(out), host(cache), m.launch_count() - before))
+        m.step(dev(hidden), cache, idx_dev(act), idx_dev(act), None, 0.0, out, None, ws)
+        got.append((*of_active_rows(host(out), host(cache[:, 0]), host(cache[:, 1])), m.launch_count() - before))
+        assert all(rel_l2(g, w) <= limit for g, w in zip(got[-1], want)), [rel_l2(g, w) for g, w in zip(got[-1], want)]
     m.debug_repeat_classes(())
     assert got[1][2] - got[0][2] == 2 * cfg.L + 2 * cfg.L - 1              # all but the first are gone, and the hook doubles them
-    rel = 2e-4 if operand == "f16" else 1.6e-3
-    assert rel_l2(got[0][0], got[1][0]) <= rel and rel_l2(got[0][1], got[1][1]) <= 8 * rel
+    assert got[2][2] - got[0][2] == cfg.L                                  # the write-back's launches
+    assert np.array_equal(got[2][0], got[0][0]) and np.array_equal(got[2][1], got[0][1])
     assert m.device_status() == 0
 
 

@@ -130,9 +130,9 @@ typedef struct {
 /* Creates the host-side context for one model shape on the current device.
  * `blocks` is a host array of cfg->n_blocks structs (copied).  Synchronous; no
  * device memory is allocated.  MARCHE_ESHAPE for unsupported dimensions, MARCHE_EINVAL for a
- * NULL or misaligned parameter array.  Weight matrices and biases must be complete in memory
- * before any call that uses them is enqueued (the projection kernels start fetching weight tiles
- * before they wait for the preceding kernel of the stream). */
+ * NULL or misaligned parameter array.  Weight matrices, biases and LayerNorm parameters must be complete
+ * in memory before any call that uses them is enqueued (the kernels start fetching them before they wait
+ * for the preceding kernel of the stream). */
 int marche_create(const marche_config* cfg, const marche_block_weights* blocks, marche_ctx** out);
 void marche_destroy(marche_ctx* ctx);
 
@@ -443,7 +443,7 @@ int marche_attention_two_segment(marche_ctx* ctx, const void* qkv, int ld, int n
 enum { MARCHE_ATTENTION_AUTO = 0, MARCHE_ATTENTION_MMA = 1, MARCHE_ATTENTION_TCGEN05 = 2,
        MARCHE_ATTENTION_TCGEN05_TWO_PASS = 3 /* the two-pass tcgen05 kernel also where no scores are taken */ };
 enum { MARCHE_GEMM_AUTO = 0, MARCHE_GEMM_SINGLE = 1 /* split-K: one CTA, or a cluster that shares K, per tile */,
-       MARCHE_GEMM_PAIR = 2 /* CTA pairs on 256-row tiles */ };
+       MARCHE_GEMM_PAIR = 2 /* CTA pairs on 256-row tiles */ };   /* (AUTO alone reaches the mma.sync kernel) */
 typedef struct {
   int32_t stream_k;              /* 1: fc2-sized residual projections use stream-K with ordered reduce-adds   */
   int32_t fuse_qkv_scatter;      /* 1: the QKV projection's epilogue writes K, V into the cache (no K5 launch)*/
@@ -453,7 +453,9 @@ typedef struct {
                                     where long sequences or head_dim 80 make them faster; at head_dim 80 up to
                                     four thirds of it not with one item per SM or fewer                        */
   int32_t two_segment_attention; /* 1: the step uses marche_attention_two_segment instead of K5 + K3           */
-  int32_t gemm_kernel;           /* MARCHE_GEMM_*: AUTO = the kernel with the shorter estimated time           */
+  int32_t gemm_kernel;           /* MARCHE_GEMM_*: AUTO = up to 32 rows, by size, the mma.sync kernel, which also
+                                    normalises the rows of QKV and fc1; else the one with the shorter estimated
+                                    time of the other two                                                      */
   int32_t tail_split;            /* 0 off, 1 cost model, 2 / 4 forced: column slices in a partial last round   */
   int32_t tile_n;                /* CTA-pair kernel: 0 = tile width by estimated time, 128 = narrow tiles      */
   int32_t pdl;                   /* 1: programmatic dependent launch along the kernel chain (process-wide)     */
@@ -503,7 +505,9 @@ int marche_debug_skip_classes(marche_ctx* ctx, unsigned class_mask);
  * arguments).  (time with the class doubled) - (time of the normal step) is the class's cost in the real
  * chain under the clocks and power the real chain runs at, which leaving a class out does not preserve
  * on a power-capped GPU.  Doubling is harmless for the values except that the two residual projections
- * add their result twice; use it for timing only.  Same classes, same errors. */
+ * add their result twice; use it for timing only.  On up to 32 rows, where the projections normalise their rows
+ * themselves, naming MARCHE_KC_GATHER_LN here or above brings the LayerNorm launches back: a step with one launch of them
+ * (marche_tuning.gemm_kernel = MARCHE_GEMM_SINGLE) is what to compare with.  Same classes, same errors. */
 int marche_debug_repeat_classes(marche_ctx* ctx, unsigned class_mask);
 void marche_clear_device_status(marche_ctx* ctx);
 

@@ -6,7 +6,7 @@
 //   K3 attention over the whole cache (+ score partials at the scoring block, in the same
 //   kernel or in one of their own before it) -> K2 output projection (+residual) -> K1
 //   LayerNorm -> K2 fc1 (+GELU) -> K2 fc2 (+residual);
-// on up to 32 rows the projections after a LayerNorm do it themselves (K1 remains at block 0);
+// on a handful of rows (gemm_few_wins) the projections after a LayerNorm do it themselves (K1 remains at block 0);
 // then once per step the fp32 row scatter into hidden_out and K4 (score reduction +
 // top-K).  Nothing here allocates device memory or synchronises, except where the
 // header says a call is synchronous.
@@ -181,7 +181,7 @@ bool use_pair(const marche_ctx* ctx, int M, int N, int K) {
   return gemm_splitk_cost(M, N, K, gemm_splitk_pick(M, N, K)) > (wide < narrow ? wide : narrow);
 }
 
-// A handful of rows: the mma.sync kernel (use_pair is not asked then).
+// A handful of rows: the mma.sync kernel, whatever use_pair says (which says no for so few).
 bool use_few(const marche_ctx* ctx, int M, int N, int K, bool norm = false) {
   return ctx->bf16 && ctx->tune.gemm_kernel == MARCHE_GEMM_AUTO && gemm_few_wins(M, N, K, norm);
 }
@@ -257,7 +257,7 @@ int do_attention(marche_ctx* ctx, const void* q, int ld_q, int n, const void* ca
   for (int rep_i = 0; rep_i < launches_of(ctx, MARCHE_KC_ATTENTION); ++rep_i) {
   if (n > 0) mark(ctx, MARCHE_KC_ATTENTION, st);
   // The plain attention has four tensor-core kernels; which one runs is a matter of query rows, keys, head_dim and items, by
-  // rules that stand beside the kernels with both sides measured:
+  // rules that stand beside the kernels with both sides measured (where they are no longer the faster choice, that stands there, too):
   //   few items (or few key tiles)      all tiles in flight, split over a cluster and over warps (attention_split_wins)
   //   more than 48 rows, or nearly so   tcgen05 streams, up to four per SM (attention_tc_stream_wins)
   //   32 rows or fewer                  the persistent mma.sync launch (31 vs 34 us at n = 8, 32 vs 36 us at n = 24..32, S 320)

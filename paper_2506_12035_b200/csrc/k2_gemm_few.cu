@@ -1,4 +1,4 @@
-// K2 for a handful of rows (16, or 32 where that fits the chip): out = epilogue(a * w^T + bias), with the LayerNorm of the rows (K1)
+// K2 for a handful of rows (up to 16, or 32, by size: gemm_few_wins): out = epilogue(a * w^T + bias), with the LayerNorm of the rows (K1)
 // in the same launch where the caller has the fp32 rows.
 //
 // What bounds it: latency.  One image without refresh has 4 to 26 active rows; a launch is a chain of hand-over, first operands,
@@ -15,8 +15,9 @@
 //     other CTAs, and the LayerNorm launch before it is gone;
 //   * partial sums meet in the CTA's shared memory, then in the CTA that owns the pair of columns, both in a fixed order; what
 //     crosses the cluster goes by st.async, whose bytes the receiver's barrier counts (no fence, no barrier of the cluster).
-// A block of a step (7 launches before, 5 now), us: width 768, 4 rows 22.9 -> 16.7, 16 rows 22.8 -> 17.3, 32 rows 23.9 -> 21.7; width 1024,
-// 16 rows 25.6 -> 19.7; width 1280, 16 rows 30.1 -> 26.0.  All waits are bounded.
+// A block of a step (six blocks over 320 tokens; 7 launches with the split-K kernel, 5 with this one), us: width 768, 4 rows 24.9 and 18.8,
+// 16 rows 24.6 and 19.6, 32 rows 24.9 and 22.8; width 1024, 16 rows 27.9 and 23.2; width 1280, 16 rows 31.2 and 27.9.  Waits on barriers
+// of shared memory are bounded; those on the cluster's barrier return once every CTA has arrived or left, which none of them delays.
 #include "common.cuh"
 #include "kernels.h"
 #include "launch_pdl.h"
@@ -355,8 +356,9 @@ gemm_few_kernel(const void* __restrict__ a, int lda, int M, const uint16_t* __re
 struct Plan { int nt, cs, warps, kbw, n_m, ctas; size_t smem; };
 
 // Columns per CTA and CTAs per cluster.  With the LayerNorm every warp has one K block, so that the slice of K is at most 512 columns, and
-// as many columns as the registers hold, since every CTA reads and normalises the rows anew (16 rows, a block of a step, us: 8 NT = 64
-// columns and pairs of CTAs 17.3, 48 columns 17.1, 32 columns 17.9, clusters of four 17.6; width 1024 19.7, 20.6, 21.3 and 21.5).
+// as many columns as the registers hold, since every CTA reads and normalises the rows anew (16 rows, a block of a step of 24 blocks, us, as the
+// kernel was when the plan was chosen: 8 NT = 64 columns and pairs of CTAs 17.3, 48 columns 17.1, 32 columns 17.9, clusters of four 17.6;
+// width 1024 19.7, 20.6, 21.3 and 21.5).
 // Without it 16 columns: whole K up to 2048 (17.2 us; pairs 17.1, of 32 columns 17.1), then pairs (17.1; whole K 18.6, of 32
 // columns 17.4; width 1024 19.7 and 21.8), with two groups of rows pairs of 32 columns (21.8 -> 21.2).
 bool make_plan(int M, int N, int K, bool norm, Plan* p) {

@@ -345,11 +345,13 @@ bool attention_split_plan(int n, int S, int dh, int items, int* cs, int* nk) {
   // CTAs do better.  64 rows, S 320, eight blocks of a step: 64 items 342 us on pairs, 315 on one, mma.sync kernel 320; 32 items
   // 295 either way; 16 items on four CTAs 6.4 us against 6.7 back to back.)
   if (dh == 80 && nq == 4 && n_kv <= 5 && 2 * c * items > device_sm_count()) c = 1;
-  // Two or three groups of query rows over four or five tiles: a single CTA whose groups of warps take a tile each, where there are
-  // enough items that pairs of CTAs would be the alternative (a block of a step, us, five tiles: 43 rows, 32 items 30.8 -> 29.8, 48 items
-  // 30.3 -> 29.0; 20 rows, 64 items 32.1 -> 29.6, 72 items 30.4 -> 28.9; head_dim 80, 32 items 37.9 -> 35.7, 20 rows, 64 items 35.8 -> 34.5;
-  // with fewer items clusters of four do better: 43 rows, 24 items 26.6 and 27.2).  At head_dim 80 three groups from 49 items on stay on
-  // pairs of CTAs.
+  // Two or three groups of query rows over four or five tiles: a single CTA whose groups of warps take a tile each, in place of clusters of
+  // four (up to a quarter of the SMs in items) and of two.  A block of a step, us, clusters and single CTAs: five tiles, 43 rows: 32 items
+  // (of four) 33.5 and 32.1, 48 items (of two) 34.4 and 33.7, 72 items 34.3 and 33.6, 20 rows, 64 items 32.8 and 30.5; four tiles, 43 rows:
+  // 32 items 31.9 and 31.3, 48 items 30.7 and 29.1, 72 items 33.7 and 32.6; head_dim 80, 43 rows, 32 items: five tiles 39.2 and 36.7, four
+  // 37.4 and 36.0.  (Back to back, without the launches around it, four tiles of 32 items are slower: 4.0 and 4.2, head_dim 80 4.7 and 5.2.)
+  // With fewer items clusters of four do better (43 rows, 24 items 26.6 and 27.2); 25 to 31 were not measured.  At head_dim 80 three groups
+  // from 49 items on stay on pairs of CTAs.
   if ((nq == 2 || nq == 3) && (n_kv == 4 || n_kv == 5) && items > 28 && 2 * items <= device_sm_count() && !(dh == 80 && nq == 3 && items > 48)) {
     *cs = 1;
     *nk = n_kv;
@@ -358,8 +360,9 @@ bool attention_split_plan(int n, int S, int dh, int items, int* cs, int* nk) {
   while (c < 8 && (n_kv + c - 1) / c > (dh == 64 ? 10 : 8)) c *= 2;
   const int tiles = (n_kv + c - 1) / c;
   if (tiles > kMaxTiles || tiles * stage > 160 * 1024) return false;
-  // Warps beyond the query groups: free where the merge over the cluster happens anyway; in a single CTA they pay for one
-  // group (S 320, 5 rows: 4.5 -> 3.1 us) and two groups of queries with four tiles or more, not for three (4.8 -> 5.3).
+  // Warps beyond the query groups: free where the merge over the cluster happens anyway; in a single CTA, with the queries by loads and the
+  // merge in a loop, they pay for one group (S 320, 5 rows: 4.5 -> 3.1 us) and two groups of queries with four tiles or more, not for
+  // three (4.8 -> 5.3).
   int k = 1;
   if (nq == 1) k = tiles < 5 ? tiles : 5;
   else if ((c > 1 && tiles > 1) || (nq == 2 && tiles > 3)) k = 2;

@@ -4,7 +4,7 @@
 //
 // Persistent CTAs (one per SM).  The work of a CTA is a list of units, one unit = one 128-row query
 // tile of one (sample, head) item against all S keys; three independent streams inside the CTA (one where a CTA has a single unit,
-// four where that saves a round) take the units in turn.  A unit is a latency chain (Q K^T -> read logits -> exponentials -> write
+// four where that saves rounds that count, see attention_tc_streams) take the units in turn.  A unit is a latency chain (Q K^T -> read logits -> exponentials -> write
 // weights -> P V), and the exponentials - 16 per clock and SM - are the scarce resource once the active set
 // is large; the chains in flight per SM partition keep those units busy while each waits on its hand-overs.
 // Each stream owns a query buffer, TMA rings of 64-key tiles (three of K, two of V: a K tile is used up a step earlier)
@@ -16,7 +16,7 @@
 // without, 128 x 16 items, S 320, us: 320 rows 107 and 122, 128 rows 42.5 and 50.5, 60 rows 36 and 40; 64 x 16 items, S 1088: 151
 // rows 98 and 104, 1088 rows 528 and 590; one stream, with and without: S 1088, 144 items, 116 rows 17.1 and 19.5, S 2048, 64
 // items, 200 rows 28.2 and 33.0.
-// Roles, for three streams (18 warps of 112 registers a thread; numbers for four in brackets):
+// Roles, for three streams (18 warps of 96 registers a thread, 112 would fit; for four, in brackets, 24 of 80):
 //   warps 0-11    [0-15] softmax: warps 4j .. 4j+3 serve stream j, one thread per query row.  A thread pulls its
 //                 S row into registers (tcgen05.ld; without columns for P_j the first half again for its exponentials, since 80
 //                 registers do not hold a row and its weights) and writes the weights to tensor memory
@@ -563,11 +563,14 @@ cudaError_t launch_stream(const void* q, int ld_q, int B, int n, int S, int H, c
 
 }  // namespace
 
-// Against the mma.sync kernels (us), which take 48 rows or fewer (min_rows, marche_tuning) with up to five CTAs per SM and
-// drop to two from 49 rows: S 320, head_dim 64: 60 rows 42 and 58, 77 rows 47 and 110, 320 rows 125 and 303; head_dim 80: 60
-// rows 46 and 98, 320 rows 134 and 350.  33 to 48 rows: over long sequences at head_dim 64 (S 1088, 41 rows: 57 and 62; S 320:
-// 41 and 42, nothing in a whole step); at head_dim 80 over five key tiles or more (S 320: 45 and 49), unless the last
-// round of units leaves the streams (three per SM) idle: 576 items on 444 streams 19 and 16, 1024 items 29 either way.
+// Against the mma.sync kernels (alone, us, 2048 items over 320 keys), which take 48 rows or fewer (min_rows, marche_tuning) with up to
+// five CTAs per SM and drop to two from 49 rows: head_dim 64: 60 rows 37 and 56, 77 rows 42 and 109, 320 rows 107 and 307; head_dim 80: 60
+// rows 47 and 99, 320 rows 133 and 352.  33 to 48 rows at head_dim 64: over long sequences (S 1088, 1024 items, 41 rows: 56 and 62).  Over
+// shorter ones the line dates from four streams whose weights shared the logits' columns (41 and 42, nothing in a step); the streams of today are
+// faster there, too, from about 700 items on: S 320, 41 rows, 2048 items 36.5 and 40.9, 1024 items 22.3 and 24.0, 512 items 13.4 and 13.5,
+// and a block of a step: width 1024, 128 samples 199 and 205, 64 samples 116 and 117, 32 samples 74.0 and 73.6; width 768, 64 samples 78.5 and
+// 82.4.  At head_dim 80 over five key tiles or more (S 320, 2048 items, 41 rows: 46 and 52), unless the last round of units leaves the streams
+// (three per SM) idle: 512 items on 444 streams 18.2 and 15.3, 1024 items 27.1 and 27.9.
 // One item per SM or fewer at head_dim 80, 49 to 64 rows: the mma.sync kernel's four warps take an item faster than a stream that
 // nothing overlaps with (S 1088, 128 items, 60 rows, back to back 18.1 and 20.5, eight blocks of a step 465 and 503; 41 rows, on three
 // warps, 530 and 481).  At head_dim 64 the one-stream CTAs are slower back to back (S 1088, 128 items, 41 rows 18.6 and 17.8, 64 rows

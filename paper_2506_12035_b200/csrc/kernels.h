@@ -99,7 +99,7 @@ cudaError_t launch_gemm_splitk(const void* a, int lda, int M, const void* w, con
                                void* out, bool a_bf16, int* status, cudaStream_t st, SplitKShape shape,
                                const KvScatter* kv_scatter = nullptr);
 
-// K2 for up to 32 rows on mma.sync.  Same operand rules.  gamma (and beta) given: a is fp32 [M][lda] and its rows are normalised
+// K2 for up to 32 rows on mma.sync, where gemm_few_wins.  Same operand rules.  gamma (and beta) given: a is fp32 [M][lda] and its rows are normalised
 // first (epilogues 0, 2 and 4).  Weights, bias, gamma and beta are read ahead of the dependency wait: they were complete before the
 // preceding launch.  (The scatter's token indices, which kernels write, are read behind it.)
 bool gemm_few_wins(int M, int N, int K, bool norm);

@@ -163,7 +163,7 @@ MARCHE_DEVINL float ex2_approx(float x) {
 // items, 300 rows 62 and 55; S 320, 512 items, 230 rows 25.4 and 24.1; level with many.)  Stream j of a CTA takes k = j, j + NS, ...
 // An item's last tile can be much shorter than the others, and no CTA or stream should get the short ones only, or none: where
 // there is more than one turn, a CTA's place in the row of CTAs moves on by `rotate` with every k and by `rotate_turn` with
-// every turn of its streams (chosen by the launch so that the tile number changes along both).
+// every turn of its streams (attention_tc_rotation chooses them so that the tile number changes along both).
 struct Deal {
   int units, grid, rotate, rotate_turn;
   template <int NS> MARCHE_DEVINL int place(int k) const {
